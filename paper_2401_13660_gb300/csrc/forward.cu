@@ -1,0 +1,490 @@
+// Forward scan of the selective-scan layer core (MambaByte Section 2,
+// "Implementation: parallel scans"; Eq. 2-3; Table 6 output and gating):
+// prefill, and the training forward, which also keeps the state before every
+// chunk. (Verify and the fused Delta projection: prefill.cu.)
+//
+// Work decomposition. Every (batch row, channel) is an independent recurrence
+// over L with a 16-float state (A is diagonal). A CTA of four warps owns 32
+// channels of one batch row for its span of L; a warp 8 channels, four lanes
+// per channel, each with 4 states in registers. Chunks of 16 steps come through
+// a ring of TMA tiles (bounded waits); iteration i scans chunk i and converts
+// chunk i + 1.
+//
+// What bounds it: per (step, channel) 16 decays on the SFU and 64 multiply-adds,
+// which leave the SM at about 0.6 instructions per scheduler and clock, because
+// packed and scalar fp32 operations with three register operands take more
+// than their pipe's cycles (a register-only loop of just these instructions
+// runs at 0.57-0.61), and the shared-memory pipe, which every operand passes.
+// The layout therefore spends as few instructions and shared-memory wavefronts
+// as it can on everything else:
+//  * Pairs of adjacent steps, not of states, fill the packed operations:
+//    Delta_t, Delta_t+1 and (Delta x)_t, (Delta x)_t+1 of a channel lie in one
+//    16-byte slot, B and C are widened to fp32 in pairs (t, t + 1), so decay
+//    exponents, B Delta x and the sum C.h need no copies that duplicate a
+//    scalar and no add across a pair; only the recurrence itself is scalar.
+//    (Pairs of states: 35.3 instructions per lane and step; this: 29.6.)
+//  * A 128-bit shared load takes 2 wavefronts instead of 4 if lanes that differ
+//    in lane bit 0 (or in bit 1) read the same address. Lane bit 0 is a channel
+//    bit and bit 1 a state bit (channel bits 0, 2, 3; state bits 1, 4), so that
+//    both B, C (by state) and Delta (by channel) are read at that rate.
+//  * The four lanes' shares of C.h are added through a warp's own tile instead
+//    of shuffles and selects; the lane that adds them is the one that converts
+//    those channels and steps, so that D x and silu(z) stay in its registers.
+//  * Nothing is stored to shared memory between the loads of a chunk's scan:
+//    the shares and the converted chunk i + 1 wait in registers, so that the
+//    compiler may move every load ahead.
+//  * Token tiles are swizzled by TMA: a warp reads 16-byte columns of them.
+//
+// Measured (B x L x D, bf16; before: pairs of states, shuffles): 8 x 8192 x 2048
+// 850 -> 764 us, 4 x 8192 x 3584 708 -> 592 us, 1 x 8192 x 2048 (time split) 176
+// -> 152 us, fp32 3 x 1003 x 1544 56 -> 48 us. Two channels per lane (B and C
+// loaded once for both: 17 % fewer wavefronts) measured 758 / 750 us on the
+// first two: half the warps; two-warp CTAs (16 channels) 784 / 640 us.
+#include <stddef.h>
+#include <string.h>
+
+#include <atomic>
+
+#include "common.cuh"
+#include "tma.cuh"
+
+namespace mbscan {
+namespace {
+
+constexpr int kT = 16;        // steps per chunk
+constexpr int kTP = kT / 2;   // step pairs per chunk
+constexpr int kWarps = 4;
+constexpr int kThreads = 32 * kWarps;
+constexpr int kWCh = 8;                     // channels per warp
+constexpr int kCh = kWarps * kWCh;          // channels per CTA
+constexpr int kPairs = kWCh / 2;            // channel pairs per warp
+constexpr int kPartQ = kTP * kPairs + 4;    // float4s between the shares of two lanes q (the pad keeps them on other banks)
+
+template <typename T>
+constexpr int kStages = sizeof(T) == 2 ? 4 : 3;
+
+template <typename T>
+struct Raw {   // TMA destinations; token tiles swizzled in their 64- (bf16) or 128-byte (fp32) rows
+    T dt[kT][kCh];
+    T x[kT][kCh];
+    T z[kT][kCh];
+    T B[kT][kDState];
+    T C[kT][kDState];
+};
+
+template <typename T>
+struct alignas(1024) Smem {
+    Raw<T> raw[kStages<T>];
+    T ys[2][kT][kCh];                              // output tiles (TMA stores), swizzled like the inputs
+    float4 dg[2][kWarps][kTP][kWCh];   // (Delta_t, Delta_t+1, (Delta x)_t, (Delta x)_t+1), see dg_slot
+    float4 bc[2][2][2][kTP][4];                    // [buffer][B, C][states 4q, 4q+1 or 4q+2, 4q+3][tp][q]
+    float4 part[kWarps][4 * kPartQ];   // shares of C.h of lane q: [q][tp][channel pair]
+    uint64_t full[kStages<T>];
+};
+
+struct FwdArgs {
+    CUtensorMap tm_dt, tm_x, tm_z, tm_B, tm_C, tm_y;
+    ScanParams p;
+    int has_gate;
+    int grid_segs;   // segments of L covered by the grid (blockIdx = (b, segment, channel tile))
+};
+
+// Slot of channel c of a warp at step pair tp in its dg tile. A lane stores channels 2 pp and 2 pp + 1 one after
+// the other, eight lanes (four pp, two tp) at a time: the two halves change places on odd tp, so that these eight
+// 16-byte stores fall on different banks. The scan's loads of all 8 channels at one tp cover 128 bytes either way.
+__device__ __forceinline__ int dg_slot(int tp, int c) { return (((c ^ tp) & 1) << 2) | (c >> 1); }
+
+// Byte offset of channels c, c + 1 of the CTA at step t in a swizzled token tile
+template <typename T>
+__device__ __forceinline__ int tile_off(int t, int c) {
+    constexpr int kRow = kCh * (int)sizeof(T);
+    const int by = c * (int)sizeof(T), x = kRow == 128 ? t & 7 : (t >> 1) & 3;
+    return t * kRow + (((by >> 4) ^ x) << 4) + (by & 15);
+}
+
+template <typename T>
+__device__ __forceinline__ float2 ld2(const void *base, int off) {
+    if constexpr (sizeof(T) == 2) {
+        const unsigned u = *reinterpret_cast<const unsigned *>(static_cast<const char *>(base) + off);
+        return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
+    } else {
+        return *reinterpret_cast<const float2 *>(static_cast<const char *>(base) + off);
+    }
+}
+template <typename T>
+__device__ __forceinline__ void st2(void *base, int off, float2 v) {
+    if constexpr (sizeof(T) == 2) {
+        const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
+        *reinterpret_cast<__nv_bfloat162 *>(static_cast<char *>(base) + off) = b;
+    } else {
+        *reinterpret_cast<float2 *>(static_cast<char *>(base) + off) = v;
+    }
+}
+
+template <typename T, bool kSummary>
+__device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int stage, int chunk, int d0, int b) {
+    constexpr uint32_t tok = kT * kCh * sizeof(T), bc = kT * kDState * sizeof(T);
+    const uint32_t bytes = ((a.has_gate ? 3 : 2) * tok) + (kSummary ? 1 : 2) * bc;
+    uint64_t *bar = &s.full[stage];
+    mbar_arrive_expect_tx(bar, bytes);
+    const int t = chunk * kT;
+    Raw<T> &r = s.raw[stage];
+    tma_load_3d(&r.dt[0][0], &a.tm_dt, bar, d0, t, b);
+    tma_load_3d(&r.x[0][0], &a.tm_x, bar, d0, t, b);
+    if (a.has_gate) tma_load_3d(&r.z[0][0], &a.tm_z, bar, d0, t, b);
+    tma_load_3d(&r.B[0][0], &a.tm_B, bar, 0, t, b);
+    if (!kSummary) tma_load_3d(&r.C[0][0], &a.tm_C, bar, 0, t, b);
+}
+
+__device__ __forceinline__ float rcp(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// Delta = softplus(v) of a pair, as softplus() of common.cuh
+__device__ __forceinline__ float2 softplus2(float2 v) {
+    const float2 w = mul2(v, make_float2(kLog2e, kLog2e));
+    const float2 u = make_float2(ex2(w.x), ex2(w.y));
+    float2 r = fma2(u, make_float2(0.33333334f, 0.33333334f), make_float2(-0.5f, -0.5f));
+    r = mul2(u, fma2(u, r, make_float2(1.f, 1.f)));
+    const float2 o = add2(u, make_float2(1.f, 1.f));
+    const float2 lw = mul2(make_float2(lg2(o.x), lg2(o.y)), make_float2(kLn2, kLn2));
+    r.x = u.x < 0.03125f ? r.x : lw.x;
+    r.y = u.y < 0.03125f ? r.y : lw.y;
+    return make_float2(v.x > 15.f ? v.x : r.x, v.y > 15.f ? v.y : r.y);
+}
+
+// silu(z) of a pair
+__device__ __forceinline__ float2 silu2(float2 z) {
+    const float2 w = mul2(z, make_float2(-kLog2e, -kLog2e));
+    const float2 d = add2(make_float2(ex2(w.x), ex2(w.y)), make_float2(1.f, 1.f));
+    return mul2(z, make_float2(rcp(d.x), rcp(d.y)));
+}
+
+// kCkpt (training forward): also stores the state before every chunk.
+// kSummary (first pass of a time-split span): scans each segment but the last
+// from a zero state (segment 0: from h0) and records its end state and the
+// product of its decays, 2^(A log2 e * sum of Delta); no outputs. In the second
+// pass (the plain kernel) segment s starts from those, folded with the
+// associative operator of Section 2: h <- P_s' * h + H_s'.
+template <typename T, bool kCkpt, bool kSummary>
+__global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_constant__ FwdArgs a) {
+    using S = Smem<T>;
+    using R = Raw<T>;
+    constexpr int STAGES = kStages<T>, kRowB = kCh * (int)sizeof(T);
+    static_assert(sizeof(R) % (8 * kRowB) == 0 && offsetof(R, x) % (8 * kRowB) == 0 &&
+                      offsetof(R, z) % (8 * kRowB) == 0 && offsetof(R, B) % 128 == 0 && offsetof(R, C) % 128 == 0 &&
+                      offsetof(S, ys) % (8 * kRowB) == 0 && sizeof(T) * kT * kCh % (8 * kRowB) == 0,
+                  "swizzled TMA tiles start on their pattern's boundary");
+    extern __shared__ unsigned char smem_dyn[];
+    S &s = *reinterpret_cast<S *>(smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u));
+    const ScanParams &p = a.p;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int64_t D = p.d_inner;
+    // blockIdx.x = (batch row, segment of L, channel tile), channel tile fastest
+    const int ntd = (int)((D + kCh - 1) / kCh);
+    const int L = (int)p.seqlen;
+    const int nchunks = (L + kT - 1) / kT;   // chunks of the whole span
+    const int seg = (int)((blockIdx.x / ntd) % a.grid_segs);
+    const int b = (int)(blockIdx.x / ntd / a.grid_segs);
+    const int nseg = p.nseg > 1 ? (int)p.nseg : 1;
+    const int cps = (nchunks + nseg - 1) / nseg;                        // chunks per segment
+    const int c0 = seg * cps, nch = min(nchunks - c0, cps);             // this CTA's: c0 .. c0 + nch - 1
+    const int d0 = (int)(blockIdx.x % ntd) * kCh;
+    const bool gate = a.has_gate != 0;
+
+    if (tid == 0) {
+        for (int st = 0; st < STAGES; ++st) mbar_init(&s.full[st], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    pdl_wait();   // everything below reads or writes global memory
+    if (tid == 0)
+        for (int st = 0; st < STAGES && st < nch; ++st) issue_chunk<T, kSummary>(s, a, st, c0 + st, d0, b);
+
+    // ---- conversion and output role: channels 8 warp + 2 pp + {0, 1} of the tile, steps 2 tp, 2 tp + 1
+    const int pp = lane % kPairs, tp = lane / kPairs;
+    const int off0 = tile_off<T>(2 * tp, kWCh * warp + 2 * pp), off1 = tile_off<T>(2 * tp + 1, kWCh * warp + 2 * pp);
+    float2 bias = make_float2(0.f, 0.f), dsk = make_float2(0.f, 0.f);
+    {
+        const int64_t dc = (int64_t)d0 + kWCh * warp + 2 * pp;   // D % 8 == 0: both channels valid or neither
+        if (dc < D) {
+            if (p.dt_bias) bias = __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc));
+            if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
+        }
+    }
+    // widening role: two states of B or C at a step pair (s.bc in the order of the threads)
+    const int bc_off = ((2 * ((tid >> 2) & 7)) * kDState + 4 * (tid & 3) + 2 * ((tid >> 5) & 1)) * (int)sizeof(T);
+    const bool bc_is_c = tid >= 64;
+
+    // ---- scan role: channel c of the warp, states 4 q .. 4 q + 3 (the lane order of the file comment)
+    const int c = (lane & 1) | ((lane >> 1) & 6), q = ((lane >> 1) & 1) | ((lane >> 4) << 1);
+    const int64_t d = (int64_t)d0 + kWCh * warp + c;
+    const bool chan_ok = d < D;
+    float h[4], a2[4];
+    float2 dsum = make_float2(0.f, 0.f);   // kSummary: sum of Delta over even and odd steps
+    {
+        float4 av = make_float4(0.f, 0.f, 0.f, 0.f), hv = av;
+        if (chan_ok) {
+            av = ldg4(p.A + d * kDState + 4 * q);
+            if (seg == 0 && p.h0) hv = ldg4(p.h0 + ((int64_t)b * D + d) * kDState + 4 * q);
+            if constexpr (!kSummary) {
+                for (int sp = 0; sp < seg; ++sp) {
+                    const int64_t o = (((int64_t)b * nseg + sp) * D + d) * kDState + 4 * q;
+                    const float4 he = *reinterpret_cast<const float4 *>(p.seg_h + o);
+                    const float4 pe = *reinterpret_cast<const float4 *>(p.seg_p + o);
+                    hv = sp == 0 ? he : make_float4(fmaf(pe.x, hv.x, he.x), fmaf(pe.y, hv.y, he.y),
+                                                    fmaf(pe.z, hv.z, he.z), fmaf(pe.w, hv.w, he.w));
+                }
+            }
+        }
+        a2[0] = av.x * kLog2e; a2[1] = av.y * kLog2e; a2[2] = av.z * kLog2e; a2[3] = av.w * kLog2e;
+        h[0] = hv.x; h[1] = hv.y; h[2] = hv.z; h[3] = hv.w;
+    }
+    const int slot_e = dg_slot(0, c), slot_o = dg_slot(1, c);
+
+    struct Conv {
+        float4 c0, c1, bc;
+    };
+    auto convert = [&](const R &r, int t0) {
+        const float2 x0 = ld2<T>(&r.x[0][0], off0), x1 = ld2<T>(&r.x[0][0], off1);
+        float2 D0 = softplus2(add2(ld2<T>(&r.dt[0][0], off0), bias));
+        float2 D1 = softplus2(add2(ld2<T>(&r.dt[0][0], off1), bias));
+        const int rest = L - t0 - 2 * tp;   // steps left from this pair on
+        const float m0 = rest < 1 ? 0.f : 1.f, m1 = rest < 2 ? 0.f : 1.f;
+        D0 = mul2(D0, make_float2(m0, m0));   // Delta = 0 past the end leaves h unchanged
+        D1 = mul2(D1, make_float2(m1, m1));
+        const float2 g0 = mul2(D0, x0), g1 = mul2(D1, x1);
+        Conv v;
+        v.c0 = make_float4(D0.x, D1.x, g0.x, g1.x);
+        v.c1 = make_float4(D0.y, D1.y, g0.y, g1.y);
+        const T *src = !kSummary && bc_is_c ? &r.C[0][0] : &r.B[0][0];
+        const float2 v0 = ld2<T>(src, bc_off), v1 = ld2<T>(src, bc_off + kDState * (int)sizeof(T));
+        v.bc = make_float4(v0.x, v1.x, v0.y, v1.y);
+        return v;
+    };
+    auto put = [&](int buf, const Conv &v) {
+        s.dg[buf][warp][tp][dg_slot(tp, 2 * pp)] = v.c0;
+        s.dg[buf][warp][tp][dg_slot(tp, 2 * pp + 1)] = v.c1;
+        (&s.bc[buf][0][0][0][0])[tid] = v.bc;
+    };
+
+    // ---- prologue: chunk 0
+    bool ok = mbar_wait(&s.full[0], 0);   // nch >= 1
+    if (ok) put(0, convert(s.raw[0], c0 * kT));
+    if (__syncthreads_or(ok ? 0 : 1)) {
+        if (tid == 0) {
+            report(p.status, 4 /* MB_ERR_TIMEOUT */, 0);
+            for (int j = 0; j < STAGES && j < nch; ++j) mbar_wait(&s.full[j], 0);
+        }
+        return;
+    }
+
+    int st = 0;        // ring stage of chunk i
+    uint32_t ph = 0;   // and its phase parity
+    for (int i = 0; i < nch; ++i) {
+        const int t0 = (c0 + i) * kT;
+        // (1) chunk i + 1: wait for its tiles and convert them (stored after the scan below)
+        const int nst = st + 1 == STAGES ? 0 : st + 1;
+        const uint32_t nph = st + 1 == STAGES ? ph ^ 1u : ph;
+        ok = i + 1 < nch ? mbar_wait(&s.full[nst], nph) : true;
+        const Conv nv = convert(s.raw[nst], t0 + kT);   // past the last chunk: of no use, and not read
+        // (2) chunk i: D x and silu(z) of this lane's outputs
+        const R &r = s.raw[st];
+        float2 xd0, xd1, sz0 = make_float2(1.f, 1.f), sz1 = sz0;
+        if constexpr (!kSummary) {
+            xd0 = mul2(dsk, ld2<T>(&r.x[0][0], off0));
+            xd1 = mul2(dsk, ld2<T>(&r.x[0][0], off1));
+            if (gate) {
+                sz0 = silu2(ld2<T>(&r.z[0][0], off0));
+                sz1 = silu2(ld2<T>(&r.z[0][0], off1));
+            }
+        }
+        if constexpr (kCkpt) {   // state before chunk i, for the backward's recompute
+            static_assert(kT == kCkptSteps, "checkpoints are taken per chunk");
+            if (chan_ok)
+                *reinterpret_cast<float4 *>(p.h_ckpt + (((int64_t)b * nchunks + c0 + i) * D + d) * kDState + 4 * q) =
+                    make_float4(h[0], h[1], h[2], h[3]);
+        }
+        // (3) chunk i: decays, recurrence, shares of C.h, a step pair at a time
+        const float4(&dgw)[kTP][kWCh] = s.dg[i & 1][warp];
+        const float4(&bcw)[2][2][kTP][4] = s.bc[i & 1];
+        float2 part[kTP], csum;
+#pragma unroll
+        for (int k = 0; k < kTP; ++k) {
+            const float4 v = dgw[k][(k & 1) ? slot_o : slot_e];
+            const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
+            const float4 b01 = bcw[0][0][k][q], b23 = bcw[0][1][k][q];
+            const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w), make_float2(b23.x, b23.y),
+                                  make_float2(b23.z, b23.w)};
+            float2 hp[4];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                const float2 e = mul2(dd, make_float2(a2[n], a2[n]));
+                const float2 ab = make_float2(ex2(e.x), ex2(e.y));
+                const float2 bg = mul2(bp[n], gg);
+                hp[n].x = fmaf(ab.x, h[n], bg.x);
+                hp[n].y = fmaf(ab.y, hp[n].x, bg.y);
+                h[n] = hp[n].y;
+            }
+            if constexpr (kSummary) {
+                csum = k == 0 ? dd : add2(csum, dd);
+            } else {
+                const float4 c01 = bcw[1][0][k][q], c23 = bcw[1][1][k][q];
+                part[k] = mul2(make_float2(c01.x, c01.y), hp[0]);
+                part[k] = fma2(make_float2(c01.z, c01.w), hp[1], part[k]);
+                part[k] = fma2(make_float2(c23.x, c23.y), hp[2], part[k]);
+                part[k] = fma2(make_float2(c23.z, c23.w), hp[3], part[k]);
+            }
+        }
+        if constexpr (kSummary) dsum = add2(dsum, csum);
+        put((i + 1) & 1, nv);
+        // (4) chunk i: add the four lanes' shares of each channel, skip term, gate
+        if constexpr (!kSummary) {
+            float4 *pw = s.part[warp];
+#pragma unroll
+            for (int k = 0; k < kTP; ++k) reinterpret_cast<float2 *>(pw + q * kPartQ + k * kPairs)[c] = part[k];
+            __syncwarp();
+            const float4 *src = pw + tp * kPairs + pp;   // (channel, step): (0, 0), (0, 1), (1, 0), (1, 1)
+            const float4 s0 = src[0], s1 = src[kPartQ], s2 = src[2 * kPartQ], s3 = src[3 * kPartQ];
+            const float2 ca = add2(add2(make_float2(s0.x, s0.y), make_float2(s1.x, s1.y)),
+                                   add2(make_float2(s2.x, s2.y), make_float2(s3.x, s3.y)));
+            const float2 cb = add2(add2(make_float2(s0.z, s0.w), make_float2(s1.z, s1.w)),
+                                   add2(make_float2(s2.z, s2.w), make_float2(s3.z, s3.w)));
+            st2<T>(&s.ys[i & 1][0][0], off0, mul2(add2(make_float2(ca.x, cb.x), xd0), sz0));
+            st2<T>(&s.ys[i & 1][0][0], off1, mul2(add2(make_float2(ca.y, cb.y), xd1), sz1));
+            fence_proxy_async_smem();   // y tile -> visible to the TMA store below
+            if (tid == 0) bulk_wait_read_all();   // the store of chunk i - 1 no longer reads its tile
+        }
+        if (__syncthreads_or(ok ? 0 : 1)) {
+            if (tid == 0) {
+                report(p.status, 4 /* MB_ERR_TIMEOUT */, c0 + i + 1);
+                for (int j = i + 1; j < i + STAGES && j < nch; ++j)
+                    mbar_wait(&s.full[j % STAGES], (uint32_t)((j / STAGES) & 1));
+                bulk_wait_all();
+            }
+            return;
+        }
+        if (tid == 0) {
+            if constexpr (!kSummary) {
+                tma_store_3d(&a.tm_y, &s.ys[i & 1][0][0], d0, t0, b);
+                bulk_commit();
+            }
+            if (i + STAGES < nch) {   // stage st is free: refill it with chunk i + STAGES
+                fence_proxy_async_smem();
+                issue_chunk<T, kSummary>(s, a, st, c0 + i + STAGES, d0, b);
+            }
+        }
+        st = nst;
+        ph = nph;
+    }
+    if (tid == 0) bulk_wait_all();
+
+    if (!chan_ok) return;
+    if constexpr (kSummary) {
+        const int64_t o = (((int64_t)b * nseg + seg) * D + d) * kDState + 4 * q;
+        const float sd = dsum.x + dsum.y;
+        *reinterpret_cast<float4 *>(p.seg_h + o) = make_float4(h[0], h[1], h[2], h[3]);
+        *reinterpret_cast<float4 *>(p.seg_p + o) =
+            make_float4(ex2(a2[0] * sd), ex2(a2[1] * sd), ex2(a2[2] * sd), ex2(a2[3] * sd));
+    } else if (p.h_out && seg == nseg - 1) {   // the span's last state
+        *reinterpret_cast<float4 *>(p.h_out + ((int64_t)b * D + d) * kDState + 4 * q) =
+            make_float4(h[0], h[1], h[2], h[3]);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Host side: tensor maps and the launch.
+
+// [batch, L, inner] tensor with a (box_inner x kT x 1) box; rows (b, t) are
+// `row` elements apart (row >= inner).
+bool make_map(CUtensorMap *m, const void *base, int es, int64_t batch, int64_t L, int64_t inner, int box_inner,
+              int64_t row, int swizzle) {
+    const uint64_t dims[3] = {(uint64_t)inner, (uint64_t)L, (uint64_t)batch};
+    const uint64_t strides[2] = {(uint64_t)(row * es), (uint64_t)(L * row * es)};
+    const uint32_t box[3] = {(uint32_t)box_inner, (uint32_t)kT, 1};
+    return encode_tmap(m, base, es, 3, dims, strides, box, swizzle);
+}
+
+template <typename T, bool kCkpt>
+cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
+    constexpr int es = sizeof(T), sw = kCh * es;   // one token row of a tile
+    FwdArgs a;
+    memset(&a, 0, sizeof(a));
+    a.p = p;
+    a.has_gate = p.z != nullptr;
+    if (p.nseg < 2 || !p.seg_h || !p.seg_p) a.p.nseg = 1;
+    const int64_t nseg = a.p.nseg, D = p.d_inner;
+    auto tok = [&](CUtensorMap *m, const void *base) {
+        return make_map(m, base, es, p.batch, p.seqlen, D, kCh, D, sw);
+    };
+    if (!tok(&a.tm_dt, p.dt) || !tok(&a.tm_x, p.x) || (p.z && !tok(&a.tm_z, p.z)) || !tok(&a.tm_y, p.y) ||
+        !make_map(&a.tm_B, p.B, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0) ||
+        !make_map(&a.tm_C, p.C, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0))
+        return cudaErrorInvalidValue;
+    const size_t smem = sizeof(Smem<T>) + 1024;
+    const int64_t ctas = ((D + kCh - 1) / kCh) * p.batch;   // per segment of L
+    cudaError_t e;
+    if (nseg > 1) {   // first pass: summaries of segments 0 .. nseg-2
+        FwdArgs a1 = a;
+        a1.has_gate = 0;   // no outputs: the gate is not read
+        a1.grid_segs = (int)(nseg - 1);
+        auto k1 = forward_kernel<T, false, true>;
+        if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+            return e;
+        if ((e = launch_pdl(false, k1, dim3((unsigned)(ctas * (nseg - 1))), dim3(kThreads), smem, s, a1)) !=
+            cudaSuccess)
+            return e;
+    }
+    a.grid_segs = (int)nseg;
+    auto k = forward_kernel<T, kCkpt, false>;
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(false, k, dim3((unsigned)(ctas * nseg)), dim3(kThreads), smem, s, a);
+}
+
+}  // namespace
+
+// Time split: only when the batch rows and channel tiles give at most one CTA
+// per SM (a CTA alone on an SM leaves most of its issue slots idle); then into
+// as many segments as fill the resident slots (4 per SM),
+// each at least kMinSegChunks chunks long. The summary pass repeats most of a
+// scan, so at 1.7 CTAs per SM (batch 4 x 2048 channels) the split measured
+// slower (604 -> 653 us) while batch 1 x 2048 channels x 8192 steps went
+// 480 -> 180 us (both before the layout above, which took the latter to 152).
+constexpr int64_t kMinSegChunks = 8;
+
+int64_t prefill_segments(const ScanParams &p) {
+    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen <= 0 || p.dt_low) return 1;
+    constexpr int kMaxDevices = 64;
+    static std::atomic<int> sm_count[kMaxDevices];   // per device, filled on first use (0: not yet)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 1;
+    int sms = sm_count[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 1;
+        sm_count[dev].store(sms, std::memory_order_relaxed);   // every writer stores the same value
+    }
+    const int64_t slots = (int64_t)sms * 4;
+    const int64_t ctas = p.batch * ((p.d_inner + kCh - 1) / kCh);
+    if (ctas > sms) return 1;
+    const int64_t nchunks = (p.seqlen + kT - 1) / kT;
+    int64_t nseg = slots / ctas;
+    if (nseg > nchunks / kMinSegChunks) nseg = nchunks / kMinSegChunks;
+    if (nseg < 2) return 1;
+    const int64_t cps = (nchunks + nseg - 1) / nseg;
+    return (nchunks + cps - 1) / cps;   // no empty segment
+}
+
+size_t prefill_split_bytes(const ScanParams &p, int64_t nseg) {
+    return nseg > 1 ? (size_t)(2 * p.batch * nseg * p.d_inner * kDState) * sizeof(float) : 0;
+}
+
+cudaError_t launch_forward(const ScanParams &p, bool bf16, cudaStream_t s) {
+    if (p.h_ckpt)
+        return bf16 ? launch_typed<__nv_bfloat16, true>(p, s) : launch_typed<float, true>(p, s);
+    return bf16 ? launch_typed<__nv_bfloat16, false>(p, s) : launch_typed<float, false>(p, s);
+}
+
+}  // namespace mbscan

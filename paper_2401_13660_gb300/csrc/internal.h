@@ -66,10 +66,12 @@ constexpr long long kMaxWaitCycles = 4000000000LL;   // the kernels' wait limit 
 // Bounded-wait diagnostic (selftest.cu): a wait that runs out after `limit` clocks.
 cudaError_t launch_wait_timeout(StatusBlock *sb, long long limit, cudaStream_t s);
 cudaError_t launch_prefill(const ScanParams &p, bool bf16, cudaStream_t s);
+// The forward scan given dt (forward.cu); with p.h_ckpt also the checkpoints. All sizes > 0.
+cudaError_t launch_forward(const ScanParams &p, bool bf16, cudaStream_t s);
 // Segments a prefill of these sizes is split into when the workspace has room
 // (1 when the batch rows and channels alone fill the GPU), and the scratch
 // bytes that split needs beyond the status block.
-int64_t prefill_segments(const ScanParams &p, bool bf16);
+int64_t prefill_segments(const ScanParams &p);
 size_t prefill_split_bytes(const ScanParams &p, int64_t nseg);
 cudaError_t launch_verify(const ScanParams &p, bool bf16, cudaStream_t s);
 // Prefill that also writes p.h_ckpt [batch, ceil(L / kCkptSteps), d_inner, 16].

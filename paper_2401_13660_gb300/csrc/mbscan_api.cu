@@ -140,11 +140,10 @@ mb_status check_ws(const mb_scan_args *a, void *ws, size_t ws_bytes) {
 // Long spans with few channels are split over L when the workspace holds the
 // segment summaries (after the status block); else they run unsplit.
 mb_status setup_split(const mb_scan_args *args, ScanParams &p, const float *h_last, void *ws, size_t ws_bytes) {
-    const bool bf16 = args->dtype == MB_BF16;
-    const int64_t nseg = mbscan::prefill_segments(p, bf16);
+    const int64_t nseg = mbscan::prefill_segments(p);
     const size_t split = mbscan::prefill_split_bytes(p, nseg);
     if (nseg < 2 || ws_bytes < mbscan::kStatusBytes + split) return MB_OK;
-    const int64_t es = bf16 ? 2 : 4;
+    const int64_t es = args->dtype == MB_BF16 ? 2 : 4;
     const int64_t tok = args->batch * args->seqlen * args->d_inner * es;
     const int64_t sbytes = args->batch * args->d_inner * args->d_state * 4;
     const Range rs = range_of(static_cast<char *>(ws) + mbscan::kStatusBytes, (int64_t)split);
@@ -193,8 +192,7 @@ extern "C" {
 size_t mb_workspace_size(const mb_scan_args *args) {
     if (check_args(args, false, false) != MB_OK) return 0;
     const ScanParams p = to_params(args, nullptr, nullptr);
-    const bool bf16 = args->dtype == MB_BF16;
-    return mbscan::kStatusBytes + mbscan::prefill_split_bytes(p, mbscan::prefill_segments(p, bf16));
+    return mbscan::kStatusBytes + mbscan::prefill_split_bytes(p, mbscan::prefill_segments(p));
 }
 
 mb_status mb_scan_prefill(const mb_scan_args *args, float *h_last, void *ws, size_t ws_bytes,

@@ -1,15 +1,14 @@
-// Prefill scan of the selective-scan layer core (MambaByte Section 2,
-// "Implementation: parallel scans"; Eq. 2-3; Table 6 output and gating), and
-// the speculative-decoding verify scan (Algorithm 1), which is the same scan
-// that also streams every per-position state to h_all.
+// The speculative-decoding verify scan of the selective-scan layer core
+// (Algorithm 1: every per-position state is streamed to h_all), and, in the
+// same kernel, prefill and verify with the fused Delta projection (Eq. 3).
+// Prefill given dt and the training forward: forward.cu.
 //
 // Work decomposition. Every (batch row, channel) pair is an independent
 // linear recurrence over L steps with a 16-float state (A is diagonal, so the
 // scan of Section 2 is element-wise). The kernel is channel-parallel and runs
 // each channel's recurrence sequentially in time, the evaluation order with
 // the fewest operations (one Abar, one FMA for h and one FMA for C.h per state
-// and step); the associative operator of Section 2 is only needed to split a
-// span, which the h0 / h_last interface does across calls.
+// and step).
 //
 // A CTA of kWarps warps owns CH = 32 kWarps / LPC channels of one batch row
 // for the whole span (small CTAs spread the channels evenly over the SMs).
@@ -23,13 +22,12 @@
 //    waits, tma.cuh);
 //  * the CTA converts a chunk once per (t, channel) into fp32 in shared
 //    memory: (Delta, Delta*x) with Delta = softplus(dt + bias), (D*x, silu z);
-//    a bf16 prefill also widens the chunk's B and C rows to fp32 once, so
+//    a fused prefill also widens the chunk's B and C rows to fp32 once, so
 //    that the scan does not convert them again in every lane;
 //  * each lane scans the chunk: Abar = 2^(Delta * A*log2 e) on the SFU for all
 //    kT steps, then h = Abar*h + B*(Delta*x) and its share of C.h in packed
 //    f32x2 arithmetic, reading B and C (four states each) from those fp32
-//    rows, or, in verify and for fp32 inputs, straight from the TMA tile in
-//    the input dtype; groups of LPC steps are reduced across the LPC
+//    rows, or, in verify, straight from the TMA tile in the input dtype; groups of LPC steps are reduced across the LPC
 //    lanes of a channel with log2(LPC) shuffle rounds, each lane finishing one
 //    output y = (C.h + D*x) * silu(z), which goes to a shared-memory tile that
 //    one thread writes out with a TMA store.
@@ -48,7 +46,6 @@
 #include <stddef.h>
 #include <string.h>
 
-#include <atomic>
 
 #include "common.cuh"
 #include "tma.cuh"
@@ -106,7 +103,7 @@ struct Conv {
     float2 xs[kT][CH];          // (D*x, silu(z)); silu(z) = 1 without a gate
 };
 
-// B and C rows widened to fp32 once per chunk (bf16 prefill): the scan then
+// B and C rows widened to fp32 once per chunk (fused prefill): the scan then
 // reads four states of each with one shared load and no per-lane conversion.
 // Verify spans are a single chunk, where the extra pass only lengthens the
 // critical path; they read the bf16 tiles directly.
@@ -138,7 +135,6 @@ struct PrefillArgs {
     ScanParams p;
     int has_gate;
     int nbox;      // ceil(dt_rank / kRankTile)
-    int grid_segs; // segments of L covered by the grid (blockIdx = (b, segment, channel tile))
 };
 
 // Shared-memory layout of the fused Delta projection, after the Smem struct:
@@ -305,12 +301,7 @@ __device__ __forceinline__ float reduce_steps(const float (&part)[LPC], int q) {
     }
 }
 
-// kSummary (first pass of a time-split prefill): scan each segment of L from a
-// zero state and record its end state and the product of its decays in the
-// scratch (no outputs). The second pass is the plain kernel: its segment s
-// starts from the state the summaries of segments 0 .. s-1 give (folded with
-// the associative operator of Section 2: h <- P_s' * h + H_s').
-template <typename T, int LPC, int STAGES, bool kStoreAll, bool kCkpt, bool kFuse, bool kSummary = false>
+template <typename T, int LPC, int STAGES, bool kStoreAll, bool kFuse>
 __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED_MINB : MB_VERIFY_MINB) : 1)
     prefill_kernel(const __grid_constant__ PrefillArgs a) {
     using G = Geom<LPC>;
@@ -341,22 +332,10 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
     const ScanParams &p = a.p;
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
-    // blockIdx.x = (batch row, segment of L, channel tile), channel tile fastest;
-    // only the plain prefill is ever split over L
-    constexpr bool kSplit = !kStoreAll && !kFuse;
-    const int ntd = (int)((p.d_inner + CH - 1) / CH);
+    const int ntd = (int)((p.d_inner + CH - 1) / CH);   // blockIdx.x = (batch row, channel tile), tile fastest
+    const int b = (int)(blockIdx.x / ntd);
     const int64_t L = p.seqlen, D = p.d_inner;
-    const int64_t nchunks = (L + kT - 1) / kT;   // chunks of the whole span
-    int seg = 0, b = (int)(blockIdx.x / ntd);
-    int64_t nseg = 1, c0 = 0, nch = nchunks;    // this CTA's chunks: c0 .. c0 + nch - 1
-    if constexpr (kSplit) {
-        seg = (int)((blockIdx.x / ntd) % a.grid_segs);
-        b = (int)(blockIdx.x / ntd / a.grid_segs);
-        nseg = p.nseg > 1 ? p.nseg : 1;
-        const int64_t cps = (nchunks + nseg - 1) / nseg;   // chunks per segment
-        c0 = seg * cps;
-        nch = nchunks - c0 < cps ? nchunks - c0 : cps;
-    }
+    const int64_t nch = (L + kT - 1) / kT;   // chunks
     const int d0 = (blockIdx.x % ntd) * CH;
     const bool gate = a.has_gate != 0;
 
@@ -382,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
             // the CTA's W_dt slice rides on chunk 0's barrier (its bytes are
             // part of that arrival's expected count)
             const bool wslice = kFuse && st == 0;
-            issue_chunk(s, a, st, c0 + st, d0, b, fz, wslice ? (uint32_t)a.nbox * FuseLayout<CH>::kWBox : 0u);
+            issue_chunk(s, a, st, st, d0, b, fz, wslice ? (uint32_t)a.nbox * FuseLayout<CH>::kWBox : 0u);
             if (wslice)
                 for (int bx = 0; bx < a.nbox; ++bx)
                     tma_load_2d(fz + (uint32_t)(STAGES * a.nbox) * kDtlBox + (uint32_t)bx * FuseLayout<CH>::kWBox,
@@ -425,21 +404,9 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
         for (int k = 0; k < G::kPairs; ++k) {
             const float2 av = __ldg(Ap + k);
             a2[k] = make_float2(av.x * kLog2e, av.y * kLog2e);
-            if (hp && !kSummary) h[k] = __ldg(hp + k);   // a summary starts from zero
-        }
-        if constexpr (kSplit && !kSummary) {   // segment s > 0 of a split span: fold the summaries before it
-            for (int sp = 0; sp < seg; ++sp) {
-                const int64_t off = (((int64_t)b * nseg + sp) * D + d) * kDState + G::kSPL * q;
-                const float2 *hs_ = reinterpret_cast<const float2 *>(p.seg_h + off);
-                const float2 *ps_ = reinterpret_cast<const float2 *>(p.seg_p + off);
-#pragma unroll
-                for (int k = 0; k < G::kPairs; ++k) h[k] = fma2(ps_[k], h[k], hs_[k]);
-            }
+            if (hp) h[k] = __ldg(hp + k);
         }
     }
-    float2 prod[G::kPairs];   // kSummary: product of the segment's decays
-#pragma unroll
-    for (int k = 0; k < G::kPairs; ++k) prod[k] = make_float2(1.f, 1.f);
 
     // ---- prologue: chunk 0
     bool ok = nch > 0 ? mbar_wait(&s.full[0], 0) : true;
@@ -449,7 +416,7 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
         if constexpr (kFuse) f.dtl = fz_addr + (uint32_t)(st * a.nbox) * kDtlBox;
         return f;
     };
-    if (ok && nch > 0) convert(s.cv[0], s.wbc[0], s.raw[0], cr, c0 * kT, L, gate, stage_fx(0));
+    if (ok && nch > 0) convert(s.cv[0], s.wbc[0], s.raw[0], cr, 0, L, gate, stage_fx(0));
     if (__syncthreads_or(ok ? 0 : 1)) {
         if (tid == 0) {
             report(p.status, 4 /* MB_ERR_TIMEOUT */, 0);
@@ -458,8 +425,8 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
         return;
     }
 
-    for (int64_t i = 0; i < nch; ++i) {   // i: chunk c0 + i of the span, ring slot i % STAGES
-        const int64_t t0 = (c0 + i) * kT;
+    for (int64_t i = 0; i < nch; ++i) {   // ring slot i % STAGES
+        const int64_t t0 = i * kT;
         const bool has_next = i + 1 < nch;
         // (1) chunk i+1: wait for its tiles and convert them
         const int nst = (int)((i + 1) % STAGES);
@@ -469,16 +436,6 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
             convert(s.cv[(i + 1) & 1], s.wbc[(i + 1) & 1], s.raw[nst], cr, t0 + kT, L, gate, stage_fx(nst));
 
         // (2) chunk i: decays of all kT steps, recurrence, shares of C.h
-        if constexpr (kCkpt) {   // state before chunk i, for the backward's recompute
-            static_assert(kT == kCkptSteps, "checkpoints are taken per chunk");
-            if (chan_ok) {
-                float2 *dst = reinterpret_cast<float2 *>(
-                    p.h_ckpt + (((int64_t)b * nchunks + c0 + i) * D + d) * kDState + G::kSPL * q);
-#pragma unroll
-                for (int k = 0; k < G::kPairs; k += 2)
-                    *reinterpret_cast<float4 *>(dst + k) = make_float4(h[k].x, h[k].y, h[k + 1].x, h[k + 1].y);
-            }
-        }
         const Conv<CH> &cv = s.cv[i & 1];
         const Raw<T, CH, kFuse> &rs = s.raw[i % STAGES];   // without kWide: B, C straight from the TMA tile
         const WideBC<kWide> &wb = s.wbc[i & 1];
@@ -517,13 +474,10 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
 #pragma unroll
             for (int k = 0; k < G::kPairs; ++k) {
                 h[k] = fma2(ab[t][k], h[k], mul2(bp[k], gg));
-                if constexpr (kSummary) prod[k] = mul2(prod[k], ab[t][k]);
-                else acc[k & 1] = k < 2 ? mul2(cp[k], h[k]) : fma2(cp[k], h[k], acc[k & 1]);
+                acc[k & 1] = k < 2 ? mul2(cp[k], h[k]) : fma2(cp[k], h[k], acc[k & 1]);
             }
-            if constexpr (!kSummary) {
-                const float2 sum = add2(acc[0], acc[1]);
-                part[t] = sum.x + sum.y;
-            }
+            const float2 sum = add2(acc[0], acc[1]);
+            part[t] = sum.x + sum.y;
             if constexpr (kStoreAll) {
                 if (chan_ok && t0 + t < L) {
                     float2 *dst = reinterpret_cast<float2 *>(
@@ -538,7 +492,7 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
         // (3) chunk i: reduce across the lanes of each channel, gate, stage y
         T(&ys)[kT][CH] = s.ys[i & 1];
 #pragma unroll
-        for (int m = 0; m < (kSummary ? 0 : kT / LPC); ++m) {
+        for (int m = 0; m < kT / LPC; ++m) {
             float grp[LPC];
 #pragma unroll
             for (int u = 0; u < LPC; ++u) grp[u] = part[LPC * m + u];
@@ -551,7 +505,7 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
         if (tid == 0) bulk_wait_read_all();   // the store of chunk i-1 no longer reads its tile
         if (__syncthreads_or(ok ? 0 : 1)) {
             if (tid == 0) {
-                report(p.status, 4 /* MB_ERR_TIMEOUT */, c0 + i + 1);
+                report(p.status, 4 /* MB_ERR_TIMEOUT */, i + 1);
                 for (int64_t j = i + 1; j < i + STAGES && j < nch; ++j)
                     mbar_wait(&s.full[j % STAGES], (uint32_t)((j / STAGES) & 1));
                 bulk_wait_all();
@@ -559,29 +513,19 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
             return;
         }
         if (tid == 0) {
-            if constexpr (!kSummary) {
-                tma_store_3d(&a.tm_y, &ys[0][0], d0, (int)t0, b);
-                bulk_commit();
-            }
+            tma_store_3d(&a.tm_y, &ys[0][0], d0, (int)t0, b);
+            bulk_commit();
             // stage i % STAGES (chunk i: converted last iteration, scanned
             // now) is free: refill it with chunk i + STAGES
             if (i + STAGES < nch) {
                 fence_proxy_async_smem();
-                issue_chunk(s, a, (int)(i % STAGES), c0 + i + STAGES, d0, b, fz);
+                issue_chunk(s, a, (int)(i % STAGES), i + STAGES, d0, b, fz);
             }
         }
     }
     if (tid == 0) bulk_wait_all();
 
-    if constexpr (kSummary) {   // this segment's end state from a zero start, and its decay product
-        if (chan_ok) {
-            const int64_t off = (((int64_t)b * nseg + seg) * D + d) * kDState + G::kSPL * q;
-            float2 *hd = reinterpret_cast<float2 *>(p.seg_h + off);
-            float2 *pd = reinterpret_cast<float2 *>(p.seg_p + off);
-#pragma unroll
-            for (int k = 0; k < G::kPairs; ++k) { hd[k] = h[k]; pd[k] = prod[k]; }
-        }
-    } else if (!kStoreAll && p.h_out && chan_ok && seg == nseg - 1) {   // the span's last state
+    if (!kStoreAll && p.h_out && chan_ok) {   // the span's last state
         float2 *hp = reinterpret_cast<float2 *>(p.h_out + ((int64_t)b * D + d) * kDState + G::kSPL * q);
 #pragma unroll
         for (int k = 0; k < G::kPairs; ++k) hp[k] = h[k];
@@ -603,7 +547,7 @@ bool make_map(CUtensorMap *m, const void *base, bool bf16, int64_t batch, int64_
     return encode_tmap(m, base, (int)es, 3, dims, strides, box);
 }
 
-template <typename T, int LPC, int STAGES, bool kStoreAll, bool kCkpt = false, bool kFuse = false>
+template <typename T, int LPC, int STAGES, bool kStoreAll, bool kFuse>
 cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     constexpr int kCh = Geom<LPC>::kCh;
     const bool bf16 = sizeof(T) == 2;
@@ -611,9 +555,6 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     memset(&a, 0, sizeof(a));
     a.p = p;
     a.has_gate = p.z != nullptr;
-    constexpr bool kSplittable = !kStoreAll && !kFuse;
-    if (!kSplittable || p.nseg < 2 || !p.seg_h || !p.seg_p) a.p.nseg = 1;
-    const int64_t nseg = a.p.nseg;
     size_t fuse_bytes = 0;
     if constexpr (kFuse) {
         // dt_low [batch, L, r] (rows dt_low_stride apart) and W_dt [D, r], both
@@ -639,65 +580,14 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
         !make_map(&a.tm_y, p.y, bf16, p.batch, p.seqlen, p.d_inner, kCh))
         return cudaErrorInvalidValue;
     const size_t smem = sizeof(Smem<T, kCh, STAGES, kFuse, kWideBC<T, kStoreAll>>) + 128 + fuse_bytes;
-    const int64_t ctas = ((p.d_inner + kCh - 1) / kCh) * p.batch;   // per segment of L
-    cudaError_t e;
-    if constexpr (kSplittable) {
-        if (nseg > 1) {   // first pass: summaries of segments 0 .. nseg-2
-            PrefillArgs a1 = a;
-            a1.has_gate = 0;   // no outputs: the gate is not read
-            a1.grid_segs = (int)(nseg - 1);
-            auto k1 = prefill_kernel<T, LPC, STAGES, false, false, false, true>;
-            if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
-                return e;
-            if ((e = launch_pdl(false, k1, dim3((unsigned)(ctas * (nseg - 1))), dim3(kThreads), smem, s, a1)) !=
-                cudaSuccess)
-                return e;
-        }
-    }
-    a.grid_segs = (int)nseg;
-    auto k = prefill_kernel<T, LPC, STAGES, kStoreAll, kCkpt, kFuse>;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const int64_t ctas = ((p.d_inner + kCh - 1) / kCh) * p.batch;
+    auto k = prefill_kernel<T, LPC, STAGES, kStoreAll, kFuse>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(false, k, dim3((unsigned)(ctas * nseg)), dim3(kThreads), smem, s, a);
+    return launch_pdl(false, k, dim3((unsigned)ctas), dim3(kThreads), smem, s, a);
 }
 
 }  // namespace
-
-// Time split: only when the batch rows and channel tiles give at most one CTA
-// per SM (a CTA alone on an SM leaves most of its issue slots idle); then into
-// as many segments as fill the resident slots (4 per SM for bf16, 3 for fp32),
-// each at least kMinSegChunks chunks long. The summary pass repeats most of a
-// scan, so at 1.7 CTAs per SM (batch 4 x 2048 channels) the split measured
-// slower (604 -> 653 us) while batch 1 x 2048 channels x 8192 steps went
-// 480 -> 180 us.
-constexpr int64_t kMinSegChunks = 8;
-
-int64_t prefill_segments(const ScanParams &p, bool bf16) {
-    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen <= 0 || p.dt_low) return 1;
-    constexpr int kMaxDevices = 64;
-    static std::atomic<int> sm_count[kMaxDevices];   // per device, filled on first use (0: not yet)
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 1;
-    int sms = sm_count[dev].load(std::memory_order_relaxed);
-    if (sms == 0) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 1;
-        sm_count[dev].store(sms, std::memory_order_relaxed);   // every writer stores the same value
-    }
-    constexpr int kCh = Geom<kPrefillLanesPerChannel>::kCh;
-    const int64_t slots = (int64_t)sms * (bf16 ? 4 : 3);
-    const int64_t ctas = p.batch * ((p.d_inner + kCh - 1) / kCh);
-    if (ctas > sms) return 1;
-    const int64_t nchunks = (p.seqlen + kT - 1) / kT;
-    int64_t nseg = slots / ctas;
-    if (nseg > nchunks / kMinSegChunks) nseg = nchunks / kMinSegChunks;
-    if (nseg < 2) return 1;
-    const int64_t cps = (nchunks + nseg - 1) / nseg;
-    return (nchunks + cps - 1) / cps;   // no empty segment
-}
-
-size_t prefill_split_bytes(const ScanParams &p, int64_t nseg) {
-    return nseg > 1 ? (size_t)(2 * p.batch * nseg * p.d_inner * kDState) * sizeof(float) : 0;
-}
 
 cudaError_t launch_prefill(const ScanParams &p, bool bf16, cudaStream_t s) {
     if (p.batch == 0 || p.d_inner == 0) return cudaSuccess;
@@ -714,18 +604,15 @@ cudaError_t launch_prefill(const ScanParams &p, bool bf16, cudaStream_t s) {
     constexpr int LPC = kPrefillLanesPerChannel;
     if (p.dt_low)   // fused Delta projection (bf16 only; the API checks)
         return !bf16 ? cudaErrorInvalidValue
-               : p.dt_rank <= kRankTile ? launch_typed<__nv_bfloat16, LPC, kPrefillStages, false, false, true>(p, s)
-                                        : launch_typed<__nv_bfloat16, LPC, kPrefillStagesWide, false, false, true>(p, s);
-    return bf16 ? launch_typed<__nv_bfloat16, LPC, kPrefillStages, false>(p, s)
-                : launch_typed<float, LPC, kPrefillStages, false>(p, s);
+               : p.dt_rank <= kRankTile ? launch_typed<__nv_bfloat16, LPC, kPrefillStages, false, true>(p, s)
+                                        : launch_typed<__nv_bfloat16, LPC, kPrefillStagesWide, false, true>(p, s);
+    return launch_forward(p, bf16, s);
 }
 
 cudaError_t launch_prefill_ckpt(const ScanParams &p, bool bf16, cudaStream_t s) {
     if (p.batch == 0 || p.d_inner == 0) return cudaSuccess;
     if (p.seqlen == 0) return launch_prefill(p, bf16, s);   // no chunks: no checkpoints
-    constexpr int LPC = kPrefillLanesPerChannel;
-    return bf16 ? launch_typed<__nv_bfloat16, LPC, kPrefillStages, false, true>(p, s)
-                : launch_typed<float, LPC, kPrefillStages, false, true>(p, s);
+    return launch_forward(p, bf16, s);
 }
 
 cudaError_t launch_verify(const ScanParams &p, bool bf16, cudaStream_t s) {
@@ -733,14 +620,14 @@ cudaError_t launch_verify(const ScanParams &p, bool bf16, cudaStream_t s) {
     constexpr int LPC = kPrefillLanesPerChannel;
     if (p.dt_low) {   // fused Delta projection (bf16 only; the API checks)
         if (!bf16) return cudaErrorInvalidValue;
-        return p.seqlen <= kT ? launch_typed<__nv_bfloat16, LPC, 1, true, false, true>(p, s)
-                              : launch_typed<__nv_bfloat16, LPC, kVerifyStages, true, false, true>(p, s);
+        return p.seqlen <= kT ? launch_typed<__nv_bfloat16, LPC, 1, true, true>(p, s)
+                              : launch_typed<__nv_bfloat16, LPC, kVerifyStages, true, true>(p, s);
     }
     if (p.seqlen <= kT)   // one chunk: a single ring stage suffices (smaller CTAs, more resident)
-        return bf16 ? launch_typed<__nv_bfloat16, LPC, 1, true>(p, s)
-                    : launch_typed<float, LPC, 1, true>(p, s);
-    return bf16 ? launch_typed<__nv_bfloat16, LPC, kVerifyStages, true>(p, s)
-                : launch_typed<float, LPC, kVerifyStages, true>(p, s);
+        return bf16 ? launch_typed<__nv_bfloat16, LPC, 1, true, false>(p, s)
+                    : launch_typed<float, LPC, 1, true, false>(p, s);
+    return bf16 ? launch_typed<__nv_bfloat16, LPC, kVerifyStages, true, false>(p, s)
+                : launch_typed<float, LPC, kVerifyStages, true, false>(p, s);
 }
 
 }  // namespace mbscan
