@@ -11,53 +11,67 @@
 //   g *= Abar;  ddt = dDelta * sigmoid(dt + bias);  dbias += ddt;  dD += dy x
 // and dh0 = g at the end.
 //
-// Work decomposition (the lane geometry of the forward kernel): a CTA of 4
-// warps owns 32 channels of one batch row; lane = 8 q + c8 keeps the 4 states
-// 4q .. 4q+3 of channel warp*8 + c8. Chunks of kCkptSteps steps are taken in
-// reverse order through a ring of 3-D TMA tile loads (dt, x, z, dout, B, C).
-// Per chunk:
-//  * conversion (once per (t, channel pair)): Delta, Delta*x and dy into
-//    shared memory; for bf16 inputs also the chunk's B and C rows, widened
-//    to fp32 once instead of in every lane of both sweeps (x, needed only
-//    where a step is finished, is read there from the input tile);
-//  * recompute: from the chunk's checkpoint, the forward states of the 16
-//    steps and each lane's share of C.h (for y); the states of the even steps
-//    go to shared memory (one float4 per lane and even step): the sweep forms
-//    an odd step's state again from the even state below it, with the decay
-//    and inputs of that step that it needs anyway, bit for bit the same value
-//    (half the shared-memory traffic of keeping every state: 3.41 -> 3.24 ms
-//    on the 353M layer);
-//  * reverse sweep: the adjoint g, dA in registers; per step the lane's
-//    shares of dB, dC (8 values) are summed over the 8 channels of its
-//    quarter-warp with a transposed 3-round shuffle reduction and left in
-//    shared memory per warp; S1, S2 and y are summed over the 4 lanes of a
-//    channel with a transposed 2-round reduction per 4 steps, after which lane
-//    q finishes step 4m+q (dx, ddt, dz to output tiles written by TMA stores);
-//    The finishing lane evaluates sigmoid(dt + bias) and silu'(z) itself from
-//    the chunk's tiles;
-//  * after the chunk's barrier (in the next iteration), the CTA's dB, dC sums
-//    are sent to global memory with vector atomics.
-// Two barriers per chunk (after the conversion, after the sweep) keep one
-// conversion buffer and one dB/dC buffer, so that 4 CTAs fit on an SM.
-// dA, dD, dbias are accumulated in registers and added atomically at the end
-// (one contribution per batch row); dh0 is stored directly.
+// Work decomposition. A CTA of two warps owns 32 channels of one batch row;
+// four lanes share a channel pair, each with 4 states of both channels. Chunks
+// of kCkptSteps steps are taken in reverse order through a ring of TMA tiles
+// (dt, x, z, dout, B, C). Per chunk:
+//  * conversion, once per (step, channel): Delta, Delta x, dy, sigmoid(dt +
+//    bias) and the gate's factor of dz; B and C widened to fp32. Everything is
+//    kept for pairs of adjacent steps, which fill the packed operations as in
+//    forward.cu;
+//  * the state before step 8, from the checkpoint; then for steps 8..15 and
+//    then 0..7: their states and decays, forward, into registers (with each
+//    lane's share of C.h), and the reverse sweep over them: the adjoint g and
+//    dA in registers, each lane's shares of S1 and S2, and dB, dC;
+//  * dB, dC of a step are sums over channels. A lane adds its own two; lanes
+//    that differ in a channel bit exchange what they do not keep. Lanes hold
+//    their four states in the order r -> r ^ perm with perm = their two low
+//    channel bits (B and C lie in shared memory in both orders of a pair), so
+//    that what is kept and sent is the same register on every lane: 7 shuffles
+//    and 2 selects for 8 values. The warps' sums are added when the chunk is
+//    done and sent to global memory with vector atomics;
+//  * the shares of C.h, S1 and S2 are added through a warp's own tile; the lane
+//    that adds them finishes dx, ddt, dz of those channels and steps (output
+//    tiles written by TMA stores).
+// dA, dD, dbias are accumulated in registers and added atomically at the end;
+// dh0 is stored directly. Segments of a time-split span (backward_segments)
+// start from the adjoints that a first pass (kSummary) leaves: each segment's
+// adjoint from a zero one at its end, and its product of decays.
+//
+// What bounds it: issue at 2 warps per scheduler (registers hold half a chunk's
+// states and decays: 254 of them), of which a loop of the core instructions
+// alone reaches 0.52 per clock; it runs at 0.48. Two channels per lane halve
+// the loads of B and C and the exchange of dB, dC per channel. Measured (8 x
+// 8192 x 2048 bf16): 3.23 -> 2.51 ms, 2.08 -> 1.36 G warp instructions; before,
+// the four warps added dB, dC with shared float atomics, a compare-and-swap loop
+// that cost 5.5 clocks per instruction and kept the compiler from moving code
+// across steps. Variants: quarters of a chunk in registers (193 registers, a
+// longer first pass over the states) 2.63 ms, eighths 4.28 ms; both halves
+// unrolled 3.38 ms (spills); states of the halves in registers instead of
+// shared memory 2.74 ms.
 #include <stddef.h>
 #include <string.h>
 
 #include "common.cuh"
+#include "pairs.cuh"
 #include "tma.cuh"
 
 namespace mbscan {
 namespace {
 
-constexpr int kBT = kCkptSteps;   // steps per chunk
-constexpr int kBWarps = 4;
+constexpr int kBT = kCkptSteps;            // steps per chunk
+constexpr int kBTP = kBT / 2;              // step pairs per chunk
+constexpr int kHTP = kBTP / 2;             // step pairs per half chunk
+constexpr int kBWarps = 2;
 constexpr int kBThreads = 32 * kBWarps;
-constexpr int kBCh = 8 * kBWarps;  // channels per CTA
+constexpr int kBWCh = 16;                  // channels per warp, two per lane
+constexpr int kBPairs = kBWCh / 2;
+constexpr int kBCh = kBWarps * kBWCh;      // channels per CTA
 constexpr int kBStages = 2;
+constexpr int kShareQ = kHTP * kBPairs + 2;   // float4s between the shares of two lanes q (the pad moves them to other banks)
 
 template <typename T>
-struct BRaw {  // TMA destinations; member offsets are multiples of 128 B
+struct BRaw {   // TMA destinations; token tiles swizzled in their 64- (bf16) or 128-byte (fp32) rows
     T dt[kBT][kBCh];
     T x[kBT][kBCh];
     T z[kBT][kBCh];
@@ -66,29 +80,17 @@ struct BRaw {  // TMA destinations; member offsets are multiples of 128 B
     T C[kBT][kDState];
 };
 
-template <bool kWide>
-struct BConv {
-    float2 dg[kBT][kBCh];   // (Delta, Delta*x)
-    float dy[kBT][kBCh];    // dJ/dy * silu(z)
-};
-// bf16 inputs: B and C rows widened to fp32 once per chunk (both sweeps read
-// four states of each per step; the space comes from keeping x out of the
-// conversion tile: the few readers of x take it from the input tile)
-template <>
-struct BConv<true> {
-    float2 dg[kBT][kBCh];
-    float dy[kBT][kBCh];
-    float B[kBT][kDState];
-    float C[kBT][kDState];
-};
-
 template <typename T>
-struct BSmem {
+struct alignas(1024) BSmem {
     BRaw<T> raw[kBStages];
-    BConv<sizeof(T) == 2> cv;
-    float4 hs[kBT / 2][kBThreads];    // recomputed states of the chunk's even steps, per lane
-    T gx[kBT][kBCh], gdt[kBT][kBCh], gz[kBT][kBCh];   // output tiles (TMA stores)
-    float bc[kBT][32];   // per step: slot 8q + j, j < 4 dB[4q+j], else dC[4q+j-4]
+    T gx[kBT][kBCh], gdt[kBT][kBCh], gz[kBT][kBCh];   // output tiles (TMA stores), swizzled like the inputs
+    float4 dg[kBWarps][kBTP][2][kBPairs];   // (Delta_t, Delta_t+1, (Delta x)_t, (Delta x)_t+1) of channel 2 j + k: [k][j]
+    float4 dy[kBWarps][kBTP][kBPairs];      // dJ/dy: channel 2 j (t, t+1), channel 2 j + 1 (t, t+1)
+    float4 bc[2][kBTP][4][4];               // B, C: [tp][q][2 h + s]: states 4q + 2h + s, 4q + 2h + 1 - s (t, t+1 each)
+    float4 share[kBWarps][3][4 * kShareQ];  // shares of C.h, g.B, sum g Abar h A log2 e of lane q: [q][tp of the half][j]
+    float4 fin[kBWarps][2][kBTP][kBPairs];  // sigmoid(dt + bias); dout d(gate)/dz: channels 2 j, 2 j + 1 at t, at t + 1
+    float4 hq[kBWarps][2][2][32];           // states before each half of the chunk: [half][channel][lane]
+    float2 sum[kBWarps][kBTP][32];          // the warp's dB, dC (t, t+1): [tp][8 q + 4 (dC) + state]
     uint64_t full[kBStages];
 };
 
@@ -97,408 +99,472 @@ struct BwdArgs {
     ScanParams p;
     GradParams g;
     int has_gate;
+    int grid_segs, seg0;   // segments of L covered by the grid (blockIdx = (b, segment - seg0, channel tile))
 };
 
-template <typename T>
-__device__ __forceinline__ void issue_bchunk(BSmem<T> &s, const BwdArgs &a, int stage, int64_t chunk,
-                                             int d0, int b) {
+template <typename T, bool kSummary>
+__device__ __forceinline__ void issue_bchunk(BSmem<T> &s, const BwdArgs &a, int stage, int chunk, int d0, int b) {
     constexpr uint32_t tok = kBT * kBCh * sizeof(T), bc = kBT * kDState * sizeof(T);
-    const uint32_t bytes = (a.has_gate ? 4 : 3) * tok + 2 * bc;
+    const uint32_t bytes = ((a.has_gate ? 3 : 2) + (kSummary ? 0 : 1)) * tok + (kSummary ? 1 : 2) * bc;
     uint64_t *bar = &s.full[stage];
     mbar_arrive_expect_tx(bar, bytes);
-    const int t = (int)(chunk * kBT);
+    const int t = chunk * kBT;
     BRaw<T> &r = s.raw[stage];
     tma_load_3d(&r.dt[0][0], &a.tm_dt, bar, d0, t, b);
-    tma_load_3d(&r.x[0][0], &a.tm_x, bar, d0, t, b);
+    if (!kSummary) tma_load_3d(&r.x[0][0], &a.tm_x, bar, d0, t, b);
     if (a.has_gate) tma_load_3d(&r.z[0][0], &a.tm_z, bar, d0, t, b);
     tma_load_3d(&r.dout[0][0], &a.tm_dout, bar, d0, t, b);
-    tma_load_3d(&r.B[0][0], &a.tm_B, bar, 0, t, b);
+    if (!kSummary) tma_load_3d(&r.B[0][0], &a.tm_B, bar, 0, t, b);
     tma_load_3d(&r.C[0][0], &a.tm_C, bar, 0, t, b);
 }
 
-__device__ __forceinline__ float2 ld_pair(const float *p) { return *reinterpret_cast<const float2 *>(p); }
-__device__ __forceinline__ float2 ld_pair(const __nv_bfloat16 *p) {
-    const unsigned u = *reinterpret_cast<const unsigned *>(p);
-    return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
-}
-__device__ __forceinline__ float4 ld_quad(const float *p) { return *reinterpret_cast<const float4 *>(p); }
-__device__ __forceinline__ float4 ld_quad(const __nv_bfloat16 *p) {
-    const uint2 u = *reinterpret_cast<const uint2 *>(p);
-    return make_float4(__uint_as_float(u.x << 16), __uint_as_float(u.x & 0xffff0000u),
-                       __uint_as_float(u.y << 16), __uint_as_float(u.y & 0xffff0000u));
-}
-
-// sigmoid(v) = u / (1 + u) with u = e^v, 1 where u overflows (v > 15 gives
-// 1 - 3e-7, below fp32 resolution of the product it scales).
-__device__ __forceinline__ float sigmoid_v(float v) {
-    if (v > 15.f) return 1.f;
-    const float u = ex2(v * kLog2e);
-    return __fdividef(u, 1.f + u);
+// Delta = softplus(v) (as softplus2) and sigmoid(v) = u / (1 + u), u = e^v, 1 above v = 15 (1 - 3e-7 there)
+__device__ __forceinline__ void softplus_sigmoid2(float2 v, float2 &delta, float2 &sig) {
+    const float2 w = mul2(v, splat(kLog2e));
+    const float2 u = make_float2(ex2(w.x), ex2(w.y));
+    const float2 o = add2(u, splat(1.f));
+    delta = softplus_of(v, u, o);
+    sig = mul2(u, make_float2(rcp(o.x), rcp(o.y)));
+    sig.x = v.x > 15.f ? 1.f : sig.x;
+    sig.y = v.y > 15.f ? 1.f : sig.y;
 }
 
-// Conversion of one chunk by one thread: channel pair cp at steps th, th + 8
-// (and, for bf16, a quarter row of B or C).
+// Four values of a lane's permuted state order (register r: state r ^ perm) from a row of four
+__device__ __forceinline__ void load_perm(float (&v)[4], const float *row, int perm) {
+    const float2 lo = __ldg(reinterpret_cast<const float2 *>(row + (perm & 2)));
+    const float2 hi = __ldg(reinterpret_cast<const float2 *>(row + 2 - (perm & 2)));
+    const bool s = perm & 1;
+    v[0] = s ? lo.y : lo.x;
+    v[1] = s ? lo.x : lo.y;
+    v[2] = s ? hi.y : hi.x;
+    v[3] = s ? hi.x : hi.y;
+}
+__device__ __forceinline__ void store_perm(float *row, const float (&v)[4], int perm) {
+    const bool s = perm & 1;
+    *reinterpret_cast<float2 *>(row + (perm & 2)) = s ? make_float2(v[1], v[0]) : make_float2(v[0], v[1]);
+    *reinterpret_cast<float2 *>(row + 2 - (perm & 2)) = s ? make_float2(v[3], v[2]) : make_float2(v[2], v[3]);
+}
+
+// dB, dC of one chunk: add the warps' sums to global memory (thread: step pair tid / 8, states 4q..4q+3 of dB or dC)
 template <typename T>
-__device__ __forceinline__ void bconvert(BConv<sizeof(T) == 2> &cv, const BRaw<T> &r, int cp, int th, float2 bias,
-                                         bool ok, int64_t t0, int64_t L, bool gate) {
+__device__ __forceinline__ void flush_sums(const BSmem<T> &s, const GradParams &g, int64_t b, int t0, int64_t L) {
+    static_assert(kBTP * 8 == kBThreads, "one thread per step pair and group of four");
+    const int k = threadIdx.x >> 3, grp = threadIdx.x & 7;
+    float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;   // steps t, t + 1
 #pragma unroll
-    for (int k = 0; k < kBT / 8; ++k) {
-        const int t = th + 8 * k;
-        const int c = 2 * cp;
-        float4 dg = make_float4(0.f, 0.f, 0.f, 0.f);   // (Delta, Delta*x) of channels c, c + 1
-        float2 dy = make_float2(0.f, 0.f);
-        if (ok && t0 + t < L) {
-            const float2 xv = ld_pair(&r.x[t][c]);
-            const float2 dv = ld_pair(&r.dt[t][c]);
-            const float2 ov = ld_pair(&r.dout[t][c]);
-            const float d0 = softplus(dv.x + bias.x), d1 = softplus(dv.y + bias.y);   // as in the forward
-            dy = ov;
-            if (gate) {
-                const float2 zv = ld_pair(&r.z[t][c]);
-                dy = make_float2(ov.x * silu(zv.x), ov.y * silu(zv.y));
-            }
-            dg = make_float4(d0, d0 * xv.x, d1, d1 * xv.y);
-        }
-        *reinterpret_cast<float4 *>(&cv.dg[t][c]) = dg;
-        *reinterpret_cast<float2 *>(&cv.dy[t][c]) = dy;
+    for (int w = 0; w < kBWarps; ++w) {
+        const float4 *r = reinterpret_cast<const float4 *>(&s.sum[w][k][4 * grp]);
+        const float4 u = r[0], v = r[1];
+        lo = make_float4(lo.x + u.x, lo.y + u.z, lo.z + v.x, lo.w + v.z);
+        hi = make_float4(hi.x + u.y, hi.y + u.w, hi.z + v.y, hi.w + v.w);
     }
-    if constexpr (sizeof(T) == 2) {   // thread (t, j): four states of B (j < 4) or C (j >= 4) at step t
-        static_assert(kBThreads == kBT * 8 && kDState == 16, "one quarter row of B or C per thread");
-        const int t = threadIdx.x >> 3, j = threadIdx.x & 7;
-        const float4 v = ld_quad(j < 4 ? &r.B[t][4 * j] : &r.C[t][4 * (j - 4)]);
-        *reinterpret_cast<float4 *>(j < 4 ? &cv.B[t][4 * j] : &cv.C[t][4 * (j - 4)]) = v;
-    }
+    float *dst = ((grp & 1) ? g.dC : g.dB) + ((b * L + t0 + 2 * k) * kDState + 4 * (grp >> 1));
+    if (t0 + 2 * k < L) atomicAdd(reinterpret_cast<float4 *>(dst), lo);
+    if (t0 + 2 * k + 1 < L) atomicAdd(reinterpret_cast<float4 *>(dst + kDState), hi);
 }
 
-// Four states of B and C at step t: the widened rows (bf16) or the tile (fp32).
-template <typename T>
-__device__ __forceinline__ void load_bc(const BConv<sizeof(T) == 2> &cv, const BRaw<T> &r, int t, int q,
-                                        float4 &b4, float4 &c4) {
-    if constexpr (sizeof(T) == 2) {
-        b4 = *reinterpret_cast<const float4 *>(&cv.B[t][4 * q]);
-        c4 = *reinterpret_cast<const float4 *>(&cv.C[t][4 * q]);
-    } else {
-        b4 = ld_quad(&r.B[t][4 * q]);
-        c4 = ld_quad(&r.C[t][4 * q]);
-    }
-}
-
-// Transposed sum over the 4 lanes of a channel (8 apart) for 4 consecutive
-// steps: lane q ends with the full sum of step q.
-__device__ __forceinline__ float reduce4(float p0, float p1, float p2, float p3, int q) {
-    const bool hi = (q & 2) != 0;
-    float k0 = hi ? p2 : p0, k1 = hi ? p3 : p1;
-    const float s0 = hi ? p0 : p2, s1 = hi ? p1 : p3;
-    k0 += __shfl_xor_sync(kFull, s0, 16);
-    k1 += __shfl_xor_sync(kFull, s1, 16);
-    const bool odd = (q & 1) != 0;
-    const float keep = odd ? k1 : k0, send = odd ? k0 : k1;
-    return keep + __shfl_xor_sync(kFull, send, 8);
-}
-
-// Transposed sum of 8 values over the 8 lanes c8 = 0..7 of a quarter-warp
-// (lanes 1, 2, 4 apart): lane c8 ends with the sum of value c8.
-__device__ __forceinline__ float reduce8(const float (&v)[8], int c8) {
-    const bool h4 = (c8 & 4) != 0, h2 = (c8 & 2) != 0, h1 = (c8 & 1) != 0;
-    float k[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float keep = h4 ? v[4 + i] : v[i], send = h4 ? v[i] : v[4 + i];
-        k[i] = keep + __shfl_xor_sync(kFull, send, 4);
-    }
-    float k2[2];
-#pragma unroll
-    for (int i = 0; i < 2; ++i) {
-        const float keep = h2 ? k[2 + i] : k[i], send = h2 ? k[i] : k[2 + i];
-        k2[i] = keep + __shfl_xor_sync(kFull, send, 2);
-    }
-    const float keep = h1 ? k2[1] : k2[0], send = h1 ? k2[0] : k2[1];
-    return keep + __shfl_xor_sync(kFull, send, 1);
-}
-
-template <typename T>
-__device__ __forceinline__ void store_out(T (&tile)[kBT][kBCh], int t, int c, float v) {
-    tile[t][c] = from_f32<T>(v);
-}
-
-// dB, dC of one chunk: send the CTA's sums to global memory and clear the
-// buffer for its next use (thread: step tid / 8, slots 4 sg .. 4 sg + 3).
-__device__ __forceinline__ void flush_bc(float (&bc)[kBT][32], const GradParams &g, int64_t b, int64_t t0,
-                                         int64_t L) {
-    static_assert(kBT * 8 == kBThreads, "one thread per step and slot group");
-    const int t = threadIdx.x >> 3, sg = threadIdx.x & 7;
-    float4 &v = *reinterpret_cast<float4 *>(&bc[t][4 * sg]);
-    if (t0 + t < L) {
-        const int q = sg >> 1;
-        float *dst = ((sg & 1) ? g.dC : g.dB) + ((b * L + t0 + t) * kDState + 4 * q);
-        atomicAdd(reinterpret_cast<float4 *>(dst), v);
-    }
-    v = make_float4(0.f, 0.f, 0.f, 0.f);
-}
-
-template <typename T>
+template <typename T, bool kSummary>
 __global__ void __launch_bounds__(kBThreads, 4) backward_kernel(const __grid_constant__ BwdArgs a) {
-    constexpr int S = kBStages;
+    constexpr int S = kBStages, kRowB = kBCh * (int)sizeof(T);
     using R = BRaw<T>;
     using SM = BSmem<T>;
-    // every TMA source or destination starts on a 128-byte boundary
-    static_assert(sizeof(R) % 128 == 0 && offsetof(R, x) % 128 == 0 && offsetof(R, z) % 128 == 0 &&
-                      offsetof(R, dout) % 128 == 0 && offsetof(R, B) % 128 == 0 && offsetof(R, C) % 128 == 0 &&
-                      offsetof(SM, raw) % 128 == 0 && offsetof(SM, gx) % 128 == 0 &&
-                      offsetof(SM, gdt) % 128 == 0 && offsetof(SM, gz) % 128 == 0,
-                  "TMA tiles must be 128-byte aligned");
+    static_assert(sizeof(R) % (8 * kRowB) == 0 && offsetof(R, x) % (8 * kRowB) == 0 && offsetof(R, z) % (8 * kRowB) == 0 &&
+                      offsetof(R, dout) % (8 * kRowB) == 0 && offsetof(R, B) % 128 == 0 && offsetof(R, C) % 128 == 0 &&
+                      offsetof(SM, gx) % (8 * kRowB) == 0 && offsetof(SM, gdt) % (8 * kRowB) == 0 &&
+                      offsetof(SM, gz) % (8 * kRowB) == 0,
+                  "swizzled TMA tiles start on their pattern's boundary");
     extern __shared__ unsigned char smem_dyn[];
-    BSmem<T> &s = smem_aligned<BSmem<T>>(smem_dyn);
+    SM &s = *reinterpret_cast<SM *>(smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u));
     const ScanParams &p = a.p;
     const GradParams &gp = a.g;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ntd = (int)((p.d_inner + kBCh - 1) / kBCh);
-    const int b = blockIdx.x / ntd;
-    const int d0 = (blockIdx.x % ntd) * kBCh;
-    const int64_t L = p.seqlen, D = p.d_inner;
-    const int64_t nchunks = (L + kBT - 1) / kBT;   // >= 1: L > 0 here
+    const int64_t D = p.d_inner;
+    const int ntd = (int)((D + kBCh - 1) / kBCh);
+    const int L = (int)p.seqlen;
+    const int nchunks = (L + kBT - 1) / kBT;
+    const int seg = a.seg0 + (int)((blockIdx.x / ntd) % a.grid_segs);
+    const int b = (int)(blockIdx.x / ntd / a.grid_segs);
+    const int nseg = p.nseg > 1 ? (int)p.nseg : 1;
+    const int cps = (nchunks + nseg - 1) / nseg;
+    const int c0 = seg * cps, nch = min(nchunks - c0, cps);   // chunks c0 + nch - 1 down to c0
+    const int d0 = (int)(blockIdx.x % ntd) * kBCh;
     const bool gate = a.has_gate != 0;
 
     if (tid == 0) {
         for (int st = 0; st < S; ++st) mbar_init(&s.full[st], 1);
         fence_mbar_init();
     }
-    for (int i = tid; i < kBT * 32; i += kBThreads) (&s.bc[0][0])[i] = 0.f;
     __syncthreads();
     pdl_wait();   // everything below reads or writes global memory
-    // ring slot j holds chunk nchunks-1-j (reverse order)
     if (tid == 0)
-        for (int j = 0; j < S && j < nchunks; ++j) issue_bchunk(s, a, j, nchunks - 1 - j, d0, b);
+        for (int j = 0; j < S && j < nch; ++j) issue_bchunk<T, kSummary>(s, a, j, c0 + nch - 1 - j, d0, b);
 
-    // ---- conversion role: channel pair cp at steps th, th + 8
-    const int cp = tid % (kBCh / 2), th = tid / (kBCh / 2);
-    const int64_t dc = d0 + 2 * cp;
-    const bool cok = dc < D;
-    const float2 bias2 = (cok && p.dt_bias) ? __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc))
-                                            : make_float2(0.f, 0.f);
-
-    // ---- scan role: channel c, states 4q .. 4q+3
-    const int c8 = lane & 7, q = lane >> 3;
-    const int c = warp * 8 + c8;
-    const int64_t d = d0 + c;
-    const bool chan_ok = d < D;
-    float2 a2[2], Ar[2], g[2], dA[2];
-    float dsk = 0.f, dtb = 0.f, dD_acc = 0.f, db_acc = 0.f;
+    // ---- conversion and finishing role: channels 16 warp + 2 pp + {0, 1} of the tile, step pairs ts and ts + 4
+    const int wc0 = kBWCh * warp, pp = lane & 7, ts = lane >> 3;
+    int off[2][2];
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-        a2[k] = make_float2(0.f, 0.f); Ar[k] = a2[k]; g[k] = a2[k]; dA[k] = a2[k];
+    for (int u = 0; u < 2; ++u)
+#pragma unroll
+        for (int e = 0; e < 2; ++e) off[u][e] = tile_off<T, kBCh>(2 * (ts + kHTP * u) + e, wc0 + 2 * pp);
+    float2 bias = make_float2(0.f, 0.f), dsk = bias, dD_acc = bias, db_acc = bias;
+    const int64_t dc = (int64_t)d0 + wc0 + 2 * pp;   // D % 8 == 0: both channels valid or neither
+    if (dc < D) {
+        if (p.dt_bias) bias = __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc));
+        if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
     }
-    if (chan_ok) {
-        const float4 av = __ldg(reinterpret_cast<const float4 *>(p.A + d * kDState + 4 * q));
-        Ar[0] = make_float2(av.x, av.y);
-        Ar[1] = make_float2(av.z, av.w);
-        a2[0] = make_float2(av.x * kLog2e, av.y * kLog2e);
-        a2[1] = make_float2(av.z * kLog2e, av.w * kLog2e);
-        dsk = p.D ? __ldg(p.D + d) : 0.f;
-        dtb = p.dt_bias ? __ldg(p.dt_bias + d) : 0.f;
-        if (gp.dh_last) {
-            const float4 gv = __ldg(reinterpret_cast<const float4 *>(gp.dh_last + ((int64_t)b * D + d) * kDState + 4 * q));
-            g[0] = make_float2(gv.x, gv.y);
-            g[1] = make_float2(gv.z, gv.w);
+
+    // ---- scan role: channels 2 cl, 2 cl + 1 of the warp, states 4 q .. 4 q + 3 in the order r -> r ^ perm
+    const int cl = ((lane >> 2) & 3) | ((lane & 1) << 2), q = ((lane >> 1) & 1) | ((lane >> 4) << 1);
+    const int perm = cl & 3;
+    const int ix0 = perm, ix1 = perm ^ 2;   // slots of s.bc that hold registers 0, 1 and 2, 3
+    const int64_t d = (int64_t)d0 + wc0 + 2 * cl;
+    const bool chan_ok = d < D;
+    float a2[2][4], g[2][4];   // A log2 e; the adjoint Abar_{t+1} g_{t+1} on its way down
+    float2 dA[2][4];           // even and odd steps
+    float2 dsum[2];            // kSummary: sum of Delta
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            a2[j][n] = g[j][n] = 0.f;
+            dA[j][n] = make_float2(0.f, 0.f);
+        }
+        dsum[j] = make_float2(0.f, 0.f);
+        if (chan_ok) {
+            load_perm(a2[j], p.A + (d + j) * kDState + 4 * q, perm);
+#pragma unroll
+            for (int n = 0; n < 4; ++n) a2[j][n] *= kLog2e;
+            if (seg == nseg - 1) {
+                if (gp.dh_last) load_perm(g[j], gp.dh_last + ((int64_t)b * D + d + j) * kDState + 4 * q, perm);
+            } else if (!kSummary) {   // the last segment's summary starts from dh_last: fold down to this one
+                for (int sp = nseg - 1; sp > seg; --sp) {
+                    const int64_t o = (((int64_t)b * nseg + sp) * D + d + j) * kDState + 4 * q;
+                    float ge[4], pe[4];
+                    load_perm(ge, p.seg_h + o, perm);
+                    load_perm(pe, p.seg_p + o, perm);
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) g[j][n] = sp == nseg - 1 ? ge[n] : fmaf(pe[n], g[j][n], ge[n]);
+                }
+            }
         }
     }
 
-    // checkpoint of chunk i, loaded one iteration ahead (its latency overlaps
-    // the previous chunk's sweep)
-    auto load_ckpt = [&](int64_t i) {
-        return chan_ok ? __ldg(reinterpret_cast<const float4 *>(
-                             gp.h_ckpt + (((int64_t)b * nchunks + i) * D + d) * kDState + 4 * q))
-                       : make_float4(0.f, 0.f, 0.f, 0.f);
-    };
-    float4 ck_next = load_ckpt(nchunks - 1);
-
     bool ok = true;
-    for (int64_t j = 0; j < nchunks; ++j) {
-        const int64_t i = nchunks - 1 - j;   // chunk of this iteration
-        const int64_t t0 = i * kBT;
-        // (1) wait for chunk i's tiles and convert them; dB, dC of chunk i + 1
-        ok = mbar_wait(&s.full[j % S], (uint32_t)((j / S) & 1));
-        if (ok) bconvert(s.cv, s.raw[j % S], cp, th, bias2, cok, t0, L, gate);
-        if (j >= 1) flush_bc(s.bc, gp, b, t0 + kBT, L);
+    for (int it = 0; it < nch; ++it) {
+        const int i = c0 + nch - 1 - it;   // chunk of this iteration
+        const int t0 = i * kBT;
+        const R &r = s.raw[it % S];
+        // the chunk's checkpoint, in flight during the conversion; the next one's on its way to L2
+        float hm[2][4];
+        if constexpr (!kSummary) {
+            const float *ck = gp.h_ckpt + (((int64_t)b * nchunks + i) * D + d) * kDState + 4 * q;
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+#pragma unroll
+                for (int n = 0; n < 4; ++n) hm[j][n] = 0.f;
+                if (chan_ok) load_perm(hm[j], ck + j * kDState, perm);
+            }
+            if (chan_ok && it + 1 < nch) asm volatile("prefetch.global.L2 [%0];" ::"l"(ck - D * kDState + (q & 1) * kDState));
+        }
+        // (1) convert chunk i; add dB, dC of chunk i + 1 to global memory
+        ok = mbar_wait(&s.full[it % S], (uint32_t)((it / S) & 1));
+        if (ok) {
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int tp = ts + kHTP * u;
+                float2 de[2], dyv[2], gxv[2], sig[2], qz[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    softplus_sigmoid2(add2(ld2<T>(&r.dt[0][0], off[u][e]), bias), de[e], sig[e]);
+                    const float m = t0 + 2 * tp + e < L ? 1.f : 0.f;   // Delta = 0 past the end: h and g unchanged
+                    de[e] = mul2(de[e], splat(m));
+                    sig[e] = mul2(sig[e], splat(m));
+                    dyv[e] = ld2<T>(&r.dout[0][0], off[u][e]);
+                    if constexpr (!kSummary) gxv[e] = mul2(de[e], ld2<T>(&r.x[0][0], off[u][e]));
+                    qz[e] = make_float2(0.f, 0.f);
+                    if (gate) {
+                        const float2 z = ld2<T>(&r.z[0][0], off[u][e]);
+                        const float2 w = mul2(z, splat(-kLog2e));
+                        const float2 o = add2(make_float2(ex2(w.x), ex2(w.y)), splat(1.f));
+                        const float2 sz = make_float2(rcp(o.x), rcp(o.y));
+                        qz[e] = mul2(mul2(dyv[e], sz), fma2(z, fma2(sz, splat(-1.f), splat(1.f)), splat(1.f)));
+                        dyv[e] = mul2(dyv[e], mul2(z, sz));
+                    }
+                }
+                if constexpr (kSummary) gxv[0] = gxv[1] = make_float2(0.f, 0.f);
+                s.dg[warp][tp][0][pp] = make_float4(de[0].x, de[1].x, gxv[0].x, gxv[1].x);
+                s.dg[warp][tp][1][pp] = make_float4(de[0].y, de[1].y, gxv[0].y, gxv[1].y);
+                s.dy[warp][tp][pp] = make_float4(dyv[0].x, dyv[1].x, dyv[0].y, dyv[1].y);
+                if constexpr (!kSummary) {
+                    s.fin[warp][0][tp][pp] = make_float4(sig[0].x, sig[0].y, sig[1].x, sig[1].y);
+                    s.fin[warp][1][tp][pp] = make_float4(qz[0].x, qz[0].y, qz[1].x, qz[1].y);
+                }
+            }
+            {   // two states of B and of C at a step pair, in both orders
+                const int wh = tid & 1, wq = (tid >> 1) & 3, wt = tid >> 3;
+                const bool swap = wq & 2;   // which order first: eight stores at a time on different banks
+#pragma unroll
+                for (int u = kSummary ? 1 : 0; u < 2; ++u) {
+                    const T *src = u ? &r.C[2 * wt][4 * wq + 2 * wh] : &r.B[2 * wt][4 * wq + 2 * wh];
+                    const float2 v0 = ld2<T>(src, 0), v1 = ld2<T>(src, kDState * (int)sizeof(T));
+                    float4 *dst = &s.bc[u][wt][wq][2 * wh];
+                    const float4 f = make_float4(v0.x, v1.x, v0.y, v1.y), rv = make_float4(v0.y, v1.y, v0.x, v1.x);
+                    dst[swap ? 1 : 0] = swap ? rv : f;
+                    dst[swap ? 0 : 1] = swap ? f : rv;
+                }
+            }
+        }
+        if constexpr (!kSummary) {
+            if (it >= 1) flush_sums(s, gp, b, t0 + kBT, L);
+            if (tid == 0) bulk_wait_read_all();   // the output tiles may be written again
+        }
         if (__syncthreads_or(ok ? 0 : 1)) {
             if (tid == 0) {
-                report(p.status, 4 /* MB_ERR_TIMEOUT */, j);
-                int64_t last = j + S - 1;   // ring slots issued so far: 0 .. j+S-1
-                if (last > nchunks - 1) last = nchunks - 1;
-                for (int64_t jj = j; jj <= last; ++jj)
+                report(p.status, 4 /* MB_ERR_TIMEOUT */, it);
+                for (int jj = it; jj <= it + S - 1 && jj < nch; ++jj)
                     mbar_wait(&s.full[jj % S], (uint32_t)((jj / S) & 1));
                 bulk_wait_all();
             }
             return;
         }
 
-        // (2) chunk i
-        const BConv<sizeof(T) == 2> &cv = s.cv;
-        const BRaw<T> &rs = s.raw[j % S];
-        const float2 hc[2] = {make_float2(ck_next.x, ck_next.y), make_float2(ck_next.z, ck_next.w)};
-        if (i > 0) ck_next = load_ckpt(i - 1);
-        // recompute the chunk's forward states (same arithmetic as the forward)
-        float4(&hs)[kBT / 2][kBThreads] = s.hs;
-        float yv[kBT / 4];   // lane q: share-summed y of step 4m + q
-        {
-            float2 h0v = hc[0], h1v = hc[1];
-            float part[4];
+        const float4(&dgw)[kBTP][2][kBPairs] = s.dg[warp];
+        const float4(&dyw)[kBTP][kBPairs] = s.dy[warp];
+        if constexpr (kSummary) {
+            float2 cs[2];
 #pragma unroll
-            for (int t = 0; t < kBT; ++t) {
-                const float2 av = cv.dg[t][c];
-                const float2 dd = make_float2(av.x, av.x), gg = make_float2(av.y, av.y);
-                const float2 e0 = mul2(dd, a2[0]), e1 = mul2(dd, a2[1]);
-                float4 b4, c4;
-                load_bc(cv, rs, t, q, b4, c4);
-                h0v = fma2(make_float2(ex2(e0.x), ex2(e0.y)), h0v, mul2(make_float2(b4.x, b4.y), gg));
-                h1v = fma2(make_float2(ex2(e1.x), ex2(e1.y)), h1v, mul2(make_float2(b4.z, b4.w), gg));
-                if ((t & 1) == 0) hs[t / 2][tid] = make_float4(h0v.x, h0v.y, h1v.x, h1v.y);
-                const float2 acc = fma2(make_float2(c4.z, c4.w), h1v, mul2(make_float2(c4.x, c4.y), h0v));
-                part[t & 3] = acc.x + acc.y;
-                if ((t & 3) == 3) yv[t >> 2] = reduce4(part[0], part[1], part[2], part[3], q);
-            }
-        }
-        // reverse sweep over the chunk. Only the even steps' states were kept:
-        // an odd step's state is one recurrence step from the even state below
-        // it, with that step's decay and inputs, which the sweep forms anyway
-        // (one step ahead), so the result is bit for bit the recompute's.
-        float (&bcs)[kBT][32] = s.bc;
-        float s1[4], s2[4];
-        struct StepVals {
-            float2 dd, gx, ab0, ab1;
-            float4 b4, c4;
-            float dyv;
-        };
-        auto stepvals = [&](int t) {
-            StepVals v;
-            const float2 av = cv.dg[t][c];   // (Delta, Delta*x)
-            v.dd = make_float2(av.x, av.x);
-            v.gx = make_float2(av.y, av.y);
-            v.dyv = cv.dy[t][c];
-            const float2 e0 = mul2(v.dd, a2[0]), e1 = mul2(v.dd, a2[1]);
-            v.ab0 = make_float2(ex2(e0.x), ex2(e0.y));
-            v.ab1 = make_float2(ex2(e1.x), ex2(e1.y));
-            load_bc(cv, rs, t, q, v.b4, v.c4);
-            return v;
-        };
-        auto advance = [&](const StepVals &v, float4 hp) {   // the forward step from hp
-            const float2 n0 = fma2(v.ab0, make_float2(hp.x, hp.y), mul2(make_float2(v.b4.x, v.b4.y), v.gx));
-            const float2 n1 = fma2(v.ab1, make_float2(hp.z, hp.w), mul2(make_float2(v.b4.z, v.b4.w), v.gx));
-            return make_float4(n0.x, n0.y, n1.x, n1.y);
-        };
-        StepVals cur = stepvals(kBT - 1);
-        float4 heven = hs[kBT / 2 - 1][tid];   // h_{kBT-2}
-        float4 hcur = advance(cur, heven);     // h_{kBT-1}
+            for (int k = kBTP - 1; k >= 0; --k) {
+                const float4 c01 = s.bc[1][k][q][ix0], c23 = s.bc[1][k][q][ix1];
+                const float2 cp[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w),
+                                      make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
+                const float4 yv = dyw[k][cl];
+                const float2 dyp[2] = {make_float2(yv.x, yv.y), make_float2(yv.z, yv.w)};
 #pragma unroll
-        for (int t = kBT - 1; t >= 0; --t) {
-            const float2 dd = cur.dd, gx = cur.gx;
-            const float2 dy = make_float2(cur.dyv, cur.dyv);
-            const float2 ab0 = cur.ab0, ab1 = cur.ab1;
-            const float4 b4 = cur.b4, c4 = cur.c4;
-            float4 hprev;
-            StepVals nxt = cur;
-            if (t == 0) {
-                hprev = make_float4(hc[0].x, hc[0].y, hc[1].x, hc[1].y);
-            } else if (t & 1) {
-                hprev = heven;                   // h_{t-1}, even: kept
-                nxt = stepvals(t - 1);
-            } else {
-                nxt = stepvals(t - 1);
-                heven = hs[t / 2 - 1][tid];      // h_{t-2}
-                hprev = advance(nxt, heven);     // h_{t-1}, odd
-            }
-            const float2 hp0 = make_float2(hprev.x, hprev.y), hp1 = make_float2(hprev.z, hprev.w);
-            const float2 ht0 = make_float2(hcur.x, hcur.y), ht1 = make_float2(hcur.z, hcur.w);
-            hcur = hprev;
-            cur = nxt;
-            g[0] = fma2(dy, make_float2(c4.x, c4.y), g[0]);
-            g[1] = fma2(dy, make_float2(c4.z, c4.w), g[1]);
-            const float2 dc0 = mul2(dy, ht0), dc1 = mul2(dy, ht1);
-            const float2 sb = fma2(g[1], make_float2(b4.z, b4.w), mul2(g[0], make_float2(b4.x, b4.y)));
-            const float2 db0 = mul2(g[0], gx), db1 = mul2(g[1], gx);
-            const float2 ga0 = mul2(g[0], ab0), ga1 = mul2(g[1], ab1);
-            const float2 w0 = mul2(ga0, hp0), w1 = mul2(ga1, hp1);
-            const float2 sa = fma2(w1, Ar[1], mul2(w0, Ar[0]));
-            dA[0] = fma2(w0, dd, dA[0]);
-            dA[1] = fma2(w1, dd, dA[1]);
-            g[0] = ga0;
-            g[1] = ga1;
-            s1[t & 3] = sb.x + sb.y;
-            s2[t & 3] = sa.x + sa.y;
-            const float v8[8] = {db0.x, db0.y, db1.x, db1.y, dc0.x, dc0.y, dc1.x, dc1.y};
-            atomicAdd(&bcs[t][lane], reduce8(v8, c8));   // the 4 warps' shares
-            if ((t & 3) == 0) {   // steps t .. t+3 done: finish step t + q on this lane
-                const float S1 = reduce4(s1[0], s1[1], s1[2], s1[3], q);
-                const float S2 = reduce4(s2[0], s2[1], s2[2], s2[3], q);
-                const int tq = t + q;
-                const bool live = chan_ok && t0 + tq < L;
-                const float delta = cv.dg[tq][c].x, dyq = cv.dy[tq][c];
-                const float xq = live ? to_f32(rs.x[tq][c]) : 0.f;
-                const float sig = live ? sigmoid_v(to_f32(rs.dt[tq][c]) + dtb) : 0.f;
-                float qz = 0.f;
-                if (gate && live) {
-                    const float zt = to_f32(rs.z[tq][c]);
-                    const float sz = __fdividef(1.f, 1.f + ex2(-zt * kLog2e));
-                    qz = to_f32(rs.dout[tq][c]) * sz * fmaf(zt, 1.f - sz, 1.f);
+                for (int j = 0; j < 2; ++j) {
+                    const float2 dd = *reinterpret_cast<const float2 *>(&dgw[k][j][cl]);
+                    cs[j] = k == kBTP - 1 ? dd : add2(cs[j], dd);
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        const float2 e = mul2(dd, splat(a2[j][n]));
+                        const float g1 = fmaf(dyp[j].y, cp[n].y, g[j][n]) * ex2(e.y);
+                        g[j][n] = fmaf(dyp[j].x, cp[n].x, g1) * ex2(e.x);
+                    }
                 }
-                const float dx = fmaf(delta, S1, dyq * dsk);
-                const float ddt = fmaf(xq, S1, S2) * sig;
-                const float y = fmaf(dsk, xq, yv[t >> 2]);
-                dD_acc = fmaf(dyq, xq, dD_acc);
-                db_acc += ddt;
-                store_out(s.gx, tq, c, dx);
-                store_out(s.gdt, tq, c, ddt);
-                if (gate) store_out(s.gz, tq, c, y * qz);
             }
+            dsum[0] = add2(dsum[0], cs[0]);
+            dsum[1] = add2(dsum[1], cs[1]);
+        } else {
+            // (2) the state before step 8: steps 0 .. 7 from the checkpoint
+            float4(&hq)[2][2][32] = s.hq[warp];
+#pragma unroll
+            for (int j = 0; j < 2; ++j) hq[0][j][lane] = make_float4(hm[j][0], hm[j][1], hm[j][2], hm[j][3]);
+#pragma unroll
+            for (int k = 0; k < kHTP; ++k) {
+                const float4 b01 = s.bc[0][k][q][ix0], b23 = s.bc[0][k][q][ix1];
+                const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w), make_float2(b23.x, b23.y),
+                                      make_float2(b23.z, b23.w)};
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+                    const float4 v = dgw[k][j][cl];
+                    const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        const float2 e = mul2(dd, splat(a2[j][n]));
+                        const float2 bg = mul2(bp[n], gg);
+                        hm[j][n] = fmaf(ex2(e.y), fmaf(ex2(e.x), hm[j][n], bg.x), bg.y);
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 2; ++j) hq[1][j][lane] = make_float4(hm[j][0], hm[j][1], hm[j][2], hm[j][3]);
+            float4(&sh)[3][4 * kShareQ] = s.share[warp];
+            // (3) the two halves, the later one first (not unrolled: both at once spill registers)
+#pragma unroll 1
+            for (int u = 1; u >= 0; --u) {
+                const int k0 = kHTP * u;
+                const float4 ha = hq[u][0][lane], hb = hq[u][1][lane];
+                const float hs[2][4] = {{ha.x, ha.y, ha.z, ha.w}, {hb.x, hb.y, hb.z, hb.w}};   // state before this half
+                // its decays and states, kept in registers, and the shares of C.h
+                float2 ab[kHTP][2][4], hp[kHTP][2][4];
+                float4 shy[kHTP];
+#pragma unroll
+                for (int k = 0; k < kHTP; ++k) {
+                    const float4 b01 = s.bc[0][k0 + k][q][ix0], b23 = s.bc[0][k0 + k][q][ix1];
+                    const float4 c01 = s.bc[1][k0 + k][q][ix0], c23 = s.bc[1][k0 + k][q][ix1];
+                    const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
+                                          make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
+                    const float2 cp[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w),
+                                          make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
+                    float2 acc[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const float4 v = dgw[k0 + k][j][cl];
+                        const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
+#pragma unroll
+                        for (int n = 0; n < 4; ++n) {
+                            const float2 e = mul2(dd, splat(a2[j][n]));
+                            ab[k][j][n] = make_float2(ex2(e.x), ex2(e.y));
+                            const float2 bg = mul2(bp[n], gg);
+                            const float hl = k == 0 ? hs[j][n] : hp[k - 1][j][n].y;
+                            hp[k][j][n].x = fmaf(ab[k][j][n].x, hl, bg.x);
+                            hp[k][j][n].y = fmaf(ab[k][j][n].y, hp[k][j][n].x, bg.y);
+                            acc[j] = n == 0 ? mul2(cp[0], hp[k][j][0]) : fma2(cp[n], hp[k][j][n], acc[j]);
+                        }
+                    }
+                    shy[k] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
+                }
+#pragma unroll
+                for (int k = 0; k < kHTP; ++k) sh[0][q * kShareQ + k * kBPairs + cl] = shy[k];
+                // reverse sweep
+                float4 sh1[kHTP], sh2[kHTP];
+                float2 sums[kHTP];
+#pragma unroll
+                for (int k = kHTP - 1; k >= 0; --k) {
+                    const float4 b01 = s.bc[0][k0 + k][q][ix0], b23 = s.bc[0][k0 + k][q][ix1];
+                    const float4 c01 = s.bc[1][k0 + k][q][ix0], c23 = s.bc[1][k0 + k][q][ix1];
+                    const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
+                                          make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
+                    const float2 cp[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w),
+                                          make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
+                    const float4 yv = dyw[k0 + k][cl];
+                    const float2 dyp[2] = {make_float2(yv.x, yv.y), make_float2(yv.z, yv.w)};
+                    float2 dBv[4], dCv[4], s1[2], s2[2];
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const float4 v = dgw[k0 + k][j][cl];
+                        const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
+#pragma unroll
+                        for (int n = 0; n < 4; ++n) {
+                            const float2 A = ab[k][j][n], H = hp[k][j][n];
+                            float2 gv, ga, w;
+                            gv.y = fmaf(dyp[j].y, cp[n].y, g[j][n]);
+                            ga.y = gv.y * A.y;
+                            gv.x = fmaf(dyp[j].x, cp[n].x, ga.y);
+                            ga.x = gv.x * A.x;
+                            g[j][n] = ga.x;
+                            w.x = ga.x * (k == 0 ? hs[j][n] : hp[k - 1][j][n].y);
+                            w.y = ga.y * H.x;
+                            dCv[n] = j == 0 ? mul2(dyp[0], H) : fma2(dyp[1], H, dCv[n]);
+                            dBv[n] = j == 0 ? mul2(gg, gv) : fma2(gg, gv, dBv[n]);
+                            s1[j] = n == 0 ? mul2(bp[0], gv) : fma2(bp[n], gv, s1[j]);
+                            s2[j] = n == 0 ? mul2(splat(a2[j][0]), w) : fma2(splat(a2[j][n]), w, s2[j]);
+                            dA[j][n] = fma2(dd, w, dA[j][n]);
+                        }
+                    }
+                    sh1[k] = make_float4(s1[0].x, s1[0].y, s1[1].x, s1[1].y);
+                    sh2[k] = make_float4(s2[0].x, s2[0].y, s2[1].x, s2[1].y);
+                    // dB, dC over the warp's 16 channels: lanes that differ in channel bits exchange the states they do
+                    // not keep; the state order r -> r ^ perm makes those registers 2, 3, then 1, on every lane
+#pragma unroll
+                    for (int n = 0; n < 2; ++n) {
+                        dBv[n] = add2(dBv[n], shfl2(dBv[n + 2], 8));
+                        dCv[n] = add2(dCv[n], shfl2(dCv[n + 2], 8));
+                    }
+                    dBv[0] = add2(dBv[0], shfl2(dBv[1], 4));
+                    dCv[0] = add2(dCv[0], shfl2(dCv[1], 4));
+                    const bool keepC = lane & 1;   // channel bit 2: this lane ends with dC of its state, or dB
+                    const float2 keep = keepC ? dCv[0] : dBv[0], send = keepC ? dBv[0] : dCv[0];
+                    sums[k] = add2(keep, shfl2(send, 1));
+                }
+#pragma unroll
+                for (int k = 0; k < kHTP; ++k) {
+                    sh[1][q * kShareQ + k * kBPairs + cl] = sh1[k];
+                    sh[2][q * kShareQ + k * kBPairs + cl] = sh2[k];
+                    s.sum[warp][k0 + k][8 * q + 4 * (lane & 1) + perm] = sums[k];
+                }
+                // finish this half's outputs
+                __syncwarp();
+                float2 tot[3][2];   // C.h, g.B, sum g Abar h A log2 e: [step] of (channel 2 pp, channel 2 pp + 1)
+#pragma unroll
+                for (int v = 0; v < 3; ++v) {
+                    const float4 *src = &sh[v][ts * kBPairs + pp];
+                    const float4 x0 = src[0], x1 = src[kShareQ], x2 = src[2 * kShareQ], x3 = src[3 * kShareQ];
+                    const float2 ca = add2(add2(make_float2(x0.x, x0.y), make_float2(x1.x, x1.y)),
+                                           add2(make_float2(x2.x, x2.y), make_float2(x3.x, x3.y)));
+                    const float2 cb = add2(add2(make_float2(x0.z, x0.w), make_float2(x1.z, x1.w)),
+                                           add2(make_float2(x2.z, x2.w), make_float2(x3.z, x3.w)));
+                    tot[v][0] = make_float2(ca.x, cb.x);
+                    tot[v][1] = make_float2(ca.y, cb.y);
+                }
+                const float4 va = dgw[k0 + ts][0][pp], vb = dgw[k0 + ts][1][pp], yv = dyw[k0 + ts][pp];
+                const float4 fs = s.fin[warp][0][k0 + ts][pp], fq = s.fin[warp][1][k0 + ts][pp];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int o = u ? off[1][e] : off[0][e];
+                    const float2 sg = e ? make_float2(fs.z, fs.w) : make_float2(fs.x, fs.y);
+                    const float2 qv = e ? make_float2(fq.z, fq.w) : make_float2(fq.x, fq.y);
+                    const float2 de = e ? make_float2(va.y, vb.y) : make_float2(va.x, vb.x);
+                    const float2 dyv = e ? make_float2(yv.y, yv.w) : make_float2(yv.x, yv.z);
+                    const float2 xv = ld2<T>(&r.x[0][0], o);
+                    const float2 ddt = mul2(fma2(xv, tot[1][e], mul2(tot[2][e], splat(kLn2))), sg);
+                    st2<T>(&s.gx[0][0], o, fma2(de, tot[1][e], mul2(dyv, dsk)));
+                    st2<T>(&s.gdt[0][0], o, ddt);
+                    if (gate) st2<T>(&s.gz[0][0], o, mul2(fma2(dsk, xv, tot[0][e]), qv));
+                    dD_acc = fma2(dyv, xv, dD_acc);
+                    db_acc = add2(db_acc, ddt);
+                }
+                __syncwarp();   // the shares may be written again
+            }
+            fence_proxy_async_smem();   // output tiles -> visible to the TMA stores
         }
-        fence_proxy_async_smem();   // output tiles -> visible to the TMA stores
         __syncthreads();
         if (tid == 0) {
-            tma_store_3d(&a.tm_dx, &s.gx[0][0], d0, (int)t0, b);
-            tma_store_3d(&a.tm_ddt, &s.gdt[0][0], d0, (int)t0, b);
-            if (gate) tma_store_3d(&a.tm_dz, &s.gz[0][0], d0, (int)t0, b);
-            bulk_commit();
-            // slot j (chunk i) is converted and consumed: refill it with the
-            // chunk of slot j + S
-            if (j + S < nchunks) {
-                fence_proxy_async_smem();
-                issue_bchunk(s, a, (int)(j % S), nchunks - 1 - (j + S), d0, b);
+            if constexpr (!kSummary) {
+                tma_store_3d(&a.tm_dx, &s.gx[0][0], d0, t0, b);
+                tma_store_3d(&a.tm_ddt, &s.gdt[0][0], d0, t0, b);
+                if (gate) tma_store_3d(&a.tm_dz, &s.gz[0][0], d0, t0, b);
+                bulk_commit();
             }
-            // the output tiles are rewritten after the next conversion
-            // barrier: wait until these stores have read them
-            bulk_wait_read_all();
+            if (it + S < nch) {   // the stage is consumed: refill it
+                fence_proxy_async_smem();
+                issue_bchunk<T, kSummary>(s, a, it % S, c0 + nch - 1 - (it + S), d0, b);
+            }
         }
     }
-    // dB, dC of chunk 0
-    flush_bc(s.bc, gp, b, 0, L);
-
-    // per-channel sums: dD, dbias over the 4 lanes of the channel
-    dD_acc += __shfl_xor_sync(kFull, dD_acc, 8);
-    dD_acc += __shfl_xor_sync(kFull, dD_acc, 16);
-    db_acc += __shfl_xor_sync(kFull, db_acc, 8);
-    db_acc += __shfl_xor_sync(kFull, db_acc, 16);
-    if (chan_ok) {
-        atomicAdd(reinterpret_cast<float4 *>(gp.dA + d * kDState + 4 * q),
-                  make_float4(dA[0].x, dA[0].y, dA[1].x, dA[1].y));
-        if (gp.dh0)
-            *reinterpret_cast<float4 *>(gp.dh0 + ((int64_t)b * D + d) * kDState + 4 * q) =
-                make_float4(g[0].x, g[0].y, g[1].x, g[1].y);
-        if (q == 0) {
-            if (gp.dD) atomicAdd(gp.dD + d, dD_acc);
-            if (gp.ddt_bias) atomicAdd(gp.ddt_bias + d, db_acc);
+    if constexpr (kSummary) {   // Abar g at the segment's start from a zero adjoint at its end; the product of its decays
+        if (!chan_ok) return;
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+            const int64_t o = (((int64_t)b * nseg + seg) * D + d + j) * kDState + 4 * q;
+            const float sd = dsum[j].x + dsum[j].y;
+            float pe[4];
+#pragma unroll
+            for (int n = 0; n < 4; ++n) pe[n] = ex2(a2[j][n] * sd);
+            store_perm(p.seg_h + o, g[j], perm);
+            store_perm(p.seg_p + o, pe, perm);
         }
+    } else {
+        flush_sums(s, gp, b, c0 * kBT, L);   // the last chunk's
+#pragma unroll
+        for (int o = 8; o <= 16; o += 8) {   // over the four lanes of a channel pair
+            dD_acc = add2(dD_acc, shfl2(dD_acc, o));
+            db_acc = add2(db_acc, shfl2(db_acc, o));
+        }
+        if (ts == 0 && dc < D) {
+            if (gp.dD) atomicAdd(reinterpret_cast<float2 *>(gp.dD + dc), dD_acc);
+            if (gp.ddt_bias) atomicAdd(reinterpret_cast<float2 *>(gp.ddt_bias + dc), db_acc);
+        }
+        if (chan_ok) {
+#pragma unroll
+            for (int j = 0; j < 2; ++j) {
+#pragma unroll
+                for (int n = 0; n < 4; ++n)
+                    atomicAdd(gp.dA + (d + j) * kDState + 4 * q + (n ^ perm), dA[j][n].x + dA[j][n].y);
+                if (gp.dh0 && seg == 0)
+                    store_perm(gp.dh0 + ((int64_t)b * D + d + j) * kDState + 4 * q, g[j], perm);
+            }
+        }
+        if (tid == 0) bulk_wait_all();
     }
-    if (tid == 0) bulk_wait_all();
 }
 
 bool make_map3(CUtensorMap *m, const void *base, bool bf16, int64_t batch, int64_t L, int64_t inner,
-               int box_inner, int64_t row = 0) {
+               int box_inner, int64_t row, int swizzle) {
     const int64_t es = bf16 ? 2 : 4;
-    if (row == 0) row = inner;
     const uint64_t dims[3] = {(uint64_t)inner, (uint64_t)L, (uint64_t)batch};
     const uint64_t strides[2] = {(uint64_t)(row * es), (uint64_t)(L * row * es)};
     const uint32_t box[3] = {(uint32_t)box_inner, (uint32_t)kBT, 1};
-    return encode_tmap(m, base, (int)es, 3, dims, strides, box);
+    return encode_tmap(m, base, (int)es, 3, dims, strides, box, swizzle);
 }
 
 template <typename T>
@@ -510,25 +576,59 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
     a.g = g;
     a.has_gate = p.z != nullptr;
     const int64_t Bn = p.batch, L = p.seqlen, D = p.d_inner;
-    if (!make_map3(&a.tm_dt, p.dt, bf16, Bn, L, D, kBCh) || !make_map3(&a.tm_x, p.x, bf16, Bn, L, D, kBCh) ||
-        (p.z && !make_map3(&a.tm_z, p.z, bf16, Bn, L, D, kBCh)) ||
-        !make_map3(&a.tm_dout, g.dout, bf16, Bn, L, D, kBCh) ||
-        !make_map3(&a.tm_B, p.B, bf16, Bn, L, kDState, kDState, p.bc_stride) ||
-        !make_map3(&a.tm_C, p.C, bf16, Bn, L, kDState, kDState, p.bc_stride) ||
-        !make_map3(&a.tm_dx, g.dx, bf16, Bn, L, D, kBCh) || !make_map3(&a.tm_ddt, g.ddt, bf16, Bn, L, D, kBCh) ||
-        (p.z && !make_map3(&a.tm_dz, g.dz, bf16, Bn, L, D, kBCh)))
+    if (p.nseg < 2 || !p.seg_h || !p.seg_p) a.p.nseg = 1;
+    const int64_t nseg = a.p.nseg;
+    auto tok = [&](CUtensorMap *m, const void *base) {
+        return make_map3(m, base, bf16, Bn, L, D, kBCh, D, kBCh * (int)sizeof(T));
+    };
+    if (!tok(&a.tm_dt, p.dt) || !tok(&a.tm_x, p.x) || (p.z && !tok(&a.tm_z, p.z)) || !tok(&a.tm_dout, g.dout) ||
+        !make_map3(&a.tm_B, p.B, bf16, Bn, L, kDState, kDState, p.bc_stride, 0) ||
+        !make_map3(&a.tm_C, p.C, bf16, Bn, L, kDState, kDState, p.bc_stride, 0) || !tok(&a.tm_dx, g.dx) ||
+        !tok(&a.tm_ddt, g.ddt) || (p.z && !tok(&a.tm_dz, g.dz)))
         return cudaErrorInvalidValue;
-    const size_t smem = sizeof(BSmem<T>) + 128;
-    auto k = backward_kernel<T>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const dim3 grid((unsigned)(((D + kBCh - 1) / kBCh) * Bn));
-    e = launch_pdl(false, k, grid, dim3(kBThreads), smem, s, a);
-    if (e != cudaSuccess) return e;
-    return cudaGetLastError();
+    const size_t smem = sizeof(BSmem<T>) + 1024;
+    const int64_t ctas = ((D + kBCh - 1) / kBCh) * Bn;   // per segment of L
+    cudaError_t e;
+    if (nseg > 1) {   // first pass: summaries of segments 1 .. nseg - 1
+        BwdArgs a1 = a;
+        a1.seg0 = 1;
+        a1.grid_segs = (int)(nseg - 1);
+        auto k1 = backward_kernel<T, true>;
+        if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+            return e;
+        if ((e = launch_pdl(false, k1, dim3((unsigned)(ctas * (nseg - 1))), dim3(kBThreads), smem, s, a1)) !=
+            cudaSuccess)
+            return e;
+    }
+    a.grid_segs = (int)nseg;
+    auto k = backward_kernel<T, false>;
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
+    return launch_pdl(false, k, dim3((unsigned)(ctas * nseg)), dim3(kBThreads), smem, s, a);
 }
 
 }  // namespace
+
+// Time split: when the batch rows and channel tiles fill at most half of the
+// resident slots (4 CTAs per SM), into as many segments as fill them, each at
+// least kMinBwdSegChunks chunks long. Only the adjoint is carried across a
+// boundary (the states come from the checkpoints), so the first pass is short:
+// decays and dy C, no sums over channels or states. Measured (2 x 777 x 1544:
+// 98 CTAs) 190 us unsplit, 91 us in 6 segments; with every slot but a few
+// filled (8 x 8192 x 2048: 512 CTAs) 2.63 ms unsplit, 2.90 ms in 6.
+constexpr int64_t kMinBwdSegChunks = 4;
+
+int64_t backward_segments(const ScanParams &p) {
+    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen <= 0 || p.dt_low) return 1;
+    const int64_t slots = (int64_t)device_sms() * 4;
+    const int64_t ctas = p.batch * ((p.d_inner + kBCh - 1) / kBCh);
+    if (2 * ctas > slots) return 1;
+    const int64_t nchunks = (p.seqlen + kBT - 1) / kBT;
+    int64_t nseg = slots / ctas;
+    if (nseg > nchunks / kMinBwdSegChunks) nseg = nchunks / kMinBwdSegChunks;
+    if (nseg < 2) return 1;
+    const int64_t cps = (nchunks + nseg - 1) / nseg;
+    return (nchunks + cps - 1) / cps;   // no empty segment
+}
 
 cudaError_t launch_backward(const ScanParams &p, const GradParams &g, bool bf16, cudaStream_t s) {
     const int64_t Bn = p.batch, L = p.seqlen, D = p.d_inner;

@@ -43,9 +43,8 @@
 #include <stddef.h>
 #include <string.h>
 
-#include <atomic>
-
 #include "common.cuh"
+#include "pairs.cuh"
 #include "tma.cuh"
 
 namespace mbscan {
@@ -94,33 +93,6 @@ struct FwdArgs {
 // 16-byte stores fall on different banks. The scan's loads of all 8 channels at one tp cover 128 bytes either way.
 __device__ __forceinline__ int dg_slot(int tp, int c) { return (((c ^ tp) & 1) << 2) | (c >> 1); }
 
-// Byte offset of channels c, c + 1 of the CTA at step t in a swizzled token tile
-template <typename T>
-__device__ __forceinline__ int tile_off(int t, int c) {
-    constexpr int kRow = kCh * (int)sizeof(T);
-    const int by = c * (int)sizeof(T), x = kRow == 128 ? t & 7 : (t >> 1) & 3;
-    return t * kRow + (((by >> 4) ^ x) << 4) + (by & 15);
-}
-
-template <typename T>
-__device__ __forceinline__ float2 ld2(const void *base, int off) {
-    if constexpr (sizeof(T) == 2) {
-        const unsigned u = *reinterpret_cast<const unsigned *>(static_cast<const char *>(base) + off);
-        return make_float2(__uint_as_float(u << 16), __uint_as_float(u & 0xffff0000u));
-    } else {
-        return *reinterpret_cast<const float2 *>(static_cast<const char *>(base) + off);
-    }
-}
-template <typename T>
-__device__ __forceinline__ void st2(void *base, int off, float2 v) {
-    if constexpr (sizeof(T) == 2) {
-        const __nv_bfloat162 b = __floats2bfloat162_rn(v.x, v.y);
-        *reinterpret_cast<__nv_bfloat162 *>(static_cast<char *>(base) + off) = b;
-    } else {
-        *reinterpret_cast<float2 *>(static_cast<char *>(base) + off) = v;
-    }
-}
-
 template <typename T, bool kSummary>
 __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int stage, int chunk, int d0, int b) {
     constexpr uint32_t tok = kT * kCh * sizeof(T), bc = kT * kDState * sizeof(T);
@@ -134,32 +106,6 @@ __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int st
     if (a.has_gate) tma_load_3d(&r.z[0][0], &a.tm_z, bar, d0, t, b);
     tma_load_3d(&r.B[0][0], &a.tm_B, bar, 0, t, b);
     if (!kSummary) tma_load_3d(&r.C[0][0], &a.tm_C, bar, 0, t, b);
-}
-
-__device__ __forceinline__ float rcp(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// Delta = softplus(v) of a pair, as softplus() of common.cuh
-__device__ __forceinline__ float2 softplus2(float2 v) {
-    const float2 w = mul2(v, make_float2(kLog2e, kLog2e));
-    const float2 u = make_float2(ex2(w.x), ex2(w.y));
-    float2 r = fma2(u, make_float2(0.33333334f, 0.33333334f), make_float2(-0.5f, -0.5f));
-    r = mul2(u, fma2(u, r, make_float2(1.f, 1.f)));
-    const float2 o = add2(u, make_float2(1.f, 1.f));
-    const float2 lw = mul2(make_float2(lg2(o.x), lg2(o.y)), make_float2(kLn2, kLn2));
-    r.x = u.x < 0.03125f ? r.x : lw.x;
-    r.y = u.y < 0.03125f ? r.y : lw.y;
-    return make_float2(v.x > 15.f ? v.x : r.x, v.y > 15.f ? v.y : r.y);
-}
-
-// silu(z) of a pair
-__device__ __forceinline__ float2 silu2(float2 z) {
-    const float2 w = mul2(z, make_float2(-kLog2e, -kLog2e));
-    const float2 d = add2(make_float2(ex2(w.x), ex2(w.y)), make_float2(1.f, 1.f));
-    return mul2(z, make_float2(rcp(d.x), rcp(d.y)));
 }
 
 // kCkpt (training forward): also stores the state before every chunk.
@@ -205,7 +151,7 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
 
     // ---- conversion and output role: channels 8 warp + 2 pp + {0, 1} of the tile, steps 2 tp, 2 tp + 1
     const int pp = lane % kPairs, tp = lane / kPairs;
-    const int off0 = tile_off<T>(2 * tp, kWCh * warp + 2 * pp), off1 = tile_off<T>(2 * tp + 1, kWCh * warp + 2 * pp);
+    const int off0 = tile_off<T, kCh>(2 * tp, kWCh * warp + 2 * pp), off1 = tile_off<T, kCh>(2 * tp + 1, kWCh * warp + 2 * pp);
     float2 bias = make_float2(0.f, 0.f), dsk = make_float2(0.f, 0.f);
     {
         const int64_t dc = (int64_t)d0 + kWCh * warp + 2 * pp;   // D % 8 == 0: both channels valid or neither
@@ -253,8 +199,8 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
         float2 D1 = softplus2(add2(ld2<T>(&r.dt[0][0], off1), bias));
         const int rest = L - t0 - 2 * tp;   // steps left from this pair on
         const float m0 = rest < 1 ? 0.f : 1.f, m1 = rest < 2 ? 0.f : 1.f;
-        D0 = mul2(D0, make_float2(m0, m0));   // Delta = 0 past the end leaves h unchanged
-        D1 = mul2(D1, make_float2(m1, m1));
+        D0 = mul2(D0, splat(m0));   // Delta = 0 past the end leaves h unchanged
+        D1 = mul2(D1, splat(m1));
         const float2 g0 = mul2(D0, x0), g1 = mul2(D1, x1);
         Conv v;
         v.c0 = make_float4(D0.x, D1.x, g0.x, g1.x);
@@ -321,7 +267,7 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
             float2 hp[4];
 #pragma unroll
             for (int n = 0; n < 4; ++n) {
-                const float2 e = mul2(dd, make_float2(a2[n], a2[n]));
+                const float2 e = mul2(dd, splat(a2[n]));
                 const float2 ab = make_float2(ex2(e.x), ex2(e.y));
                 const float2 bg = mul2(bp[n], gg);
                 hp[n].x = fmaf(ab.x, h[n], bg.x);
@@ -457,16 +403,8 @@ constexpr int64_t kMinSegChunks = 8;
 
 int64_t prefill_segments(const ScanParams &p) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen <= 0 || p.dt_low) return 1;
-    constexpr int kMaxDevices = 64;
-    static std::atomic<int> sm_count[kMaxDevices];   // per device, filled on first use (0: not yet)
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 1;
-    int sms = sm_count[dev].load(std::memory_order_relaxed);
-    if (sms == 0) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 1;
-        sm_count[dev].store(sms, std::memory_order_relaxed);   // every writer stores the same value
-    }
-    const int64_t slots = (int64_t)sms * 4;
+    const int64_t sms = device_sms();
+    const int64_t slots = sms * 4;
     const int64_t ctas = p.batch * ((p.d_inner + kCh - 1) / kCh);
     if (ctas > sms) return 1;
     const int64_t nchunks = (p.seqlen + kT - 1) / kT;

@@ -60,6 +60,9 @@ constexpr int kCkptSteps = 16;   // steps between the state checkpoints of the t
 bool encode_tmap(CUtensorMap *m, const void *base, int elem_bytes, int rank, const uint64_t *dims,
                  const uint64_t *strides, const uint32_t *box, int swizzle = 0);
 
+// SMs of the current device; 0 if they cannot be read (no device).
+int device_sms();
+
 constexpr long long kMaxWaitCycles = 4000000000LL;   // the kernels' wait limit (~2 s at 2 GHz)
 
 // Launchers: return the cudaError_t of the launch.
@@ -72,6 +75,8 @@ cudaError_t launch_forward(const ScanParams &p, bool bf16, cudaStream_t s);
 // (1 when the batch rows and channels alone fill the GPU), and the scratch
 // bytes that split needs beyond the status block.
 int64_t prefill_segments(const ScanParams &p);
+// The same for the backward (its adjoint summaries need the same scratch per segment).
+int64_t backward_segments(const ScanParams &p);
 size_t prefill_split_bytes(const ScanParams &p, int64_t nseg);
 cudaError_t launch_verify(const ScanParams &p, bool bf16, cudaStream_t s);
 // Prefill that also writes p.h_ckpt [batch, ceil(L / kCkptSteps), d_inner, 16].

@@ -192,7 +192,8 @@ extern "C" {
 size_t mb_workspace_size(const mb_scan_args *args) {
     if (check_args(args, false, false) != MB_OK) return 0;
     const ScanParams p = to_params(args, nullptr, nullptr);
-    return mbscan::kStatusBytes + mbscan::prefill_split_bytes(p, mbscan::prefill_segments(p));
+    const int64_t fwd = mbscan::prefill_segments(p), bwd = mbscan::backward_segments(p);
+    return mbscan::kStatusBytes + mbscan::prefill_split_bytes(p, fwd > bwd ? fwd : bwd);
 }
 
 mb_status mb_scan_prefill(const mb_scan_args *args, float *h_last, void *ws, size_t ws_bytes,
@@ -431,7 +432,7 @@ mb_status mb_scan_backward(const mb_scan_args *args, const float *h_ckpt, const 
                          range_of(args->D, Dn * 4), range_of(args->dt_bias, Dn * 4), range_of(args->h0, st_b),
                          range_of(h_ckpt, chans * nchunks * N * 4), range_of(dout, tok),
                          range_of(dh_last, st_b), range_of(ws, ws_bytes)};
-    constexpr int kOuts = sizeof(outs) / sizeof(outs[0]);
+    constexpr int kOuts = sizeof(outs) / sizeof(outs[0]), kIns = sizeof(ins) / sizeof(ins[0]);   // ins: ws is the last
     for (int i = 0; i < kOuts; ++i) {
         for (const Range &r : ins)
             if (overlap(outs[i], r)) return MB_ERR_INVALID_ARG;
@@ -439,6 +440,19 @@ mb_status mb_scan_backward(const mb_scan_args *args, const float *h_ckpt, const 
             if (overlap(outs[i], outs[j])) return MB_ERR_INVALID_ARG;
     }
     ScanParams p = to_params(args, nullptr, static_cast<StatusBlock *>(ws));
+    // Split over L when the workspace holds the adjoint summaries and nothing that is read lies there.
+    const int64_t nseg = mbscan::backward_segments(p);
+    const size_t split = mbscan::prefill_split_bytes(p, nseg);
+    if (nseg > 1 && ws_bytes >= mbscan::kStatusBytes + split) {
+        float *scratch = reinterpret_cast<float *>(static_cast<char *>(ws) + mbscan::kStatusBytes);
+        bool clear = true;
+        for (int i = 0; i < kIns - 1; ++i) clear = clear && !overlap(range_of(scratch, (int64_t)split), ins[i]);
+        if (clear) {
+            p.nseg = nseg;
+            p.seg_h = scratch;
+            p.seg_p = scratch + split / (2 * sizeof(float));
+        }
+    }
     mbscan::GradParams gp;
     gp.h_ckpt = h_ckpt;
     gp.dout = dout;

@@ -1,8 +1,10 @@
-// TMA tensor-map encoding shared by the kernels. cuTensorMapEncodeTiled is
+// What the launchers share on the host: TMA tensor-map encoding, the SM count. cuTensorMapEncodeTiled is
 // fetched through the runtime's driver entry point, so the library does not
 // link libcuda directly.
 #include <cuda.h>
 #include <cuda_runtime.h>
+
+#include <atomic>
 
 #include "internal.h"
 
@@ -49,6 +51,19 @@ bool encode_tmap(CUtensorMap *m, const void *base, int elem_bytes, int rank, con
                swizzle == 128 ? CU_TENSOR_MAP_SWIZZLE_128B
                               : (swizzle == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE),
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
+int device_sms() {
+    constexpr int kMaxDevices = 64;
+    static std::atomic<int> count[kMaxDevices];   // per device, filled on first use (0: not yet)
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
+    int sms = count[dev].load(std::memory_order_relaxed);
+    if (sms == 0) {
+        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 0;
+        count[dev].store(sms, std::memory_order_relaxed);   // every writer stores the same value
+    }
+    return sms;
 }
 
 }  // namespace mbscan
