@@ -1,9 +1,12 @@
-"""Build libmbscan.so (the C-ABI CUDA library) in-tree for sm_103a.
+"""Build libmbscan.so (the C-ABI CUDA library) in-tree for sm_103a, and the
+native part of its Python binding.
 
 Each .cu under csrc/ is compiled to an object file by nvcc (in parallel),
 then linked into _build/libmbscan.so with the CUDA runtime linked statically,
 so the library loads on a machine without a GPU (for the export checks) and
-needs nothing but the driver on a GPU machine.
+needs nothing but the driver on a GPU machine. csrc/binding.cpp (argument
+marshalling on torch tensors) is compiled by g++ into _build/_mbcall.so beside
+it; only that file depends on torch.
 
     python -m paper_2401_13660_gb300.build [--force] [--verbose]
 """
@@ -11,15 +14,18 @@ from __future__ import annotations
 
 import argparse
 import concurrent.futures as cf
+import importlib.util
 import os
 import shutil
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.environ.get("MBSCAN_BUILD_DIR") or os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libmbscan.so")
+BINDING = os.path.join(BUILD, "_mbcall.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
@@ -42,13 +48,13 @@ def sources():
 
 def _deps():
     return sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC)
-                        if f.endswith((".cuh", ".h"))] + [os.path.join(INCLUDE, "mbscan.h")]
+                        if f.endswith((".cuh", ".h", ".cpp"))] + [os.path.join(INCLUDE, "mbscan.h")]
 
 
 def up_to_date() -> bool:
-    if not os.path.exists(LIB):
+    if not (os.path.exists(LIB) and os.path.exists(BINDING)):
         return False
-    t = os.path.getmtime(LIB)
+    t = min(os.path.getmtime(LIB), os.path.getmtime(BINDING))
     return all(os.path.getmtime(d) <= t for d in _deps())
 
 
@@ -65,14 +71,31 @@ def _compile(src: str, verbose: bool) -> str:
     return obj
 
 
+def _compile_binding() -> None:
+    torch_dir = os.path.dirname(importlib.util.find_spec("torch").origin)   # found without importing it
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(nvcc())))
+    inc = [INCLUDE, sysconfig.get_paths()["include"], os.path.join(torch_dir, "include"),
+           os.path.join(torch_dir, "include", "torch", "csrc", "api", "include"), os.path.join(cuda, "include")]
+    tmp = BINDING + f".tmp{os.getpid()}"
+    cmd = ["g++", "-O2", "-std=c++20", "-fPIC", "-shared", *(f"-I{d}" for d in inc),
+           os.path.join(CSRC, "binding.cpp"), "-o", tmp, f"-L{os.path.join(torch_dir, 'lib')}",
+           "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch", "-ltorch_python"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError(f"g++ failed on binding.cpp:\n{r.stdout}\n{r.stderr}")
+    os.replace(tmp, BINDING)
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile every kernel for sm_103a and link libmbscan.so; returns its path."""
     if not force and up_to_date():
         return LIB
     os.makedirs(BUILD, exist_ok=True)
     srcs = sources()
-    with cf.ThreadPoolExecutor(max_workers=min(8, len(srcs))) as ex:
+    with cf.ThreadPoolExecutor(max_workers=min(12, len(srcs) + 1)) as ex:
+        binding = ex.submit(_compile_binding)
         objs = list(ex.map(lambda s: _compile(s, verbose), srcs))
+        binding.result()
     tmp = LIB + f".tmp{os.getpid()}"
     cmd = [nvcc(), *ARCH, "-shared", "-cudart", "static", "-o", tmp, *objs]
     r = subprocess.run(cmd, capture_output=True, text=True)
