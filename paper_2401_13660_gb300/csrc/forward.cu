@@ -51,6 +51,7 @@ namespace mbscan {
 namespace {
 
 constexpr int kT = 16;        // steps per chunk
+constexpr int kSegUnit = 32;  // segments of a time split are multiples of this many steps
 constexpr int kTP = kT / 2;   // step pairs per chunk
 constexpr int kWarps = 4;
 constexpr int kThreads = 32 * kWarps;
@@ -59,26 +60,30 @@ constexpr int kCh = kWarps * kWCh;          // channels per CTA
 constexpr int kPairs = kWCh / 2;            // channel pairs per warp
 constexpr int kPartQ = kTP * kPairs + 4;    // float4s between the shares of two lanes q (the pad keeps them on other banks)
 
+constexpr int kStages = 3;
+// Chunks per ring stage, one after the other between two CTA barriers (two for fp32 would leave 2 CTAs per SM)
 template <typename T>
-constexpr int kStages = sizeof(T) == 2 ? 4 : 3;
+constexpr int kSub = sizeof(T) == 2 ? 2 : 1;
+template <typename T>
+constexpr int kRT = kT * kSub<T>;   // steps per stage
 
 template <typename T>
 struct Raw {   // TMA destinations; token tiles swizzled in their 64- (bf16) or 128-byte (fp32) rows
-    T dt[kT][kCh];
-    T x[kT][kCh];
-    T z[kT][kCh];
-    T B[kT][kDState];
-    T C[kT][kDState];
+    T dt[kRT<T>][kCh];
+    T x[kRT<T>][kCh];
+    T z[kRT<T>][kCh];
+    T B[kRT<T>][kDState];
+    T C[kRT<T>][kDState];
 };
 
 template <typename T>
 struct alignas(1024) Smem {
-    Raw<T> raw[kStages<T>];
-    T ys[2][kT][kCh];                              // output tiles (TMA stores), swizzled like the inputs
+    Raw<T> raw[kStages];
+    T ys[2][kRT<T>][kCh];                          // output tiles (TMA stores), swizzled like the inputs
     float4 dg[2][kWarps][kTP][kWCh];   // (Delta_t, Delta_t+1, (Delta x)_t, (Delta x)_t+1), see dg_slot
-    float4 bc[2][2][2][kTP][4];                    // [buffer][B, C][states 4q, 4q+1 or 4q+2, 4q+3][tp][q]
+    float4 bc[2][kSub<T>][2][2][kTP][4];           // [buffer][chunk][B, C][states 4q, 4q+1 or 4q+2, 4q+3][tp][q]
     float4 part[kWarps][4 * kPartQ];   // shares of C.h of lane q: [q][tp][channel pair]
-    uint64_t full[kStages<T>];
+    uint64_t full[kStages];
 };
 
 struct FwdArgs {
@@ -94,12 +99,11 @@ struct FwdArgs {
 __device__ __forceinline__ int dg_slot(int tp, int c) { return (((c ^ tp) & 1) << 2) | (c >> 1); }
 
 template <typename T, bool kSummary>
-__device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int stage, int chunk, int d0, int b) {
-    constexpr uint32_t tok = kT * kCh * sizeof(T), bc = kT * kDState * sizeof(T);
+__device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int stage, int t, int d0, int b) {
+    constexpr uint32_t tok = kRT<T> * kCh * sizeof(T), bc = kRT<T> * kDState * sizeof(T);
     const uint32_t bytes = ((a.has_gate ? 3 : 2) * tok) + (kSummary ? 1 : 2) * bc;
     uint64_t *bar = &s.full[stage];
     mbar_arrive_expect_tx(bar, bytes);
-    const int t = chunk * kT;
     Raw<T> &r = s.raw[stage];
     tma_load_3d(&r.dt[0][0], &a.tm_dt, bar, d0, t, b);
     tma_load_3d(&r.x[0][0], &a.tm_x, bar, d0, t, b);
@@ -118,10 +122,10 @@ template <typename T, bool kCkpt, bool kSummary>
 __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_constant__ FwdArgs a) {
     using S = Smem<T>;
     using R = Raw<T>;
-    constexpr int STAGES = kStages<T>, kRowB = kCh * (int)sizeof(T);
+    constexpr int STAGES = kStages, SUB = kSub<T>, RT = kRT<T>, kRowB = kCh * (int)sizeof(T);
     static_assert(sizeof(R) % (8 * kRowB) == 0 && offsetof(R, x) % (8 * kRowB) == 0 &&
                       offsetof(R, z) % (8 * kRowB) == 0 && offsetof(R, B) % 128 == 0 && offsetof(R, C) % 128 == 0 &&
-                      offsetof(S, ys) % (8 * kRowB) == 0 && sizeof(T) * kT * kCh % (8 * kRowB) == 0,
+                      offsetof(S, ys) % (8 * kRowB) == 0 && sizeof(T) * RT * kCh % (8 * kRowB) == 0,
                   "swizzled TMA tiles start on their pattern's boundary");
     extern __shared__ unsigned char smem_dyn[];
     S &s = *reinterpret_cast<S *>(smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u));
@@ -131,12 +135,12 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
     // blockIdx.x = (batch row, segment of L, channel tile), channel tile fastest
     const int ntd = (int)((D + kCh - 1) / kCh);
     const int L = (int)p.seqlen;
-    const int nchunks = (L + kT - 1) / kT;   // chunks of the whole span
     const int seg = (int)((blockIdx.x / ntd) % a.grid_segs);
     const int b = (int)(blockIdx.x / ntd / a.grid_segs);
     const int nseg = p.nseg > 1 ? (int)p.nseg : 1;
-    const int cps = (nchunks + nseg - 1) / nseg;                        // chunks per segment
-    const int c0 = seg * cps, nch = min(nchunks - c0, cps);             // this CTA's: c0 .. c0 + nch - 1
+    const int units = (L + kSegUnit - 1) / kSegUnit, ups = (units + nseg - 1) / nseg;   // of the span, per segment
+    const int tb = seg * ups * kSegUnit, te = min(L, tb + ups * kSegUnit);              // this CTA's steps: tb .. te - 1
+    const int nch = (te - tb + RT - 1) / RT;                                           // its stages
     const int d0 = (int)(blockIdx.x % ntd) * kCh;
     const bool gate = a.has_gate != 0;
 
@@ -147,7 +151,7 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
     __syncthreads();
     pdl_wait();   // everything below reads or writes global memory
     if (tid == 0)
-        for (int st = 0; st < STAGES && st < nch; ++st) issue_chunk<T, kSummary>(s, a, st, c0 + st, d0, b);
+        for (int st = 0; st < STAGES && st < nch; ++st) issue_chunk<T, kSummary>(s, a, st, tb + st * RT, d0, b);
 
     // ---- conversion and output role: channels 8 warp + 2 pp + {0, 1} of the tile, steps 2 tp, 2 tp + 1
     const int pp = lane % kPairs, tp = lane / kPairs;
@@ -160,7 +164,7 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
             if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
         }
     }
-    // widening role: two states of B or C at a step pair (s.bc in the order of the threads)
+    // widening role: two states of B or C at a step pair of every chunk (s.bc in the order of the threads)
     const int bc_off = ((2 * ((tid >> 2) & 7)) * kDState + 4 * (tid & 3) + 2 * ((tid >> 5) & 1)) * (int)sizeof(T);
     const bool bc_is_c = tid >= 64;
 
@@ -191,34 +195,49 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
     const int slot_e = dg_slot(0, c), slot_o = dg_slot(1, c);
 
     struct Conv {
-        float4 c0, c1, bc;
+        float4 c0, c1;
     };
-    auto convert = [&](const R &r, int t0) {
-        const float2 x0 = ld2<T>(&r.x[0][0], off0), x1 = ld2<T>(&r.x[0][0], off1);
-        float2 D0 = softplus2(add2(ld2<T>(&r.dt[0][0], off0), bias));
-        float2 D1 = softplus2(add2(ld2<T>(&r.dt[0][0], off1), bias));
+    auto convert = [&](const R &r, int sub, int t0) {   // chunk `sub` of a stage, its first step t0
+        constexpr int kSubB = kT * kRowB;
+        const float2 x0 = ld2<T>(&r.x[0][0], off0 + sub * kSubB), x1 = ld2<T>(&r.x[0][0], off1 + sub * kSubB);
+        float2 D0 = softplus2(add2(ld2<T>(&r.dt[0][0], off0 + sub * kSubB), bias));
+        float2 D1 = softplus2(add2(ld2<T>(&r.dt[0][0], off1 + sub * kSubB), bias));
         const int rest = L - t0 - 2 * tp;   // steps left from this pair on
         const float m0 = rest < 1 ? 0.f : 1.f, m1 = rest < 2 ? 0.f : 1.f;
         D0 = mul2(D0, splat(m0));   // Delta = 0 past the end leaves h unchanged
         D1 = mul2(D1, splat(m1));
         const float2 g0 = mul2(D0, x0), g1 = mul2(D1, x1);
-        Conv v;
-        v.c0 = make_float4(D0.x, D1.x, g0.x, g1.x);
-        v.c1 = make_float4(D0.y, D1.y, g0.y, g1.y);
-        const T *src = !kSummary && bc_is_c ? &r.C[0][0] : &r.B[0][0];
-        const float2 v0 = ld2<T>(src, bc_off), v1 = ld2<T>(src, bc_off + kDState * (int)sizeof(T));
-        v.bc = make_float4(v0.x, v1.x, v0.y, v1.y);
-        return v;
+        return Conv{make_float4(D0.x, D1.x, g0.x, g1.x), make_float4(D0.y, D1.y, g0.y, g1.y)};
     };
     auto put = [&](int buf, const Conv &v) {
         s.dg[buf][warp][tp][dg_slot(tp, 2 * pp)] = v.c0;
         s.dg[buf][warp][tp][dg_slot(tp, 2 * pp + 1)] = v.c1;
-        (&s.bc[buf][0][0][0][0])[tid] = v.bc;
+    };
+    struct Wide {
+        float4 v[SUB];
+    };
+    auto widen = [&](const R &r) {
+        Wide w;
+        const T *src = !kSummary && bc_is_c ? &r.C[0][0] : &r.B[0][0];
+#pragma unroll
+        for (int u = 0; u < SUB; ++u) {
+            const int o = bc_off + u * kT * kDState * (int)sizeof(T);
+            const float2 v0 = ld2<T>(src, o), v1 = ld2<T>(src, o + kDState * (int)sizeof(T));
+            w.v[u] = make_float4(v0.x, v1.x, v0.y, v1.y);
+        }
+        return w;
+    };
+    auto put_bc = [&](int buf, const Wide &w) {
+#pragma unroll
+        for (int u = 0; u < SUB; ++u) (&s.bc[buf][u][0][0][0][0])[tid] = w.v[u];
     };
 
-    // ---- prologue: chunk 0
+    // ---- prologue: the first chunk, the first stage's B and C
     bool ok = mbar_wait(&s.full[0], 0);   // nch >= 1
-    if (ok) put(0, convert(s.raw[0], c0 * kT));
+    if (ok) {
+        put(0, convert(s.raw[0], 0, tb));
+        put_bc(0, widen(s.raw[0]));
+    }
     if (__syncthreads_or(ok ? 0 : 1)) {
         if (tid == 0) {
             report(p.status, 4 /* MB_ERR_TIMEOUT */, 0);
@@ -227,85 +246,103 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
         return;
     }
 
-    int st = 0;        // ring stage of chunk i
+    int st = 0;        // ring slot of stage i
     uint32_t ph = 0;   // and its phase parity
     for (int i = 0; i < nch; ++i) {
-        const int t0 = (c0 + i) * kT;
-        // (1) chunk i + 1: wait for its tiles and convert them (stored after the scan below)
+        const int ts = tb + i * RT;   // its first step
+        const R &r = s.raw[st];
         const int nst = st + 1 == STAGES ? 0 : st + 1;
         const uint32_t nph = st + 1 == STAGES ? ph ^ 1u : ph;
-        ok = i + 1 < nch ? mbar_wait(&s.full[nst], nph) : true;
-        const Conv nv = convert(s.raw[nst], t0 + kT);   // past the last chunk: of no use, and not read
-        // (2) chunk i: D x and silu(z) of this lane's outputs
-        const R &r = s.raw[st];
-        float2 xd0, xd1, sz0 = make_float2(1.f, 1.f), sz1 = sz0;
+#pragma unroll
+        for (int sub = 0; sub < SUB; ++sub) {
+            const int t0 = ts + sub * kT;
+            if (sub > 0 && t0 >= te) break;   // the span ends in an earlier chunk of this stage
+            const int buf = SUB == 1 ? i & 1 : sub & 1;
+            // (1) convert the next chunk, of this stage or (waiting for its tiles) the next one; past the last
+            // chunk that is of no use, and not read. Stored after the scan below.
+            const bool last = sub == SUB - 1;
+            if (last) ok = i + 1 < nch ? mbar_wait(&s.full[nst], nph) : true;
+            const Conv nv = last ? convert(s.raw[nst], 0, t0 + kT) : convert(r, sub + 1, t0 + kT);
+            Wide nw;
+            if (last) nw = widen(s.raw[nst]);
+            // (2) D x and silu(z) of this lane's outputs
+            const int o0 = off0 + sub * kT * kRowB, o1 = off1 + sub * kT * kRowB;
+            float2 xd0, xd1, sz0 = splat(1.f), sz1 = sz0;
+            if constexpr (!kSummary) {
+                xd0 = mul2(dsk, ld2<T>(&r.x[0][0], o0));
+                xd1 = mul2(dsk, ld2<T>(&r.x[0][0], o1));
+                if (gate) {
+                    sz0 = silu2(ld2<T>(&r.z[0][0], o0));
+                    sz1 = silu2(ld2<T>(&r.z[0][0], o1));
+                }
+            }
+            if constexpr (kCkpt) {   // state before the chunk, for the backward's recompute
+                static_assert(kT == kCkptSteps, "checkpoints are taken per chunk");
+                const int64_t nck = (L + kT - 1) / kT;
+                if (chan_ok)
+                    *reinterpret_cast<float4 *>(p.h_ckpt + (((int64_t)b * nck + t0 / kT) * D + d) * kDState + 4 * q) =
+                        make_float4(h[0], h[1], h[2], h[3]);
+            }
+            // (3) decays, recurrence, shares of C.h, a step pair at a time
+            const float4(&dgw)[kTP][kWCh] = s.dg[buf][warp];
+            const float4(&bcw)[2][2][kTP][4] = s.bc[i & 1][sub];
+            float2 part[kTP], csum;
+#pragma unroll
+            for (int k = 0; k < kTP; ++k) {
+                const float4 v = dgw[k][(k & 1) ? slot_o : slot_e];
+                const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
+                const float4 b01 = bcw[0][0][k][q], b23 = bcw[0][1][k][q];
+                const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
+                                      make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
+                float2 hp[4];
+#pragma unroll
+                for (int n = 0; n < 4; ++n) {
+                    const float2 e = mul2(dd, splat(a2[n]));
+                    const float2 ab = make_float2(ex2(e.x), ex2(e.y));
+                    const float2 bg = mul2(bp[n], gg);
+                    hp[n].x = fmaf(ab.x, h[n], bg.x);
+                    hp[n].y = fmaf(ab.y, hp[n].x, bg.y);
+                    h[n] = hp[n].y;
+                }
+                if constexpr (kSummary) {
+                    csum = k == 0 ? dd : add2(csum, dd);
+                } else {
+                    const float4 c01 = bcw[1][0][k][q], c23 = bcw[1][1][k][q];
+                    part[k] = mul2(make_float2(c01.x, c01.y), hp[0]);
+                    part[k] = fma2(make_float2(c01.z, c01.w), hp[1], part[k]);
+                    part[k] = fma2(make_float2(c23.x, c23.y), hp[2], part[k]);
+                    part[k] = fma2(make_float2(c23.z, c23.w), hp[3], part[k]);
+                }
+            }
+            if constexpr (kSummary) dsum = add2(dsum, csum);
+            put(buf ^ 1, nv);
+            if (last) put_bc((i + 1) & 1, nw);
+            // (4) add the four lanes' shares of each channel, skip term, gate
+            if constexpr (!kSummary) {
+                float4 *pw = s.part[warp];
+                if (sub > 0) __syncwarp();   // the shares of the chunk before have been read
+#pragma unroll
+                for (int k = 0; k < kTP; ++k) reinterpret_cast<float2 *>(pw + q * kPartQ + k * kPairs)[c] = part[k];
+                __syncwarp();
+                const float4 *src = pw + tp * kPairs + pp;   // (channel, step): (0, 0), (0, 1), (1, 0), (1, 1)
+                const float4 s0 = src[0], s1 = src[kPartQ], s2 = src[2 * kPartQ], s3 = src[3 * kPartQ];
+                const float2 ca = add2(add2(make_float2(s0.x, s0.y), make_float2(s1.x, s1.y)),
+                                       add2(make_float2(s2.x, s2.y), make_float2(s3.x, s3.y)));
+                const float2 cb = add2(add2(make_float2(s0.z, s0.w), make_float2(s1.z, s1.w)),
+                                       add2(make_float2(s2.z, s2.w), make_float2(s3.z, s3.w)));
+                st2<T>(&s.ys[i & 1][0][0], o0, mul2(add2(make_float2(ca.x, cb.x), xd0), sz0));
+                st2<T>(&s.ys[i & 1][0][0], o1, mul2(add2(make_float2(ca.y, cb.y), xd1), sz1));
+            } else if (!last) {
+                __syncwarp();
+            }
+        }
         if constexpr (!kSummary) {
-            xd0 = mul2(dsk, ld2<T>(&r.x[0][0], off0));
-            xd1 = mul2(dsk, ld2<T>(&r.x[0][0], off1));
-            if (gate) {
-                sz0 = silu2(ld2<T>(&r.z[0][0], off0));
-                sz1 = silu2(ld2<T>(&r.z[0][0], off1));
-            }
-        }
-        if constexpr (kCkpt) {   // state before chunk i, for the backward's recompute
-            static_assert(kT == kCkptSteps, "checkpoints are taken per chunk");
-            if (chan_ok)
-                *reinterpret_cast<float4 *>(p.h_ckpt + (((int64_t)b * nchunks + c0 + i) * D + d) * kDState + 4 * q) =
-                    make_float4(h[0], h[1], h[2], h[3]);
-        }
-        // (3) chunk i: decays, recurrence, shares of C.h, a step pair at a time
-        const float4(&dgw)[kTP][kWCh] = s.dg[i & 1][warp];
-        const float4(&bcw)[2][2][kTP][4] = s.bc[i & 1];
-        float2 part[kTP], csum;
-#pragma unroll
-        for (int k = 0; k < kTP; ++k) {
-            const float4 v = dgw[k][(k & 1) ? slot_o : slot_e];
-            const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
-            const float4 b01 = bcw[0][0][k][q], b23 = bcw[0][1][k][q];
-            const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w), make_float2(b23.x, b23.y),
-                                  make_float2(b23.z, b23.w)};
-            float2 hp[4];
-#pragma unroll
-            for (int n = 0; n < 4; ++n) {
-                const float2 e = mul2(dd, splat(a2[n]));
-                const float2 ab = make_float2(ex2(e.x), ex2(e.y));
-                const float2 bg = mul2(bp[n], gg);
-                hp[n].x = fmaf(ab.x, h[n], bg.x);
-                hp[n].y = fmaf(ab.y, hp[n].x, bg.y);
-                h[n] = hp[n].y;
-            }
-            if constexpr (kSummary) {
-                csum = k == 0 ? dd : add2(csum, dd);
-            } else {
-                const float4 c01 = bcw[1][0][k][q], c23 = bcw[1][1][k][q];
-                part[k] = mul2(make_float2(c01.x, c01.y), hp[0]);
-                part[k] = fma2(make_float2(c01.z, c01.w), hp[1], part[k]);
-                part[k] = fma2(make_float2(c23.x, c23.y), hp[2], part[k]);
-                part[k] = fma2(make_float2(c23.z, c23.w), hp[3], part[k]);
-            }
-        }
-        if constexpr (kSummary) dsum = add2(dsum, csum);
-        put((i + 1) & 1, nv);
-        // (4) chunk i: add the four lanes' shares of each channel, skip term, gate
-        if constexpr (!kSummary) {
-            float4 *pw = s.part[warp];
-#pragma unroll
-            for (int k = 0; k < kTP; ++k) reinterpret_cast<float2 *>(pw + q * kPartQ + k * kPairs)[c] = part[k];
-            __syncwarp();
-            const float4 *src = pw + tp * kPairs + pp;   // (channel, step): (0, 0), (0, 1), (1, 0), (1, 1)
-            const float4 s0 = src[0], s1 = src[kPartQ], s2 = src[2 * kPartQ], s3 = src[3 * kPartQ];
-            const float2 ca = add2(add2(make_float2(s0.x, s0.y), make_float2(s1.x, s1.y)),
-                                   add2(make_float2(s2.x, s2.y), make_float2(s3.x, s3.y)));
-            const float2 cb = add2(add2(make_float2(s0.z, s0.w), make_float2(s1.z, s1.w)),
-                                   add2(make_float2(s2.z, s2.w), make_float2(s3.z, s3.w)));
-            st2<T>(&s.ys[i & 1][0][0], off0, mul2(add2(make_float2(ca.x, cb.x), xd0), sz0));
-            st2<T>(&s.ys[i & 1][0][0], off1, mul2(add2(make_float2(ca.y, cb.y), xd1), sz1));
             fence_proxy_async_smem();   // y tile -> visible to the TMA store below
-            if (tid == 0) bulk_wait_read_all();   // the store of chunk i - 1 no longer reads its tile
+            if (tid == 0) bulk_wait_read_all();   // the store of stage i - 1 no longer reads its tile
         }
         if (__syncthreads_or(ok ? 0 : 1)) {
             if (tid == 0) {
-                report(p.status, 4 /* MB_ERR_TIMEOUT */, c0 + i + 1);
+                report(p.status, 4 /* MB_ERR_TIMEOUT */, i + 1);
                 for (int j = i + 1; j < i + STAGES && j < nch; ++j)
                     mbar_wait(&s.full[j % STAGES], (uint32_t)((j / STAGES) & 1));
                 bulk_wait_all();
@@ -314,12 +351,12 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
         }
         if (tid == 0) {
             if constexpr (!kSummary) {
-                tma_store_3d(&a.tm_y, &s.ys[i & 1][0][0], d0, t0, b);
+                tma_store_3d(&a.tm_y, &s.ys[i & 1][0][0], d0, ts, b);
                 bulk_commit();
             }
-            if (i + STAGES < nch) {   // stage st is free: refill it with chunk i + STAGES
+            if (i + STAGES < nch) {   // the slot is free: refill it with stage i + STAGES
                 fence_proxy_async_smem();
-                issue_chunk<T, kSummary>(s, a, st, c0 + i + STAGES, d0, b);
+                issue_chunk<T, kSummary>(s, a, st, tb + (i + STAGES) * RT, d0, b);
             }
         }
         st = nst;
@@ -343,13 +380,13 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
 // ---------------------------------------------------------------------------
 // Host side: tensor maps and the launch.
 
-// [batch, L, inner] tensor with a (box_inner x kT x 1) box; rows (b, t) are
+// [batch, L, inner] tensor with a (box_inner x rows x 1) box; rows (b, t) are
 // `row` elements apart (row >= inner).
 bool make_map(CUtensorMap *m, const void *base, int es, int64_t batch, int64_t L, int64_t inner, int box_inner,
-              int64_t row, int swizzle) {
+              int64_t row, int swizzle, int rows) {
     const uint64_t dims[3] = {(uint64_t)inner, (uint64_t)L, (uint64_t)batch};
     const uint64_t strides[2] = {(uint64_t)(row * es), (uint64_t)(L * row * es)};
-    const uint32_t box[3] = {(uint32_t)box_inner, (uint32_t)kT, 1};
+    const uint32_t box[3] = {(uint32_t)box_inner, (uint32_t)rows, 1};
     return encode_tmap(m, base, es, 3, dims, strides, box, swizzle);
 }
 
@@ -363,11 +400,11 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     if (p.nseg < 2 || !p.seg_h || !p.seg_p) a.p.nseg = 1;
     const int64_t nseg = a.p.nseg, D = p.d_inner;
     auto tok = [&](CUtensorMap *m, const void *base) {
-        return make_map(m, base, es, p.batch, p.seqlen, D, kCh, D, sw);
+        return make_map(m, base, es, p.batch, p.seqlen, D, kCh, D, sw, kRT<T>);
     };
     if (!tok(&a.tm_dt, p.dt) || !tok(&a.tm_x, p.x) || (p.z && !tok(&a.tm_z, p.z)) || !tok(&a.tm_y, p.y) ||
-        !make_map(&a.tm_B, p.B, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0) ||
-        !make_map(&a.tm_C, p.C, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0))
+        !make_map(&a.tm_B, p.B, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0, kRT<T>) ||
+        !make_map(&a.tm_C, p.C, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0, kRT<T>))
         return cudaErrorInvalidValue;
     const size_t smem = sizeof(Smem<T>) + 1024;
     const int64_t ctas = ((D + kCh - 1) / kCh) * p.batch;   // per segment of L
@@ -395,11 +432,11 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
 // Time split: only when the batch rows and channel tiles give at most one CTA
 // per SM (a CTA alone on an SM leaves most of its issue slots idle); then into
 // as many segments as fill the resident slots (4 per SM),
-// each at least kMinSegChunks chunks long. The summary pass repeats most of a
+// each at least kMinSegSteps long. The summary pass repeats most of a
 // scan, so at 1.7 CTAs per SM (batch 4 x 2048 channels) the split measured
 // slower (604 -> 653 us) while batch 1 x 2048 channels x 8192 steps went
 // 480 -> 180 us (both before the layout above, which took the latter to 152).
-constexpr int64_t kMinSegChunks = 8;
+constexpr int64_t kMinSegSteps = 128;
 
 int64_t prefill_segments(const ScanParams &p) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen <= 0 || p.dt_low) return 1;
@@ -407,12 +444,12 @@ int64_t prefill_segments(const ScanParams &p) {
     const int64_t slots = sms * 4;
     const int64_t ctas = p.batch * ((p.d_inner + kCh - 1) / kCh);
     if (ctas > sms) return 1;
-    const int64_t nchunks = (p.seqlen + kT - 1) / kT;
+    const int64_t units = (p.seqlen + kSegUnit - 1) / kSegUnit;
     int64_t nseg = slots / ctas;
-    if (nseg > nchunks / kMinSegChunks) nseg = nchunks / kMinSegChunks;
+    if (nseg > p.seqlen / kMinSegSteps) nseg = p.seqlen / kMinSegSteps;
     if (nseg < 2) return 1;
-    const int64_t cps = (nchunks + nseg - 1) / nseg;
-    return (nchunks + cps - 1) / cps;   // no empty segment
+    const int64_t ups = (units + nseg - 1) / nseg;
+    return (units + ups - 1) / ups;   // no empty segment
 }
 
 size_t prefill_split_bytes(const ScanParams &p, int64_t nseg) {
