@@ -138,6 +138,8 @@ mb_status mb_scan_prefill(const mb_scan_args *args, float *h_last, void *ws, siz
  *   h_all[b, j, d, n] = state after drafted byte j (j = 0..k-1), fp32,
  *   shape [batch, k, d_inner, d_state]; y as in prefill.
  * h_all must not alias h0.
+ * The kernel lets the next one launch while its last blocks drain (the launch
+ * overlap described at mb_step; mb_scan_verify_resume too).
  */
 mb_status mb_scan_verify(const mb_scan_args *args, float *h_all, void *ws, size_t ws_bytes,
                          void *stream);
@@ -189,7 +191,8 @@ mb_status mb_rollback(const float *h0, const float *h_all, const int32_t *accept
  *   accept  : [streams] int32 output, the index of the first drafted byte that
  *             is not accepted, or k when all are; this is the accept count
  *             that mb_rollback takes.
- * Device pointers; logits 16-byte aligned.
+ * Device pointers; logits 16-byte aligned. Launched with the launch overlap
+ * described at mb_step.
  */
 mb_status mb_accept_topk(const void *logits, int32_t dtype, const uint8_t *drafted, int64_t streams,
                          int64_t k, int32_t beta, int32_t *accept, void *stream);

@@ -44,15 +44,20 @@ __global__ void __launch_bounds__(32 * kAccWarps) accept_kernel(const T *__restr
     const int64_t s = blockIdx.x;
     if (threadIdx.x == 0) first_reject = (int)k;
     __syncthreads();
+    pdl_trigger();   // a step that resumes from these counts may set up meanwhile
     pdl_wait();
     for (int64_t base = 0; base < k; base += kAccWarps) {
         const int64_t i = base + warp;
         if (i < k) {
             const T *row = logits + (s * k + i) * 256;
             const int byte = __ldg(drafted + s * k + i);
-            const float target = to_f32(row[byte]);
             float v[8];
             load8(row + 8 * lane, v);
+            // the drafted byte's own score, from the lane that has it (no second, dependent load)
+            const float w0 = byte & 1 ? v[1] : v[0], w1 = byte & 1 ? v[3] : v[2], w2 = byte & 1 ? v[5] : v[4],
+                        w3 = byte & 1 ? v[7] : v[6];
+            const float u0 = byte & 2 ? w1 : w0, u1 = byte & 2 ? w3 : w2;
+            const float target = __shfl_sync(kFull, byte & 4 ? u1 : u0, byte >> 3);
             int greater = 0;
 #pragma unroll
             for (int j = 0; j < 8; ++j) greater += v[j] > target ? 1 : 0;
@@ -74,9 +79,9 @@ cudaError_t launch_accept(const void *logits, bool bf16, const uint8_t *drafted,
     if (streams == 0) return cudaSuccess;
     const unsigned grid = (unsigned)streams;
     if (bf16)
-        return launch_pdl(false, accept_kernel<__nv_bfloat16>, dim3(grid), dim3(32 * kAccWarps), 0, s,
+        return launch_pdl(true, accept_kernel<__nv_bfloat16>, dim3(grid), dim3(32 * kAccWarps), 0, s,
                           static_cast<const __nv_bfloat16 *>(logits), drafted, k, beta, accept);
-    return launch_pdl(false, accept_kernel<float>, dim3(grid), dim3(32 * kAccWarps), 0, s,
+    return launch_pdl(true, accept_kernel<float>, dim3(grid), dim3(32 * kAccWarps), 0, s,
                       static_cast<const float *>(logits), drafted, k, beta, accept);
 }
 

@@ -538,6 +538,7 @@ __global__ void __launch_bounds__(kBThreads, 4) backward_kernel(const __grid_con
             }
         }
     }
+    if constexpr (kSummary) pdl_trigger();   // the second pass may set up while the last summaries are written
     if constexpr (kSummary) {   // Abar g at the segment's start from a zero adjoint at its end; the product of its decays
         if (!chan_ok) return;
 #pragma unroll
@@ -637,7 +638,7 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
     a.grid_segs = (int)nseg;
     auto k = backward_kernel<T, false>;
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    return launch_pdl(nseg < 2, k, dim3((unsigned)(ctas * nseg)), dim3(kBThreads), smem, s, a);
+    return launch_pdl(true, k, dim3((unsigned)(ctas * nseg)), dim3(kBThreads), smem, s, a);
 }
 
 }  // namespace

@@ -362,6 +362,7 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
         st = nst;
         ph = nph;
     }
+    if constexpr (kSummary) pdl_trigger();   // the second pass may set up while the last summaries are written
     if (tid == 0) bulk_wait_all();
 
     if (!chan_ok) return;
@@ -424,7 +425,7 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     auto k = forward_kernel<T, kCkpt, false>;
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    return launch_pdl(false, k, dim3((unsigned)(ctas * nseg)), dim3(kThreads), smem, s, a);
+    return launch_pdl(nseg > 1, k, dim3((unsigned)(ctas * nseg)), dim3(kThreads), smem, s, a);
 }
 
 }  // namespace

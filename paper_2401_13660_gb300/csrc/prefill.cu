@@ -523,6 +523,7 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
             }
         }
     }
+    pdl_trigger();   // late: what follows may be launched while the last CTAs drain
     if (tid == 0) bulk_wait_all();
 
     if (!kStoreAll && p.h_out && chan_ok) {   // the span's last state
