@@ -49,6 +49,7 @@
 // longer first pass over the states) 2.63 ms, eighths 4.28 ms; both halves
 // unrolled 3.38 ms (spills); states of the halves in registers instead of
 // shared memory 2.74 ms.
+#include <math.h>
 #include <stddef.h>
 #include <string.h>
 
@@ -645,21 +646,25 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
 
 // Time split: when the batch rows and channel tiles fill at most half of the
 // resident slots (4 CTAs per SM), into as many segments as fill them, each at
-// least kMinBwdSegChunks chunks long. Only the adjoint is carried across a
-// boundary (the states come from the checkpoints), so the first pass is short:
-// decays and dy C, no sums over channels or states. Measured (2 x 777 x 1544:
-// 98 CTAs) 190 us unsplit, 91 us in 6 segments; with every slot but a few
+// least two chunks long. Only the adjoint is carried across a boundary (the
+// states come from the checkpoints), so the first pass is short: decays and
+// dy C, no sums over channels or states. Every lane folds the segments after
+// its own; beyond sqrt(2 L) segments that costs more than shorter segments
+// give. Measured: 2 x 777 x 1544 (98 CTAs) 156 us unsplit, 66 in 5 segments;
+// 1 x 8192 x 64 1537 us unsplit, 53 in 128, 84 in 256; with the slots nearly
 // filled (8 x 8192 x 2048: 512 CTAs) 2.63 ms unsplit, 2.90 ms in 6.
-constexpr int64_t kMinBwdSegChunks = 4;
+constexpr int64_t kMinBwdSplitSteps = 128;
 
 int64_t backward_segments(const ScanParams &p) {
-    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen <= 0 || p.dt_low) return 1;
+    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinBwdSplitSteps || p.dt_low) return 1;
     const int64_t slots = (int64_t)device_sms() * 4;
     const int64_t ctas = p.batch * ((p.d_inner + kBCh - 1) / kBCh);
     if (2 * ctas > slots) return 1;
     const int64_t nchunks = (p.seqlen + kBT - 1) / kBT;
     int64_t nseg = slots / ctas;
-    if (nseg > nchunks / kMinBwdSegChunks) nseg = nchunks / kMinBwdSegChunks;
+    const int64_t most = (int64_t)sqrt(2.0 * (double)p.seqlen);
+    if (nseg > most) nseg = most;
+    if (nseg > nchunks / 2) nseg = nchunks / 2;
     if (nseg < 2) return 1;
     const int64_t cps = (nchunks + nseg - 1) / nseg;
     return (nchunks + cps - 1) / cps;   // no empty segment

@@ -40,6 +40,7 @@
 // -> 152 us, fp32 3 x 1003 x 1544 56 -> 48 us. Two channels per lane (B and C
 // loaded once for both: 17 % fewer wavefronts) measured 758 / 750 us on the
 // first two: half the warps; two-warp CTAs (16 channels) 784 / 640 us.
+#include <math.h>
 #include <stddef.h>
 #include <string.h>
 
@@ -431,23 +432,28 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
 }  // namespace
 
 // Time split: only when the batch rows and channel tiles give at most one CTA
-// per SM (a CTA alone on an SM leaves most of its issue slots idle); then into
-// as many segments as fill the resident slots (4 per SM),
-// each at least kMinSegSteps long. The summary pass repeats most of a
-// scan, so at 1.7 CTAs per SM (batch 4 x 2048 channels) the split measured
-// slower (604 -> 653 us) while batch 1 x 2048 channels x 8192 steps went
-// 480 -> 180 us (both before the layout above, which took the latter to 152).
-constexpr int64_t kMinSegSteps = 128;
+// per SM (a CTA alone on an SM leaves most of its issue slots idle; the summary
+// pass repeats most of a scan, so at 1.7 CTAs per SM, batch 4 x 2048 channels,
+// the split measured slower) and the span is long enough to pay for the second
+// launch: at 128 steps x 2048 channels unsplit 8.5 us, split 10.3; at 256 steps
+// 14.4 and 12.3. Then into as many segments as fill the resident slots (4 per
+// SM), each at least kSegUnit long. Every lane folds the summaries before its
+// segment, about 0.07 us each, while a step costs about 0.1 us over both passes:
+// their sum is least at sqrt(1.4 L) segments, which bounds spans of very few
+// channels (8192 x 64: 86 segments 20 us, 256 segments 35 us, 16 segments 37 us;
+// fp32 256 x 64: 8 segments 8.4 us, 2 segments 14.4 us).
+constexpr int64_t kMinSplitSteps = 256;
 
 int64_t prefill_segments(const ScanParams &p) {
-    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen <= 0 || p.dt_low) return 1;
+    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinSplitSteps || p.dt_low) return 1;
     const int64_t sms = device_sms();
-    const int64_t slots = sms * 4;
     const int64_t ctas = p.batch * ((p.d_inner + kCh - 1) / kCh);
     if (ctas > sms) return 1;
     const int64_t units = (p.seqlen + kSegUnit - 1) / kSegUnit;
-    int64_t nseg = slots / ctas;
-    if (nseg > p.seqlen / kMinSegSteps) nseg = p.seqlen / kMinSegSteps;
+    int64_t nseg = 4 * sms / ctas;
+    const int64_t most = (int64_t)sqrt(1.4 * (double)p.seqlen);
+    if (nseg > most) nseg = most;
+    if (nseg > units) nseg = units;
     if (nseg < 2) return 1;
     const int64_t ups = (units + nseg - 1) / nseg;
     return (units + ups - 1) / ups;   // no empty segment
