@@ -25,6 +25,10 @@
  *    MB_ERR_INVALID_ARG or MB_ERR_UNSUPPORTED; nothing is launched then.
  *    A failed launch returns MB_ERR_CUDA.
  *  - Outputs must not alias inputs unless stated.
+ *  - Calls overlap the tail of the kernel before them where that is safe (each
+ *    waits for it before touching memory), and several let the next kernel
+ *    launch before they complete: the launch overlap described at mb_step
+ *    holds for all of them. Plainly launched work is ordered as usual.
  *  - Supported today: d_state == 16, dtype MB_F32 or MB_BF16,
  *    d_inner % 8 == 0, batch*seqlen*d_inner <= 2^31.
  */
@@ -138,8 +142,6 @@ mb_status mb_scan_prefill(const mb_scan_args *args, float *h_last, void *ws, siz
  *   h_all[b, j, d, n] = state after drafted byte j (j = 0..k-1), fp32,
  *   shape [batch, k, d_inner, d_state]; y as in prefill.
  * h_all must not alias h0.
- * The kernel lets the next one launch while its last blocks drain (the launch
- * overlap described at mb_step; mb_scan_verify_resume too).
  */
 mb_status mb_scan_verify(const mb_scan_args *args, float *h_all, void *ws, size_t ws_bytes,
                          void *stream);
@@ -191,8 +193,7 @@ mb_status mb_rollback(const float *h0, const float *h_all, const int32_t *accept
  *   accept  : [streams] int32 output, the index of the first drafted byte that
  *             is not accepted, or k when all are; this is the accept count
  *             that mb_rollback takes.
- * Device pointers; logits 16-byte aligned. Launched with the launch overlap
- * described at mb_step.
+ * Device pointers; logits 16-byte aligned.
  */
 mb_status mb_accept_topk(const void *logits, int32_t dtype, const uint8_t *drafted, int64_t streams,
                          int64_t k, int32_t beta, int32_t *accept, void *stream);

@@ -69,6 +69,7 @@ constexpr int kBWCh = 16;                  // channels per warp, two per lane
 constexpr int kBPairs = kBWCh / 2;
 constexpr int kBCh = kBWarps * kBWCh;      // channels per CTA
 constexpr int kBStages = 2;
+constexpr int kBResident = 4;              // CTAs per SM (registers)
 constexpr int kShareQ = kHTP * kBPairs + 2;   // float4s between the shares of two lanes q (the pad moves them to other banks)
 
 template <typename T>
@@ -165,7 +166,7 @@ __device__ __forceinline__ void flush_sums(const BSmem<T> &s, const GradParams &
 }
 
 template <typename T, bool kSummary>
-__global__ void __launch_bounds__(kBThreads, 4) backward_kernel(const __grid_constant__ BwdArgs a) {
+__global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const __grid_constant__ BwdArgs a) {
     constexpr int S = kBStages, kRowB = kBCh * (int)sizeof(T);
     using R = BRaw<T>;
     using SM = BSmem<T>;
@@ -623,6 +624,8 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
         !tok(&a.tm_ddt, g.ddt) || (p.z && !tok(&a.tm_dz, g.dz)))
         return cudaErrorInvalidValue;
     const size_t smem = sizeof(BSmem<T>) + 1024;
+    const DeviceLimits *lim = device_limits();
+    if (!lim) return cudaErrorInvalidDevice;
     const int64_t ctas = ((D + kBCh - 1) / kBCh) * Bn;   // per segment of L
     cudaError_t e;
     if (nseg > 1) {   // first pass: summaries of segments 1 .. nseg - 1
@@ -630,16 +633,20 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
         a1.seg0 = 1;
         a1.grid_segs = (int)(nseg - 1);
         auto k1 = backward_kernel<T, true>;
-        if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
+            cudaSuccess)
             return e;
-        if ((e = launch_pdl(true, k1, dim3((unsigned)(ctas * (nseg - 1))), dim3(kBThreads), smem, s, a1)) !=
+        const int64_t grid = ctas * (nseg - 1);
+        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kBThreads), spread_smem(smem, grid, kBResident), s, a1)) !=
             cudaSuccess)
             return e;
     }
     a.grid_segs = (int)nseg;
     auto k = backward_kernel<T, false>;
-    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess) return e;
-    return launch_pdl(true, k, dim3((unsigned)(ctas * nseg)), dim3(kBThreads), smem, s, a);
+    if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) != cudaSuccess)
+        return e;
+    return launch_pdl(true, k, dim3((unsigned)(ctas * nseg)), dim3(kBThreads),
+                      spread_smem(smem, ctas * nseg, kBResident), s, a);
 }
 
 }  // namespace
@@ -657,7 +664,7 @@ constexpr int64_t kMinBwdSplitSteps = 128;
 
 int64_t backward_segments(const ScanParams &p) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinBwdSplitSteps || p.dt_low) return 1;
-    const int64_t slots = (int64_t)device_sms() * 4;
+    const int64_t slots = (int64_t)device_sms() * kBResident;
     const int64_t ctas = p.batch * ((p.d_inner + kBCh - 1) / kBCh);
     if (2 * ctas > slots) return 1;
     const int64_t nchunks = (p.seqlen + kBT - 1) / kBT;
@@ -687,7 +694,7 @@ cudaError_t launch_backward(const ScanParams &p, const GradParams &g, bool bf16,
     if (most > 0) {
         const int64_t want = (most + kClearThreads - 1) / kClearThreads, cap = 8 * (int64_t)device_sms();
         const int64_t grid = want < cap || cap == 0 ? want : cap;
-        if ((e = launch_pdl(false, clear_kernel, dim3((unsigned)grid), dim3(kClearThreads), 0, s, c)) != cudaSuccess)
+        if ((e = launch_pdl(true, clear_kernel, dim3((unsigned)grid), dim3(kClearThreads), 0, s, c)) != cudaSuccess)
             return e;
     }
     if (Bn == 0 || D == 0) return cudaSuccess;

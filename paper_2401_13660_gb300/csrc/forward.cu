@@ -62,6 +62,7 @@ constexpr int kPairs = kWCh / 2;            // channel pairs per warp
 constexpr int kPartQ = kTP * kPairs + 4;    // float4s between the shares of two lanes q (the pad keeps them on other banks)
 
 constexpr int kStages = 3;
+constexpr int kResident = 4;   // CTAs per SM (shared memory and the register bound)
 // Chunks per ring stage, one after the other between two CTA barriers (two for fp32 would leave 2 CTAs per SM)
 template <typename T>
 constexpr int kSub = sizeof(T) == 2 ? 2 : 1;
@@ -120,7 +121,7 @@ __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int st
 // pass (the plain kernel) segment s starts from those, folded with the
 // associative operator of Section 2: h <- P_s' * h + H_s'.
 template <typename T, bool kCkpt, bool kSummary>
-__global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_constant__ FwdArgs a) {
+__global__ void __launch_bounds__(kThreads, kResident) forward_kernel(const __grid_constant__ FwdArgs a) {
     using S = Smem<T>;
     using R = Raw<T>;
     constexpr int STAGES = kStages, SUB = kSub<T>, RT = kRT<T>, kRowB = kCh * (int)sizeof(T);
@@ -316,6 +317,9 @@ __global__ void __launch_bounds__(kThreads, 4) forward_kernel(const __grid_const
                 }
             }
             if constexpr (kSummary) dsum = add2(dsum, csum);
+            // Not needed for order (other slots are read above): it keeps these stores behind the scan, 717 -> 711 us
+            // on 8 x 8192 x 2048.
+            if (!last) __syncwarp();
             put(buf ^ 1, nv);
             if (last) put_bc((i + 1) & 1, nw);
             // (4) add the four lanes' shares of each channel, skip term, gate
@@ -409,6 +413,8 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
         !make_map(&a.tm_C, p.C, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0, kRT<T>))
         return cudaErrorInvalidValue;
     const size_t smem = sizeof(Smem<T>) + 1024;
+    const DeviceLimits *lim = device_limits();
+    if (!lim) return cudaErrorInvalidDevice;
     const int64_t ctas = ((D + kCh - 1) / kCh) * p.batch;   // per segment of L
     cudaError_t e;
     if (nseg > 1) {   // first pass: summaries of segments 0 .. nseg-2
@@ -416,17 +422,20 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
         a1.has_gate = 0;   // no outputs: the gate is not read
         a1.grid_segs = (int)(nseg - 1);
         auto k1 = forward_kernel<T, false, true>;
-        if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+        if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
+            cudaSuccess)
             return e;
-        if ((e = launch_pdl(false, k1, dim3((unsigned)(ctas * (nseg - 1))), dim3(kThreads), smem, s, a1)) !=
+        const int64_t grid = ctas * (nseg - 1);
+        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kThreads), spread_smem(smem, grid, kResident), s, a1)) !=
             cudaSuccess)
             return e;
     }
     a.grid_segs = (int)nseg;
     auto k = forward_kernel<T, kCkpt, false>;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin);
     if (e != cudaSuccess) return e;
-    return launch_pdl(nseg > 1, k, dim3((unsigned)(ctas * nseg)), dim3(kThreads), smem, s, a);
+    return launch_pdl(true, k, dim3((unsigned)(ctas * nseg)), dim3(kThreads), spread_smem(smem, ctas * nseg, kResident), s,
+                      a);
 }
 
 }  // namespace
@@ -450,7 +459,7 @@ int64_t prefill_segments(const ScanParams &p) {
     const int64_t ctas = p.batch * ((p.d_inner + kCh - 1) / kCh);
     if (ctas > sms) return 1;
     const int64_t units = (p.seqlen + kSegUnit - 1) / kSegUnit;
-    int64_t nseg = 4 * sms / ctas;
+    int64_t nseg = kResident * sms / ctas;
     const int64_t most = (int64_t)sqrt(1.4 * (double)p.seqlen);
     if (nseg > most) nseg = most;
     if (nseg > units) nseg = units;

@@ -60,8 +60,19 @@ constexpr int kCkptSteps = 16;   // steps between the state checkpoints of the t
 bool encode_tmap(CUtensorMap *m, const void *base, int elem_bytes, int rank, const uint64_t *dims,
                  const uint64_t *strides, const uint32_t *box, int swizzle = 0);
 
-// SMs of the current device; 0 if they cannot be read (no device).
-int device_sms();
+// Limits of the current device, read once per device; null if they cannot be read (no device).
+struct DeviceLimits {
+    int sms;
+    size_t smem_sm, smem_reserved, smem_optin;   // shared memory per SM; reserved per CTA; most per CTA
+};
+const DeviceLimits *device_limits();
+int device_sms();   // 0 if there is no device
+// Dynamic shared memory to ask for, at least `smem`, so that a grid of less
+// than `per` CTAs per SM (the resident limit at `smem`) is spread evenly: left
+// to itself the block scheduler puts up to `per` of them on the SMs that are
+// free first and leaves others idle, above all when the launch overlaps the
+// tail of the kernel before.
+size_t spread_smem(size_t smem, int64_t grid, int per);
 
 constexpr long long kMaxWaitCycles = 4000000000LL;   // the kernels' wait limit (~2 s at 2 GHz)
 

@@ -583,9 +583,13 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     const size_t smem = sizeof(Smem<T, kCh, STAGES, kFuse, kWideBC<T, kStoreAll>>) + 128 + fuse_bytes;
     const int64_t ctas = ((p.d_inner + kCh - 1) / kCh) * p.batch;
     auto k = prefill_kernel<T, LPC, STAGES, kStoreAll, kFuse>;
-    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const DeviceLimits *lim = device_limits();
+    if (!lim) return cudaErrorInvalidDevice;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin);
     if (e != cudaSuccess) return e;
-    return launch_pdl(false, k, dim3((unsigned)ctas), dim3(kThreads), smem, s, a);
+    // verify: overlaps the tail of the kernel before it
+    const size_t ask = kStoreAll ? spread_smem(smem, ctas, kFuse ? MB_VERIFY_FUSED_MINB : MB_VERIFY_MINB) : smem;
+    return launch_pdl(kStoreAll, k, dim3((unsigned)ctas), dim3(kThreads), ask, s, a);
 }
 
 }  // namespace

@@ -1,10 +1,11 @@
-// What the launchers share on the host: TMA tensor-map encoding, the SM count. cuTensorMapEncodeTiled is
+// What the launchers share on the host: TMA tensor-map encoding, device limits. cuTensorMapEncodeTiled is
 // fetched through the runtime's driver entry point, so the library does not
 // link libcuda directly.
 #include <cuda.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
+#include <mutex>
 
 #include "internal.h"
 
@@ -53,17 +54,42 @@ bool encode_tmap(CUtensorMap *m, const void *base, int elem_bytes, int rank, con
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-int device_sms() {
+const DeviceLimits *device_limits() {
     constexpr int kMaxDevices = 64;
-    static std::atomic<int> count[kMaxDevices];   // per device, filled on first use (0: not yet)
+    static DeviceLimits lim[kMaxDevices];
+    static std::atomic<int> ready[kMaxDevices];   // 0: not read yet, 1: lim[] is filled
+    static std::mutex mu;
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 0;
-    int sms = count[dev].load(std::memory_order_relaxed);
-    if (sms == 0) {
-        if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || sms <= 0) return 0;
-        count[dev].store(sms, std::memory_order_relaxed);   // every writer stores the same value
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    if (!ready[dev].load(std::memory_order_acquire)) {
+        std::lock_guard<std::mutex> guard(mu);
+        if (!ready[dev].load(std::memory_order_relaxed)) {
+            int v[4];
+            const cudaDeviceAttr attr[4] = {cudaDevAttrMultiProcessorCount, cudaDevAttrMaxSharedMemoryPerMultiprocessor,
+                                            cudaDevAttrReservedSharedMemoryPerBlock,
+                                            cudaDevAttrMaxSharedMemoryPerBlockOptin};
+            for (int i = 0; i < 4; ++i)
+                if (cudaDeviceGetAttribute(&v[i], attr[i], dev) != cudaSuccess) return nullptr;
+            if (v[0] <= 0) return nullptr;
+            lim[dev] = DeviceLimits{v[0], (size_t)v[1], (size_t)v[2], (size_t)v[3]};
+            ready[dev].store(1, std::memory_order_release);
+        }
     }
-    return sms;
+    return &lim[dev];
+}
+
+int device_sms() {
+    const DeviceLimits *l = device_limits();
+    return l ? l->sms : 0;
+}
+
+size_t spread_smem(size_t smem, int64_t grid, int per) {
+    const DeviceLimits *l = device_limits();
+    if (!l) return smem;
+    const int64_t m = (grid + l->sms - 1) / l->sms;
+    if (m >= per) return smem;
+    const size_t want = l->smem_sm / (size_t)(m + 1) - l->smem_reserved + 128;   // m of these fit, m + 1 do not
+    return want > smem && want <= l->smem_optin ? want : smem;
 }
 
 }  // namespace mbscan

@@ -212,24 +212,32 @@ __global__ void __launch_bounds__(kXpThreads) conv_xproj_kernel(const __grid_con
 // 64 groups of four adjacent outputs x 4 interleaved subsets of the splits
 // (subset q sums splits q, q + 4, ... in order); the four subset sums are then
 // added in order q = 0..3, so the result does not depend on timing.
+constexpr int kRedLoads = 9;   // loads in flight per thread: all of a subset's at width 4608 (36 splits)
 constexpr int kRedQuads = 64, kRedSub = 4, kRedThreads = kRedQuads * kRedSub;
 __global__ void __launch_bounds__(kRedThreads) xproj_reduce_kernel(const float *__restrict__ part,
                                                                   __nv_bfloat16 *__restrict__ out,
                                                                   int64_t quads, int splits) {
     __shared__ float4 sub[kRedSub][kRedQuads];
+    pdl_trigger();   // the Delta GEMM that follows when a model decodes may set up meanwhile (it waits, as CUDA requires)
     pdl_wait();
     const int qi = threadIdx.x % kRedQuads, q = threadIdx.x / kRedQuads;
     const int64_t i = (int64_t)blockIdx.x * kRedQuads + qi;
     float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
     if (i < quads) {
         const float4 *p = reinterpret_cast<const float4 *>(part) + i;
-#pragma unroll 4
-        for (int k = q; k < splits; k += kRedSub) {
-            const float4 v = __ldg(p + (int64_t)k * quads);
-            s.x += v.x;
-            s.y += v.y;
-            s.z += v.z;
-            s.w += v.w;
+        for (int k0 = q; k0 < splits; k0 += kRedSub * kRedLoads) {
+            float4 v[kRedLoads];
+#pragma unroll
+            for (int u = 0; u < kRedLoads; ++u)
+                if (k0 + u * kRedSub < splits) v[u] = __ldg(p + (int64_t)(k0 + u * kRedSub) * quads);
+#pragma unroll
+            for (int u = 0; u < kRedLoads; ++u) {
+                if (k0 + u * kRedSub >= splits) break;
+                s.x += v[u].x;
+                s.y += v[u].y;
+                s.z += v[u].z;
+                s.w += v[u].w;
+            }
         }
     }
     sub[q][qi] = s;
