@@ -109,15 +109,17 @@ typedef struct {
 } mb_scan_args;
 
 /* Bytes of device workspace to pass with `args`: a 256-byte status block
- * (written by bounded device-side waits), plus, when the batch rows and
- * channels of a long span fill less than half of the GPU, scratch that lets
- * mb_scan_prefill split the span over L (two passes: per-segment summaries,
- * then the scan of every segment from its folded start state; Section 2's
- * associative operator). Any workspace of at least 256 bytes is accepted: a
- * smaller one than this runs such spans unsplit. The caller allocates it
- * (256-byte aligned) and may reuse it across calls on one stream; calls that
- * overlap on the GPU need distinct workspaces. Returns 0 for invalid
- * arguments. */
+ * (written by bounded device-side waits), plus scratch for the spans that run
+ * faster with it: when the batch rows and channels of a long span fill only
+ * part of the GPU, prefill and backward split it over L (two passes:
+ * per-segment summaries, then every segment from its folded start; Section
+ * 2's associative operator); when they fill it unevenly, prefill runs in equal
+ * shares that hand the state on where a share ends inside a channel's span.
+ * Any workspace of at least 256 bytes is accepted: with a smaller one than
+ * this such spans run as they are. The scratch needs no clearing. The caller
+ * allocates it (256-byte aligned) and may reuse it across calls on one stream;
+ * calls that overlap on the GPU need distinct workspaces. Returns 0 for
+ * invalid arguments. */
 size_t mb_workspace_size(const mb_scan_args *args);
 
 /*

@@ -86,6 +86,7 @@ struct alignas(1024) Smem {
     float4 bc[2][kSub<T>][2][2][kTP][4];           // [buffer][chunk][B, C][states 4q, 4q+1 or 4q+2, 4q+3][tp][q]
     float4 part[kWarps][4 * kPartQ];   // shares of C.h of lane q: [q][tp][channel pair]
     uint64_t full[kStages];
+    int ticket;
 };
 
 struct FwdArgs {
@@ -99,6 +100,18 @@ struct FwdArgs {
 // the other, eight lanes (four pp, two tp) at a time: the two halves change places on odd tp, so that these eight
 // 16-byte stores fall on different banks. The scan's loads of all 8 channels at one tp cover 128 bytes either way.
 __device__ __forceinline__ int dg_slot(int tp, int c) { return (((c ^ tp) & 1) << 2) | (c >> 1); }
+
+// A share's flag in global memory: set after its state has been written, and waited for (bounded).
+__device__ __forceinline__ void flag_set(int *f) { asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(f) : "memory"); }
+__device__ __forceinline__ bool flag_wait(const int *f) {
+    const long long t0 = clock64();
+    for (;;) {
+        int v;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+        if (v) return true;
+        if (clock64() - t0 > kWaitCycles) return false;
+    }
+}
 
 template <typename T, bool kSummary>
 __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int stage, int t, int d0, int b) {
@@ -120,8 +133,16 @@ __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int st
 // product of its decays, 2^(A log2 e * sum of Delta); no outputs. In the second
 // pass (the plain kernel) segment s starts from those, folded with the
 // associative operator of Section 2: h <- P_s' * h + H_s'.
-template <typename T, bool kCkpt, bool kSummary>
-__global__ void __launch_bounds__(kThreads, kResident) forward_kernel(const __grid_constant__ FwdArgs a) {
+// kShares: the grid is p.shares CTAs; the channel tiles' spans, laid end to end,
+// are cut into that many equal lengths, and a CTA scans the pieces in its own,
+// the highest first. Its highest piece starts a tile (or it is all of a CTA's
+// part of one) and depends on nothing; where it ends inside a tile, the CTA
+// leaves the state for the next share. Only its lowest piece may start inside a
+// tile: it comes last and waits (bounded) for the state that the share before
+// has left as the first thing it did. Shares are numbered in the order in which
+// their CTAs start (a ticket), so the one waited for is always running.
+template <typename T, bool kCkpt, bool kSummary, bool kShares = false>
+__global__ void __launch_bounds__(kThreads, kShares ? kResident - 1 : kResident) forward_kernel(const __grid_constant__ FwdArgs a) {
     using S = Smem<T>;
     using R = Raw<T>;
     constexpr int STAGES = kStages, SUB = kSub<T>, RT = kRT<T>, kRowB = kCh * (int)sizeof(T);
@@ -137,13 +158,9 @@ __global__ void __launch_bounds__(kThreads, kResident) forward_kernel(const __gr
     // blockIdx.x = (batch row, segment of L, channel tile), channel tile fastest
     const int ntd = (int)((D + kCh - 1) / kCh);
     const int L = (int)p.seqlen;
-    const int seg = (int)((blockIdx.x / ntd) % a.grid_segs);
-    const int b = (int)(blockIdx.x / ntd / a.grid_segs);
+    const int seg = kShares ? 0 : (int)((blockIdx.x / ntd) % a.grid_segs);
     const int nseg = p.nseg > 1 ? (int)p.nseg : 1;
     const int units = (L + kSegUnit - 1) / kSegUnit, ups = (units + nseg - 1) / nseg;   // of the span, per segment
-    const int tb = seg * ups * kSegUnit, te = min(L, tb + ups * kSegUnit);              // this CTA's steps: tb .. te - 1
-    const int nch = (te - tb + RT - 1) / RT;                                           // its stages
-    const int d0 = (int)(blockIdx.x % ntd) * kCh;
     const bool gate = a.has_gate != 0;
 
     if (tid == 0) {
@@ -152,235 +169,291 @@ __global__ void __launch_bounds__(kThreads, kResident) forward_kernel(const __gr
     }
     __syncthreads();
     pdl_wait();   // everything below reads or writes global memory
-    if (tid == 0)
-        for (int st = 0; st < STAGES && st < nch; ++st) issue_chunk<T, kSummary>(s, a, st, tb + st * RT, d0, b);
 
-    // ---- conversion and output role: channels 8 warp + 2 pp + {0, 1} of the tile, steps 2 tp, 2 tp + 1
-    const int pp = lane % kPairs, tp = lane / kPairs;
-    const int off0 = tile_off<T, kCh>(2 * tp, kWCh * warp + 2 * pp), off1 = tile_off<T, kCh>(2 * tp + 1, kWCh * warp + 2 * pp);
-    float2 bias = make_float2(0.f, 0.f), dsk = make_float2(0.f, 0.f);
-    {
-        const int64_t dc = (int64_t)d0 + kWCh * warp + 2 * pp;   // D % 8 == 0: both channels valid or neither
-        if (dc < D) {
-            if (p.dt_bias) bias = __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc));
-            if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
-        }
-    }
-    // widening role: two states of B or C at a step pair of every chunk (s.bc in the order of the threads)
-    const int bc_off = ((2 * ((tid >> 2) & 7)) * kDState + 4 * (tid & 3) + 2 * ((tid >> 5) & 1)) * (int)sizeof(T);
-    const bool bc_is_c = tid >= 64;
-
-    // ---- scan role: channel c of the warp, states 4 q .. 4 q + 3 (the lane order of the file comment)
-    const int c = (lane & 1) | ((lane >> 1) & 6), q = ((lane >> 1) & 1) | ((lane >> 4) << 1);
-    const int64_t d = (int64_t)d0 + kWCh * warp + c;
-    const bool chan_ok = d < D;
-    float h[4], a2[4];
-    float2 dsum = make_float2(0.f, 0.f);   // kSummary: sum of Delta over even and odd steps
-    {
-        float4 av = make_float4(0.f, 0.f, 0.f, 0.f), hv = av;
-        if (chan_ok) {
-            av = ldg4(p.A + d * kDState + 4 * q);
-            if (seg == 0 && p.h0) hv = ldg4(p.h0 + ((int64_t)b * D + d) * kDState + 4 * q);
-            if constexpr (!kSummary) {
-                for (int sp = 0; sp < seg; ++sp) {
-                    const int64_t o = (((int64_t)b * nseg + sp) * D + d) * kDState + 4 * q;
-                    const float4 he = *reinterpret_cast<const float4 *>(p.seg_h + o);
-                    const float4 pe = *reinterpret_cast<const float4 *>(p.seg_p + o);
-                    hv = sp == 0 ? he : make_float4(fmaf(pe.x, hv.x, he.x), fmaf(pe.y, hv.y, he.y),
-                                                    fmaf(pe.z, hv.z, he.z), fmaf(pe.w, hv.w, he.w));
-                }
-            }
-        }
-        a2[0] = av.x * kLog2e; a2[1] = av.y * kLog2e; a2[2] = av.z * kLog2e; a2[3] = av.w * kLog2e;
-        h[0] = hv.x; h[1] = hv.y; h[2] = hv.z; h[3] = hv.w;
-    }
-    const int slot_e = dg_slot(0, c), slot_o = dg_slot(1, c);
-
-    struct Conv {
-        float4 c0, c1;
-    };
-    auto convert = [&](const R &r, int sub, int t0) {   // chunk `sub` of a stage, its first step t0
-        constexpr int kSubB = kT * kRowB;
-        const float2 x0 = ld2<T>(&r.x[0][0], off0 + sub * kSubB), x1 = ld2<T>(&r.x[0][0], off1 + sub * kSubB);
-        float2 D0 = softplus2(add2(ld2<T>(&r.dt[0][0], off0 + sub * kSubB), bias));
-        float2 D1 = softplus2(add2(ld2<T>(&r.dt[0][0], off1 + sub * kSubB), bias));
-        const int rest = L - t0 - 2 * tp;   // steps left from this pair on
-        const float m0 = rest < 1 ? 0.f : 1.f, m1 = rest < 2 ? 0.f : 1.f;
-        D0 = mul2(D0, splat(m0));   // Delta = 0 past the end leaves h unchanged
-        D1 = mul2(D1, splat(m1));
-        const float2 g0 = mul2(D0, x0), g1 = mul2(D1, x1);
-        return Conv{make_float4(D0.x, D1.x, g0.x, g1.x), make_float4(D0.y, D1.y, g0.y, g1.y)};
-    };
-    auto put = [&](int buf, const Conv &v) {
-        s.dg[buf][warp][tp][dg_slot(tp, 2 * pp)] = v.c0;
-        s.dg[buf][warp][tp][dg_slot(tp, 2 * pp + 1)] = v.c1;
-    };
-    struct Wide {
-        float4 v[SUB];
-    };
-    auto widen = [&](const R &r) {
-        Wide w;
-        const T *src = !kSummary && bc_is_c ? &r.C[0][0] : &r.B[0][0];
-#pragma unroll
-        for (int u = 0; u < SUB; ++u) {
-            const int o = bc_off + u * kT * kDState * (int)sizeof(T);
-            const float2 v0 = ld2<T>(src, o), v1 = ld2<T>(src, o + kDState * (int)sizeof(T));
-            w.v[u] = make_float4(v0.x, v1.x, v0.y, v1.y);
-        }
-        return w;
-    };
-    auto put_bc = [&](int buf, const Wide &w) {
-#pragma unroll
-        for (int u = 0; u < SUB; ++u) (&s.bc[buf][u][0][0][0][0])[tid] = w.v[u];
-    };
-
-    // ---- prologue: the first chunk, the first stage's B and C
-    bool ok = mbar_wait(&s.full[0], 0);   // nch >= 1
-    if (ok) {
-        put(0, convert(s.raw[0], 0, tb));
-        put_bc(0, widen(s.raw[0]));
-    }
-    if (__syncthreads_or(ok ? 0 : 1)) {
-        if (tid == 0) {
-            report(p.status, 4 /* MB_ERR_TIMEOUT */, 0);
-            for (int j = 0; j < STAGES && j < nch; ++j) mbar_wait(&s.full[j], 0);
-        }
-        return;
-    }
-
-    int st = 0;        // ring slot of stage i
+    int st = 0;        // ring slot of the next stage
     uint32_t ph = 0;   // and its phase parity
-    for (int i = 0; i < nch; ++i) {
-        const int ts = tb + i * RT;   // its first step
-        const R &r = s.raw[st];
-        const int nst = st + 1 == STAGES ? 0 : st + 1;
-        const uint32_t nph = st + 1 == STAGES ? ph ^ 1u : ph;
-#pragma unroll
-        for (int sub = 0; sub < SUB; ++sub) {
-            const int t0 = ts + sub * kT;
-            if (sub > 0 && t0 >= te) break;   // the span ends in an earlier chunk of this stage
-            const int buf = SUB == 1 ? i & 1 : sub & 1;
-            // (1) convert the next chunk, of this stage or (waiting for its tiles) the next one; past the last
-            // chunk that is of no use, and not read. Stored after the scan below.
-            const bool last = sub == SUB - 1;
-            if (last) ok = i + 1 < nch ? mbar_wait(&s.full[nst], nph) : true;
-            const Conv nv = last ? convert(s.raw[nst], 0, t0 + kT) : convert(r, sub + 1, t0 + kT);
-            Wide nw;
-            if (last) nw = widen(s.raw[nst]);
-            // (2) D x and silu(z) of this lane's outputs
-            const int o0 = off0 + sub * kT * kRowB, o1 = off1 + sub * kT * kRowB;
-            float2 xd0, xd1, sz0 = splat(1.f), sz1 = sz0;
-            if constexpr (!kSummary) {
-                xd0 = mul2(dsk, ld2<T>(&r.x[0][0], o0));
-                xd1 = mul2(dsk, ld2<T>(&r.x[0][0], o1));
-                if (gate) {
-                    sz0 = silu2(ld2<T>(&r.z[0][0], o0));
-                    sz1 = silu2(ld2<T>(&r.z[0][0], o1));
-                }
-            }
-            if constexpr (kCkpt) {   // state before the chunk, for the backward's recompute
-                static_assert(kT == kCkptSteps, "checkpoints are taken per chunk");
-                const int64_t nck = (L + kT - 1) / kT;
-                if (chan_ok)
-                    *reinterpret_cast<float4 *>(p.h_ckpt + (((int64_t)b * nck + t0 / kT) * D + d) * kDState + 4 * q) =
-                        make_float4(h[0], h[1], h[2], h[3]);
-            }
-            // (3) decays, recurrence, shares of C.h, a step pair at a time
-            const float4(&dgw)[kTP][kWCh] = s.dg[buf][warp];
-            const float4(&bcw)[2][2][kTP][4] = s.bc[i & 1][sub];
-            float2 part[kTP], csum;
-#pragma unroll
-            for (int k = 0; k < kTP; ++k) {
-                const float4 v = dgw[k][(k & 1) ? slot_o : slot_e];
-                const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
-                const float4 b01 = bcw[0][0][k][q], b23 = bcw[0][1][k][q];
-                const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
-                                      make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
-                float2 hp[4];
-#pragma unroll
-                for (int n = 0; n < 4; ++n) {
-                    const float2 e = mul2(dd, splat(a2[n]));
-                    const float2 ab = make_float2(ex2(e.x), ex2(e.y));
-                    const float2 bg = mul2(bp[n], gg);
-                    hp[n].x = fmaf(ab.x, h[n], bg.x);
-                    hp[n].y = fmaf(ab.y, hp[n].x, bg.y);
-                    h[n] = hp[n].y;
-                }
-                if constexpr (kSummary) {
-                    csum = k == 0 ? dd : add2(csum, dd);
-                } else {
-                    const float4 c01 = bcw[1][0][k][q], c23 = bcw[1][1][k][q];
-                    part[k] = mul2(make_float2(c01.x, c01.y), hp[0]);
-                    part[k] = fma2(make_float2(c01.z, c01.w), hp[1], part[k]);
-                    part[k] = fma2(make_float2(c23.x, c23.y), hp[2], part[k]);
-                    part[k] = fma2(make_float2(c23.z, c23.w), hp[3], part[k]);
-                }
-            }
-            if constexpr (kSummary) dsum = add2(dsum, csum);
-            // Not needed for order (other slots are read above): it keeps these stores behind the scan, 717 -> 711 us
-            // on 8 x 8192 x 2048.
-            if (!last) __syncwarp();
-            put(buf ^ 1, nv);
-            if (last) put_bc((i + 1) & 1, nw);
-            // (4) add the four lanes' shares of each channel, skip term, gate
-            if constexpr (!kSummary) {
-                float4 *pw = s.part[warp];
-                if (sub > 0) __syncwarp();   // the shares of the chunk before have been read
-#pragma unroll
-                for (int k = 0; k < kTP; ++k) reinterpret_cast<float2 *>(pw + q * kPartQ + k * kPairs)[c] = part[k];
-                __syncwarp();
-                const float4 *src = pw + tp * kPairs + pp;   // (channel, step): (0, 0), (0, 1), (1, 0), (1, 1)
-                const float4 s0 = src[0], s1 = src[kPartQ], s2 = src[2 * kPartQ], s3 = src[3 * kPartQ];
-                const float2 ca = add2(add2(make_float2(s0.x, s0.y), make_float2(s1.x, s1.y)),
-                                       add2(make_float2(s2.x, s2.y), make_float2(s3.x, s3.y)));
-                const float2 cb = add2(add2(make_float2(s0.z, s0.w), make_float2(s1.z, s1.w)),
-                                       add2(make_float2(s2.z, s2.w), make_float2(s3.z, s3.w)));
-                st2<T>(&s.ys[i & 1][0][0], o0, mul2(add2(make_float2(ca.x, cb.x), xd0), sz0));
-                st2<T>(&s.ys[i & 1][0][0], o1, mul2(add2(make_float2(ca.y, cb.y), xd1), sz1));
-            } else if (!last) {
-                __syncwarp();
+    // this CTA's tile (batch row, 32 channels); with kShares the units of 32 steps lo .. hi - 1 of all tiles' spans
+    // end to end, which it takes tile by tile from the highest
+    int tile = (int)(blockIdx.x / ntd / a.grid_segs) * ntd + (int)(blockIdx.x % ntd);
+    int share = 0, lo = 0, hi = 0;
+    if constexpr (kShares) {
+        if (tid == 0) s.ticket = atomicAdd(p.share_sync, 1);
+        __syncthreads();
+        share = s.ticket;
+        const int total = (int)p.batch * ntd * units, len = (total + (int)p.shares - 1) / (int)p.shares;
+        lo = min(share * len, total);
+        hi = min(lo + len, total);
+        if (lo == hi) return;
+        tile = (hi - 1) / units;
+    }
+    for (;;) {   // pieces: one without kShares
+        const int b = tile / ntd, d0 = (tile % ntd) * kCh;
+        const int tb = kShares ? max(lo - tile * units, 0) * kSegUnit : seg * ups * kSegUnit;   // its steps: tb .. te - 1
+        const int te = min(L, kShares ? (hi - tile * units) * kSegUnit : tb + ups * kSegUnit);
+        const int nch = (te - tb + RT - 1) / RT;                                               // its stages
+        if (tid == 0) {
+            fence_proxy_async_smem();
+            for (int j = 0, sl = st; j < STAGES && j < nch; ++j, sl = sl + 1 == STAGES ? 0 : sl + 1)
+                issue_chunk<T, kSummary>(s, a, sl, tb + j * RT, d0, b);
+        }
+
+        // ---- conversion and output role: channels 8 warp + 2 pp + {0, 1} of the tile, steps 2 tp, 2 tp + 1
+        const int pp = lane % kPairs, tp = lane / kPairs;
+        const int off0 = tile_off<T, kCh>(2 * tp, kWCh * warp + 2 * pp), off1 = tile_off<T, kCh>(2 * tp + 1, kWCh * warp + 2 * pp);
+        float2 bias = make_float2(0.f, 0.f), dsk = make_float2(0.f, 0.f);
+        {
+            const int64_t dc = (int64_t)d0 + kWCh * warp + 2 * pp;   // D % 8 == 0: both channels valid or neither
+            if (dc < D) {
+                if (p.dt_bias) bias = __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc));
+                if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
             }
         }
-        if constexpr (!kSummary) {
-            fence_proxy_async_smem();   // y tile -> visible to the TMA store below
-            if (tid == 0) bulk_wait_read_all();   // the store of stage i - 1 no longer reads its tile
+        // widening role: two states of B or C at a step pair of every chunk (s.bc in the order of the threads)
+        const int bc_off = ((2 * ((tid >> 2) & 7)) * kDState + 4 * (tid & 3) + 2 * ((tid >> 5) & 1)) * (int)sizeof(T);
+        const bool bc_is_c = tid >= 64;
+
+        // ---- scan role: channel c of the warp, states 4 q .. 4 q + 3 (the lane order of the file comment)
+        const int c = (lane & 1) | ((lane >> 1) & 6), q = ((lane >> 1) & 1) | ((lane >> 4) << 1);
+        const int64_t d = (int64_t)d0 + kWCh * warp + c;
+        const bool chan_ok = d < D;
+        float h[4], a2[4];
+        float2 dsum = make_float2(0.f, 0.f);   // kSummary: sum of Delta over even and odd steps
+        {
+            float4 av = make_float4(0.f, 0.f, 0.f, 0.f), hv = av;
+            if (chan_ok) {
+                av = ldg4(p.A + d * kDState + 4 * q);
+                if (seg == 0 && tb == 0 && p.h0) hv = ldg4(p.h0 + ((int64_t)b * D + d) * kDState + 4 * q);
+                if constexpr (!kSummary) {
+                    for (int sp = 0; sp < seg; ++sp) {
+                        const int64_t o = (((int64_t)b * nseg + sp) * D + d) * kDState + 4 * q;
+                        const float4 he = *reinterpret_cast<const float4 *>(p.seg_h + o);
+                        const float4 pe = *reinterpret_cast<const float4 *>(p.seg_p + o);
+                        hv = sp == 0 ? he : make_float4(fmaf(pe.x, hv.x, he.x), fmaf(pe.y, hv.y, he.y),
+                                                        fmaf(pe.z, hv.z, he.z), fmaf(pe.w, hv.w, he.w));
+                    }
+                }
+            }
+            a2[0] = av.x * kLog2e; a2[1] = av.y * kLog2e; a2[2] = av.z * kLog2e; a2[3] = av.w * kLog2e;
+            h[0] = hv.x; h[1] = hv.y; h[2] = hv.z; h[3] = hv.w;
+        }
+        const int slot_e = dg_slot(0, c), slot_o = dg_slot(1, c);
+
+        struct Conv {
+            float4 c0, c1;
+        };
+        auto convert = [&](const R &r, int sub, int t0) {   // chunk `sub` of a stage, its first step t0
+            constexpr int kSubB = kT * kRowB;
+            const float2 x0 = ld2<T>(&r.x[0][0], off0 + sub * kSubB), x1 = ld2<T>(&r.x[0][0], off1 + sub * kSubB);
+            float2 D0 = softplus2(add2(ld2<T>(&r.dt[0][0], off0 + sub * kSubB), bias));
+            float2 D1 = softplus2(add2(ld2<T>(&r.dt[0][0], off1 + sub * kSubB), bias));
+            const int rest = L - t0 - 2 * tp;   // steps left from this pair on
+            const float m0 = rest < 1 ? 0.f : 1.f, m1 = rest < 2 ? 0.f : 1.f;
+            D0 = mul2(D0, splat(m0));   // Delta = 0 past the end leaves h unchanged
+            D1 = mul2(D1, splat(m1));
+            const float2 g0 = mul2(D0, x0), g1 = mul2(D1, x1);
+            return Conv{make_float4(D0.x, D1.x, g0.x, g1.x), make_float4(D0.y, D1.y, g0.y, g1.y)};
+        };
+        auto put = [&](int buf, const Conv &v) {
+            s.dg[buf][warp][tp][dg_slot(tp, 2 * pp)] = v.c0;
+            s.dg[buf][warp][tp][dg_slot(tp, 2 * pp + 1)] = v.c1;
+        };
+        struct Wide {
+            float4 v[SUB];
+        };
+        auto widen = [&](const R &r) {
+            Wide w;
+            const T *src = !kSummary && bc_is_c ? &r.C[0][0] : &r.B[0][0];
+#pragma unroll
+            for (int u = 0; u < SUB; ++u) {
+                const int o = bc_off + u * kT * kDState * (int)sizeof(T);
+                const float2 v0 = ld2<T>(src, o), v1 = ld2<T>(src, o + kDState * (int)sizeof(T));
+                w.v[u] = make_float4(v0.x, v1.x, v0.y, v1.y);
+            }
+            return w;
+        };
+        auto put_bc = [&](int buf, const Wide &w) {
+#pragma unroll
+            for (int u = 0; u < SUB; ++u) (&s.bc[buf][u][0][0][0][0])[tid] = w.v[u];
+        };
+
+        // ---- prologue: the first chunk, the first stage's B and C
+        bool ok = mbar_wait(&s.full[st], ph);   // nch >= 1
+        if (ok) {
+            put(0, convert(s.raw[st], 0, tb));
+            put_bc(0, widen(s.raw[st]));
+        }
+        if constexpr (kShares) {
+            if (tid == 0) {
+                bulk_wait_read_all();   // the piece before's last store no longer reads its output tile
+                if (tb > 0) ok = flag_wait(p.share_sync + share) && ok;   // share - 1's flag
+            }
         }
         if (__syncthreads_or(ok ? 0 : 1)) {
             if (tid == 0) {
-                report(p.status, 4 /* MB_ERR_TIMEOUT */, i + 1);
-                for (int j = i + 1; j < i + STAGES && j < nch; ++j)
-                    mbar_wait(&s.full[j % STAGES], (uint32_t)((j / STAGES) & 1));
+                report(p.status, 4 /* MB_ERR_TIMEOUT */, 0);
+                for (int j = 0; j < STAGES && j < nch; ++j) {
+                    mbar_wait(&s.full[st], ph);
+                    st = st + 1 == STAGES ? 0 : st + 1;
+                    ph ^= st == 0 ? 1u : 0u;
+                }
                 bulk_wait_all();
             }
             return;
         }
-        if (tid == 0) {
-            if constexpr (!kSummary) {
-                tma_store_3d(&a.tm_y, &s.ys[i & 1][0][0], d0, ts, b);
-                bulk_commit();
-            }
-            if (i + STAGES < nch) {   // the slot is free: refill it with stage i + STAGES
-                fence_proxy_async_smem();
-                issue_chunk<T, kSummary>(s, a, st, tb + (i + STAGES) * RT, d0, b);
+        if constexpr (kShares) {
+            if (tb > 0 && chan_ok) {
+                const float4 hv = __ldcg(reinterpret_cast<const float4 *>(
+                    p.share_h + ((int64_t)(share - 1) * kCh + kWCh * warp + c) * kDState + 4 * q));
+                h[0] = hv.x; h[1] = hv.y; h[2] = hv.z; h[3] = hv.w;
             }
         }
-        st = nst;
-        ph = nph;
-    }
-    if constexpr (kSummary) pdl_trigger();   // the second pass may set up while the last summaries are written
-    if (tid == 0) bulk_wait_all();
 
-    if (!chan_ok) return;
-    if constexpr (kSummary) {
-        const int64_t o = (((int64_t)b * nseg + seg) * D + d) * kDState + 4 * q;
-        const float sd = dsum.x + dsum.y;
-        *reinterpret_cast<float4 *>(p.seg_h + o) = make_float4(h[0], h[1], h[2], h[3]);
-        *reinterpret_cast<float4 *>(p.seg_p + o) =
-            make_float4(ex2(a2[0] * sd), ex2(a2[1] * sd), ex2(a2[2] * sd), ex2(a2[3] * sd));
-    } else if (p.h_out && seg == nseg - 1) {   // the span's last state
-        *reinterpret_cast<float4 *>(p.h_out + ((int64_t)b * D + d) * kDState + 4 * q) =
-            make_float4(h[0], h[1], h[2], h[3]);
+        for (int i = 0; i < nch; ++i) {
+            const int ts = tb + i * RT;   // its first step
+            const R &r = s.raw[st];
+            const int nst = st + 1 == STAGES ? 0 : st + 1;
+            const uint32_t nph = st + 1 == STAGES ? ph ^ 1u : ph;
+#pragma unroll
+            for (int sub = 0; sub < SUB; ++sub) {
+                const int t0 = ts + sub * kT;
+                if (sub > 0 && t0 >= te) break;   // the span ends in an earlier chunk of this stage
+                const int buf = SUB == 1 ? i & 1 : sub & 1;
+                // (1) convert the next chunk, of this stage or (waiting for its tiles) the next one; past the last
+                // chunk that is of no use, and not read. Stored after the scan below.
+                const bool last = sub == SUB - 1;
+                if (last) ok = i + 1 < nch ? mbar_wait(&s.full[nst], nph) : true;
+                const Conv nv = last ? convert(s.raw[nst], 0, t0 + kT) : convert(r, sub + 1, t0 + kT);
+                Wide nw;
+                if (last) nw = widen(s.raw[nst]);
+                // (2) D x and silu(z) of this lane's outputs
+                const int o0 = off0 + sub * kT * kRowB, o1 = off1 + sub * kT * kRowB;
+                float2 xd0, xd1, sz0 = splat(1.f), sz1 = sz0;
+                if constexpr (!kSummary) {
+                    xd0 = mul2(dsk, ld2<T>(&r.x[0][0], o0));
+                    xd1 = mul2(dsk, ld2<T>(&r.x[0][0], o1));
+                    if (gate) {
+                        sz0 = silu2(ld2<T>(&r.z[0][0], o0));
+                        sz1 = silu2(ld2<T>(&r.z[0][0], o1));
+                    }
+                }
+                if constexpr (kCkpt) {   // state before the chunk, for the backward's recompute
+                    static_assert(kT == kCkptSteps, "checkpoints are taken per chunk");
+                    const int64_t nck = (L + kT - 1) / kT;
+                    if (chan_ok)
+                        *reinterpret_cast<float4 *>(p.h_ckpt + (((int64_t)b * nck + t0 / kT) * D + d) * kDState + 4 * q) =
+                            make_float4(h[0], h[1], h[2], h[3]);
+                }
+                // (3) decays, recurrence, shares of C.h, a step pair at a time
+                const float4(&dgw)[kTP][kWCh] = s.dg[buf][warp];
+                const float4(&bcw)[2][2][kTP][4] = s.bc[i & 1][sub];
+                float2 part[kTP], csum;
+#pragma unroll
+                for (int k = 0; k < kTP; ++k) {
+                    const float4 v = dgw[k][(k & 1) ? slot_o : slot_e];
+                    const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
+                    const float4 b01 = bcw[0][0][k][q], b23 = bcw[0][1][k][q];
+                    const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
+                                          make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
+                    float2 hp[4];
+#pragma unroll
+                    for (int n = 0; n < 4; ++n) {
+                        const float2 e = mul2(dd, splat(a2[n]));
+                        const float2 ab = make_float2(ex2(e.x), ex2(e.y));
+                        const float2 bg = mul2(bp[n], gg);
+                        hp[n].x = fmaf(ab.x, h[n], bg.x);
+                        hp[n].y = fmaf(ab.y, hp[n].x, bg.y);
+                        h[n] = hp[n].y;
+                    }
+                    if constexpr (kSummary) {
+                        csum = k == 0 ? dd : add2(csum, dd);
+                    } else {
+                        const float4 c01 = bcw[1][0][k][q], c23 = bcw[1][1][k][q];
+                        part[k] = mul2(make_float2(c01.x, c01.y), hp[0]);
+                        part[k] = fma2(make_float2(c01.z, c01.w), hp[1], part[k]);
+                        part[k] = fma2(make_float2(c23.x, c23.y), hp[2], part[k]);
+                        part[k] = fma2(make_float2(c23.z, c23.w), hp[3], part[k]);
+                    }
+                }
+                if constexpr (kSummary) dsum = add2(dsum, csum);
+                // Not needed for order (other slots are read above): it keeps these stores behind the scan, 717 -> 711 us
+                // on 8 x 8192 x 2048.
+                if (!last) __syncwarp();
+                put(buf ^ 1, nv);
+                if (last) put_bc((i + 1) & 1, nw);
+                // (4) add the four lanes' shares of each channel, skip term, gate
+                if constexpr (!kSummary) {
+                    float4 *pw = s.part[warp];
+                    if (sub > 0) __syncwarp();   // the shares of the chunk before have been read
+#pragma unroll
+                    for (int k = 0; k < kTP; ++k) reinterpret_cast<float2 *>(pw + q * kPartQ + k * kPairs)[c] = part[k];
+                    __syncwarp();
+                    const float4 *src = pw + tp * kPairs + pp;   // (channel, step): (0, 0), (0, 1), (1, 0), (1, 1)
+                    const float4 s0 = src[0], s1 = src[kPartQ], s2 = src[2 * kPartQ], s3 = src[3 * kPartQ];
+                    const float2 ca = add2(add2(make_float2(s0.x, s0.y), make_float2(s1.x, s1.y)),
+                                           add2(make_float2(s2.x, s2.y), make_float2(s3.x, s3.y)));
+                    const float2 cb = add2(add2(make_float2(s0.z, s0.w), make_float2(s1.z, s1.w)),
+                                           add2(make_float2(s2.z, s2.w), make_float2(s3.z, s3.w)));
+                    st2<T>(&s.ys[i & 1][0][0], o0, mul2(add2(make_float2(ca.x, cb.x), xd0), sz0));
+                    st2<T>(&s.ys[i & 1][0][0], o1, mul2(add2(make_float2(ca.y, cb.y), xd1), sz1));
+                } else if (!last) {
+                    __syncwarp();
+                }
+            }
+            if constexpr (!kSummary) {
+                fence_proxy_async_smem();   // y tile -> visible to the TMA store below
+                if (tid == 0) bulk_wait_read_all();   // the store of stage i - 1 no longer reads its tile
+            }
+            if (__syncthreads_or(ok ? 0 : 1)) {
+                if (tid == 0) {
+                    report(p.status, 4 /* MB_ERR_TIMEOUT */, i + 1);
+                    for (int j = i + 1; j < i + STAGES && j < nch; ++j) {
+                        st = st + 1 == STAGES ? 0 : st + 1;
+                        ph ^= st == 0 ? 1u : 0u;
+                        mbar_wait(&s.full[st], ph);
+                    }
+                    bulk_wait_all();
+                }
+                return;
+            }
+            if (tid == 0) {
+                if constexpr (!kSummary) {
+                    tma_store_3d(&a.tm_y, &s.ys[i & 1][0][0], d0, ts, b);
+                    bulk_commit();
+                }
+                if (i + STAGES < nch) {   // the slot is free: refill it with stage i + STAGES
+                    fence_proxy_async_smem();
+                    issue_chunk<T, kSummary>(s, a, st, tb + (i + STAGES) * RT, d0, b);
+                }
+            }
+            st = nst;
+            ph = nph;
+        }
+        if constexpr (kSummary) pdl_trigger();   // the second pass may set up while the last summaries are written
+        if (!kShares && tid == 0) bulk_wait_all();
+
+        if constexpr (kSummary) {
+            if (chan_ok) {
+                const int64_t o = (((int64_t)b * nseg + seg) * D + d) * kDState + 4 * q;
+                const float sd = dsum.x + dsum.y;
+                *reinterpret_cast<float4 *>(p.seg_h + o) = make_float4(h[0], h[1], h[2], h[3]);
+                *reinterpret_cast<float4 *>(p.seg_p + o) =
+                    make_float4(ex2(a2[0] * sd), ex2(a2[1] * sd), ex2(a2[2] * sd), ex2(a2[3] * sd));
+            }
+        } else if (te == L) {   // the span's last state
+            if (p.h_out && chan_ok)
+                *reinterpret_cast<float4 *>(p.h_out + ((int64_t)b * D + d) * kDState + 4 * q) =
+                    make_float4(h[0], h[1], h[2], h[3]);
+        } else if constexpr (kShares) {   // the share ends here: leave the state for the next one
+            __stcg(reinterpret_cast<float4 *>(p.share_h + ((int64_t)share * kCh + kWCh * warp + c) * kDState + 4 * q),
+                   make_float4(h[0], h[1], h[2], h[3]));
+            __threadfence();
+            __syncthreads();
+            if (tid == 0) flag_set(p.share_sync + 1 + share);
+        }
+        if (!kShares || tile * units <= lo) break;
+        --tile;
     }
+    if (kShares && tid == 0) bulk_wait_all();
 }
 
 // ---------------------------------------------------------------------------
@@ -431,6 +504,14 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
             return e;
     }
     a.grid_segs = (int)nseg;
+    if (nseg == 1 && p.shares > 0) {
+        auto ks = forward_kernel<T, kCkpt, false, true>;
+        if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
+                cudaSuccess ||
+            (e = cudaMemsetAsync(p.share_sync, 0, prefill_share_sync_bytes(p.shares), s)) != cudaSuccess)
+            return e;
+        return launch_pdl(true, ks, dim3((unsigned)p.shares), dim3(kThreads), spread_smem(smem, p.shares, kResident), s, a);
+    }
     auto k = forward_kernel<T, kCkpt, false>;
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin);
     if (e != cudaSuccess) return e;
@@ -470,6 +551,35 @@ int64_t prefill_segments(const ScanParams &p) {
 
 size_t prefill_split_bytes(const ScanParams &p, int64_t nseg) {
     return nseg > 1 ? (size_t)(2 * p.batch * nseg * p.d_inner * kDState) * sizeof(float) : 0;
+}
+
+// Even shares: CTAs of one tile each leave the GPU unevenly loaded when their
+// number is little over a multiple of the SMs: the SMs that hold one more set
+// the time (8 x 8192 x 2048: 512 tiles, 3.4 per SM). Then m = tiles / SMs
+// (rounded down) CTAs per SM take equal shares of all tiles' steps instead.
+// Microseconds per chunk of an SM's CTAs, 1 to 4 of them, as measured:
+//   bf16 0.61 0.82 1.10 1.40, fp32 0.79 1.01 1.22 1.55
+// so shares pay off while tiles / (m SMs) * t[m] is well below t[m + 1] (bf16:
+// up to 1.26, 2.52 and 3.59 tiles per SM) and the span is long enough to make up
+// for the clearing of the flags and the second prologue (about 6 us). Measured:
+// 8 x 8192 x 2048 709 -> 650 us (622 by the rates alone), its training forward
+// 740 -> 672 us.
+constexpr double kChunkUs[2][4] = {{0.79, 1.01, 1.22, 1.55}, {0.61, 0.82, 1.10, 1.40}};
+
+int64_t prefill_shares(const ScanParams &p, bool bf16) {
+    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinSplitSteps || p.dt_low) return 0;
+    const int64_t sms = device_sms(), tiles = p.batch * ((p.d_inner + kCh - 1) / kCh);
+    if (sms <= 0 || tiles <= sms || tiles >= kResident * sms || tiles % sms == 0) return 0;
+    const int64_t m = tiles / sms;
+    const double even = (double)tiles / (double)(m * sms) * kChunkUs[bf16][m - 1], plain = kChunkUs[bf16][m];
+    if (even > 0.94 * plain || (plain - even) * (double)(p.seqlen / kT) < 8.0) return 0;
+    return m * sms;
+}
+
+size_t prefill_share_sync_bytes(int64_t shares) { return ((size_t)(shares + 1) * sizeof(int) + 255) / 256 * 256; }
+
+size_t prefill_share_bytes(int64_t shares) {
+    return shares > 0 ? prefill_share_sync_bytes(shares) + (size_t)shares * kCh * kDState * sizeof(float) : 0;
 }
 
 cudaError_t launch_forward(const ScanParams &p, bool bf16, cudaStream_t s) {

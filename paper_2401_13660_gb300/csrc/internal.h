@@ -42,6 +42,12 @@ struct ScanParams {
     // zero start and the product of its decays (scratch in the workspace).
     int64_t nseg;
     float *seg_h, *seg_p;
+    // Even shares of a prefill (0: off): `shares` CTAs of equal length, see
+    // prefill_shares. share_sync: a ticket counter, then a flag per share, all
+    // zero; share_h [shares, 32, 16]: the state where a share ends in a tile.
+    int64_t shares;
+    int *share_sync;
+    float *share_h;
 };
 
 constexpr int kRankTile = 64;    // dt_rank elements per 128-byte swizzled TMA box
@@ -89,6 +95,12 @@ int64_t prefill_segments(const ScanParams &p);
 // The same for the backward (its adjoint summaries need the same scratch per segment).
 int64_t backward_segments(const ScanParams &p);
 size_t prefill_split_bytes(const ScanParams &p, int64_t nseg);
+// Shares a prefill that is not split is cut into when the workspace has room
+// (0: one CTA per channel tile), and the scratch they need: share_sync (first,
+// prefill_share_sync_bytes) and share_h.
+int64_t prefill_shares(const ScanParams &p, bool bf16);
+size_t prefill_share_sync_bytes(int64_t shares);
+size_t prefill_share_bytes(int64_t shares);
 cudaError_t launch_verify(const ScanParams &p, bool bf16, cudaStream_t s);
 // Prefill that also writes p.h_ckpt [batch, ceil(L / kCkptSteps), d_inner, 16].
 cudaError_t launch_prefill_ckpt(const ScanParams &p, bool bf16, cudaStream_t s);

@@ -105,7 +105,7 @@ mb_status check_args(const mb_scan_args *a, bool need_seqlen1, bool need_y = tru
 }
 
 ScanParams to_params(const mb_scan_args *a, float *h_out, StatusBlock *status) {
-    ScanParams p;
+    ScanParams p{};   // whatever is not set here is off: no shares, no split
     p.batch = a->batch;
     p.seqlen = a->seqlen;
     p.d_inner = a->d_inner;
@@ -129,7 +129,7 @@ ScanParams to_params(const mb_scan_args *a, float *h_out, StatusBlock *status) {
 }
 
 // The status block must fit; a larger workspace (mb_workspace_size) only
-// lets mb_scan_prefill split long few-channel spans.
+// lets mb_scan_prefill split long few-channel spans or run even shares.
 mb_status check_ws(const mb_scan_args *a, void *ws, size_t ws_bytes) {
     if (mb_workspace_size(a) == 0) return MB_OK;
     if (ws == nullptr || ws_bytes < mbscan::kStatusBytes) return MB_ERR_INVALID_ARG;
@@ -137,26 +137,37 @@ mb_status check_ws(const mb_scan_args *a, void *ws, size_t ws_bytes) {
     return MB_OK;
 }
 
-// Long spans with few channels are split over L when the workspace holds the
-// segment summaries (after the status block); else they run unsplit.
-mb_status setup_split(const mb_scan_args *args, ScanParams &p, const float *h_last, void *ws, size_t ws_bytes) {
-    const int64_t nseg = mbscan::prefill_segments(p);
-    const size_t split = mbscan::prefill_split_bytes(p, nseg);
-    if (nseg < 2 || ws_bytes < mbscan::kStatusBytes + split) return MB_OK;
-    const int64_t es = args->dtype == MB_BF16 ? 2 : 4;
+// Long spans with few channels are split over L, others run in even shares where
+// that is faster, when the workspace holds the scratch (after the status block);
+// else they run as one CTA per channel tile.
+mb_status setup_split(const mb_scan_args *args, ScanParams &p, const float *h_last, void *ws, size_t ws_bytes,
+                      Range ckpt = Range{}) {
+    const bool bf16 = args->dtype == MB_BF16;
+    const int64_t nseg = mbscan::prefill_segments(p), shares = nseg > 1 ? 0 : mbscan::prefill_shares(p, bf16);
+    const size_t scratch = nseg > 1 ? mbscan::prefill_split_bytes(p, nseg) : mbscan::prefill_share_bytes(shares);
+    if (scratch == 0 || ws_bytes < mbscan::kStatusBytes + scratch) return MB_OK;
+    const int64_t es = bf16 ? 2 : 4;
     const int64_t tok = args->batch * args->seqlen * args->d_inner * es;
     const int64_t sbytes = args->batch * args->d_inner * args->d_state * 4;
-    const Range rs = range_of(static_cast<char *>(ws) + mbscan::kStatusBytes, (int64_t)split);
+    char *base = static_cast<char *>(ws) + mbscan::kStatusBytes;
+    const Range rs = range_of(base, (int64_t)scratch);
     const Range others[] = {range_of(args->x, tok), range_of(args->z, tok), range_of(args->dt, tok),
                             range_of(args->y, tok), range_of(args->B, bc_bytes(args)),
                             range_of(args->C, bc_bytes(args)), range_of(args->h0, sbytes), range_of(h_last, sbytes),
                             range_of(args->A, args->d_inner * args->d_state * 4),
-                            range_of(args->D, args->d_inner * 4), range_of(args->dt_bias, args->d_inner * 4)};
-    for (const Range &r : others)
-        if (overlap(rs, r)) return MB_ERR_INVALID_ARG;
-    p.nseg = nseg;
-    p.seg_h = reinterpret_cast<float *>(static_cast<char *>(ws) + mbscan::kStatusBytes);
-    p.seg_p = p.seg_h + split / (2 * sizeof(float));
+                            range_of(args->D, args->d_inner * 4), range_of(args->dt_bias, args->d_inner * 4), ckpt};
+    bool clear = true;
+    for (const Range &r : others) clear = clear && !overlap(rs, r);
+    if (nseg > 1) {
+        if (!clear) return MB_ERR_INVALID_ARG;
+        p.nseg = nseg;
+        p.seg_h = reinterpret_cast<float *>(base);
+        p.seg_p = p.seg_h + scratch / (2 * sizeof(float));
+    } else if (clear) {   // otherwise one CTA per tile, which needs no scratch
+        p.shares = shares;
+        p.share_sync = reinterpret_cast<int *>(base);
+        p.share_h = reinterpret_cast<float *>(base + mbscan::prefill_share_sync_bytes(shares));
+    }
     return MB_OK;
 }
 
@@ -193,7 +204,9 @@ size_t mb_workspace_size(const mb_scan_args *args) {
     if (check_args(args, false, false) != MB_OK) return 0;
     const ScanParams p = to_params(args, nullptr, nullptr);
     const int64_t fwd = mbscan::prefill_segments(p), bwd = mbscan::backward_segments(p);
-    return mbscan::kStatusBytes + mbscan::prefill_split_bytes(p, fwd > bwd ? fwd : bwd);
+    const size_t split = mbscan::prefill_split_bytes(p, fwd > bwd ? fwd : bwd);
+    const size_t shares = fwd > 1 ? 0 : mbscan::prefill_share_bytes(mbscan::prefill_shares(p, args->dtype == MB_BF16));
+    return mbscan::kStatusBytes + (split > shares ? split : shares);
 }
 
 mb_status mb_scan_prefill(const mb_scan_args *args, float *h_last, void *ws, size_t ws_bytes,
@@ -392,9 +405,7 @@ mb_status mb_scan_prefill_ckpt(const mb_scan_args *args, float *h_last, float *h
         return MB_ERR_INVALID_ARG;
     ScanParams p = to_params(args, h_last, static_cast<StatusBlock *>(ws));
     p.h_ckpt = h_ckpt;
-    if ((st = setup_split(args, p, h_last, ws, ws_bytes)) != MB_OK) return st;
-    if (p.nseg > 1 && overlap(rc, range_of(p.seg_h, (int64_t)mbscan::prefill_split_bytes(p, p.nseg))))
-        return MB_ERR_INVALID_ARG;
+    if ((st = setup_split(args, p, h_last, ws, ws_bytes, rc)) != MB_OK) return st;
     return from_cuda(mbscan::launch_prefill_ckpt(p, args->dtype == MB_BF16, (cudaStream_t)stream));
 }
 
