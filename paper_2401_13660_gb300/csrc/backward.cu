@@ -94,6 +94,7 @@ struct alignas(1024) BSmem {
     float4 hq[kBWarps][2][2][32];           // states before each half of the chunk: [half][channel][lane]
     float2 sum[kBWarps][kBTP][32];          // the warp's dB, dC (t, t+1): [tp][8 q + 4 (dC) + state]
     uint64_t full[kBStages];
+    int ticket;
 };
 
 struct BwdArgs {
@@ -165,7 +166,10 @@ __device__ __forceinline__ void flush_sums(const BSmem<T> &s, const GradParams &
     if (t0 + 2 * k + 1 < L) atomicAdd(reinterpret_cast<float4 *>(dst + kDState), hi);
 }
 
-template <typename T, bool kSummary>
+// kShares: as in forward.cu, the grid is p.shares CTAs of equal shares of all
+// tiles' chunks (in the order the sweep takes them, the last chunk first); a
+// share that ends inside a tile leaves the adjoint for the next one.
+template <typename T, bool kSummary, bool kShares = false>
 __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const __grid_constant__ BwdArgs a) {
     constexpr int S = kBStages, kRowB = kBCh * (int)sizeof(T);
     using R = BRaw<T>;
@@ -185,12 +189,8 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
     const int ntd = (int)((D + kBCh - 1) / kBCh);
     const int L = (int)p.seqlen;
     const int nchunks = (L + kBT - 1) / kBT;
-    const int seg = a.seg0 + (int)((blockIdx.x / ntd) % a.grid_segs);
-    const int b = (int)(blockIdx.x / ntd / a.grid_segs);
-    const int nseg = p.nseg > 1 ? (int)p.nseg : 1;
-    const int cps = (nchunks + nseg - 1) / nseg;
-    const int c0 = seg * cps, nch = min(nchunks - c0, cps);   // chunks c0 + nch - 1 down to c0
-    const int d0 = (int)(blockIdx.x % ntd) * kBCh;
+    const int nseg = p.nseg > 1 ? (int)p.nseg : 1, cps = (nchunks + nseg - 1) / nseg;
+    const int seg = kShares ? 0 : a.seg0 + (int)((blockIdx.x / ntd) % a.grid_segs);
     const bool gate = a.has_gate != 0;
 
     if (tid == 0) {
@@ -199,390 +199,450 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
     }
     __syncthreads();
     pdl_wait();   // everything below reads or writes global memory
-    if (tid == 0)
-        for (int j = 0; j < S && j < nch; ++j) issue_bchunk<T, kSummary>(s, a, j, c0 + nch - 1 - j, d0, b);
 
-    // ---- conversion and finishing role: channels 16 warp + 2 pp + {0, 1} of the tile, step pairs ts and ts + 4
-    const int wc0 = kBWCh * warp, pp = lane & 7, ts = lane >> 3;
-    int off[2][2];
-#pragma unroll
-    for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int e = 0; e < 2; ++e) off[u][e] = tile_off<T, kBCh>(2 * (ts + kHTP * u) + e, wc0 + 2 * pp);
-    float2 bias = make_float2(0.f, 0.f), dsk = bias, dD_acc = bias, db_acc = bias;
-    const int64_t dc = (int64_t)d0 + wc0 + 2 * pp;   // D % 8 == 0: both channels valid or neither
-    if (dc < D) {
-        if (p.dt_bias) bias = __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc));
-        if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
+    int tile = (int)(blockIdx.x / ntd / a.grid_segs) * ntd + (int)(blockIdx.x % ntd);   // batch row, 32 channels
+    int share = 0, lo = 0, hi = 0;   // kShares: chunks lo .. hi - 1 of all tiles' sweeps end to end
+    int n0 = 0;                      // ring stages consumed by the pieces before
+    if constexpr (kShares) {
+        if (tid == 0) s.ticket = atomicAdd(p.share_sync, 1);
+        __syncthreads();
+        share = s.ticket;
+        const int total = (int)p.batch * ntd * nchunks, len = (total + (int)p.shares - 1) / (int)p.shares;
+        lo = min(share * len, total);
+        hi = min(lo + len, total);
+        if (lo == hi) return;
+        tile = (hi - 1) / nchunks;
     }
-
-    // ---- scan role: channels 2 cl, 2 cl + 1 of the warp, states 4 q .. 4 q + 3 in the order r -> r ^ perm
-    const int cl = ((lane >> 2) & 3) | ((lane & 1) << 2), q = ((lane >> 1) & 1) | ((lane >> 4) << 1);
-    const int perm = cl & 3;
-    const int ix0 = perm, ix1 = perm ^ 2;   // slots of s.bc that hold registers 0, 1 and 2, 3
-    const int64_t d = (int64_t)d0 + wc0 + 2 * cl;
-    const bool chan_ok = d < D;
-    float a2[2][4], g[2][4];   // A log2 e; the adjoint Abar_{t+1} g_{t+1} on its way down
-    float2 dA[2][4];           // even and odd steps
-    float2 dsum[2];            // kSummary: sum of Delta
-#pragma unroll
-    for (int j = 0; j < 2; ++j) {
-#pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            a2[j][n] = g[j][n] = 0.f;
-            dA[j][n] = make_float2(0.f, 0.f);
+    for (;;) {   // pieces: one without kShares
+        const int b = tile / ntd, d0 = (tile % ntd) * kBCh;
+        // chunks c0 + nch - 1 down to c0
+        const int c0 = kShares ? max(nchunks - (hi - tile * nchunks), 0) : seg * cps;
+        const int nch = (kShares ? nchunks - max(lo - tile * nchunks, 0) : min(nchunks, c0 + cps)) - c0;
+        if (tid == 0) {
+            fence_proxy_async_smem();
+            for (int j = 0; j < S && j < nch; ++j) issue_bchunk<T, kSummary>(s, a, (n0 + j) % S, c0 + nch - 1 - j, d0, b);
         }
-        dsum[j] = make_float2(0.f, 0.f);
-        if (chan_ok) {
-            load_perm(a2[j], p.A + (d + j) * kDState + 4 * q, perm);
+
+        // ---- conversion and finishing role: channels 16 warp + 2 pp + {0, 1} of the tile, step pairs ts and ts + 4
+        const int wc0 = kBWCh * warp, pp = lane & 7, ts = lane >> 3;
+        int off[2][2];
 #pragma unroll
-            for (int n = 0; n < 4; ++n) a2[j][n] *= kLog2e;
-            if (seg == nseg - 1) {
-                if (gp.dh_last) load_perm(g[j], gp.dh_last + ((int64_t)b * D + d + j) * kDState + 4 * q, perm);
-            } else if (!kSummary) {   // the last segment's summary starts from dh_last: fold down to this one
-                for (int sp = nseg - 1; sp > seg; --sp) {
-                    const int64_t o = (((int64_t)b * nseg + sp) * D + d + j) * kDState + 4 * q;
-                    float ge[4], pe[4];
-                    load_perm(ge, p.seg_h + o, perm);
-                    load_perm(pe, p.seg_p + o, perm);
+        for (int u = 0; u < 2; ++u)
 #pragma unroll
-                    for (int n = 0; n < 4; ++n) g[j][n] = sp == nseg - 1 ? ge[n] : fmaf(pe[n], g[j][n], ge[n]);
-                }
+            for (int e = 0; e < 2; ++e) off[u][e] = tile_off<T, kBCh>(2 * (ts + kHTP * u) + e, wc0 + 2 * pp);
+        float2 bias = make_float2(0.f, 0.f), dsk = bias, dD_acc = bias, db_acc = bias;
+        const int64_t dc = (int64_t)d0 + wc0 + 2 * pp;   // D % 8 == 0: both channels valid or neither
+        if (dc < D) {
+            if (p.dt_bias) bias = __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc));
+            if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
+        }
+
+        // ---- scan role: channels 2 cl, 2 cl + 1 of the warp, states 4 q .. 4 q + 3 in the order r -> r ^ perm
+        const int cl = ((lane >> 2) & 3) | ((lane & 1) << 2), q = ((lane >> 1) & 1) | ((lane >> 4) << 1);
+        const int perm = cl & 3;
+        const int ix0 = perm, ix1 = perm ^ 2;   // slots of s.bc that hold registers 0, 1 and 2, 3
+        const int64_t d = (int64_t)d0 + wc0 + 2 * cl;
+        const bool chan_ok = d < D;
+        float a2[2][4], g[2][4];   // A log2 e; the adjoint Abar_{t+1} g_{t+1} on its way down
+        float2 dA[2][4];           // even and odd steps
+        float2 dsum[2];            // kSummary: sum of Delta
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+#pragma unroll
+            for (int n = 0; n < 4; ++n) {
+                a2[j][n] = g[j][n] = 0.f;
+                dA[j][n] = make_float2(0.f, 0.f);
             }
-        }
-    }
-
-    // Byte offsets (from smem_dyn) of what the scan's loops read and write, opaque to the compiler: it would compute
-    // them again at every use rather than keep them.
-    auto fixed = [&](size_t o) {
-        uint32_t v = sbase + (uint32_t)o;
-        asm volatile("" : "+r"(v));
-        return v;
-    };
-    const uint32_t o_bc0 = fixed(offsetof(SM, bc) + (q * 4 + ix0) * 16), o_bc1 = o_bc0 + (ix1 - ix0) * 16;
-    const uint32_t o_dg = fixed(offsetof(SM, dg) + (warp * kBTP * 2 * kBPairs + cl) * 16);
-    const uint32_t o_dy = fixed(offsetof(SM, dy) + (warp * kBTP * kBPairs + cl) * 16);
-    const uint32_t o_sh = fixed(offsetof(SM, share) + (warp * 3 * 4 * kShareQ + q * kShareQ + cl) * 16);
-    auto at4 = [&](uint32_t o) -> float4 & { return *reinterpret_cast<float4 *>(smem_dyn + o); };
-    constexpr uint32_t kC = kBTP * 4 * 4 * 16, kStepB = 4 * 4 * 16, kStepG = 2 * kBPairs * 16, kStepY = kBPairs * 16;
-    constexpr uint32_t kShare = 4 * kShareQ * 16;
-
-    bool ok = true;
-    for (int it = 0; it < nch; ++it) {
-        const int i = c0 + nch - 1 - it;   // chunk of this iteration
-        const int t0 = i * kBT;
-        const R &r = s.raw[it % S];
-        // the chunk's checkpoint, in flight during the conversion; the next one's on its way to L2
-        float hm[2][4];
-        if constexpr (!kSummary) {
-            const float *ck = gp.h_ckpt + (((int64_t)b * nchunks + i) * D + d) * kDState + 4 * q;
+            dsum[j] = make_float2(0.f, 0.f);
+            if (chan_ok) {
+                load_perm(a2[j], p.A + (d + j) * kDState + 4 * q, perm);
 #pragma unroll
-            for (int j = 0; j < 2; ++j) {
+                for (int n = 0; n < 4; ++n) a2[j][n] *= kLog2e;
+                if (kShares ? c0 + nch == nchunks : seg == nseg - 1) {
+                    if (gp.dh_last) load_perm(g[j], gp.dh_last + ((int64_t)b * D + d + j) * kDState + 4 * q, perm);
+                } else if (!kSummary && !kShares) {   // the last segment's summary starts from dh_last: fold down to this one
+                    for (int sp = nseg - 1; sp > seg; --sp) {
+                        const int64_t o = (((int64_t)b * nseg + sp) * D + d + j) * kDState + 4 * q;
+                        float ge[4], pe[4];
+                        load_perm(ge, p.seg_h + o, perm);
+                        load_perm(pe, p.seg_p + o, perm);
 #pragma unroll
-                for (int n = 0; n < 4; ++n) hm[j][n] = 0.f;
-                if (chan_ok) load_perm(hm[j], ck + j * kDState, perm);
-            }
-            if (chan_ok && it + 1 < nch) asm volatile("prefetch.global.L2 [%0];" ::"l"(ck - D * kDState + (q & 1) * kDState));
-        }
-        // (1) convert chunk i; add dB, dC of chunk i + 1 to global memory
-        ok = mbar_wait(&s.full[it % S], (uint32_t)((it / S) & 1));
-        if (ok) {
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int tp = ts + kHTP * u;
-                float2 de[2], dyv[2], gxv[2], sig[2], qz[2];
-#pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    softplus_sigmoid2(add2(ld2<T>(&r.dt[0][0], off[u][e]), bias), de[e], sig[e]);
-                    const float m = t0 + 2 * tp + e < L ? 1.f : 0.f;   // Delta = 0 past the end: h and g unchanged
-                    de[e] = mul2(de[e], splat(m));
-                    sig[e] = mul2(sig[e], splat(m));
-                    dyv[e] = ld2<T>(&r.dout[0][0], off[u][e]);
-                    if constexpr (!kSummary) gxv[e] = mul2(de[e], ld2<T>(&r.x[0][0], off[u][e]));
-                    qz[e] = make_float2(0.f, 0.f);
-                    if (gate) {
-                        const float2 z = ld2<T>(&r.z[0][0], off[u][e]);
-                        const float2 w = mul2(z, splat(-kLog2e));
-                        const float2 o = add2(make_float2(ex2(w.x), ex2(w.y)), splat(1.f));
-                        const float2 sz = make_float2(rcp(o.x), rcp(o.y));
-                        qz[e] = mul2(mul2(dyv[e], sz), fma2(z, fma2(sz, splat(-1.f), splat(1.f)), splat(1.f)));
-                        dyv[e] = mul2(dyv[e], mul2(z, sz));
+                        for (int n = 0; n < 4; ++n) g[j][n] = sp == nseg - 1 ? ge[n] : fmaf(pe[n], g[j][n], ge[n]);
                     }
                 }
-                if constexpr (kSummary) gxv[0] = gxv[1] = make_float2(0.f, 0.f);
-                s.dg[warp][tp][0][pp] = make_float4(de[0].x, de[1].x, gxv[0].x, gxv[1].x);
-                s.dg[warp][tp][1][pp] = make_float4(de[0].y, de[1].y, gxv[0].y, gxv[1].y);
-                s.dy[warp][tp][pp] = make_float4(dyv[0].x, dyv[1].x, dyv[0].y, dyv[1].y);
-                if constexpr (!kSummary) {
-                    s.fin[warp][0][tp][pp] = make_float4(sig[0].x, sig[0].y, sig[1].x, sig[1].y);
-                    s.fin[warp][1][tp][pp] = make_float4(qz[0].x, qz[0].y, qz[1].x, qz[1].y);
-                }
             }
-            {   // two states of B and of C at a step pair, in both orders
-                const int wh = tid & 1, wq = (tid >> 1) & 3, wt = tid >> 3;
-                const bool swap = wq & 2;   // which order first: eight stores at a time on different banks
-#pragma unroll
-                for (int u = kSummary ? 1 : 0; u < 2; ++u) {
-                    const T *src = u ? &r.C[2 * wt][4 * wq + 2 * wh] : &r.B[2 * wt][4 * wq + 2 * wh];
-                    const float2 v0 = ld2<T>(src, 0), v1 = ld2<T>(src, kDState * (int)sizeof(T));
-                    float4 *dst = &s.bc[u][wt][wq][2 * wh];
-                    const float4 f = make_float4(v0.x, v1.x, v0.y, v1.y), rv = make_float4(v0.y, v1.y, v0.x, v1.x);
-                    dst[swap ? 1 : 0] = swap ? rv : f;
-                    dst[swap ? 0 : 1] = swap ? f : rv;
-                }
-            }
-        }
-        if constexpr (!kSummary) {
-            if (it >= 1) flush_sums(s, gp, b, t0 + kBT, L);
-            if (tid == 0) bulk_wait_read_all();   // the output tiles may be written again
-        }
-        if (__syncthreads_or(ok ? 0 : 1)) {
-            if (tid == 0) {
-                report(p.status, 4 /* MB_ERR_TIMEOUT */, it);
-                for (int jj = it; jj <= it + S - 1 && jj < nch; ++jj)
-                    mbar_wait(&s.full[jj % S], (uint32_t)((jj / S) & 1));
-                bulk_wait_all();
-            }
-            return;
         }
 
-        const float4(&dgw)[kBTP][2][kBPairs] = s.dg[warp];
-        const float4(&dyw)[kBTP][kBPairs] = s.dy[warp];
-        if constexpr (kSummary) {
-            float2 cs[2];
-#pragma unroll
-            for (int k = kBTP - 1; k >= 0; --k) {
-                const float4 c01 = s.bc[1][k][q][ix0], c23 = s.bc[1][k][q][ix1];
-                const float2 cp[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w),
-                                      make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
-                const float4 yv = dyw[k][cl];
-                const float2 dyp[2] = {make_float2(yv.x, yv.y), make_float2(yv.z, yv.w)};
+        // Byte offsets (from smem_dyn) of what the scan's loops read and write, opaque to the compiler: it would compute
+        // them again at every use rather than keep them.
+        auto fixed = [&](size_t o) {
+            uint32_t v = sbase + (uint32_t)o;
+            asm volatile("" : "+r"(v));
+            return v;
+        };
+        const uint32_t o_bc0 = fixed(offsetof(SM, bc) + (q * 4 + ix0) * 16), o_bc1 = o_bc0 + (ix1 - ix0) * 16;
+        const uint32_t o_dg = fixed(offsetof(SM, dg) + (warp * kBTP * 2 * kBPairs + cl) * 16);
+        const uint32_t o_dy = fixed(offsetof(SM, dy) + (warp * kBTP * kBPairs + cl) * 16);
+        const uint32_t o_sh = fixed(offsetof(SM, share) + (warp * 3 * 4 * kShareQ + q * kShareQ + cl) * 16);
+        auto at4 = [&](uint32_t o) -> float4 & { return *reinterpret_cast<float4 *>(smem_dyn + o); };
+        constexpr uint32_t kC = kBTP * 4 * 4 * 16, kStepB = 4 * 4 * 16, kStepG = 2 * kBPairs * 16, kStepY = kBPairs * 16;
+        constexpr uint32_t kShare = 4 * kShareQ * 16;
+
+        if constexpr (kShares) {
+            if (c0 + nch < nchunks) {   // the share before has left the adjoint
+                bool set = true;
+                if (tid == 0) set = flag_wait(p.share_sync + share);
+                if (__syncthreads_or(set ? 0 : 1)) {
+                    if (tid == 0) {
+                        report(p.status, 4 /* MB_ERR_TIMEOUT */, share);
+                        for (int jj = 0; jj < S && jj < nch; ++jj)
+                            mbar_wait(&s.full[(n0 + jj) % S], (uint32_t)(((n0 + jj) / S) & 1));
+                        bulk_wait_all();
+                    }
+                    return;
+                }
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const float2 dd = *reinterpret_cast<const float2 *>(&dgw[k][j][cl]);
-                    cs[j] = k == kBTP - 1 ? dd : add2(cs[j], dd);
-#pragma unroll
-                    for (int n = 0; n < 4; ++n) {
-                        const float2 e = mul2(dd, splat(a2[j][n]));
-                        const float g1 = fmaf(dyp[j].y, cp[n].y, g[j][n]) * ex2(e.y);
-                        g[j][n] = fmaf(dyp[j].x, cp[n].x, g1) * ex2(e.x);
-                    }
+                    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p.share_h) +
+                                            ((int64_t)(share - 1) * 2 + j) * kBThreads + tid);
+                    g[j][0] = v.x; g[j][1] = v.y; g[j][2] = v.z; g[j][3] = v.w;
                 }
             }
-            dsum[0] = add2(dsum[0], cs[0]);
-            dsum[1] = add2(dsum[1], cs[1]);
-        } else {
-            // (2) the state before step 8: steps 0 .. 7 from the checkpoint
-            float4(&hq)[2][2][32] = s.hq[warp];
-#pragma unroll
-            for (int j = 0; j < 2; ++j) hq[0][j][lane] = make_float4(hm[j][0], hm[j][1], hm[j][2], hm[j][3]);
-#pragma unroll
-            for (int k = 0; k < kHTP; ++k) {
-                const float4 b01 = at4(o_bc0 + k * kStepB), b23 = at4(o_bc1 + k * kStepB);
-                const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w), make_float2(b23.x, b23.y),
-                                      make_float2(b23.z, b23.w)};
+        }
+        bool ok = true;
+        for (int it = 0; it < nch; ++it) {
+            const int sl = (n0 + it) % S;   // ring slot
+            const int i = c0 + nch - 1 - it;   // chunk of this iteration
+            const int t0 = i * kBT;
+            const R &r = s.raw[sl];
+            // the chunk's checkpoint, in flight during the conversion; the next one's on its way to L2
+            float hm[2][4];
+            if constexpr (!kSummary) {
+                const float *ck = gp.h_ckpt + (((int64_t)b * nchunks + i) * D + d) * kDState + 4 * q;
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const float4 v = at4(o_dg + k * kStepG + j * kBPairs * 16);
-                    const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
 #pragma unroll
-                    for (int n = 0; n < 4; ++n) {
-                        const float2 e = mul2(dd, splat(a2[j][n]));
-                        const float2 bg = mul2(bp[n], gg);
-                        hm[j][n] = fmaf(ex2(e.y), fmaf(ex2(e.x), hm[j][n], bg.x), bg.y);
+                    for (int n = 0; n < 4; ++n) hm[j][n] = 0.f;
+                    if (chan_ok) load_perm(hm[j], ck + j * kDState, perm);
+                }
+                if (chan_ok && it + 1 < nch) asm volatile("prefetch.global.L2 [%0];" ::"l"(ck - D * kDState + (q & 1) * kDState));
+            }
+            // (1) convert chunk i; add dB, dC of chunk i + 1 to global memory
+            ok = mbar_wait(&s.full[sl], (uint32_t)(((n0 + it) / S) & 1));
+            if (ok) {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int tp = ts + kHTP * u;
+                    float2 de[2], dyv[2], gxv[2], sig[2], qz[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        softplus_sigmoid2(add2(ld2<T>(&r.dt[0][0], off[u][e]), bias), de[e], sig[e]);
+                        const float m = t0 + 2 * tp + e < L ? 1.f : 0.f;   // Delta = 0 past the end: h and g unchanged
+                        de[e] = mul2(de[e], splat(m));
+                        sig[e] = mul2(sig[e], splat(m));
+                        dyv[e] = ld2<T>(&r.dout[0][0], off[u][e]);
+                        if constexpr (!kSummary) gxv[e] = mul2(de[e], ld2<T>(&r.x[0][0], off[u][e]));
+                        qz[e] = make_float2(0.f, 0.f);
+                        if (gate) {
+                            const float2 z = ld2<T>(&r.z[0][0], off[u][e]);
+                            const float2 w = mul2(z, splat(-kLog2e));
+                            const float2 o = add2(make_float2(ex2(w.x), ex2(w.y)), splat(1.f));
+                            const float2 sz = make_float2(rcp(o.x), rcp(o.y));
+                            qz[e] = mul2(mul2(dyv[e], sz), fma2(z, fma2(sz, splat(-1.f), splat(1.f)), splat(1.f)));
+                            dyv[e] = mul2(dyv[e], mul2(z, sz));
+                        }
+                    }
+                    if constexpr (kSummary) gxv[0] = gxv[1] = make_float2(0.f, 0.f);
+                    s.dg[warp][tp][0][pp] = make_float4(de[0].x, de[1].x, gxv[0].x, gxv[1].x);
+                    s.dg[warp][tp][1][pp] = make_float4(de[0].y, de[1].y, gxv[0].y, gxv[1].y);
+                    s.dy[warp][tp][pp] = make_float4(dyv[0].x, dyv[1].x, dyv[0].y, dyv[1].y);
+                    if constexpr (!kSummary) {
+                        s.fin[warp][0][tp][pp] = make_float4(sig[0].x, sig[0].y, sig[1].x, sig[1].y);
+                        s.fin[warp][1][tp][pp] = make_float4(qz[0].x, qz[0].y, qz[1].x, qz[1].y);
+                    }
+                }
+                {   // two states of B and of C at a step pair, in both orders
+                    const int wh = tid & 1, wq = (tid >> 1) & 3, wt = tid >> 3;
+                    const bool swap = wq & 2;   // which order first: eight stores at a time on different banks
+#pragma unroll
+                    for (int u = kSummary ? 1 : 0; u < 2; ++u) {
+                        const T *src = u ? &r.C[2 * wt][4 * wq + 2 * wh] : &r.B[2 * wt][4 * wq + 2 * wh];
+                        const float2 v0 = ld2<T>(src, 0), v1 = ld2<T>(src, kDState * (int)sizeof(T));
+                        float4 *dst = &s.bc[u][wt][wq][2 * wh];
+                        const float4 f = make_float4(v0.x, v1.x, v0.y, v1.y), rv = make_float4(v0.y, v1.y, v0.x, v1.x);
+                        dst[swap ? 1 : 0] = swap ? rv : f;
+                        dst[swap ? 0 : 1] = swap ? f : rv;
                     }
                 }
             }
+            if constexpr (!kSummary) {
+                if (it >= 1) flush_sums(s, gp, b, t0 + kBT, L);
+                if (tid == 0) bulk_wait_read_all();   // the output tiles may be written again
+            }
+            if (__syncthreads_or(ok ? 0 : 1)) {
+                if (tid == 0) {
+                    report(p.status, 4 /* MB_ERR_TIMEOUT */, it);
+                    for (int jj = it; jj <= it + S - 1 && jj < nch; ++jj)
+                        mbar_wait(&s.full[(n0 + jj) % S], (uint32_t)(((n0 + jj) / S) & 1));
+                    bulk_wait_all();
+                }
+                return;
+            }
+
+            const float4(&dgw)[kBTP][2][kBPairs] = s.dg[warp];
+            const float4(&dyw)[kBTP][kBPairs] = s.dy[warp];
+            if constexpr (kSummary) {
+                float2 cs[2];
 #pragma unroll
-            for (int j = 0; j < 2; ++j) hq[1][j][lane] = make_float4(hm[j][0], hm[j][1], hm[j][2], hm[j][3]);
-            float4(&sh)[3][4 * kShareQ] = s.share[warp];
-            // (3) the two halves, the later one first (not unrolled: both at once spill registers)
-#pragma unroll 1
-            for (int u = 1; u >= 0; --u) {
-                const int k0 = kHTP * u;
-                const uint32_t ub0 = o_bc0 + u * kHTP * kStepB, ub1 = o_bc1 + u * kHTP * kStepB, ug = o_dg + u * kHTP * kStepG;
-                const float4 ha = hq[u][0][lane], hb = hq[u][1][lane];
-                const float hs[2][4] = {{ha.x, ha.y, ha.z, ha.w}, {hb.x, hb.y, hb.z, hb.w}};   // state before this half
-                // its decays and states, kept in registers, and the shares of C.h
-                float2 ab[kHTP][2][4], hp[kHTP][2][4];
-                float4 shy[kHTP];
-#pragma unroll
-                for (int k = 0; k < kHTP; ++k) {
-                    const float4 b01 = at4(ub0 + k * kStepB), b23 = at4(ub1 + k * kStepB);
-                    const float4 c01 = at4(ub0 + kC + k * kStepB), c23 = at4(ub1 + kC + k * kStepB);
-                    const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
-                                          make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
+                for (int k = kBTP - 1; k >= 0; --k) {
+                    const float4 c01 = s.bc[1][k][q][ix0], c23 = s.bc[1][k][q][ix1];
                     const float2 cp[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w),
                                           make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
-                    float2 acc[2];
+                    const float4 yv = dyw[k][cl];
+                    const float2 dyp[2] = {make_float2(yv.x, yv.y), make_float2(yv.z, yv.w)};
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        const float4 v = at4(ug + k * kStepG + j * kBPairs * 16);
+                        const float2 dd = *reinterpret_cast<const float2 *>(&dgw[k][j][cl]);
+                        cs[j] = k == kBTP - 1 ? dd : add2(cs[j], dd);
+#pragma unroll
+                        for (int n = 0; n < 4; ++n) {
+                            const float2 e = mul2(dd, splat(a2[j][n]));
+                            const float g1 = fmaf(dyp[j].y, cp[n].y, g[j][n]) * ex2(e.y);
+                            g[j][n] = fmaf(dyp[j].x, cp[n].x, g1) * ex2(e.x);
+                        }
+                    }
+                }
+                dsum[0] = add2(dsum[0], cs[0]);
+                dsum[1] = add2(dsum[1], cs[1]);
+            } else {
+                // (2) the state before step 8: steps 0 .. 7 from the checkpoint
+                float4(&hq)[2][2][32] = s.hq[warp];
+#pragma unroll
+                for (int j = 0; j < 2; ++j) hq[0][j][lane] = make_float4(hm[j][0], hm[j][1], hm[j][2], hm[j][3]);
+#pragma unroll
+                for (int k = 0; k < kHTP; ++k) {
+                    const float4 b01 = at4(o_bc0 + k * kStepB), b23 = at4(o_bc1 + k * kStepB);
+                    const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w), make_float2(b23.x, b23.y),
+                                          make_float2(b23.z, b23.w)};
+#pragma unroll
+                    for (int j = 0; j < 2; ++j) {
+                        const float4 v = at4(o_dg + k * kStepG + j * kBPairs * 16);
                         const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
 #pragma unroll
                         for (int n = 0; n < 4; ++n) {
                             const float2 e = mul2(dd, splat(a2[j][n]));
-                            ab[k][j][n] = make_float2(ex2(e.x), ex2(e.y));
                             const float2 bg = mul2(bp[n], gg);
-                            const float hl = k == 0 ? hs[j][n] : hp[k - 1][j][n].y;
-                            hp[k][j][n].x = fmaf(ab[k][j][n].x, hl, bg.x);
-                            hp[k][j][n].y = fmaf(ab[k][j][n].y, hp[k][j][n].x, bg.y);
-                            acc[j] = n == 0 ? mul2(cp[0], hp[k][j][0]) : fma2(cp[n], hp[k][j][n], acc[j]);
+                            hm[j][n] = fmaf(ex2(e.y), fmaf(ex2(e.x), hm[j][n], bg.x), bg.y);
                         }
                     }
-                    shy[k] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
                 }
 #pragma unroll
-                for (int k = 0; k < kHTP; ++k) at4(o_sh + k * kBPairs * 16) = shy[k];
-                // reverse sweep
-                float4 sh1[kHTP], sh2[kHTP];
-                float2 sums[kHTP];
+                for (int j = 0; j < 2; ++j) hq[1][j][lane] = make_float4(hm[j][0], hm[j][1], hm[j][2], hm[j][3]);
+                float4(&sh)[3][4 * kShareQ] = s.share[warp];
+                // (3) the two halves, the later one first (not unrolled: both at once spill registers)
+#pragma unroll 1
+                for (int u = 1; u >= 0; --u) {
+                    const int k0 = kHTP * u;
+                    const uint32_t ub0 = o_bc0 + u * kHTP * kStepB, ub1 = o_bc1 + u * kHTP * kStepB, ug = o_dg + u * kHTP * kStepG;
+                    const float4 ha = hq[u][0][lane], hb = hq[u][1][lane];
+                    const float hs[2][4] = {{ha.x, ha.y, ha.z, ha.w}, {hb.x, hb.y, hb.z, hb.w}};   // state before this half
+                    // its decays and states, kept in registers, and the shares of C.h
+                    float2 ab[kHTP][2][4], hp[kHTP][2][4];
+                    float4 shy[kHTP];
 #pragma unroll
-                for (int k = kHTP - 1; k >= 0; --k) {
-                    const float4 b01 = at4(ub0 + k * kStepB), b23 = at4(ub1 + k * kStepB);
-                    const float4 c01 = at4(ub0 + kC + k * kStepB), c23 = at4(ub1 + kC + k * kStepB);
-                    const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
-                                          make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
-                    const float2 cp[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w),
-                                          make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
-                    const float4 yv = at4(o_dy + u * kHTP * kStepY + k * kStepY);
-                    const float2 dyp[2] = {make_float2(yv.x, yv.y), make_float2(yv.z, yv.w)};
-                    float2 dBv[4], dCv[4], s1[2], s2[2];
+                    for (int k = 0; k < kHTP; ++k) {
+                        const float4 b01 = at4(ub0 + k * kStepB), b23 = at4(ub1 + k * kStepB);
+                        const float4 c01 = at4(ub0 + kC + k * kStepB), c23 = at4(ub1 + kC + k * kStepB);
+                        const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
+                                              make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
+                        const float2 cp[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w),
+                                              make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
+                        float2 acc[2];
 #pragma unroll
-                    for (int j = 0; j < 2; ++j) {
-                        const float4 v = at4(ug + k * kStepG + j * kBPairs * 16);
-                        const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
+                        for (int j = 0; j < 2; ++j) {
+                            const float4 v = at4(ug + k * kStepG + j * kBPairs * 16);
+                            const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
 #pragma unroll
-                        for (int n = 0; n < 4; ++n) {
-                            const float2 A = ab[k][j][n], H = hp[k][j][n];
-                            float2 gv, ga, w;
-                            gv.y = fmaf(dyp[j].y, cp[n].y, g[j][n]);
-                            ga.y = gv.y * A.y;
-                            gv.x = fmaf(dyp[j].x, cp[n].x, ga.y);
-                            ga.x = gv.x * A.x;
-                            g[j][n] = ga.x;
-                            w.x = ga.x * (k == 0 ? hs[j][n] : hp[k - 1][j][n].y);
-                            w.y = ga.y * H.x;
-                            dCv[n] = j == 0 ? mul2(dyp[0], H) : fma2(dyp[1], H, dCv[n]);
-                            dBv[n] = j == 0 ? mul2(gg, gv) : fma2(gg, gv, dBv[n]);
-                            s1[j] = n == 0 ? mul2(bp[0], gv) : fma2(bp[n], gv, s1[j]);
-                            s2[j] = n == 0 ? mul2(splat(a2[j][0]), w) : fma2(splat(a2[j][n]), w, s2[j]);
-                            dA[j][n] = fma2(dd, w, dA[j][n]);
+                            for (int n = 0; n < 4; ++n) {
+                                const float2 e = mul2(dd, splat(a2[j][n]));
+                                ab[k][j][n] = make_float2(ex2(e.x), ex2(e.y));
+                                const float2 bg = mul2(bp[n], gg);
+                                const float hl = k == 0 ? hs[j][n] : hp[k - 1][j][n].y;
+                                hp[k][j][n].x = fmaf(ab[k][j][n].x, hl, bg.x);
+                                hp[k][j][n].y = fmaf(ab[k][j][n].y, hp[k][j][n].x, bg.y);
+                                acc[j] = n == 0 ? mul2(cp[0], hp[k][j][0]) : fma2(cp[n], hp[k][j][n], acc[j]);
+                            }
                         }
+                        shy[k] = make_float4(acc[0].x, acc[0].y, acc[1].x, acc[1].y);
                     }
-                    sh1[k] = make_float4(s1[0].x, s1[0].y, s1[1].x, s1[1].y);
-                    sh2[k] = make_float4(s2[0].x, s2[0].y, s2[1].x, s2[1].y);
-                    // dB, dC over the warp's 16 channels: lanes that differ in channel bits exchange the states they do
-                    // not keep; the state order r -> r ^ perm makes those registers 2, 3, then 1, on every lane
 #pragma unroll
-                    for (int n = 0; n < 2; ++n) {
-                        dBv[n] = add2(dBv[n], shfl2(dBv[n + 2], 8));
-                        dCv[n] = add2(dCv[n], shfl2(dCv[n + 2], 8));
+                    for (int k = 0; k < kHTP; ++k) at4(o_sh + k * kBPairs * 16) = shy[k];
+                    // reverse sweep
+                    float4 sh1[kHTP], sh2[kHTP];
+                    float2 sums[kHTP];
+#pragma unroll
+                    for (int k = kHTP - 1; k >= 0; --k) {
+                        const float4 b01 = at4(ub0 + k * kStepB), b23 = at4(ub1 + k * kStepB);
+                        const float4 c01 = at4(ub0 + kC + k * kStepB), c23 = at4(ub1 + kC + k * kStepB);
+                        const float2 bp[4] = {make_float2(b01.x, b01.y), make_float2(b01.z, b01.w),
+                                              make_float2(b23.x, b23.y), make_float2(b23.z, b23.w)};
+                        const float2 cp[4] = {make_float2(c01.x, c01.y), make_float2(c01.z, c01.w),
+                                              make_float2(c23.x, c23.y), make_float2(c23.z, c23.w)};
+                        const float4 yv = at4(o_dy + u * kHTP * kStepY + k * kStepY);
+                        const float2 dyp[2] = {make_float2(yv.x, yv.y), make_float2(yv.z, yv.w)};
+                        float2 dBv[4], dCv[4], s1[2], s2[2];
+#pragma unroll
+                        for (int j = 0; j < 2; ++j) {
+                            const float4 v = at4(ug + k * kStepG + j * kBPairs * 16);
+                            const float2 dd = make_float2(v.x, v.y), gg = make_float2(v.z, v.w);
+#pragma unroll
+                            for (int n = 0; n < 4; ++n) {
+                                const float2 A = ab[k][j][n], H = hp[k][j][n];
+                                float2 gv, ga, w;
+                                gv.y = fmaf(dyp[j].y, cp[n].y, g[j][n]);
+                                ga.y = gv.y * A.y;
+                                gv.x = fmaf(dyp[j].x, cp[n].x, ga.y);
+                                ga.x = gv.x * A.x;
+                                g[j][n] = ga.x;
+                                w.x = ga.x * (k == 0 ? hs[j][n] : hp[k - 1][j][n].y);
+                                w.y = ga.y * H.x;
+                                dCv[n] = j == 0 ? mul2(dyp[0], H) : fma2(dyp[1], H, dCv[n]);
+                                dBv[n] = j == 0 ? mul2(gg, gv) : fma2(gg, gv, dBv[n]);
+                                s1[j] = n == 0 ? mul2(bp[0], gv) : fma2(bp[n], gv, s1[j]);
+                                // scalar: a packed form would copy a2 into a pair at every use (2459 -> 2435 us)
+                                s2[j].x = n == 0 ? a2[j][0] * w.x : fmaf(a2[j][n], w.x, s2[j].x);
+                                s2[j].y = n == 0 ? a2[j][0] * w.y : fmaf(a2[j][n], w.y, s2[j].y);
+                                dA[j][n] = fma2(dd, w, dA[j][n]);
+                            }
+                        }
+                        sh1[k] = make_float4(s1[0].x, s1[0].y, s1[1].x, s1[1].y);
+                        sh2[k] = make_float4(s2[0].x, s2[0].y, s2[1].x, s2[1].y);
+                        // dB, dC over the warp's 16 channels: lanes that differ in channel bits exchange the states they do
+                        // not keep; the state order r -> r ^ perm makes those registers 2, 3, then 1, on every lane
+#pragma unroll
+                        for (int n = 0; n < 2; ++n) {
+                            dBv[n] = add2(dBv[n], shfl2(dBv[n + 2], 8));
+                            dCv[n] = add2(dCv[n], shfl2(dCv[n + 2], 8));
+                        }
+                        dBv[0] = add2(dBv[0], shfl2(dBv[1], 4));
+                        dCv[0] = add2(dCv[0], shfl2(dCv[1], 4));
+                        const bool keepC = lane & 1;   // channel bit 2: this lane ends with dC of its state, or dB
+                        const float2 keep = keepC ? dCv[0] : dBv[0], send = keepC ? dBv[0] : dCv[0];
+                        sums[k] = add2(keep, shfl2(send, 1));
                     }
-                    dBv[0] = add2(dBv[0], shfl2(dBv[1], 4));
-                    dCv[0] = add2(dCv[0], shfl2(dCv[1], 4));
-                    const bool keepC = lane & 1;   // channel bit 2: this lane ends with dC of its state, or dB
-                    const float2 keep = keepC ? dCv[0] : dBv[0], send = keepC ? dBv[0] : dCv[0];
-                    sums[k] = add2(keep, shfl2(send, 1));
-                }
 #pragma unroll
-                for (int k = 0; k < kHTP; ++k) {
-                    at4(o_sh + kShare + k * kBPairs * 16) = sh1[k];
-                    at4(o_sh + 2 * kShare + k * kBPairs * 16) = sh2[k];
-                    s.sum[warp][k0 + k][8 * q + 4 * (lane & 1) + perm] = sums[k];
-                }
-                // finish this half's outputs
-                __syncwarp();
-                float2 tot[3][2];   // C.h, g.B, sum g Abar h A log2 e: [step] of (channel 2 pp, channel 2 pp + 1)
+                    for (int k = 0; k < kHTP; ++k) {
+                        at4(o_sh + kShare + k * kBPairs * 16) = sh1[k];
+                        at4(o_sh + 2 * kShare + k * kBPairs * 16) = sh2[k];
+                        s.sum[warp][k0 + k][8 * q + 4 * (lane & 1) + perm] = sums[k];
+                    }
+                    // finish this half's outputs
+                    __syncwarp();
+                    float2 tot[3][2];   // C.h, g.B, sum g Abar h A log2 e: [step] of (channel 2 pp, channel 2 pp + 1)
 #pragma unroll
-                for (int v = 0; v < 3; ++v) {
-                    const float4 *src = &sh[v][ts * kBPairs + pp];
-                    const float4 x0 = src[0], x1 = src[kShareQ], x2 = src[2 * kShareQ], x3 = src[3 * kShareQ];
-                    const float2 ca = add2(add2(make_float2(x0.x, x0.y), make_float2(x1.x, x1.y)),
-                                           add2(make_float2(x2.x, x2.y), make_float2(x3.x, x3.y)));
-                    const float2 cb = add2(add2(make_float2(x0.z, x0.w), make_float2(x1.z, x1.w)),
-                                           add2(make_float2(x2.z, x2.w), make_float2(x3.z, x3.w)));
-                    tot[v][0] = make_float2(ca.x, cb.x);
-                    tot[v][1] = make_float2(ca.y, cb.y);
-                }
-                const float4 va = dgw[k0 + ts][0][pp], vb = dgw[k0 + ts][1][pp], yv = dyw[k0 + ts][pp];
-                const float4 fs = s.fin[warp][0][k0 + ts][pp], fq = s.fin[warp][1][k0 + ts][pp];
+                    for (int v = 0; v < 3; ++v) {
+                        const float4 *src = &sh[v][ts * kBPairs + pp];
+                        const float4 x0 = src[0], x1 = src[kShareQ], x2 = src[2 * kShareQ], x3 = src[3 * kShareQ];
+                        const float2 ca = add2(add2(make_float2(x0.x, x0.y), make_float2(x1.x, x1.y)),
+                                               add2(make_float2(x2.x, x2.y), make_float2(x3.x, x3.y)));
+                        const float2 cb = add2(add2(make_float2(x0.z, x0.w), make_float2(x1.z, x1.w)),
+                                               add2(make_float2(x2.z, x2.w), make_float2(x3.z, x3.w)));
+                        tot[v][0] = make_float2(ca.x, cb.x);
+                        tot[v][1] = make_float2(ca.y, cb.y);
+                    }
+                    const float4 va = dgw[k0 + ts][0][pp], vb = dgw[k0 + ts][1][pp], yv = dyw[k0 + ts][pp];
+                    const float4 fs = s.fin[warp][0][k0 + ts][pp], fq = s.fin[warp][1][k0 + ts][pp];
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const int o = u ? off[1][e] : off[0][e];
-                    const float2 sg = e ? make_float2(fs.z, fs.w) : make_float2(fs.x, fs.y);
-                    const float2 qv = e ? make_float2(fq.z, fq.w) : make_float2(fq.x, fq.y);
-                    const float2 de = e ? make_float2(va.y, vb.y) : make_float2(va.x, vb.x);
-                    const float2 dyv = e ? make_float2(yv.y, yv.w) : make_float2(yv.x, yv.z);
-                    const float2 xv = ld2<T>(&r.x[0][0], o);
-                    const float2 ddt = mul2(fma2(xv, tot[1][e], mul2(tot[2][e], splat(kLn2))), sg);
-                    st2<T>(&s.gx[0][0], o, fma2(de, tot[1][e], mul2(dyv, dsk)));
-                    st2<T>(&s.gdt[0][0], o, ddt);
-                    if (gate) st2<T>(&s.gz[0][0], o, mul2(fma2(dsk, xv, tot[0][e]), qv));
-                    dD_acc = fma2(dyv, xv, dD_acc);
-                    db_acc = add2(db_acc, ddt);
+                    for (int e = 0; e < 2; ++e) {
+                        const int o = u ? off[1][e] : off[0][e];
+                        const float2 sg = e ? make_float2(fs.z, fs.w) : make_float2(fs.x, fs.y);
+                        const float2 qv = e ? make_float2(fq.z, fq.w) : make_float2(fq.x, fq.y);
+                        const float2 de = e ? make_float2(va.y, vb.y) : make_float2(va.x, vb.x);
+                        const float2 dyv = e ? make_float2(yv.y, yv.w) : make_float2(yv.x, yv.z);
+                        const float2 xv = ld2<T>(&r.x[0][0], o);
+                        const float2 ddt = mul2(fma2(xv, tot[1][e], mul2(tot[2][e], splat(kLn2))), sg);
+                        st2<T>(&s.gx[0][0], o, fma2(de, tot[1][e], mul2(dyv, dsk)));
+                        st2<T>(&s.gdt[0][0], o, ddt);
+                        if (gate) st2<T>(&s.gz[0][0], o, mul2(fma2(dsk, xv, tot[0][e]), qv));
+                        dD_acc = fma2(dyv, xv, dD_acc);
+                        db_acc = add2(db_acc, ddt);
+                    }
+                    __syncwarp();   // the shares may be written again
                 }
-                __syncwarp();   // the shares may be written again
+                fence_proxy_async_smem();   // output tiles -> visible to the TMA stores
             }
-            fence_proxy_async_smem();   // output tiles -> visible to the TMA stores
-        }
-        __syncthreads();
-        if (tid == 0) {
-            if constexpr (!kSummary) {
-                tma_store_3d(&a.tm_dx, &s.gx[0][0], d0, t0, b);
-                tma_store_3d(&a.tm_ddt, &s.gdt[0][0], d0, t0, b);
-                if (gate) tma_store_3d(&a.tm_dz, &s.gz[0][0], d0, t0, b);
-                bulk_commit();
-            }
-            if (it + S < nch) {   // the stage is consumed: refill it
-                fence_proxy_async_smem();
-                issue_bchunk<T, kSummary>(s, a, it % S, c0 + nch - 1 - (it + S), d0, b);
+            __syncthreads();
+            if (tid == 0) {
+                if constexpr (!kSummary) {
+                    tma_store_3d(&a.tm_dx, &s.gx[0][0], d0, t0, b);
+                    tma_store_3d(&a.tm_ddt, &s.gdt[0][0], d0, t0, b);
+                    if (gate) tma_store_3d(&a.tm_dz, &s.gz[0][0], d0, t0, b);
+                    bulk_commit();
+                }
+                if (it + S < nch) {   // the stage is consumed: refill it
+                    fence_proxy_async_smem();
+                    issue_bchunk<T, kSummary>(s, a, sl, c0 + nch - 1 - (it + S), d0, b);
+                }
             }
         }
-    }
-    if constexpr (kSummary) pdl_trigger();   // the second pass may set up while the last summaries are written
-    if constexpr (kSummary) {   // Abar g at the segment's start from a zero adjoint at its end; the product of its decays
-        if (!chan_ok) return;
-#pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int64_t o = (((int64_t)b * nseg + seg) * D + d + j) * kDState + 4 * q;
-            const float sd = dsum[j].x + dsum[j].y;
-            float pe[4];
-#pragma unroll
-            for (int n = 0; n < 4; ++n) pe[n] = ex2(a2[j][n] * sd);
-            store_perm(p.seg_h + o, g[j], perm);
-            store_perm(p.seg_p + o, pe, perm);
-        }
-    } else {
-        flush_sums(s, gp, b, c0 * kBT, L);   // the last chunk's
-#pragma unroll
-        for (int o = 8; o <= 16; o += 8) {   // over the four lanes of a channel pair
-            dD_acc = add2(dD_acc, shfl2(dD_acc, o));
-            db_acc = add2(db_acc, shfl2(db_acc, o));
-        }
-        if (ts == 0 && dc < D) {
-            if (gp.dD) atomicAdd(reinterpret_cast<float2 *>(gp.dD + dc), dD_acc);
-            if (gp.ddt_bias) atomicAdd(reinterpret_cast<float2 *>(gp.ddt_bias + dc), db_acc);
-        }
-        if (chan_ok) {
+        if constexpr (kSummary) pdl_trigger();   // the second pass may set up while the last summaries are written
+        if constexpr (kSummary) {   // Abar g at the segment's start from a zero adjoint at its end; the product of its decays
 #pragma unroll
             for (int j = 0; j < 2; ++j) {
+                if (!chan_ok) break;
+                const int64_t o = (((int64_t)b * nseg + seg) * D + d + j) * kDState + 4 * q;
+                const float sd = dsum[j].x + dsum[j].y;
+                float pe[4];
 #pragma unroll
-                for (int n = 0; n < 4; ++n)
-                    atomicAdd(gp.dA + (d + j) * kDState + 4 * q + (n ^ perm), dA[j][n].x + dA[j][n].y);
-                if (gp.dh0 && seg == 0)
-                    store_perm(gp.dh0 + ((int64_t)b * D + d + j) * kDState + 4 * q, g[j], perm);
+                for (int n = 0; n < 4; ++n) pe[n] = ex2(a2[j][n] * sd);
+                store_perm(p.seg_h + o, g[j], perm);
+                store_perm(p.seg_p + o, pe, perm);
+            }
+        } else {
+            flush_sums(s, gp, b, c0 * kBT, L);   // the last chunk's
+#pragma unroll
+            for (int o = 8; o <= 16; o += 8) {   // over the four lanes of a channel pair
+                dD_acc = add2(dD_acc, shfl2(dD_acc, o));
+                db_acc = add2(db_acc, shfl2(db_acc, o));
+            }
+            if (ts == 0 && dc < D) {
+                if (gp.dD) atomicAdd(reinterpret_cast<float2 *>(gp.dD + dc), dD_acc);
+                if (gp.ddt_bias) atomicAdd(reinterpret_cast<float2 *>(gp.ddt_bias + dc), db_acc);
+            }
+            if (chan_ok) {
+#pragma unroll
+                for (int j = 0; j < 2; ++j) {
+#pragma unroll
+                    for (int n = 0; n < 4; ++n)
+                        atomicAdd(gp.dA + (d + j) * kDState + 4 * q + (n ^ perm), dA[j][n].x + dA[j][n].y);
+                    if (gp.dh0 && c0 == 0)
+                        store_perm(gp.dh0 + ((int64_t)b * D + d + j) * kDState + 4 * q, g[j], perm);
+                }
+            }
+            if constexpr (kShares) {
+                if (c0 > 0) {   // the share ends inside the tile: leave the adjoint for the next one
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+                        __stcg(reinterpret_cast<float4 *>(p.share_h) + ((int64_t)share * 2 + j) * kBThreads + tid,
+                               make_float4(g[j][0], g[j][1], g[j][2], g[j][3]));
+                    __threadfence();
+                    __syncthreads();
+                    if (tid == 0) flag_set(p.share_sync + 1 + share);
+                }
             }
         }
-        if (tid == 0) bulk_wait_all();
+        if (!kShares || tile * nchunks <= lo) break;
+        n0 += nch;
+        --tile;
     }
+    if (!kSummary && tid == 0) bulk_wait_all();
 }
 
 // Zero the gradients that are accumulated atomically (16-byte aligned, sizes multiples of 16 bytes): one launch
 // instead of five memsets, which with their gaps took a small span's backward from 70 to 89 us (2 x 777 x 1544).
 struct ClearArgs {
-    float4 *p[5];
-    int64_t n[5];   // float4s
+    float4 *p[6];
+    int64_t n[6];   // float4s
 };
 constexpr int kClearThreads = 256;
 __global__ void __launch_bounds__(kClearThreads) clear_kernel(const __grid_constant__ ClearArgs a) {
@@ -590,7 +650,7 @@ __global__ void __launch_bounds__(kClearThreads) clear_kernel(const __grid_const
     pdl_wait();
     const int64_t step = (int64_t)gridDim.x * kClearThreads;
 #pragma unroll
-    for (int k = 0; k < 5; ++k)
+    for (int k = 0; k < 6; ++k)
         for (int64_t i = (int64_t)blockIdx.x * kClearThreads + threadIdx.x; i < a.n[k]; i += step)
             a.p[k][i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
@@ -642,6 +702,14 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
             return e;
     }
     a.grid_segs = (int)nseg;
+    if (nseg == 1 && p.shares > 0) {
+        auto ks = backward_kernel<T, false, true>;
+        if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
+            cudaSuccess)
+            return e;
+        return launch_pdl(true, ks, dim3((unsigned)p.shares), dim3(kBThreads), spread_smem(smem, p.shares, kBResident),
+                          s, a);
+    }
     auto k = backward_kernel<T, false>;
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) != cudaSuccess)
         return e;
@@ -677,16 +745,36 @@ int64_t backward_segments(const ScanParams &p) {
     return (nchunks + cps - 1) / cps;   // no empty segment
 }
 
+// Even shares (as prefill_shares), where the tiles are little over two per SM
+// or over a multiple of the slots. Microseconds per chunk of an SM's 1 to 4
+// CTAs, as measured (bf16), one CTA per tile: 3.2 3.4 4.7 4.8 (two CTAs of two
+// warps fill the four schedulers once, so a third costs as much as two more);
+// shares: 3.6 with two per SM, 5.05 with four. Measured, spans of 2048 steps at
+// 2.1, 4.2, 5.05 and 8.2 tiles per SM: 600 -> 486, 1000 -> 681, 1003 -> 815,
+// 1582 -> 1315 us.
+int64_t backward_shares(const ScanParams &p) {
+    if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinBwdSplitSteps || p.dt_low) return 0;
+    const int64_t sms = device_sms(), tiles = p.batch * ((p.d_inner + kBCh - 1) / kBCh);
+    if (sms <= 0 || tiles <= 2 * sms) return 0;
+    constexpr double t[4] = {3.17, 3.35, 4.69, 4.84};
+    const int64_t m = tiles < kBResident * sms ? 2 : kBResident, rest = tiles % (kBResident * sms);
+    const double plain = (double)(tiles / (kBResident * sms)) * t[kBResident - 1] + (rest ? t[(rest - 1) / sms] : 0.0);
+    const double even = (double)tiles / (double)(m * sms) * (m == 2 ? 3.6 : 5.05);
+    const double chunks = (double)(p.seqlen / kBT);
+    return even * chunks + 7.0 < 0.97 * plain * chunks ? m * sms : 0;
+}
+
 cudaError_t launch_backward(const ScanParams &p, const GradParams &g, bool bf16, cudaStream_t s) {
     const int64_t Bn = p.batch, L = p.seqlen, D = p.d_inner;
     // The sums are accumulated atomically: clear them first.
     cudaError_t e;
     ClearArgs c;
     const int64_t nbc = Bn * L * kDState / 4;
-    float *const ptr[5] = {g.dB, g.dC, g.dA, g.dD, g.ddt_bias};
-    const int64_t num[5] = {nbc, nbc, D * kDState / 4, g.dD ? D / 4 : 0, g.ddt_bias ? D / 4 : 0};
+    void *const ptr[6] = {g.dB, g.dC, g.dA, g.dD, g.ddt_bias, p.share_sync};
+    const int64_t num[6] = {nbc, nbc, D * kDState / 4, g.dD ? D / 4 : 0, g.ddt_bias ? D / 4 : 0,
+                            p.shares > 0 ? (int64_t)prefill_share_sync_bytes(p.shares) / 16 : 0};
     int64_t most = 0;
-    for (int k = 0; k < 5; ++k) {
+    for (int k = 0; k < 6; ++k) {
         c.p[k] = reinterpret_cast<float4 *>(ptr[k]);
         c.n[k] = num[k];
         if (num[k] > most) most = num[k];

@@ -101,18 +101,6 @@ struct FwdArgs {
 // 16-byte stores fall on different banks. The scan's loads of all 8 channels at one tp cover 128 bytes either way.
 __device__ __forceinline__ int dg_slot(int tp, int c) { return (((c ^ tp) & 1) << 2) | (c >> 1); }
 
-// A share's flag in global memory: set after its state has been written, and waited for (bounded).
-__device__ __forceinline__ void flag_set(int *f) { asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(f) : "memory"); }
-__device__ __forceinline__ bool flag_wait(const int *f) {
-    const long long t0 = clock64();
-    for (;;) {
-        int v;
-        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
-        if (v) return true;
-        if (clock64() - t0 > kWaitCycles) return false;
-    }
-}
-
 template <typename T, bool kSummary>
 __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int stage, int t, int d0, int b) {
     constexpr uint32_t tok = kRT<T> * kCh * sizeof(T), bc = kRT<T> * kDState * sizeof(T);
@@ -133,7 +121,7 @@ __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int st
 // product of its decays, 2^(A log2 e * sum of Delta); no outputs. In the second
 // pass (the plain kernel) segment s starts from those, folded with the
 // associative operator of Section 2: h <- P_s' * h + H_s'.
-// kShares: the grid is p.shares CTAs; the channel tiles' spans, laid end to end,
+// kShares (if not 0: the CTAs per SM it is compiled for): the grid is p.shares CTAs; the channel tiles' spans, laid end to end,
 // are cut into that many equal lengths, and a CTA scans the pieces in its own,
 // the highest first. Its highest piece starts a tile (or it is all of a CTA's
 // part of one) and depends on nothing; where it ends inside a tile, the CTA
@@ -141,8 +129,8 @@ __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int st
 // tile: it comes last and waits (bounded) for the state that the share before
 // has left as the first thing it did. Shares are numbered in the order in which
 // their CTAs start (a ticket), so the one waited for is always running.
-template <typename T, bool kCkpt, bool kSummary, bool kShares = false>
-__global__ void __launch_bounds__(kThreads, kShares ? kResident - 1 : kResident) forward_kernel(const __grid_constant__ FwdArgs a) {
+template <typename T, bool kCkpt, bool kSummary, int kShares = 0>
+__global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forward_kernel(const __grid_constant__ FwdArgs a) {
     using S = Smem<T>;
     using R = Raw<T>;
     constexpr int STAGES = kStages, SUB = kSub<T>, RT = kRT<T>, kRowB = kCh * (int)sizeof(T);
@@ -505,7 +493,8 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     }
     a.grid_segs = (int)nseg;
     if (nseg == 1 && p.shares > 0) {
-        auto ks = forward_kernel<T, kCkpt, false, true>;
+        auto ks = p.shares < kResident * lim->sms ? forward_kernel<T, kCkpt, false, kResident - 1>
+                                                  : forward_kernel<T, kCkpt, false, kResident>;
         if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
                 cudaSuccess ||
             (e = cudaMemsetAsync(p.share_sync, 0, prefill_share_sync_bytes(p.shares), s)) != cudaSuccess)
@@ -556,24 +545,31 @@ size_t prefill_split_bytes(const ScanParams &p, int64_t nseg) {
 // Even shares: CTAs of one tile each leave the GPU unevenly loaded when their
 // number is little over a multiple of the SMs: the SMs that hold one more set
 // the time (8 x 8192 x 2048: 512 tiles, 3.4 per SM). Then m = tiles / SMs
-// (rounded down) CTAs per SM take equal shares of all tiles' steps instead.
+// (rounded down, at most 4) CTAs per SM take equal shares of all tiles' steps.
 // Microseconds per chunk of an SM's CTAs, 1 to 4 of them, as measured:
-//   bf16 0.61 0.82 1.10 1.40, fp32 0.79 1.01 1.22 1.55
-// so shares pay off while tiles / (m SMs) * t[m] is well below t[m + 1] (bf16:
-// up to 1.26, 2.52 and 3.59 tiles per SM) and the span is long enough to make up
-// for the clearing of the flags and the second prologue (about 6 us). Measured:
-// 8 x 8192 x 2048 709 -> 650 us (622 by the rates alone), its training forward
-// 740 -> 672 us.
+//                        bf16                  fp32
+//   one CTA per tile     0.61 0.82 1.10 1.40   0.79 1.01 1.22 1.55
+//   shares               0.68 0.88 1.13 1.47   0.87 1.08 1.29 1.63
+// so m CTAs per SM finish tiles in tiles / (m SMs) times the second row, plus
+// about 7 us for the clearing of the flags and the second prologue, against the
+// first row's next number for one CTA per tile. More tiles than slots run in
+// waves; the last one, of r per SM, takes about 0.85 of its number (its CTAs
+// start as others end). Measured (bf16): 8 x 8192 x 2048 (3.4 tiles per SM)
+// 709 -> 650 us, its training forward 740 -> 672 us; spans of 2048 steps at 2.1,
+// 3.05, 4.2 and 5.3 tiles per SM 142 -> 126, 182 -> 158, 239 -> 206, 273 -> 254 us.
 constexpr double kChunkUs[2][4] = {{0.79, 1.01, 1.22, 1.55}, {0.61, 0.82, 1.10, 1.40}};
+constexpr double kShareUs[2][4] = {{0.87, 1.08, 1.29, 1.63}, {0.68, 0.88, 1.13, 1.47}};
 
 int64_t prefill_shares(const ScanParams &p, bool bf16) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinSplitSteps || p.dt_low) return 0;
     const int64_t sms = device_sms(), tiles = p.batch * ((p.d_inner + kCh - 1) / kCh);
-    if (sms <= 0 || tiles <= sms || tiles >= kResident * sms || tiles % sms == 0) return 0;
-    const int64_t m = tiles / sms;
-    const double even = (double)tiles / (double)(m * sms) * kChunkUs[bf16][m - 1], plain = kChunkUs[bf16][m];
-    if (even > 0.94 * plain || (plain - even) * (double)(p.seqlen / kT) < 8.0) return 0;
-    return m * sms;
+    if (sms <= 0 || tiles <= sms) return 0;
+    const int64_t m = tiles / sms < kResident ? tiles / sms : kResident, rest = tiles % (kResident * sms);
+    double plain = (double)(tiles / (kResident * sms)) * kChunkUs[bf16][kResident - 1];
+    if (rest) plain += (tiles > rest ? 0.85 : 1.0) * kChunkUs[bf16][(rest - 1) / sms];
+    const double even = (double)tiles / (double)(m * sms) * kShareUs[bf16][m - 1];
+    const double chunks = (double)(p.seqlen / kT);
+    return even * chunks + 7.0 < 0.97 * plain * chunks ? m * sms : 0;
 }
 
 size_t prefill_share_sync_bytes(int64_t shares) { return ((size_t)(shares + 1) * sizeof(int) + 255) / 256 * 256; }

@@ -42,9 +42,9 @@ struct ScanParams {
     // zero start and the product of its decays (scratch in the workspace).
     int64_t nseg;
     float *seg_h, *seg_p;
-    // Even shares of a prefill (0: off): `shares` CTAs of equal length, see
+    // Even shares of a prefill or backward (0: off): `shares` CTAs of equal length, see
     // prefill_shares. share_sync: a ticket counter, then a flag per share, all
-    // zero; share_h [shares, 32, 16]: the state where a share ends in a tile.
+    // zero; share_h [shares, 32, 16]: the state (adjoint) where a share ends in a tile.
     int64_t shares;
     int *share_sync;
     float *share_h;
@@ -99,6 +99,7 @@ size_t prefill_split_bytes(const ScanParams &p, int64_t nseg);
 // (0: one CTA per channel tile), and the scratch they need: share_sync (first,
 // prefill_share_sync_bytes) and share_h.
 int64_t prefill_shares(const ScanParams &p, bool bf16);
+int64_t backward_shares(const ScanParams &p);   // the same for the backward, with the same scratch
 size_t prefill_share_sync_bytes(int64_t shares);
 size_t prefill_share_bytes(int64_t shares);
 cudaError_t launch_verify(const ScanParams &p, bool bf16, cudaStream_t s);

@@ -205,7 +205,9 @@ size_t mb_workspace_size(const mb_scan_args *args) {
     const ScanParams p = to_params(args, nullptr, nullptr);
     const int64_t fwd = mbscan::prefill_segments(p), bwd = mbscan::backward_segments(p);
     const size_t split = mbscan::prefill_split_bytes(p, fwd > bwd ? fwd : bwd);
-    const size_t shares = fwd > 1 ? 0 : mbscan::prefill_share_bytes(mbscan::prefill_shares(p, args->dtype == MB_BF16));
+    const int64_t fs = fwd > 1 ? 0 : mbscan::prefill_shares(p, args->dtype == MB_BF16);
+    const int64_t bs = bwd > 1 ? 0 : mbscan::backward_shares(p);
+    const size_t shares = mbscan::prefill_share_bytes(fs > bs ? fs : bs);
     return mbscan::kStatusBytes + (split > shares ? split : shares);
 }
 
@@ -451,17 +453,21 @@ mb_status mb_scan_backward(const mb_scan_args *args, const float *h_ckpt, const 
             if (overlap(outs[i], outs[j])) return MB_ERR_INVALID_ARG;
     }
     ScanParams p = to_params(args, nullptr, static_cast<StatusBlock *>(ws));
-    // Split over L when the workspace holds the adjoint summaries and nothing that is read lies there.
-    const int64_t nseg = mbscan::backward_segments(p);
-    const size_t split = mbscan::prefill_split_bytes(p, nseg);
-    if (nseg > 1 && ws_bytes >= mbscan::kStatusBytes + split) {
-        float *scratch = reinterpret_cast<float *>(static_cast<char *>(ws) + mbscan::kStatusBytes);
+    // Split over L, or even shares, when the workspace holds the scratch and nothing that is read lies there.
+    const int64_t nseg = mbscan::backward_segments(p), shares = nseg > 1 ? 0 : mbscan::backward_shares(p);
+    const size_t scratch = nseg > 1 ? mbscan::prefill_split_bytes(p, nseg) : mbscan::prefill_share_bytes(shares);
+    if (scratch > 0 && ws_bytes >= mbscan::kStatusBytes + scratch) {
+        char *base = static_cast<char *>(ws) + mbscan::kStatusBytes;
         bool clear = true;
-        for (int i = 0; i < kIns - 1; ++i) clear = clear && !overlap(range_of(scratch, (int64_t)split), ins[i]);
-        if (clear) {
+        for (int i = 0; i < kIns - 1; ++i) clear = clear && !overlap(range_of(base, (int64_t)scratch), ins[i]);
+        if (clear && nseg > 1) {
             p.nseg = nseg;
-            p.seg_h = scratch;
-            p.seg_p = scratch + split / (2 * sizeof(float));
+            p.seg_h = reinterpret_cast<float *>(base);
+            p.seg_p = p.seg_h + scratch / (2 * sizeof(float));
+        } else if (clear) {
+            p.shares = shares;
+            p.share_sync = reinterpret_cast<int *>(base);
+            p.share_h = reinterpret_cast<float *>(base + mbscan::prefill_share_sync_bytes(shares));
         }
     }
     mbscan::GradParams gp;

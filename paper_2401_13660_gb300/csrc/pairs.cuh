@@ -70,4 +70,18 @@ __device__ __forceinline__ float2 silu2(float2 z) {
     return mul2(z, make_float2(rcp(o.x), rcp(o.y)));
 }
 
+// A share's flag in global memory: set after its state has been written, and waited for (bounded).
+__device__ __forceinline__ void flag_set(int *f) {
+    asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(f) : "memory");
+}
+__device__ __forceinline__ bool flag_wait(const int *f) {
+    const long long t0 = clock64();
+    for (;;) {
+        int v;
+        asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(v) : "l"(f) : "memory");
+        if (v) return true;
+        if (clock64() - t0 > kWaitCycles) return false;
+    }
+}
+
 }  // namespace mbscan
