@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
     int share = 0, lo = 0, hi = 0;   // kShares: chunks lo .. hi - 1 of all tiles' sweeps end to end
     int n0 = 0;                      // ring stages consumed by the pieces before
     if constexpr (kShares) {
-        if (tid == 0) s.ticket = atomicAdd(p.share_sync, 1);
+        if (tid == 0) s.ticket = atomicAdd(p.share_sync(), 1);
         __syncthreads();
         share = s.ticket;
         const int total = (int)p.batch * ntd * nchunks, len = (total + (int)p.shares - 1) / (int)p.shares;
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
         if constexpr (kShares) {
             if (c0 + nch < nchunks) {   // the share before has left the adjoint
                 bool set = true;
-                if (tid == 0) set = flag_wait(p.share_sync + share);
+                if (tid == 0) set = flag_wait(p.share_sync() + share);
                 if (__syncthreads_or(set ? 0 : 1)) {
                     if (tid == 0) {
                         report(p.status, 4 /* MB_ERR_TIMEOUT */, share);
@@ -303,7 +303,7 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
                 }
 #pragma unroll
                 for (int j = 0; j < 2; ++j) {
-                    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p.share_h) +
+                    const float4 v = __ldcg(reinterpret_cast<const float4 *>(p.seg_h) +
                                             ((int64_t)(share - 1) * 2 + j) * kBThreads + tid);
                     g[j][0] = v.x; g[j][1] = v.y; g[j][2] = v.z; g[j][3] = v.w;
                 }
@@ -623,11 +623,11 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
                 if (c0 > 0) {   // the share ends inside the tile: leave the adjoint for the next one
 #pragma unroll
                     for (int j = 0; j < 2; ++j)
-                        __stcg(reinterpret_cast<float4 *>(p.share_h) + ((int64_t)share * 2 + j) * kBThreads + tid,
+                        __stcg(reinterpret_cast<float4 *>(p.seg_h) + ((int64_t)share * 2 + j) * kBThreads + tid,
                                make_float4(g[j][0], g[j][1], g[j][2], g[j][3]));
                     __threadfence();
                     __syncthreads();
-                    if (tid == 0) flag_set(p.share_sync + 1 + share);
+                    if (tid == 0) flag_set(p.share_sync() + 1 + share);
                 }
             }
         }
@@ -770,7 +770,7 @@ cudaError_t launch_backward(const ScanParams &p, const GradParams &g, bool bf16,
     cudaError_t e;
     ClearArgs c;
     const int64_t nbc = Bn * L * kDState / 4;
-    void *const ptr[6] = {g.dB, g.dC, g.dA, g.dD, g.ddt_bias, p.share_sync};
+    void *const ptr[6] = {g.dB, g.dC, g.dA, g.dD, g.ddt_bias, p.share_sync()};
     const int64_t num[6] = {nbc, nbc, D * kDState / 4, g.dD ? D / 4 : 0, g.ddt_bias ? D / 4 : 0,
                             p.shares > 0 ? (int64_t)prefill_share_sync_bytes(p.shares) / 16 : 0};
     int64_t most = 0;

@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
     int tile = (int)(blockIdx.x / ntd / a.grid_segs) * ntd + (int)(blockIdx.x % ntd);
     int share = 0, lo = 0, hi = 0;
     if constexpr (kShares) {
-        if (tid == 0) s.ticket = atomicAdd(p.share_sync, 1);
+        if (tid == 0) s.ticket = atomicAdd(p.share_sync(), 1);
         __syncthreads();
         share = s.ticket;
         const int total = (int)p.batch * ntd * units, len = (total + (int)p.shares - 1) / (int)p.shares;
@@ -273,7 +273,7 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
         if constexpr (kShares) {
             if (tid == 0) {
                 bulk_wait_read_all();   // the piece before's last store no longer reads its output tile
-                if (tb > 0) ok = flag_wait(p.share_sync + share) && ok;   // share - 1's flag
+                if (tb > 0) ok = flag_wait(p.share_sync() + share) && ok;   // share - 1's flag
             }
         }
         if (__syncthreads_or(ok ? 0 : 1)) {
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
         if constexpr (kShares) {
             if (tb > 0 && chan_ok) {
                 const float4 hv = __ldcg(reinterpret_cast<const float4 *>(
-                    p.share_h + ((int64_t)(share - 1) * kCh + kWCh * warp + c) * kDState + 4 * q));
+                    p.seg_h + ((int64_t)(share - 1) * kCh + kWCh * warp + c) * kDState + 4 * q));
                 h[0] = hv.x; h[1] = hv.y; h[2] = hv.z; h[3] = hv.w;
             }
         }
@@ -432,11 +432,11 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
                 *reinterpret_cast<float4 *>(p.h_out + ((int64_t)b * D + d) * kDState + 4 * q) =
                     make_float4(h[0], h[1], h[2], h[3]);
         } else if constexpr (kShares) {   // the share ends here: leave the state for the next one
-            __stcg(reinterpret_cast<float4 *>(p.share_h + ((int64_t)share * kCh + kWCh * warp + c) * kDState + 4 * q),
+            __stcg(reinterpret_cast<float4 *>(p.seg_h + ((int64_t)share * kCh + kWCh * warp + c) * kDState + 4 * q),
                    make_float4(h[0], h[1], h[2], h[3]));
             __threadfence();
             __syncthreads();
-            if (tid == 0) flag_set(p.share_sync + 1 + share);
+            if (tid == 0) flag_set(p.share_sync() + 1 + share);
         }
         if (!kShares || tile * units <= lo) break;
         --tile;
@@ -497,7 +497,7 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
                                                   : forward_kernel<T, kCkpt, false, kResident>;
         if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
                 cudaSuccess ||
-            (e = cudaMemsetAsync(p.share_sync, 0, prefill_share_sync_bytes(p.shares), s)) != cudaSuccess)
+            (e = cudaMemsetAsync(p.share_sync(), 0, prefill_share_sync_bytes(p.shares), s)) != cudaSuccess)
             return e;
         return launch_pdl(true, ks, dim3((unsigned)p.shares), dim3(kThreads), spread_smem(smem, p.shares, kResident), s, a);
     }

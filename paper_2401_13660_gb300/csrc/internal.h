@@ -37,17 +37,18 @@ struct ScanParams {
     const float *h_prev_all;
     const int32_t *accept;
     int64_t k_prev;
-    // Time split of a prefill over nseg segments of L (1: not split): seg_h,
-    // seg_p [batch, nseg, d_inner, 16] hold each segment's end state from a
-    // zero start and the product of its decays (scratch in the workspace).
-    int64_t nseg;
+    // How a prefill or backward uses the workspace's scratch; at most one of the
+    // two is on. (Two 32-bit counts and two pointers serve both: kernel
+    // parameters 24 bytes longer made the decode step 0.1 us slower.)
+    //  * nseg > 1: time split over nseg segments of L. seg_h, seg_p [batch, nseg,
+    //    d_inner, 16]: each segment's end state from a zero start (the backward:
+    //    its adjoint at the start) and the product of its decays.
+    //  * shares > 0: equal shares, see prefill_shares. share_sync(): a ticket
+    //    counter, then a flag per share, all zero; seg_h [shares, 32, 16]: the
+    //    state (adjoint) where a share ends in a tile.
+    int32_t nseg, shares;
     float *seg_h, *seg_p;
-    // Even shares of a prefill or backward (0: off): `shares` CTAs of equal length, see
-    // prefill_shares. share_sync: a ticket counter, then a flag per share, all
-    // zero; share_h [shares, 32, 16]: the state (adjoint) where a share ends in a tile.
-    int64_t shares;
-    int *share_sync;
-    float *share_h;
+    __host__ __device__ int *share_sync() const { return reinterpret_cast<int *>(seg_p); }
 };
 
 constexpr int kRankTile = 64;    // dt_rank elements per 128-byte swizzled TMA box

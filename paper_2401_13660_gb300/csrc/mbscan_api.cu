@@ -160,13 +160,13 @@ mb_status setup_split(const mb_scan_args *args, ScanParams &p, const float *h_la
     for (const Range &r : others) clear = clear && !overlap(rs, r);
     if (nseg > 1) {
         if (!clear) return MB_ERR_INVALID_ARG;
-        p.nseg = nseg;
+        p.nseg = (int32_t)nseg;
         p.seg_h = reinterpret_cast<float *>(base);
         p.seg_p = p.seg_h + scratch / (2 * sizeof(float));
     } else if (clear) {   // otherwise one CTA per tile, which needs no scratch
-        p.shares = shares;
-        p.share_sync = reinterpret_cast<int *>(base);
-        p.share_h = reinterpret_cast<float *>(base + mbscan::prefill_share_sync_bytes(shares));
+        p.shares = (int32_t)shares;
+        p.seg_p = reinterpret_cast<float *>(base);
+        p.seg_h = reinterpret_cast<float *>(base + mbscan::prefill_share_sync_bytes(shares));
     }
     return MB_OK;
 }
@@ -461,13 +461,13 @@ mb_status mb_scan_backward(const mb_scan_args *args, const float *h_ckpt, const 
         bool clear = true;
         for (int i = 0; i < kIns - 1; ++i) clear = clear && !overlap(range_of(base, (int64_t)scratch), ins[i]);
         if (clear && nseg > 1) {
-            p.nseg = nseg;
+            p.nseg = (int32_t)nseg;
             p.seg_h = reinterpret_cast<float *>(base);
             p.seg_p = p.seg_h + scratch / (2 * sizeof(float));
         } else if (clear) {
-            p.shares = shares;
-            p.share_sync = reinterpret_cast<int *>(base);
-            p.share_h = reinterpret_cast<float *>(base + mbscan::prefill_share_sync_bytes(shares));
+            p.shares = (int32_t)shares;
+            p.seg_p = reinterpret_cast<float *>(base);
+            p.seg_h = reinterpret_cast<float *>(base + mbscan::prefill_share_sync_bytes(shares));
         }
     }
     mbscan::GradParams gp;
