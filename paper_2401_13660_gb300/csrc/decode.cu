@@ -50,20 +50,35 @@ struct StepSmem {
     uint64_t empty[kStepStages];
 };
 
+// What the kernel needs of a step, and no more: the decode step is launched for
+// every byte and layer, and kernel parameters cost time (24 bytes more: 0.1 us).
+struct StepParams {
+    int64_t batch, d_inner;
+    const float *A, *D, *dt_bias;
+    float *h_out;   // state
+    void *y;
+    StatusBlock *status;
+};
+template <bool kResume>
 struct StepArgs {
     CUtensorMap tm_state, tm_x, tm_dt, tm_z, tm_B, tm_C;
-    // resume: initial state of row s from h0 (tm_state over p.h0, box of one
-    // row) or from h_all[s, accept[s]-1] (tm_hall)
-    CUtensorMap tm_hall;
+    StepParams p;
+    int ntiles, ntiles_d, has_gate;
+};
+template <>
+struct StepArgs<true> {
+    // initial state of row s from h0 (tm_state over p.h0, box of one row) or
+    // from h_all[s, accept[s]-1] (tm_hall)
+    CUtensorMap tm_state, tm_x, tm_dt, tm_z, tm_B, tm_C, tm_hall;
+    StepParams p;
+    int ntiles, ntiles_d, has_gate, has_h0;
     const int32_t *accept;
     int64_t k;
-    ScanParams p;
-    int ntiles, ntiles_d, has_gate, has_h0;
 };
 
 // Resume: the drafted-byte index whose state row s starts from (0 .. k-1),
 // -1 for the cached state h0, or -2 when accept[s] is outside [0, k].
-__device__ __forceinline__ int resume_index(const StepArgs &a, int64_t s) {
+__device__ __forceinline__ int resume_index(const StepArgs<true> &a, int64_t s) {
     const int acc = __ldg(a.accept + s);
     return (acc < 0 || acc > a.k) ? -2 : acc - 1;
 }
@@ -115,10 +130,10 @@ __device__ __forceinline__ float4 lds4(const __nv_bfloat16 *p) {
 // [0, k] are reported and left untouched.
 // Minimum CTAs per SM: those its shared memory allows (3 for bf16, 2 for fp32).
 template <typename T, bool kResume>
-__global__ void __launch_bounds__(kStepThreads, sizeof(T) == 2 ? 3 : 2) step_kernel(const __grid_constant__ StepArgs a) {
+__global__ void __launch_bounds__(kStepThreads, sizeof(T) == 2 ? 3 : 2) step_kernel(const __grid_constant__ StepArgs<kResume> a) {
     extern __shared__ unsigned char smem_dyn[];
     StepSmem<T> &s = smem_aligned<StepSmem<T>>(smem_dyn);
-    const ScanParams &p = a.p;
+    const StepParams &p = a.p;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t D = p.d_inner;
 
@@ -300,12 +315,14 @@ template <typename T, bool kResume>
 cudaError_t launch_step_typed(const ScanParams &p, const float *h_all, const int32_t *accept, int64_t k,
                               cudaStream_t s) {
     const int es = sizeof(T);
-    StepArgs a;
+    StepArgs<kResume> a;
     memset(&a, 0, sizeof(a));
-    a.p = p;
-    a.accept = accept;
-    a.k = k;
-    a.has_h0 = p.h0 != nullptr;
+    a.p = StepParams{p.batch, p.d_inner, p.A, p.D, p.dt_bias, p.h_out, p.y, p.status};
+    if constexpr (kResume) {
+        a.accept = accept;
+        a.k = k;
+        a.has_h0 = p.h0 != nullptr;
+    }
     a.has_gate = p.z != nullptr;
     a.ntiles_d = (int)((p.d_inner + kStepCh - 1) / kStepCh);
     a.ntiles = a.ntiles_d * (int)((p.batch + kStepRows - 1) / kStepRows);
