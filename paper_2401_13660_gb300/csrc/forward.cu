@@ -44,6 +44,8 @@
 #include <stddef.h>
 #include <string.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "pairs.cuh"
 #include "tma.cuh"
@@ -93,7 +95,8 @@ struct FwdArgs {
     CUtensorMap tm_dt, tm_x, tm_z, tm_B, tm_C, tm_y;
     ScanParams p;
     int has_gate;
-    int grid_segs;   // segments of L covered by the grid (blockIdx = (b, segment, channel tile))
+    int seg0;        // first segment of L that the grid covers (blockIdx = (segment - seg0, batch row, channel tile))
+    int len0, len;   // steps of the first segment and of the others (the last may be shorter)
 };
 
 // Slot of channel c of a warp at step pair tp in its dg tile. A lane stores channels 2 pp and 2 pp + 1 one after
@@ -104,23 +107,25 @@ __device__ __forceinline__ int dg_slot(int tp, int c) { return (((c ^ tp) & 1) <
 template <typename T, bool kSummary>
 __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int stage, int t, int d0, int b) {
     constexpr uint32_t tok = kRT<T> * kCh * sizeof(T), bc = kRT<T> * kDState * sizeof(T);
-    const uint32_t bytes = ((a.has_gate ? 3 : 2) * tok) + (kSummary ? 1 : 2) * bc;
+    const bool gate = !kSummary && a.has_gate;
+    const uint32_t bytes = ((gate ? 3 : 2) * tok) + (kSummary ? 1 : 2) * bc;
     uint64_t *bar = &s.full[stage];
     mbar_arrive_expect_tx(bar, bytes);
     Raw<T> &r = s.raw[stage];
     tma_load_3d(&r.dt[0][0], &a.tm_dt, bar, d0, t, b);
     tma_load_3d(&r.x[0][0], &a.tm_x, bar, d0, t, b);
-    if (a.has_gate) tma_load_3d(&r.z[0][0], &a.tm_z, bar, d0, t, b);
+    if (gate) tma_load_3d(&r.z[0][0], &a.tm_z, bar, d0, t, b);
     tma_load_3d(&r.B[0][0], &a.tm_B, bar, 0, t, b);
     if (!kSummary) tma_load_3d(&r.C[0][0], &a.tm_C, bar, 0, t, b);
 }
 
 // kCkpt (training forward): also stores the state before every chunk.
-// kSummary (first pass of a time-split span): scans each segment but the last
-// from a zero state (segment 0: from h0) and records its end state and the
-// product of its decays, 2^(A log2 e * sum of Delta); no outputs. In the second
-// pass (the plain kernel) segment s starts from those, folded with the
-// associative operator of Section 2: h <- P_s' * h + H_s'.
+// kSummary (first pass of a time-split span, every segment but the first and the
+// last): scans the segment from a zero state and records its end state and the
+// product of its decays, 2^(A log2 e * sum of Delta); no outputs. The first
+// segment starts from h0, so that pass scans it for good and records only its
+// end state. In the second pass segment s starts from what the first recorded,
+// folded with the associative operator of Section 2: h <- P_s' * h + H_s'.
 // kShares (if not 0: the CTAs per SM it is compiled for): the grid is p.shares CTAs; the channel tiles' spans, laid end to end,
 // are cut into that many equal lengths, and a CTA scans the pieces in its own,
 // the highest first. Its highest piece starts a tile (or it is all of a CTA's
@@ -129,8 +134,8 @@ __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int st
 // tile: it comes last and waits (bounded) for the state that the share before
 // has left as the first thing it did. Shares are numbered in the order in which
 // their CTAs start (a ticket), so the one waited for is always running.
-template <typename T, bool kCkpt, bool kSummary, int kShares = 0>
-__global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forward_kernel(const __grid_constant__ FwdArgs a) {
+template <typename T, bool kCkpt, bool kSummary, int kShares>
+__device__ __forceinline__ void scan_spans(const FwdArgs &a) {
     using S = Smem<T>;
     using R = Raw<T>;
     constexpr int STAGES = kStages, SUB = kSub<T>, RT = kRT<T>, kRowB = kCh * (int)sizeof(T);
@@ -143,13 +148,13 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
     const ScanParams &p = a.p;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int64_t D = p.d_inner;
-    // blockIdx.x = (batch row, segment of L, channel tile), channel tile fastest
     const int ntd = (int)((D + kCh - 1) / kCh);
     const int L = (int)p.seqlen;
-    const int seg = kShares ? 0 : (int)((blockIdx.x / ntd) % a.grid_segs);
+    const int tiles = (int)p.batch * ntd;
+    const int seg = kShares ? 0 : a.seg0 + (int)(blockIdx.x / tiles);
     const int nseg = p.nseg > 1 ? (int)p.nseg : 1;
-    const int units = (L + kSegUnit - 1) / kSegUnit, ups = (units + nseg - 1) / nseg;   // of the span, per segment
-    const bool gate = a.has_gate != 0;
+    const int units = (L + kSegUnit - 1) / kSegUnit;   // kShares
+    const bool gate = !kSummary && a.has_gate;
 
     if (tid == 0) {
         for (int st = 0; st < STAGES; ++st) mbar_init(&s.full[st], 1);
@@ -162,13 +167,13 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
     uint32_t ph = 0;   // and its phase parity
     // this CTA's tile (batch row, 32 channels); with kShares the units of 32 steps lo .. hi - 1 of all tiles' spans
     // end to end, which it takes tile by tile from the highest
-    int tile = (int)(blockIdx.x / ntd / a.grid_segs) * ntd + (int)(blockIdx.x % ntd);
+    int tile = (int)(blockIdx.x % tiles);
     int share = 0, lo = 0, hi = 0;
     if constexpr (kShares) {
         if (tid == 0) s.ticket = atomicAdd(p.share_sync(), 1);
         __syncthreads();
         share = s.ticket;
-        const int total = (int)p.batch * ntd * units, len = (total + (int)p.shares - 1) / (int)p.shares;
+        const int total = tiles * units, len = (total + (int)p.shares - 1) / (int)p.shares;
         lo = min(share * len, total);
         hi = min(lo + len, total);
         if (lo == hi) return;
@@ -176,9 +181,10 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
     }
     for (;;) {   // pieces: one without kShares
         const int b = tile / ntd, d0 = (tile % ntd) * kCh;
-        const int tb = kShares ? max(lo - tile * units, 0) * kSegUnit : seg * ups * kSegUnit;   // its steps: tb .. te - 1
-        const int te = min(L, kShares ? (hi - tile * units) * kSegUnit : tb + ups * kSegUnit);
-        const int nch = (te - tb + RT - 1) / RT;                                               // its stages
+        // its steps: tb .. te - 1
+        const int tb = kShares ? max(lo - tile * units, 0) * kSegUnit : seg == 0 ? 0 : a.len0 + (seg - 1) * a.len;
+        const int te = min(L, kShares ? (hi - tile * units) * kSegUnit : seg == 0 ? a.len0 : tb + a.len);
+        const int nch = (te - tb + RT - 1) / RT;   // its stages
         if (tid == 0) {
             fence_proxy_async_smem();
             for (int j = 0, sl = st; j < STAGES && j < nch; ++j, sl = sl + 1 == STAGES ? 0 : sl + 1)
@@ -215,9 +221,13 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
                     for (int sp = 0; sp < seg; ++sp) {
                         const int64_t o = (((int64_t)b * nseg + sp) * D + d) * kDState + 4 * q;
                         const float4 he = *reinterpret_cast<const float4 *>(p.seg_h + o);
-                        const float4 pe = *reinterpret_cast<const float4 *>(p.seg_p + o);
-                        hv = sp == 0 ? he : make_float4(fmaf(pe.x, hv.x, he.x), fmaf(pe.y, hv.y, he.y),
-                                                        fmaf(pe.z, hv.z, he.z), fmaf(pe.w, hv.w, he.w));
+                        if (sp == 0) {
+                            hv = he;
+                        } else {
+                            const float4 pe = *reinterpret_cast<const float4 *>(p.seg_p + o);
+                            hv = make_float4(fmaf(pe.x, hv.x, he.x), fmaf(pe.y, hv.y, he.y),
+                                             fmaf(pe.z, hv.z, he.z), fmaf(pe.w, hv.w, he.w));
+                        }
                     }
                 }
             }
@@ -431,7 +441,11 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
             if (p.h_out && chan_ok)
                 *reinterpret_cast<float4 *>(p.h_out + ((int64_t)b * D + d) * kDState + 4 * q) =
                     make_float4(h[0], h[1], h[2], h[3]);
-        } else if constexpr (kShares) {   // the share ends here: leave the state for the next one
+        } else if constexpr (!kShares) {
+            if (seg == 0 && chan_ok)   // first pass: the first segment's end
+                *reinterpret_cast<float4 *>(p.seg_h + ((int64_t)b * nseg * D + d) * kDState + 4 * q) =
+                    make_float4(h[0], h[1], h[2], h[3]);
+        } else {   // the share ends here: leave the state for the next one
             __stcg(reinterpret_cast<float4 *>(p.seg_h + ((int64_t)share * kCh + kWCh * warp + c) * kDState + 4 * q),
                    make_float4(h[0], h[1], h[2], h[3]));
             __threadfence();
@@ -442,6 +456,19 @@ __global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forwa
         --tile;
     }
     if (kShares && tid == 0) bulk_wait_all();
+}
+
+template <typename T, bool kCkpt, int kShares = 0>
+__global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forward_kernel(const __grid_constant__ FwdArgs a) {
+    scan_spans<T, kCkpt, false, kShares>(a);
+}
+
+template <typename T, bool kCkpt>
+__global__ void __launch_bounds__(kThreads, kResident) first_pass_kernel(const __grid_constant__ FwdArgs a) {
+    if (blockIdx.x < a.p.batch * ((a.p.d_inner + kCh - 1) / kCh))   // segment 0
+        scan_spans<T, kCkpt, false, 0>(a);
+    else
+        scan_spans<T, kCkpt, true, 0>(a);
 }
 
 // ---------------------------------------------------------------------------
@@ -457,6 +484,21 @@ bool make_map(CUtensorMap *m, const void *base, int es, int64_t batch, int64_t L
     return encode_tmap(m, base, es, 3, dims, strides, box, swizzle);
 }
 
+// Split of a span into at most nseg segments, in multiples of `unit` steps (a stage: y is stored by stages). The first
+// is scanned for good while the others are summarised, which takes kFirst of its time per step, and is that much shorter.
+constexpr double kFirst = 0.7;
+struct Segments {
+    int64_t n, len0, len;   // n <= nseg
+};
+Segments segments(int64_t L, int64_t nseg, int64_t unit) {
+    if (nseg < 2) return {1, L, L};
+    const int64_t units = (L + unit - 1) / unit;
+    int64_t others = (int64_t)((double)units / ((double)(nseg - 1) + kFirst));
+    if (others < 1 || units - others * (nseg - 1) > others) ++others;   // the first is the shorter
+    const int64_t m = std::min(nseg - 1, (units - 1) / others);
+    return {m + 1, (units - m * others) * unit, others * unit};
+}
+
 template <typename T, bool kCkpt>
 cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     constexpr int es = sizeof(T), sw = kCh * es;   // one token row of a tile
@@ -465,7 +507,11 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     a.p = p;
     a.has_gate = p.z != nullptr;
     if (p.nseg < 2 || !p.seg_h || !p.seg_p) a.p.nseg = 1;
-    const int64_t nseg = a.p.nseg, D = p.d_inner;
+    const int64_t D = p.d_inner;
+    const Segments g = segments(p.seqlen, a.p.nseg, kRT<T>);
+    const int64_t nseg = g.n;
+    a.len0 = (int)g.len0;
+    a.len = (int)g.len;
     auto tok = [&](CUtensorMap *m, const void *base) {
         return make_map(m, base, es, p.batch, p.seqlen, D, kCh, D, sw, kRT<T>);
     };
@@ -478,34 +524,31 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     if (!lim) return cudaErrorInvalidDevice;
     const int64_t ctas = ((D + kCh - 1) / kCh) * p.batch;   // per segment of L
     cudaError_t e;
-    if (nseg > 1) {   // first pass: summaries of segments 0 .. nseg-2
-        FwdArgs a1 = a;
-        a1.has_gate = 0;   // no outputs: the gate is not read
-        a1.grid_segs = (int)(nseg - 1);
-        auto k1 = forward_kernel<T, false, true>;
+    if (nseg > 1) {   // first pass: segments 0 .. nseg-2
+        auto k1 = first_pass_kernel<T, kCkpt>;
         if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
             cudaSuccess)
             return e;
         const int64_t grid = ctas * (nseg - 1);
-        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kThreads), spread_smem(smem, grid, kResident), s, a1)) !=
+        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kThreads), spread_smem(smem, grid, kResident), s, a)) !=
             cudaSuccess)
             return e;
+        a.seg0 = 1;   // second pass: segments 1 .. nseg-1
     }
-    a.grid_segs = (int)nseg;
     if (nseg == 1 && p.shares > 0) {
-        auto ks = p.shares < kResident * lim->sms ? forward_kernel<T, kCkpt, false, kResident - 1>
-                                                  : forward_kernel<T, kCkpt, false, kResident>;
+        auto ks = p.shares < kResident * lim->sms ? forward_kernel<T, kCkpt, kResident - 1>
+                                                  : forward_kernel<T, kCkpt, kResident>;
         if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
                 cudaSuccess ||
             (e = cudaMemsetAsync(p.share_sync(), 0, prefill_share_sync_bytes(p.shares), s)) != cudaSuccess)
             return e;
         return launch_pdl(true, ks, dim3((unsigned)p.shares), dim3(kThreads), spread_smem(smem, p.shares, kResident), s, a);
     }
-    auto k = forward_kernel<T, kCkpt, false>;
+    auto k = forward_kernel<T, kCkpt>;
     e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin);
     if (e != cudaSuccess) return e;
-    return launch_pdl(true, k, dim3((unsigned)(ctas * nseg)), dim3(kThreads), spread_smem(smem, ctas * nseg, kResident), s,
-                      a);
+    const int64_t grid = ctas * (nseg - a.seg0);
+    return launch_pdl(true, k, dim3((unsigned)grid), dim3(kThreads), spread_smem(smem, grid, kResident), s, a);
 }
 
 }  // namespace
@@ -515,27 +558,45 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
 // pass repeats most of a scan, so at 1.7 CTAs per SM, batch 4 x 2048 channels,
 // the split measured slower) and the span is long enough to pay for the second
 // launch: at 128 steps x 2048 channels unsplit 8.5 us, split 10.3; at 256 steps
-// 14.4 and 12.3. Then into as many segments as fill the resident slots (4 per
-// SM), each at least kSegUnit long. Every lane folds the summaries before its
-// segment, about 0.07 us each, while a step costs about 0.1 us over both passes:
-// their sum is least at sqrt(1.4 L) segments, which bounds spans of very few
-// channels (8192 x 64: 86 segments 20 us, 256 segments 35 us, 16 segments 37 us;
-// fp32 256 x 64: 8 segments 8.4 us, 2 segments 14.4 us).
+// 14.4 and 12.3. Both passes run all segments but one, in 1 to 4 CTAs per SM:
+// more CTAs share an SM better, but not in proportion (kChunkUs), and a number
+// that leaves some SMs with one CTA less pays for it as if they had it. So, of
+// the counts that fill 1, 2, 3 or 4 per SM, the one with the least chunks x time
+// per chunk. (Microseconds with at most 3 and at most 4 per SM: bf16 1 x 8192 x
+// 2048 126.9, 129.7; 1 x 8192 x 1024 70.0, 66.7; fp32 2 x 3000 x 1536 85.9, 77.3;
+// 1 x 777 x 3584 25.8, 27.7.) Every lane folds the summaries before its segment,
+// about 0.07 us each, while a step costs about 0.1 us over both passes: their sum
+// is least at sqrt(1.4 L) segments, which bounds spans of very few channels
+// (8192 x 64: 86 segments 20 us, 256 segments 35 us, 16 segments 37 us; fp32
+// 256 x 64: 8 segments 8.4 us, 2 segments 14.4 us).
+// With the first segment summarised like the others, and scanned in the second
+// pass: bf16 1 x 8192 x 2048 139 us (now 126), fp32 3 x 1003 x 1544 42.7 (40.7).
 constexpr int64_t kMinSplitSteps = 256;
+constexpr double kFoldUs = 0.07;
+// Microseconds per chunk of an SM's CTAs, 1 to 4 of them, as measured (fp32, bf16)
+constexpr double kChunkUs[2][4] = {{0.79, 1.01, 1.22, 1.55}, {0.61, 0.82, 1.10, 1.40}};
 
-int64_t prefill_segments(const ScanParams &p) {
+int64_t prefill_segments(const ScanParams &p, bool bf16) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinSplitSteps || p.dt_low) return 1;
     const int64_t sms = device_sms();
     const int64_t ctas = p.batch * ((p.d_inner + kCh - 1) / kCh);
     if (ctas > sms) return 1;
-    const int64_t units = (p.seqlen + kSegUnit - 1) / kSegUnit;
-    int64_t nseg = kResident * sms / ctas;
-    const int64_t most = (int64_t)sqrt(1.4 * (double)p.seqlen);
-    if (nseg > most) nseg = most;
-    if (nseg > units) nseg = units;
-    if (nseg < 2) return 1;
-    const int64_t ups = (units + nseg - 1) / nseg;
-    return (units + ups - 1) / ups;   // no empty segment
+    const int64_t unit = bf16 ? kRT<__nv_bfloat16> : kRT<float>;
+    const int64_t most = std::min((p.seqlen + kSegUnit - 1) / kSegUnit, (int64_t)sqrt(1.4 * (double)p.seqlen));
+    int64_t best = 1;
+    double least = 0;
+    for (int64_t m = 1; m <= kResident; ++m) {
+        const int64_t nseg = std::min(m * sms / ctas + 1, most);
+        if (nseg < 3) continue;   // two: one after the other
+        const Segments g = segments(p.seqlen, nseg, unit);
+        const int64_t per_sm = (ctas * (g.n - 1) + sms - 1) / sms;
+        const double us = (1 + kFirst) * kChunkUs[bf16][per_sm - 1] * (double)(g.len / kT) + kFoldUs * (double)g.n;
+        if (best == 1 || us < least) {
+            best = nseg;
+            least = us;
+        }
+    }
+    return best;
 }
 
 size_t prefill_split_bytes(const ScanParams &p, int64_t nseg) {
@@ -557,7 +618,6 @@ size_t prefill_split_bytes(const ScanParams &p, int64_t nseg) {
 // start as others end). Measured (bf16): 8 x 8192 x 2048 (3.4 tiles per SM)
 // 709 -> 650 us, its training forward 740 -> 672 us; spans of 2048 steps at 2.1,
 // 3.05, 4.2 and 5.3 tiles per SM 142 -> 126, 182 -> 158, 239 -> 206, 273 -> 254 us.
-constexpr double kChunkUs[2][4] = {{0.79, 1.01, 1.22, 1.55}, {0.61, 0.82, 1.10, 1.40}};
 constexpr double kShareUs[2][4] = {{0.87, 1.08, 1.29, 1.63}, {0.68, 0.88, 1.13, 1.47}};
 
 int64_t prefill_shares(const ScanParams &p, bool bf16) {

@@ -92,7 +92,7 @@ cudaError_t launch_forward(const ScanParams &p, bool bf16, cudaStream_t s);
 // Segments a prefill of these sizes is split into when the workspace has room
 // (1 when the batch rows and channels alone fill the GPU), and the scratch
 // bytes that split needs beyond the status block.
-int64_t prefill_segments(const ScanParams &p);
+int64_t prefill_segments(const ScanParams &p, bool bf16);
 // The same for the backward (its adjoint summaries need the same scratch per segment).
 int64_t backward_segments(const ScanParams &p);
 size_t prefill_split_bytes(const ScanParams &p, int64_t nseg);

@@ -143,7 +143,7 @@ mb_status check_ws(const mb_scan_args *a, void *ws, size_t ws_bytes) {
 mb_status setup_split(const mb_scan_args *args, ScanParams &p, const float *h_last, void *ws, size_t ws_bytes,
                       Range ckpt = Range{}) {
     const bool bf16 = args->dtype == MB_BF16;
-    const int64_t nseg = mbscan::prefill_segments(p), shares = nseg > 1 ? 0 : mbscan::prefill_shares(p, bf16);
+    const int64_t nseg = mbscan::prefill_segments(p, bf16), shares = nseg > 1 ? 0 : mbscan::prefill_shares(p, bf16);
     const size_t scratch = nseg > 1 ? mbscan::prefill_split_bytes(p, nseg) : mbscan::prefill_share_bytes(shares);
     if (scratch == 0 || ws_bytes < mbscan::kStatusBytes + scratch) return MB_OK;
     const int64_t es = bf16 ? 2 : 4;
@@ -203,9 +203,10 @@ extern "C" {
 size_t mb_workspace_size(const mb_scan_args *args) {
     if (check_args(args, false, false) != MB_OK) return 0;
     const ScanParams p = to_params(args, nullptr, nullptr);
-    const int64_t fwd = mbscan::prefill_segments(p), bwd = mbscan::backward_segments(p);
+    const bool bf16 = args->dtype == MB_BF16;
+    const int64_t fwd = mbscan::prefill_segments(p, bf16), bwd = mbscan::backward_segments(p);
     const size_t split = mbscan::prefill_split_bytes(p, fwd > bwd ? fwd : bwd);
-    const int64_t fs = fwd > 1 ? 0 : mbscan::prefill_shares(p, args->dtype == MB_BF16);
+    const int64_t fs = fwd > 1 ? 0 : mbscan::prefill_shares(p, bf16);
     const int64_t bs = bwd > 1 ? 0 : mbscan::backward_shares(p);
     const size_t shares = mbscan::prefill_share_bytes(fs > bs ? fs : bs);
     return mbscan::kStatusBytes + (split > shares ? split : shares);
