@@ -243,6 +243,7 @@ def reduce_max(value, dist, device="cpu"):
 def build_gpu_state(dev):
     import torch
 
+    from paper_2401_13660_gb300 import mbscan as mb
     from paper_2401_13660_gb300.inputs import make_inputs
 
     def alloc(inp, h_last=False, h_all=False, seed_accept=False):
@@ -250,6 +251,9 @@ def build_gpu_state(dev):
         out = dict(inp)
         out["y"] = torch.empty_like(x)
         out["ws"] = torch.zeros(256, dtype=torch.uint8, device=dev)
+        if "dt" in inp and x.shape[1] > 1:   # the scratch that the library asks for (a decode step needs none)
+            out["ws"] = mb.new_workspace(mb.make_args(x, inp["dt"], inp["B"], inp["C"], inp["A"], out["y"],
+                                                      z=inp["z"]), dev)
         if h_last:
             out["h_last"] = torch.empty(x.shape[0], x.shape[2], N_STATE, device=dev)
         if h_all:
@@ -447,7 +451,7 @@ def gpu_arm(args, rank, world, dist):
     dom_launch_ms = tot[dom] / (K * launches[dom])
     dom_bytes = parts[dom] / launches[dom]
     achieved = dom_bytes / (dom_launch_ms * 1e-3) / 1e9
-    kernel_key = {"prefill": "prefill_kernel", "verify": "verify_kernel",
+    kernel_key = {"prefill": "forward_kernel", "verify": "verify_kernel",
                   "rollback": "rollback_kernel", "step": "step_kernel"}[dom]
     roofline = {"kernel": kernel_key, "bound": "hbm", "achieved": round(achieved, 1),
                 "peak": peak, "peak_kind": f"{peak_kind} (hbm_gbs)", "unit": "GB/s",
@@ -542,7 +546,7 @@ def prefill_972m_leg(args, mb, stream, dev, dist, peak):
     inp = make_inputs(**c, d_state=N_STATE, dtype="bf16", h0="normal", seed=2, device=dev)
     inp["y"] = torch.empty_like(inp["x"])
     inp["h_last"] = torch.empty(c["batch"], c["d_inner"], N_STATE, device=dev)
-    ws = torch.zeros(256, dtype=torch.uint8, device=dev)
+    ws = mb.new_workspace(mb.make_args(inp["x"], inp["dt"], inp["B"], inp["C"], inp["A"], inp["y"], z=inp["z"]), dev)
 
     def fn():
         mb.mb_scan_prefill(inp["x"], inp["dt"], inp["B"], inp["C"], inp["A"], inp["y"], z=inp["z"], D=inp["D"],

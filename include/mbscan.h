@@ -111,9 +111,9 @@ typedef struct {
 /* Bytes of device workspace to pass with `args`: a 256-byte status block
  * (written by bounded device-side waits), plus scratch for the spans that run
  * faster with it: when the batch rows and channels of a long span fill only
- * part of the GPU, prefill and backward split it over L (two passes:
- * per-segment summaries, then every segment from its folded start; Section
- * 2's associative operator); when they fill it unevenly, prefill runs in equal
+ * part of the GPU, prefill and backward split it over L (two passes: summaries
+ * of the segments, then the segments from their folded starts; Section 2's
+ * associative operator); when they fill it unevenly, they run in equal
  * shares that hand the state on where a share ends inside a channel's span.
  * Any workspace of at least 256 bytes is accepted: with a smaller one than
  * this such spans run as they are. The scratch needs no clearing. The caller

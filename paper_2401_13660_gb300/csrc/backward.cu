@@ -40,9 +40,9 @@
 //
 // What bounds it: issue at 2 warps per scheduler (registers hold half a chunk's
 // states and decays: 254 of them), of which a loop of the core instructions
-// alone reaches 0.52 per clock; it runs at 0.48. Two channels per lane halve
+// alone reaches 0.52 per clock; it runs at 0.51. Two channels per lane halve
 // the loads of B and C and the exchange of dB, dC per channel. Measured (8 x
-// 8192 x 2048 bf16): 3.23 -> 2.51 ms, 2.08 -> 1.36 G warp instructions; before,
+// 8192 x 2048 bf16): 3.23 -> 2.43 ms, 2.08 -> 1.40 G warp instructions; before,
 // the four warps added dB, dC with shared float atomics, a compare-and-swap loop
 // that cost 5.5 clocks per instruction and kept the compiler from moving code
 // across steps. Variants: quarters of a chunk in registers (193 registers, a

@@ -22,7 +22,7 @@
 //    16-byte slot, B and C are widened to fp32 in pairs (t, t + 1), so decay
 //    exponents, B Delta x and the sum C.h need no copies that duplicate a
 //    scalar and no add across a pair; only the recurrence itself is scalar.
-//    (Pairs of states: 35.3 instructions per lane and step; this: 29.6.)
+//    (Pairs of states: 35.3 instructions per lane and step; this: 29.6, 27.3 with 32-step stages.)
 //  * A 128-bit shared load takes 2 wavefronts instead of 4 if lanes that differ
 //    in lane bit 0 (or in bit 1) read the same address. Lane bit 0 is a channel
 //    bit and bit 1 a state bit (channel bits 0, 2, 3; state bits 1, 4), so that
@@ -36,10 +36,11 @@
 //  * Token tiles are swizzled by TMA: a warp reads 16-byte columns of them.
 //
 // Measured (B x L x D, bf16; before: pairs of states, shuffles): 8 x 8192 x 2048
-// 850 -> 764 us, 4 x 8192 x 3584 708 -> 592 us, 1 x 8192 x 2048 (time split) 176
-// -> 152 us, fp32 3 x 1003 x 1544 56 -> 48 us. Two channels per lane (B and C
-// loaded once for both: 17 % fewer wavefronts) measured 758 / 750 us on the
-// first two: half the warps; two-warp CTAs (16 channels) 784 / 640 us.
+// 850 -> 764 us, with 32-step stages 709, in even shares 650 (0.45 of the SFU's
+// rate); 4 x 8192 x 3584 708 -> 592 -> 553 us; 1 x 8192 x 2048 (time split) 176 ->
+// 126 us; fp32 3 x 1003 x 1544 (time split) 56 -> 40.6 us. At 764 / 592: two
+// channels per lane (B and C loaded once for both: 17 % fewer wavefronts) 758 /
+// 750 us on the first two: half the warps; two-warp CTAs (16 channels) 784 / 640.
 #include <math.h>
 #include <stddef.h>
 #include <string.h>

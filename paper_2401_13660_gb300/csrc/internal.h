@@ -38,11 +38,11 @@ struct ScanParams {
     const int32_t *accept;
     int64_t k_prev;
     // How a prefill or backward uses the workspace's scratch; at most one of the
-    // two is on. (Two 32-bit counts and two pointers serve both: kernel
-    // parameters 24 bytes longer made the decode step 0.1 us slower.)
-    //  * nseg > 1: time split over nseg segments of L. seg_h, seg_p [batch, nseg,
-    //    d_inner, 16]: each segment's end state from a zero start (the backward:
-    //    its adjoint at the start) and the product of its decays.
+    // two is on.
+    //  * nseg > 1: time split over at most nseg segments of L. seg_h, seg_p
+    //    [batch, nseg, d_inner, 16]: each segment's end state from a zero start,
+    //    the first's from h0 (the backward: its adjoint at the start, the last's
+    //    from dh_last) and the product of its decays.
     //  * shares > 0: equal shares, see prefill_shares. share_sync(): a ticket
     //    counter, then a flag per share, all zero; seg_h [shares, 32, 16]: the
     //    state (adjoint) where a share ends in a tile.
