@@ -36,9 +36,9 @@
 //  * Token tiles are swizzled by TMA: a warp reads 16-byte columns of them.
 //
 // Measured (B x L x D, bf16; before: pairs of states, shuffles): 8 x 8192 x 2048
-// 850 -> 764 us, with 32-step stages 709, in even shares 650 (0.45 of the SFU's
-// rate); 4 x 8192 x 3584 708 -> 592 -> 553 us; 1 x 8192 x 2048 (time split) 176 ->
-// 126 us; fp32 3 x 1003 x 1544 (time split) 56 -> 40.6 us. At 764 / 592: two
+// 850 -> 764 us, with 32-step stages 709, in even shares 650, of 64-step stages 623
+// (0.47 of the SFU's rate); 4 x 8192 x 3584 708 -> 592 -> 553 -> 530 us; 1 x 8192 x
+// 2048 (time split) 176 -> 122 us; fp32 3 x 1003 x 1544 (time split) 56 -> 39.8 us. At 764 / 592: two
 // channels per lane (B and C loaded once for both: 17 % fewer wavefronts) 758 /
 // 750 us on the first two: half the warps; two-warp CTAs (16 channels) 784 / 640.
 #include <math.h>
@@ -55,7 +55,8 @@ namespace mbscan {
 namespace {
 
 constexpr int kT = 16;        // steps per chunk
-constexpr int kSegUnit = 32;  // segments of a time split are multiples of this many steps
+constexpr int kSegUnit = 32;    // least steps of a segment of a time split
+constexpr int kShareUnit = 64;  // shares are multiples of this many steps (whole stages)
 constexpr int kTP = kT / 2;   // step pairs per chunk
 constexpr int kWarps = 4;
 constexpr int kThreads = 32 * kWarps;
@@ -64,31 +65,38 @@ constexpr int kCh = kWarps * kWCh;          // channels per CTA
 constexpr int kPairs = kWCh / 2;            // channel pairs per warp
 constexpr int kPartQ = kTP * kPairs + 4;    // float4s between the shares of two lanes q (the pad keeps them on other banks)
 
-constexpr int kStages = 3;
-constexpr int kResident = 4;   // CTAs per SM (shared memory and the register bound)
-// Chunks per ring stage, one after the other between two CTA barriers (two for fp32 would leave 2 CTAs per SM)
-template <typename T>
-constexpr int kSub = sizeof(T) == 2 ? 2 : 1;
-template <typename T>
-constexpr int kRT = kT * kSub<T>;   // steps per stage
+// Two forms, W: wide stages (64 steps for bf16, 32 for fp32) in a ring of 2 and at most 3 CTAs per SM, or stages of half
+// that in a ring of 3 and 4 CTAs per SM. A stage is what lies between two CTA barriers. Microseconds per chunk of an
+// SM's 1 to 4 CTAs, bf16: wide 0.56 0.78 1.07, narrow 0.61 0.82 1.10 1.40. Grids of at most 3 per SM take the wide form
+// (8 x 8192 x 2048 in shares of 3 per SM: 650 -> 623 us), others the narrow one (608 tiles, 4 per SM: 179 us, wide 197).
+template <bool W>
+constexpr int kStages = W ? 2 : 3;
+template <bool W>
+constexpr int kCtas = W ? 3 : 4;   // CTAs per SM (shared memory and the register bound)
+constexpr int kResident = kCtas<false>;
+// Chunks per ring stage, one after the other between two CTA barriers
+template <typename T, bool W>
+constexpr int kSub = (sizeof(T) == 2 ? 2 : 1) * (W ? 2 : 1);
+template <typename T, bool W>
+constexpr int kRT = kT * kSub<T, W>;   // steps per stage
 
-template <typename T>
+template <typename T, bool W>
 struct Raw {   // TMA destinations; token tiles swizzled in their 64- (bf16) or 128-byte (fp32) rows
-    T dt[kRT<T>][kCh];
-    T x[kRT<T>][kCh];
-    T z[kRT<T>][kCh];
-    T B[kRT<T>][kDState];
-    T C[kRT<T>][kDState];
+    T dt[kRT<T, W>][kCh];
+    T x[kRT<T, W>][kCh];
+    T z[kRT<T, W>][kCh];
+    T B[kRT<T, W>][kDState];
+    T C[kRT<T, W>][kDState];
 };
 
-template <typename T>
+template <typename T, bool W>
 struct alignas(1024) Smem {
-    Raw<T> raw[kStages];
-    T ys[2][kRT<T>][kCh];                          // output tiles (TMA stores), swizzled like the inputs
+    Raw<T, W> raw[kStages<W>];
+    T ys[2][kRT<T, W>][kCh];                          // output tiles (TMA stores), swizzled like the inputs
     float4 dg[2][kWarps][kTP][kWCh];   // (Delta_t, Delta_t+1, (Delta x)_t, (Delta x)_t+1), see dg_slot
-    float4 bc[2][kSub<T>][2][2][kTP][4];           // [buffer][chunk][B, C][states 4q, 4q+1 or 4q+2, 4q+3][tp][q]
+    float4 bc[2][kSub<T, W>][2][2][kTP][4];           // [buffer][chunk][B, C][states 4q, 4q+1 or 4q+2, 4q+3][tp][q]
     float4 part[kWarps][4 * kPartQ];   // shares of C.h of lane q: [q][tp][channel pair]
-    uint64_t full[kStages];
+    uint64_t full[kStages<W>];
     int ticket;
 };
 
@@ -105,14 +113,14 @@ struct FwdArgs {
 // 16-byte stores fall on different banks. The scan's loads of all 8 channels at one tp cover 128 bytes either way.
 __device__ __forceinline__ int dg_slot(int tp, int c) { return (((c ^ tp) & 1) << 2) | (c >> 1); }
 
-template <typename T, bool kSummary>
-__device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int stage, int t, int d0, int b) {
-    constexpr uint32_t tok = kRT<T> * kCh * sizeof(T), bc = kRT<T> * kDState * sizeof(T);
+template <typename T, bool kSummary, bool W>
+__device__ __forceinline__ void issue_chunk(Smem<T, W> &s, const FwdArgs &a, int stage, int t, int d0, int b) {
+    constexpr uint32_t tok = kRT<T, W> * kCh * sizeof(T), bc = kRT<T, W> * kDState * sizeof(T);
     const bool gate = !kSummary && a.has_gate;
     const uint32_t bytes = ((gate ? 3 : 2) * tok) + (kSummary ? 1 : 2) * bc;
     uint64_t *bar = &s.full[stage];
     mbar_arrive_expect_tx(bar, bytes);
-    Raw<T> &r = s.raw[stage];
+    Raw<T, W> &r = s.raw[stage];
     tma_load_3d(&r.dt[0][0], &a.tm_dt, bar, d0, t, b);
     tma_load_3d(&r.x[0][0], &a.tm_x, bar, d0, t, b);
     if (gate) tma_load_3d(&r.z[0][0], &a.tm_z, bar, d0, t, b);
@@ -127,7 +135,7 @@ __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int st
 // segment starts from h0, so that pass scans it for good and records only its
 // end state. In the second pass segment s starts from what the first recorded,
 // folded with the associative operator of Section 2: h <- P_s' * h + H_s'.
-// kShares (if not 0: the CTAs per SM it is compiled for): the grid is p.shares CTAs; the channel tiles' spans, laid end to end,
+// kShares: the grid is p.shares CTAs; the channel tiles' spans, laid end to end,
 // are cut into that many equal lengths, and a CTA scans the pieces in its own,
 // the highest first. Its highest piece starts a tile (or it is all of a CTA's
 // part of one) and depends on nothing; where it ends inside a tile, the CTA
@@ -135,11 +143,11 @@ __device__ __forceinline__ void issue_chunk(Smem<T> &s, const FwdArgs &a, int st
 // tile: it comes last and waits (bounded) for the state that the share before
 // has left as the first thing it did. Shares are numbered in the order in which
 // their CTAs start (a ticket), so the one waited for is always running.
-template <typename T, bool kCkpt, bool kSummary, int kShares>
+template <typename T, bool kCkpt, bool kSummary, bool kShares, bool W>
 __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
-    using S = Smem<T>;
-    using R = Raw<T>;
-    constexpr int STAGES = kStages, SUB = kSub<T>, RT = kRT<T>, kRowB = kCh * (int)sizeof(T);
+    using S = Smem<T, W>;
+    using R = Raw<T, W>;
+    constexpr int STAGES = kStages<W>, SUB = kSub<T, W>, RT = kRT<T, W>, kRowB = kCh * (int)sizeof(T);
     static_assert(sizeof(R) % (8 * kRowB) == 0 && offsetof(R, x) % (8 * kRowB) == 0 &&
                       offsetof(R, z) % (8 * kRowB) == 0 && offsetof(R, B) % 128 == 0 && offsetof(R, C) % 128 == 0 &&
                       offsetof(S, ys) % (8 * kRowB) == 0 && sizeof(T) * RT * kCh % (8 * kRowB) == 0,
@@ -154,7 +162,7 @@ __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
     const int tiles = (int)p.batch * ntd;
     const int seg = kShares ? 0 : a.seg0 + (int)(blockIdx.x / tiles);
     const int nseg = p.nseg > 1 ? (int)p.nseg : 1;
-    const int units = (L + kSegUnit - 1) / kSegUnit;   // kShares
+    const int units = (L + kShareUnit - 1) / kShareUnit;   // kShares
     const bool gate = !kSummary && a.has_gate;
 
     if (tid == 0) {
@@ -166,7 +174,7 @@ __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
 
     int st = 0;        // ring slot of the next stage
     uint32_t ph = 0;   // and its phase parity
-    // this CTA's tile (batch row, 32 channels); with kShares the units of 32 steps lo .. hi - 1 of all tiles' spans
+    // this CTA's tile (batch row, 32 channels); with kShares the units of 64 steps lo .. hi - 1 of all tiles' spans
     // end to end, which it takes tile by tile from the highest
     int tile = (int)(blockIdx.x % tiles);
     int share = 0, lo = 0, hi = 0;
@@ -183,13 +191,13 @@ __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
     for (;;) {   // pieces: one without kShares
         const int b = tile / ntd, d0 = (tile % ntd) * kCh;
         // its steps: tb .. te - 1
-        const int tb = kShares ? max(lo - tile * units, 0) * kSegUnit : seg == 0 ? 0 : a.len0 + (seg - 1) * a.len;
-        const int te = min(L, kShares ? (hi - tile * units) * kSegUnit : seg == 0 ? a.len0 : tb + a.len);
+        const int tb = kShares ? max(lo - tile * units, 0) * kShareUnit : seg == 0 ? 0 : a.len0 + (seg - 1) * a.len;
+        const int te = min(L, kShares ? (hi - tile * units) * kShareUnit : seg == 0 ? a.len0 : tb + a.len);
         const int nch = (te - tb + RT - 1) / RT;   // its stages
         if (tid == 0) {
             fence_proxy_async_smem();
             for (int j = 0, sl = st; j < STAGES && j < nch; ++j, sl = sl + 1 == STAGES ? 0 : sl + 1)
-                issue_chunk<T, kSummary>(s, a, sl, tb + j * RT, d0, b);
+                issue_chunk<T, kSummary, W>(s, a, sl, tb + j * RT, d0, b);
         }
 
         // ---- conversion and output role: channels 8 warp + 2 pp + {0, 1} of the tile, steps 2 tp, 2 tp + 1
@@ -416,12 +424,14 @@ __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
             }
             if (tid == 0) {
                 if constexpr (!kSummary) {
-                    tma_store_3d(&a.tm_y, &s.ys[i & 1][0][0], d0, ts, b);
+#pragma unroll
+                    for (int u = 0; u < SUB; ++u)   // the last stage may end in any chunk; what follows it is not this CTA's
+                        if (ts + u * kT < te) tma_store_3d(&a.tm_y, &s.ys[i & 1][u * kT][0], d0, ts + u * kT, b);
                     bulk_commit();
                 }
                 if (i + STAGES < nch) {   // the slot is free: refill it with stage i + STAGES
                     fence_proxy_async_smem();
-                    issue_chunk<T, kSummary>(s, a, st, tb + (i + STAGES) * RT, d0, b);
+                    issue_chunk<T, kSummary, W>(s, a, st, tb + (i + STAGES) * RT, d0, b);
                 }
             }
             st = nst;
@@ -459,17 +469,22 @@ __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
     if (kShares && tid == 0) bulk_wait_all();
 }
 
-template <typename T, bool kCkpt, int kShares = 0>
-__global__ void __launch_bounds__(kThreads, kShares ? kShares : kResident) forward_kernel(const __grid_constant__ FwdArgs a) {
-    scan_spans<T, kCkpt, false, kShares>(a);
+template <typename T, bool kCkpt, bool W>
+__global__ void __launch_bounds__(kThreads, kCtas<W>) forward_kernel(const __grid_constant__ FwdArgs a) {
+    scan_spans<T, kCkpt, false, false, W>(a);
 }
 
 template <typename T, bool kCkpt>
-__global__ void __launch_bounds__(kThreads, kResident) first_pass_kernel(const __grid_constant__ FwdArgs a) {
+__global__ void __launch_bounds__(kThreads, kCtas<true>) forward_shares_kernel(const __grid_constant__ FwdArgs a) {
+    scan_spans<T, kCkpt, false, true, true>(a);
+}
+
+template <typename T, bool kCkpt, bool W>
+__global__ void __launch_bounds__(kThreads, kCtas<W>) first_pass_kernel(const __grid_constant__ FwdArgs a) {
     if (blockIdx.x < a.p.batch * ((a.p.d_inner + kCh - 1) / kCh))   // segment 0
-        scan_spans<T, kCkpt, false, 0>(a);
+        scan_spans<T, kCkpt, false, false, W>(a);
     else
-        scan_spans<T, kCkpt, true, 0>(a);
+        scan_spans<T, kCkpt, true, false, W>(a);
 }
 
 // ---------------------------------------------------------------------------
@@ -485,71 +500,68 @@ bool make_map(CUtensorMap *m, const void *base, int es, int64_t batch, int64_t L
     return encode_tmap(m, base, es, 3, dims, strides, box, swizzle);
 }
 
-// Split of a span into at most nseg segments, in multiples of `unit` steps (a stage: y is stored by stages). The first
+// Split of a span into at most nseg segments, in whole chunks. The first
 // is scanned for good while the others are summarised, which takes kFirst of its time per step, and is that much shorter.
 constexpr double kFirst = 0.7;
 struct Segments {
     int64_t n, len0, len;   // n <= nseg
 };
-Segments segments(int64_t L, int64_t nseg, int64_t unit) {
+Segments segments(int64_t L, int64_t nseg) {
     if (nseg < 2) return {1, L, L};
-    const int64_t units = (L + unit - 1) / unit;
+    const int64_t units = (L + kT - 1) / kT;
     int64_t others = (int64_t)((double)units / ((double)(nseg - 1) + kFirst));
     if (others < 1 || units - others * (nseg - 1) > others) ++others;   // the first is the shorter
     const int64_t m = std::min(nseg - 1, (units - 1) / others);
-    return {m + 1, (units - m * others) * unit, others * unit};
+    return {m + 1, (units - m * others) * kT, others * kT};
 }
 
-template <typename T, bool kCkpt>
-cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
+template <typename T, bool kCkpt, bool W>
+cudaError_t launch_form(const ScanParams &p, const Segments &g, int64_t grid, const DeviceLimits *lim, cudaStream_t s) {
     constexpr int es = sizeof(T), sw = kCh * es;   // one token row of a tile
     FwdArgs a;
     memset(&a, 0, sizeof(a));
     a.p = p;
     a.has_gate = p.z != nullptr;
-    if (p.nseg < 2 || !p.seg_h || !p.seg_p) a.p.nseg = 1;
-    const int64_t D = p.d_inner;
-    const Segments g = segments(p.seqlen, a.p.nseg, kRT<T>);
-    const int64_t nseg = g.n;
     a.len0 = (int)g.len0;
     a.len = (int)g.len;
-    auto tok = [&](CUtensorMap *m, const void *base) {
-        return make_map(m, base, es, p.batch, p.seqlen, D, kCh, D, sw, kRT<T>);
+    const int64_t D = p.d_inner;
+    auto tok = [&](CUtensorMap *m, const void *base, int rows = kRT<T, W>) {
+        return make_map(m, base, es, p.batch, p.seqlen, D, kCh, D, sw, rows);
     };
-    if (!tok(&a.tm_dt, p.dt) || !tok(&a.tm_x, p.x) || (p.z && !tok(&a.tm_z, p.z)) || !tok(&a.tm_y, p.y) ||
-        !make_map(&a.tm_B, p.B, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0, kRT<T>) ||
-        !make_map(&a.tm_C, p.C, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0, kRT<T>))
+    if (!tok(&a.tm_dt, p.dt) || !tok(&a.tm_x, p.x) || (p.z && !tok(&a.tm_z, p.z)) || !tok(&a.tm_y, p.y, kT) ||
+        !make_map(&a.tm_B, p.B, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0, kRT<T, W>) ||
+        !make_map(&a.tm_C, p.C, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0, kRT<T, W>))
         return cudaErrorInvalidValue;
-    const size_t smem = sizeof(Smem<T>) + 1024;
+    const size_t smem = sizeof(Smem<T, W>) + 1024;
+    auto launch = [&](auto k) {
+        const cudaError_t e =
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin);
+        if (e != cudaSuccess) return e;
+        return launch_pdl(true, k, dim3((unsigned)grid), dim3(kThreads), spread_smem(smem, grid, kCtas<W>), s, a);
+    };
+    cudaError_t e;
+    if (g.n > 1) {   // first pass: segments 0 .. n-2
+        if ((e = launch(first_pass_kernel<T, kCkpt, W>)) != cudaSuccess) return e;
+        a.seg0 = 1;   // second pass: segments 1 .. n-1
+    } else if constexpr (W) {
+        if (p.shares > 0) {
+            if ((e = cudaMemsetAsync(p.share_sync(), 0, prefill_share_sync_bytes(p.shares), s)) != cudaSuccess) return e;
+            return launch(forward_shares_kernel<T, kCkpt>);
+        }
+    }
+    return launch(forward_kernel<T, kCkpt, W>);
+}
+
+template <typename T, bool kCkpt>
+cudaError_t launch_typed(ScanParams p, cudaStream_t s) {
     const DeviceLimits *lim = device_limits();
     if (!lim) return cudaErrorInvalidDevice;
-    const int64_t ctas = ((D + kCh - 1) / kCh) * p.batch;   // per segment of L
-    cudaError_t e;
-    if (nseg > 1) {   // first pass: segments 0 .. nseg-2
-        auto k1 = first_pass_kernel<T, kCkpt>;
-        if ((e = cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
-            cudaSuccess)
-            return e;
-        const int64_t grid = ctas * (nseg - 1);
-        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kThreads), spread_smem(smem, grid, kResident), s, a)) !=
-            cudaSuccess)
-            return e;
-        a.seg0 = 1;   // second pass: segments 1 .. nseg-1
-    }
-    if (nseg == 1 && p.shares > 0) {
-        auto ks = p.shares < kResident * lim->sms ? forward_kernel<T, kCkpt, kResident - 1>
-                                                  : forward_kernel<T, kCkpt, kResident>;
-        if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
-                cudaSuccess ||
-            (e = cudaMemsetAsync(p.share_sync(), 0, prefill_share_sync_bytes(p.shares), s)) != cudaSuccess)
-            return e;
-        return launch_pdl(true, ks, dim3((unsigned)p.shares), dim3(kThreads), spread_smem(smem, p.shares, kResident), s, a);
-    }
-    auto k = forward_kernel<T, kCkpt>;
-    e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin);
-    if (e != cudaSuccess) return e;
-    const int64_t grid = ctas * (nseg - a.seg0);
-    return launch_pdl(true, k, dim3((unsigned)grid), dim3(kThreads), spread_smem(smem, grid, kResident), s, a);
+    if (p.nseg < 2 || !p.seg_h || !p.seg_p) p.nseg = 1;
+    const Segments g = segments(p.seqlen, p.nseg);
+    const int64_t ctas = ((p.d_inner + kCh - 1) / kCh) * p.batch;   // per segment of L
+    const int64_t grid = g.n > 1 ? ctas * (g.n - 1) : p.shares > 0 ? p.shares : ctas;
+    return p.shares > 0 || grid <= kCtas<true> * lim->sms ? launch_form<T, kCkpt, true>(p, g, grid, lim, s)
+                                                          : launch_form<T, kCkpt, false>(p, g, grid, lim, s);
 }
 
 }  // namespace
@@ -559,40 +571,38 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
 // pass repeats most of a scan, so at 1.7 CTAs per SM, batch 4 x 2048 channels,
 // the split measured slower) and the span is long enough to pay for the second
 // launch: at 128 steps x 2048 channels unsplit 8.5 us, split 10.3; at 256 steps
-// 14.4 and 12.3. Both passes run all segments but one, in 1 to 4 CTAs per SM:
-// more CTAs share an SM better, but not in proportion (kChunkUs), and a number
-// that leaves some SMs with one CTA less pays for it as if they had it. So, of
-// the counts that fill 1, 2, 3 or 4 per SM, the one with the least chunks x time
-// per chunk. (Microseconds with at most 3 and at most 4 per SM: bf16 1 x 8192 x
-// 2048 126.9, 129.7; 1 x 8192 x 1024 70.0, 66.7; fp32 2 x 3000 x 1536 85.9, 77.3;
-// 1 x 777 x 3584 25.8, 27.7.) Every lane folds the summaries before its segment,
+// 14.4 and 12.3. Both passes run all segments but one, with at most 3 CTAs per SM
+// (wide form) or 4: of the two numbers, the one with the less chunks x time per
+// chunk of the SM that holds the most. (Microseconds with 3 and 4: bf16 1 x 4096 x
+// 4608 130, 133; fp32 2 x 3000 x 1536 84, 77; 1 x 777 x 3584 25.2, 27.7; bf16 1 x
+// 4096 x 4608 with 2: 139.) Every lane folds the summaries before its segment,
 // about 0.07 us each, while a step costs about 0.1 us over both passes: their sum
 // is least at sqrt(1.4 L) segments, which bounds spans of very few channels
 // (8192 x 64: 86 segments 20 us, 256 segments 35 us, 16 segments 37 us; fp32
 // 256 x 64: 8 segments 8.4 us, 2 segments 14.4 us).
 // With the first segment summarised like the others, and scanned in the second
-// pass: bf16 1 x 8192 x 2048 139 us (now 126), fp32 3 x 1003 x 1544 42.7 (40.7).
+// pass: bf16 1 x 8192 x 2048 139 us (then 126, wide 122), fp32 3 x 1003 x 1544 42.7
+// (then 40.7, wide 39.8).
 constexpr int64_t kMinSplitSteps = 256;
 constexpr double kFoldUs = 0.07;
 // Microseconds per chunk of an SM's CTAs, 1 to 4 of them, as measured (fp32, bf16)
-constexpr double kChunkUs[2][4] = {{0.79, 1.01, 1.22, 1.55}, {0.61, 0.82, 1.10, 1.40}};
+constexpr double kChunkUs[2][kResident] = {{0.79, 0.93, 1.20, 1.55}, {0.56, 0.78, 1.07, 1.40}};
 
 int64_t prefill_segments(const ScanParams &p, bool bf16) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinSplitSteps || p.dt_low) return 1;
     const int64_t sms = device_sms();
     const int64_t ctas = p.batch * ((p.d_inner + kCh - 1) / kCh);
     if (ctas > sms) return 1;
-    const int64_t unit = bf16 ? kRT<__nv_bfloat16> : kRT<float>;
     const int64_t most = std::min((p.seqlen + kSegUnit - 1) / kSegUnit, (int64_t)sqrt(1.4 * (double)p.seqlen));
     int64_t best = 1;
     double least = 0;
-    for (int64_t m = 1; m <= kResident; ++m) {
+    for (int64_t m = kCtas<true>; m <= kCtas<false>; ++m) {
         const int64_t nseg = std::min(m * sms / ctas + 1, most);
         if (nseg < 3) continue;   // two: one after the other
-        const Segments g = segments(p.seqlen, nseg, unit);
+        const Segments g = segments(p.seqlen, nseg);
         const int64_t per_sm = (ctas * (g.n - 1) + sms - 1) / sms;
         const double us = (1 + kFirst) * kChunkUs[bf16][per_sm - 1] * (double)(g.len / kT) + kFoldUs * (double)g.n;
-        if (best == 1 || us < least) {
+        if (best == 1 || us < 0.97 * least) {   // fewer segments at equal time: less summarised
             best = nseg;
             least = us;
         }
@@ -607,25 +617,26 @@ size_t prefill_split_bytes(const ScanParams &p, int64_t nseg) {
 // Even shares: CTAs of one tile each leave the GPU unevenly loaded when their
 // number is little over a multiple of the SMs: the SMs that hold one more set
 // the time (8 x 8192 x 2048: 512 tiles, 3.4 per SM). Then m = tiles / SMs
-// (rounded down, at most 4) CTAs per SM take equal shares of all tiles' steps.
-// Microseconds per chunk of an SM's CTAs, 1 to 4 of them, as measured:
+// (rounded down, at most 3: the wide form) CTAs per SM take equal shares of all
+// tiles' steps. Microseconds per chunk of an SM's CTAs, 1 to 4 of them, as
+// measured (kChunkUs, kShareUs; 4: the narrow form):
 //                        bf16                  fp32
-//   one CTA per tile     0.61 0.82 1.10 1.40   0.79 1.01 1.22 1.55
-//   shares               0.68 0.88 1.13 1.47   0.87 1.08 1.29 1.63
+//   one CTA per tile     0.56 0.78 1.07 1.40   0.79 0.93 1.20 1.55
+//   shares               0.63 0.83 1.10        0.87 1.02 1.22
 // so m CTAs per SM finish tiles in tiles / (m SMs) times the second row, plus
 // about 7 us for the clearing of the flags and the second prologue, against the
 // first row's next number for one CTA per tile. More tiles than slots run in
 // waves; the last one, of r per SM, takes about 0.85 of its number (its CTAs
 // start as others end). Measured (bf16): 8 x 8192 x 2048 (3.4 tiles per SM)
-// 709 -> 650 us, its training forward 740 -> 672 us; spans of 2048 steps at 2.1,
-// 3.05, 4.2 and 5.3 tiles per SM 142 -> 126, 182 -> 158, 239 -> 206, 273 -> 254 us.
-constexpr double kShareUs[2][4] = {{0.87, 1.08, 1.29, 1.63}, {0.68, 0.88, 1.13, 1.47}};
+// 709 -> 623 us, its training forward 740 -> 650 us; spans of 2048 steps at 2.1,
+// 3.2, 3.4 and 4.3 tiles per SM 136 -> 118, 182 -> 156, 182 -> 164, 242 -> 209 us.
+constexpr double kShareUs[2][kCtas<true>] = {{0.87, 1.02, 1.22}, {0.63, 0.83, 1.10}};
 
 int64_t prefill_shares(const ScanParams &p, bool bf16) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinSplitSteps || p.dt_low) return 0;
     const int64_t sms = device_sms(), tiles = p.batch * ((p.d_inner + kCh - 1) / kCh);
     if (sms <= 0 || tiles <= sms) return 0;
-    const int64_t m = tiles / sms < kResident ? tiles / sms : kResident, rest = tiles % (kResident * sms);
+    const int64_t m = std::min<int64_t>(tiles / sms, kCtas<true>), rest = tiles % (kResident * sms);
     double plain = (double)(tiles / (kResident * sms)) * kChunkUs[bf16][kResident - 1];
     if (rest) plain += (tiles > rest ? 0.85 : 1.0) * kChunkUs[bf16][(rest - 1) / sms];
     const double even = (double)tiles / (double)(m * sms) * kShareUs[bf16][m - 1];
