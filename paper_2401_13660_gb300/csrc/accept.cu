@@ -20,12 +20,12 @@ namespace {
 constexpr int kAccWarps = 16;
 
 __device__ __forceinline__ void load8(const float *p, float (&v)[8]) {
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
-    const float4 b = __ldg(reinterpret_cast<const float4 *>(p) + 1);
+    const float4 a = reinterpret_cast<const float4 *>(p)[0];
+    const float4 b = reinterpret_cast<const float4 *>(p)[1];
     v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
 }
 __device__ __forceinline__ void load8(const __nv_bfloat16 *p, float (&v)[8]) {
-    const uint4 u = __ldg(reinterpret_cast<const uint4 *>(p));
+    const uint4 u = *reinterpret_cast<const uint4 *>(p);
     const unsigned w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -35,10 +35,8 @@ __device__ __forceinline__ void load8(const __nv_bfloat16 *p, float (&v)[8]) {
 }
 
 template <typename T>
-__global__ void __launch_bounds__(32 * kAccWarps) accept_kernel(const T *__restrict__ logits,
-                                                                const uint8_t *__restrict__ drafted,
-                                                                int64_t k, int beta,
-                                                                int32_t *__restrict__ accept) {
+__global__ void __launch_bounds__(32 * kAccWarps) accept_kernel(const T *logits, const uint8_t *drafted,
+                                                                int64_t k, int beta, int32_t *accept) {
     __shared__ int first_reject;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t s = blockIdx.x;
@@ -50,7 +48,7 @@ __global__ void __launch_bounds__(32 * kAccWarps) accept_kernel(const T *__restr
         const int64_t i = base + warp;
         if (i < k) {
             const T *row = logits + (s * k + i) * 256;
-            const int byte = __ldg(drafted + s * k + i);
+            const int byte = drafted[s * k + i];
             float v[8];
             load8(row + 8 * lane, v);
             // the drafted byte's own score, from the lane that has it (no second, dependent load)

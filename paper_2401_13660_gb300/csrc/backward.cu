@@ -132,10 +132,14 @@ __device__ __forceinline__ void softplus_sigmoid2(float2 v, float2 &delta, float
     sig.y = v.y > 15.f ? 1.f : sig.y;
 }
 
-// Four values of a lane's permuted state order (register r: state r ^ perm) from a row of four
+// Four values of a lane's permuted state order (register r: state r ^ perm) from a row of four. kOnce: read this once
+// and never again (checkpoints), past the L1 cache (8 x 8192 x 2048 with the forward: 3082 us, through it 3104); the
+// few rows that every segment folds are better off in it (2 x 777 x 1544: 89.1 us, past it 89.9).
+template <bool kOnce = false>
 __device__ __forceinline__ void load_perm(float (&v)[4], const float *row, int perm) {
-    const float2 lo = __ldg(reinterpret_cast<const float2 *>(row + (perm & 2)));
-    const float2 hi = __ldg(reinterpret_cast<const float2 *>(row + 2 - (perm & 2)));
+    const float *plo = row + (perm & 2), *phi = row + 2 - (perm & 2);
+    const float2 lo = kOnce ? __ldcg(reinterpret_cast<const float2 *>(plo)) : gld2(plo);
+    const float2 hi = kOnce ? __ldcg(reinterpret_cast<const float2 *>(phi)) : gld2(phi);
     const bool s = perm & 1;
     v[0] = s ? lo.y : lo.x;
     v[1] = s ? lo.x : lo.y;
@@ -233,8 +237,8 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
         float2 bias = make_float2(0.f, 0.f), dsk = bias, dD_acc = bias, db_acc = bias;
         const int64_t dc = (int64_t)d0 + wc0 + 2 * pp;   // D % 8 == 0: both channels valid or neither
         if (dc < D) {
-            if (p.dt_bias) bias = __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc));
-            if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
+            if (p.dt_bias) bias = gld2(p.dt_bias + dc);
+            if (p.D) dsk = gld2(p.D + dc);
         }
 
         // ---- scan role: channels 2 cl, 2 cl + 1 of the warp, states 4 q .. 4 q + 3 in the order r -> r ^ perm
@@ -323,7 +327,7 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
                 for (int j = 0; j < 2; ++j) {
 #pragma unroll
                     for (int n = 0; n < 4; ++n) hm[j][n] = 0.f;
-                    if (chan_ok) load_perm(hm[j], ck + j * kDState, perm);
+                    if (chan_ok) load_perm<true>(hm[j], ck + j * kDState, perm);
                 }
                 if (chan_ok && it + 1 < nch) asm volatile("prefetch.global.L2 [%0];" ::"l"(ck - D * kDState + (q & 1) * kDState));
             }

@@ -79,7 +79,7 @@ struct StepArgs<true> {
 // Resume: the drafted-byte index whose state row s starts from (0 .. k-1),
 // -1 for the cached state h0, or -2 when accept[s] is outside [0, k].
 __device__ __forceinline__ int resume_index(const StepArgs<true> &a, int64_t s) {
-    const int acc = __ldg(a.accept + s);
+    const int acc = a.accept[s];
     return (acc < 0 || acc > a.k) ? -2 : acc - 1;
 }
 
@@ -217,9 +217,9 @@ __global__ void __launch_bounds__(kStepThreads, sizeof(T) == 2 ? 3 : 2) step_ker
         if (k < a.ntiles) {
             const int64_t dn = (int64_t)(k % a.ntiles_d) * kStepCh + c;
             if (dn < D) {
-                nav = ldg4(p.A + dn * kDState + 4 * q);
-                nbias = p.dt_bias ? __ldg(p.dt_bias + dn) : 0.f;
-                ndsk = p.D ? __ldg(p.D + dn) : 0.f;
+                nav = gld4(p.A + dn * kDState + 4 * q);
+                nbias = p.dt_bias ? p.dt_bias[dn] : 0.f;
+                ndsk = p.D ? p.D[dn] : 0.f;
             }
         }
     };
@@ -290,15 +290,14 @@ constexpr int kRbThreads = 256;
 constexpr int kRbVec = 4;
 
 __global__ void __launch_bounds__(kRbThreads)
-rollback_kernel(const float4 *h0 /* may alias h_out */, const float4 *__restrict__ h_all,
-                const int32_t *__restrict__ accept, float4 *h_out, int64_t batch, int64_t k,
-                int64_t per_stream /* float4s */, StatusBlock *status) {
+rollback_kernel(const float4 *h0 /* may alias h_out */, const float4 *h_all, const int32_t *accept, float4 *h_out,
+                int64_t batch, int64_t k, int64_t per_stream /* float4s */, StatusBlock *status) {
     pdl_wait();
     const int64_t i0 = ((int64_t)blockIdx.x * kRbThreads + threadIdx.x) * kRbVec;
     if (i0 >= batch * per_stream) return;
     const int64_t s = i0 / per_stream;
     const int64_t j0 = i0 - s * per_stream;
-    const int a = __ldg(accept + s);
+    const int a = accept[s];
     if (a < 0 || a > k) {
         if (j0 == 0) report(status, 1 /* MB_ERR_INVALID_ARG */, s);
         return;

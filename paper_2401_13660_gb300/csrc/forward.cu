@@ -207,8 +207,8 @@ __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
         {
             const int64_t dc = (int64_t)d0 + kWCh * warp + 2 * pp;   // D % 8 == 0: both channels valid or neither
             if (dc < D) {
-                if (p.dt_bias) bias = __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc));
-                if (p.D) dsk = __ldg(reinterpret_cast<const float2 *>(p.D + dc));
+                if (p.dt_bias) bias = gld2(p.dt_bias + dc);
+                if (p.D) dsk = gld2(p.D + dc);
             }
         }
         // widening role: two states of B or C at a step pair of every chunk (s.bc in the order of the threads)
@@ -224,16 +224,16 @@ __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
         {
             float4 av = make_float4(0.f, 0.f, 0.f, 0.f), hv = av;
             if (chan_ok) {
-                av = ldg4(p.A + d * kDState + 4 * q);
-                if (seg == 0 && tb == 0 && p.h0) hv = ldg4(p.h0 + ((int64_t)b * D + d) * kDState + 4 * q);
+                av = gld4(p.A + d * kDState + 4 * q);
+                if (seg == 0 && tb == 0 && p.h0) hv = gld4(p.h0 + ((int64_t)b * D + d) * kDState + 4 * q);
                 if constexpr (!kSummary) {
                     for (int sp = 0; sp < seg; ++sp) {
                         const int64_t o = (((int64_t)b * nseg + sp) * D + d) * kDState + 4 * q;
-                        const float4 he = *reinterpret_cast<const float4 *>(p.seg_h + o);
+                        const float4 he = gld4(p.seg_h + o);
                         if (sp == 0) {
                             hv = he;
                         } else {
-                            const float4 pe = *reinterpret_cast<const float4 *>(p.seg_p + o);
+                            const float4 pe = gld4(p.seg_p + o);
                             hv = make_float4(fmaf(pe.x, hv.x, he.x), fmaf(pe.y, hv.y, he.y),
                                              fmaf(pe.z, hv.z, he.z), fmaf(pe.w, hv.w, he.w));
                         }

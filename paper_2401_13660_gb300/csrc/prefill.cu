@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
     // untouched; the check comes before any copy is issued.
     int resume_a = 0;
     if (p.accept) {
-        resume_a = __ldg(p.accept + b);   // one batch row per CTA: uniform
+        resume_a = p.accept[b];   // one batch row per CTA: uniform
         if (resume_a < 0 || resume_a > p.k_prev) {
             if (tid == 0 && d0 == 0) report(p.status, 1 /* MB_ERR_INVALID_ARG */, b);
             return;
@@ -381,9 +381,8 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
     {
         const int64_t dc = d0 + 2 * cr.cp;   // D % 8 == 0: both channels valid or neither
         cr.ok = dc < D;
-        cr.bias = (cr.ok && p.dt_bias) ? __ldg(reinterpret_cast<const float2 *>(p.dt_bias + dc))
-                                       : make_float2(0.f, 0.f);
-        cr.dsk = (cr.ok && p.D) ? __ldg(reinterpret_cast<const float2 *>(p.D + dc)) : make_float2(0.f, 0.f);
+        cr.bias = (cr.ok && p.dt_bias) ? gld2(p.dt_bias + dc) : make_float2(0.f, 0.f);
+        cr.dsk = (cr.ok && p.D) ? gld2(p.D + dc) : make_float2(0.f, 0.f);
     }
 
     // ---- scan role: channel c, states kSPL*q .. kSPL*q + kSPL-1
@@ -402,9 +401,9 @@ __global__ void __launch_bounds__(kThreads, kStoreAll ? (kFuse ? MB_VERIFY_FUSED
         const float2 *hp = hrow ? reinterpret_cast<const float2 *>(hrow + G::kSPL * q) : nullptr;
 #pragma unroll
         for (int k = 0; k < G::kPairs; ++k) {
-            const float2 av = __ldg(Ap + k);
+            const float2 av = Ap[k];
             a2[k] = make_float2(av.x * kLog2e, av.y * kLog2e);
-            if (hp) h[k] = __ldg(hp + k);
+            if (hp) h[k] = hp[k];
         }
     }
 

@@ -103,11 +103,11 @@ __global__ void __launch_bounds__(kXpThreads) conv_xproj_kernel(const __grid_con
     const int kc = k0 + 8 * g;
     float4 wj[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) wj[j] = __ldg(reinterpret_cast<const float4 *>(a.cw + (int64_t)(kc + j) * 4));
+    for (int j = 0; j < 8; ++j) wj[j] = gld4(a.cw + (int64_t)(kc + j) * 4);
     float bv[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (a.cb) {
-        const float4 b0 = __ldg(reinterpret_cast<const float4 *>(a.cb + kc));
-        const float4 b1 = __ldg(reinterpret_cast<const float4 *>(a.cb + kc) + 1);
+        const float4 b0 = gld4(a.cb + kc);
+        const float4 b1 = gld4(a.cb + kc + 4);
         bv[0] = b0.x; bv[1] = b0.y; bv[2] = b0.z; bv[3] = b0.w;
         bv[4] = b1.x; bv[5] = b1.y; bv[6] = b1.z; bv[7] = b1.w;
     }
@@ -214,8 +214,7 @@ __global__ void __launch_bounds__(kXpThreads) conv_xproj_kernel(const __grid_con
 // added in order q = 0..3, so the result does not depend on timing.
 constexpr int kRedLoads = 9;   // loads in flight per thread: all of a subset's at width 4608 (36 splits)
 constexpr int kRedQuads = 64, kRedSub = 4, kRedThreads = kRedQuads * kRedSub;
-__global__ void __launch_bounds__(kRedThreads) xproj_reduce_kernel(const float *__restrict__ part,
-                                                                  __nv_bfloat16 *__restrict__ out,
+__global__ void __launch_bounds__(kRedThreads) xproj_reduce_kernel(const float *part, __nv_bfloat16 *out,
                                                                   int64_t quads, int splits) {
     __shared__ float4 sub[kRedSub][kRedQuads];
     pdl_trigger();   // the Delta GEMM that follows when a model decodes may set up meanwhile (it waits, as CUDA requires)
@@ -229,7 +228,7 @@ __global__ void __launch_bounds__(kRedThreads) xproj_reduce_kernel(const float *
             float4 v[kRedLoads];
 #pragma unroll
             for (int u = 0; u < kRedLoads; ++u)
-                if (k0 + u * kRedSub < splits) v[u] = __ldg(p + (int64_t)(k0 + u * kRedSub) * quads);
+                if (k0 + u * kRedSub < splits) v[u] = p[(int64_t)(k0 + u * kRedSub) * quads];
 #pragma unroll
             for (int u = 0; u < kRedLoads; ++u) {
                 if (k0 + u * kRedSub >= splits) break;
