@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const _
                         load_perm(ge, p.seg_h + o, perm);
                         load_perm(pe, p.seg_p + o, perm);
 #pragma unroll
-                        for (int n = 0; n < 4; ++n) g[j][n] = sp == nseg - 1 ? ge[n] : fmaf(pe[n], g[j][n], ge[n]);
+                        for (int n = 0; n < 4; ++n) g[j][n] = sp == nseg - 1 ? ge[n] : fold(pe[n], g[j][n], ge[n]);
                     }
                 }
             }

@@ -234,8 +234,8 @@ __device__ __forceinline__ void scan_spans(const FwdArgs &a) {
                             hv = he;
                         } else {
                             const float4 pe = gld4(p.seg_p + o);
-                            hv = make_float4(fmaf(pe.x, hv.x, he.x), fmaf(pe.y, hv.y, he.y),
-                                             fmaf(pe.z, hv.z, he.z), fmaf(pe.w, hv.w, he.w));
+                            hv = make_float4(fold(pe.x, hv.x, he.x), fold(pe.y, hv.y, he.y),
+                                             fold(pe.z, hv.z, he.z), fold(pe.w, hv.w, he.w));
                         }
                     }
                 }

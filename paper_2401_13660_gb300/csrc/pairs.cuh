@@ -70,6 +70,11 @@ __device__ __forceinline__ float2 silu2(float2 z) {
     return mul2(z, make_float2(rcp(o.x), rcp(o.y)));
 }
 
+// A state (adjoint) h carried over a segment with decays p and end state (adjoint) e from zero. A zero one stays out of
+// it: where states grow (A > 0) p overflows, and step by step no infinity would have met it. (The mask is on p: selecting
+// e instead makes the loop over the segments wait for its loads, 1 x 8192 x 2048 123.2 us instead of 121.9.)
+__device__ __forceinline__ float fold(float p, float h, float e) { return fmaf(h == 0.f ? 0.f : p, h, e); }
+
 // A share's flag in global memory: set after its state has been written, and waited for (bounded).
 __device__ __forceinline__ void flag_set(int *f) {
     asm volatile("st.release.gpu.global.s32 [%0], 1;" ::"l"(f) : "memory");
