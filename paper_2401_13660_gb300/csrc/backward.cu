@@ -69,7 +69,9 @@ constexpr int kBWCh = 16;                  // channels per warp, two per lane
 constexpr int kBPairs = kBWCh / 2;
 constexpr int kBCh = kBWarps * kBWCh;      // channels per CTA
 constexpr int kBStages = 2;
-constexpr int kBResident = 4;              // CTAs per SM (registers)
+// CTAs per SM: four by registers, fp32 three by shared memory (61 KB each)
+template <typename T>
+constexpr int kBResident = sizeof(T) == 2 ? 4 : 3;
 constexpr int kShareQ = kHTP * kBPairs + 2;   // float4s between the shares of two lanes q (the pad moves them to other banks)
 
 template <typename T>
@@ -174,7 +176,7 @@ __device__ __forceinline__ void flush_sums(const BSmem<T> &s, const GradParams &
 // tiles' chunks (in the order the sweep takes them, the last chunk first); a
 // share that ends inside a tile leaves the adjoint for the next one.
 template <typename T, bool kSummary, bool kShares = false>
-__global__ void __launch_bounds__(kBThreads, kBResident) backward_kernel(const __grid_constant__ BwdArgs a) {
+__global__ void __launch_bounds__(kBThreads, kBResident<T>) backward_kernel(const __grid_constant__ BwdArgs a) {
     constexpr int S = kBStages, kRowB = kBCh * (int)sizeof(T);
     using R = BRaw<T>;
     using SM = BSmem<T>;
@@ -687,7 +689,8 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
         !make_map3(&a.tm_C, p.C, bf16, Bn, L, kDState, kDState, p.bc_stride, 0) || !tok(&a.tm_dx, g.dx) ||
         !tok(&a.tm_ddt, g.ddt) || (p.z && !tok(&a.tm_dz, g.dz)))
         return cudaErrorInvalidValue;
-    const size_t smem = sizeof(BSmem<T>) + 1024;
+    constexpr size_t smem = sizeof(BSmem<T>) + 1024;
+    static_assert(kBResident<T> * (smem + 1024) <= 228 * 1024, "an SM holds this many CTAs, 1 KB reserved for each");
     const DeviceLimits *lim = device_limits();
     if (!lim) return cudaErrorInvalidDevice;
     const int64_t ctas = ((D + kBCh - 1) / kBCh) * Bn;   // per segment of L
@@ -701,7 +704,7 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
             cudaSuccess)
             return e;
         const int64_t grid = ctas * (nseg - 1);
-        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kBThreads), spread_smem(smem, grid, kBResident), s, a1)) !=
+        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kBThreads), spread_smem(smem, grid, kBResident<T>), s, a1)) !=
             cudaSuccess)
             return e;
     }
@@ -711,38 +714,43 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
         if ((e = cudaFuncSetAttribute(ks, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) !=
             cudaSuccess)
             return e;
-        return launch_pdl(true, ks, dim3((unsigned)p.shares), dim3(kBThreads), spread_smem(smem, p.shares, kBResident),
+        return launch_pdl(true, ks, dim3((unsigned)p.shares), dim3(kBThreads), spread_smem(smem, p.shares, kBResident<T>),
                           s, a);
     }
     auto k = backward_kernel<T, false>;
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) != cudaSuccess)
         return e;
     return launch_pdl(true, k, dim3((unsigned)(ctas * nseg)), dim3(kBThreads),
-                      spread_smem(smem, ctas * nseg, kBResident), s, a);
+                      spread_smem(smem, ctas * nseg, kBResident<T>), s, a);
 }
 
 }  // namespace
 
 // Time split: when the batch rows and channel tiles fill at most half of the
-// resident slots (4 CTAs per SM), into as many segments as fill them, each at
+// resident slots (kBResident per SM), into as many segments as fill them, each at
 // least two chunks long. Only the adjoint is carried across a boundary (the
 // states come from the checkpoints), so the first pass is short: decays and
 // dy C, no sums over channels or states. Every lane folds the segments after
 // its own; beyond sqrt(2 L) segments that costs more than shorter segments
 // give. Measured: 2 x 777 x 1544 (98 CTAs) 156 us unsplit, 66 in 5 segments;
 // 1 x 8192 x 64 1537 us unsplit, 53 in 128, 84 in 256; with the slots nearly
-// filled (8 x 8192 x 2048: 512 CTAs) 2.63 ms unsplit, 2.90 ms in 6.
+// filled (8 x 8192 x 2048: 512 CTAs) 2.63 ms unsplit, 2.90 ms in 6. fp32, spans
+// of 2048 steps, tiles per SM 0.5, 1, 1.2, 1.6, 2: 141, 254, 353, 446, 448 us (cut
+// for four slots per SM: 155, 270, 353, 500, 506). Three segments instead of two
+// where they are at most one per SM beyond the slots (1.2 tiles per SM: 372 us in
+// two): the CTAs of an SM do not end together, and a few more fill the gaps.
 constexpr int64_t kMinBwdSplitSteps = 128;
 
-int64_t backward_segments(const ScanParams &p) {
+int64_t backward_segments(const ScanParams &p, bool bf16) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinBwdSplitSteps || p.dt_low) return 1;
-    const int64_t slots = (int64_t)device_sms() * kBResident;
+    const int64_t slots = (int64_t)device_sms() * (bf16 ? kBResident<__nv_bfloat16> : kBResident<float>);
     const int64_t ctas = p.batch * ((p.d_inner + kBCh - 1) / kBCh);
     if (2 * ctas > slots) return 1;
     const int64_t nchunks = (p.seqlen + kBT - 1) / kBT;
     int64_t nseg = slots / ctas;
     const int64_t most = (int64_t)sqrt(2.0 * (double)p.seqlen);
     if (nseg > most) nseg = most;
+    if (!bf16 && nseg == 2 && 3 * ctas <= slots + device_sms()) nseg = 3;
     if (nseg > nchunks / 2) nseg = nchunks / 2;
     if (nseg < 2) return 1;
     const int64_t cps = (nchunks + nseg - 1) / nseg;
@@ -750,20 +758,26 @@ int64_t backward_segments(const ScanParams &p) {
 }
 
 // Even shares (as prefill_shares), where the tiles are little over two per SM
-// or over a multiple of the slots. Microseconds per chunk of an SM's 1 to 4
-// CTAs, as measured (bf16), one CTA per tile: 3.2 3.4 4.7 4.8 (two CTAs of two
-// warps fill the four schedulers once, so a third costs as much as two more);
-// shares: 3.6 with two per SM, 5.05 with four. Measured, spans of 2048 steps at
-// 2.1, 4.2, 5.05 and 8.2 tiles per SM: 600 -> 486, 1000 -> 681, 1003 -> 815,
-// 1582 -> 1315 us.
-int64_t backward_shares(const ScanParams &p) {
+// or over a multiple of the slots. Microseconds per chunk of an SM's CTAs, one
+// per tile, 1 to 4 (fp32: 3) of them, and of shares with two per SM and with
+// all, as measured:
+//   bf16   3.17 3.35 4.69 4.84   3.6  5.05
+//   fp32   3.20 3.49 4.83        3.70 5.05
+// (two CTAs of two warps fill the four schedulers once, so a third costs as much
+// as two more). The last wave of fp32 takes about 0.9 of its number, of bf16 all.
+// Measured, spans of 2048 steps: bf16 at 2.1, 4.2, 5.05 and 8.2 tiles per SM 600 ->
+// 486, 1000 -> 681, 1003 -> 815, 1582 -> 1315 us; fp32 at 2.1, 3.1, 4.2 and 6.1 618 ->
+// 501, 867 -> 670, 1007 -> 904, 1401 -> 1308 us, as it is at 2.9, 5.6 and 8.2.
+int64_t backward_shares(const ScanParams &p, bool bf16) {
     if (p.batch <= 0 || p.d_inner <= 0 || p.seqlen < kMinBwdSplitSteps || p.dt_low) return 0;
     const int64_t sms = device_sms(), tiles = p.batch * ((p.d_inner + kBCh - 1) / kBCh);
     if (sms <= 0 || tiles <= 2 * sms) return 0;
-    constexpr double t[4] = {3.17, 3.35, 4.69, 4.84};
-    const int64_t m = tiles < kBResident * sms ? 2 : kBResident, rest = tiles % (kBResident * sms);
-    const double plain = (double)(tiles / (kBResident * sms)) * t[kBResident - 1] + (rest ? t[(rest - 1) / sms] : 0.0);
-    const double even = (double)tiles / (double)(m * sms) * (m == 2 ? 3.6 : 5.05);
+    const int64_t resident = bf16 ? kBResident<__nv_bfloat16> : kBResident<float>, wave = resident * sms;
+    constexpr double t[2][4] = {{3.20, 3.49, 4.83}, {3.17, 3.35, 4.69, 4.84}}, two[2] = {3.70, 3.6}, all = 5.05;
+    const int64_t m = tiles < wave ? 2 : resident, rest = tiles % wave;
+    double plain = (double)(tiles / wave) * t[bf16][resident - 1];
+    if (rest) plain += (tiles > rest && !bf16 ? 0.9 : 1.0) * t[bf16][(rest - 1) / sms];
+    const double even = (double)tiles / (double)(m * sms) * (m == 2 ? two[bf16] : all);
     const double chunks = (double)(p.seqlen / kBT);
     return even * chunks + 7.0 < 0.97 * plain * chunks ? m * sms : 0;
 }

@@ -204,10 +204,10 @@ size_t mb_workspace_size(const mb_scan_args *args) {
     if (check_args(args, false, false) != MB_OK) return 0;
     const ScanParams p = to_params(args, nullptr, nullptr);
     const bool bf16 = args->dtype == MB_BF16;
-    const int64_t fwd = mbscan::prefill_segments(p, bf16), bwd = mbscan::backward_segments(p);
+    const int64_t fwd = mbscan::prefill_segments(p, bf16), bwd = mbscan::backward_segments(p, bf16);
     const size_t split = mbscan::prefill_split_bytes(p, fwd > bwd ? fwd : bwd);
     const int64_t fs = fwd > 1 ? 0 : mbscan::prefill_shares(p, bf16);
-    const int64_t bs = bwd > 1 ? 0 : mbscan::backward_shares(p);
+    const int64_t bs = bwd > 1 ? 0 : mbscan::backward_shares(p, bf16);
     const size_t shares = mbscan::prefill_share_bytes(fs > bs ? fs : bs);
     return mbscan::kStatusBytes + (split > shares ? split : shares);
 }
@@ -455,7 +455,8 @@ mb_status mb_scan_backward(const mb_scan_args *args, const float *h_ckpt, const 
     }
     ScanParams p = to_params(args, nullptr, static_cast<StatusBlock *>(ws));
     // Split over L, or even shares, when the workspace holds the scratch and nothing that is read lies there.
-    const int64_t nseg = mbscan::backward_segments(p), shares = nseg > 1 ? 0 : mbscan::backward_shares(p);
+    const bool bf16 = args->dtype == MB_BF16;
+    const int64_t nseg = mbscan::backward_segments(p, bf16), shares = nseg > 1 ? 0 : mbscan::backward_shares(p, bf16);
     const size_t scratch = nseg > 1 ? mbscan::prefill_split_bytes(p, nseg) : mbscan::prefill_share_bytes(shares);
     if (scratch > 0 && ws_bytes >= mbscan::kStatusBytes + scratch) {
         char *base = static_cast<char *>(ws) + mbscan::kStatusBytes;
@@ -484,7 +485,7 @@ mb_status mb_scan_backward(const mb_scan_args *args, const float *h_ckpt, const 
     gp.dD = g.dD;
     gp.ddt_bias = g.ddt_bias;
     gp.dh0 = g.dh0;
-    return from_cuda(mbscan::launch_backward(p, gp, args->dtype == MB_BF16, (cudaStream_t)stream));
+    return from_cuda(mbscan::launch_backward(p, gp, bf16, (cudaStream_t)stream));
 }
 
 mb_status mb_rmsnorm(const void *add, float *residual, const float *w, float eps, void *out,
