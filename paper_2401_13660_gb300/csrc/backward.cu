@@ -649,10 +649,11 @@ __global__ void __launch_bounds__(kBThreads, kBResident<T>) backward_kernel(cons
 struct ClearArgs {
     float4 *p[6];
     int64_t n[6];   // float4s
+    int early;      // whether the next kernel may launch early
 };
 constexpr int kClearThreads = 256;
 __global__ void __launch_bounds__(kClearThreads) clear_kernel(const __grid_constant__ ClearArgs a) {
-    pdl_trigger();   // the next kernel may set up; it waits for this one before it adds anything
+    if (a.early) pdl_trigger();   // the next kernel may set up; it waits for this one before it adds anything
     pdl_wait();
     const int64_t step = (int64_t)gridDim.x * kClearThreads;
 #pragma unroll
@@ -704,9 +705,7 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
             cudaSuccess)
             return e;
         const int64_t grid = ctas * (nseg - 1);
-        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kBThreads), spread_smem(smem, grid, kBResident<T>), s, a1)) !=
-            cudaSuccess)
-            return e;
+        if ((e = launch_pdl(true, k1, dim3((unsigned)grid), dim3(kBThreads), smem, s, a1)) != cudaSuccess) return e;
     }
     a.grid_segs = (int)nseg;
     if (nseg == 1 && p.shares > 0) {
@@ -720,8 +719,7 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
     auto k = backward_kernel<T, false>;
     if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin)) != cudaSuccess)
         return e;
-    return launch_pdl(true, k, dim3((unsigned)(ctas * nseg)), dim3(kBThreads),
-                      spread_smem(smem, ctas * nseg, kBResident<T>), s, a);
+    return launch_pdl(true, k, dim3((unsigned)(ctas * nseg)), dim3(kBThreads), smem, s, a);
 }
 
 }  // namespace
@@ -797,6 +795,10 @@ cudaError_t launch_backward(const ScanParams &p, const GradParams &g, bool bf16,
         c.n[k] = num[k];
         if (num[k] > most) most = num[k];
     }
+    // A grid that is not spread and leaves room on the SMs is placed unevenly where it launches early (2 x 2048 x 2048
+    // 417 us, and 398).
+    const int64_t tiles = Bn * ((D + kBCh - 1) / kBCh), per = bf16 ? kBResident<__nv_bfloat16> : kBResident<float>;
+    c.early = p.shares > 0 || tiles * (p.nseg > 1 ? p.nseg - 1 : 1) > (per - 1) * (int64_t)device_sms();
     if (most > 0) {
         const int64_t want = (most + kClearThreads - 1) / kClearThreads, cap = 8 * (int64_t)device_sms();
         const int64_t grid = want < cap || cap == 0 ? want : cap;

@@ -533,23 +533,25 @@ cudaError_t launch_form(const ScanParams &p, const Segments &g, int64_t grid, co
         !make_map(&a.tm_C, p.C, es, p.batch, p.seqlen, kDState, kDState, p.bc_stride, 0, kRT<T, W>))
         return cudaErrorInvalidValue;
     const size_t smem = sizeof(Smem<T, W>) + 1024;
-    auto launch = [&](auto k) {
+    auto launch = [&](auto k, Placement at) {
         const cudaError_t e =
             cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin);
         if (e != cudaSuccess) return e;
-        return launch_pdl(true, k, dim3((unsigned)grid), dim3(kThreads), spread_smem(smem, grid, kCtas<W>), s, a);
+        return launch_pdl(at.overlap, k, dim3((unsigned)grid), dim3(kThreads), at.smem, s, a);
     };
     cudaError_t e;
     if (g.n > 1) {   // first pass: segments 0 .. n-2
-        if ((e = launch(first_pass_kernel<T, kCkpt, W>)) != cudaSuccess) return e;
+        if ((e = launch(first_pass_kernel<T, kCkpt, W>, {true, smem})) != cudaSuccess) return e;
         a.seg0 = 1;   // second pass: segments 1 .. n-1
-    } else if constexpr (W) {
+        return launch(forward_kernel<T, kCkpt, W>, {true, smem});
+    }
+    if constexpr (W) {
         if (p.shares > 0) {
             if ((e = cudaMemsetAsync(p.share_sync(), 0, prefill_share_sync_bytes(p.shares), s)) != cudaSuccess) return e;
-            return launch(forward_shares_kernel<T, kCkpt>);
+            return launch(forward_shares_kernel<T, kCkpt>, {true, spread_smem(smem, grid, kCtas<W>)});
         }
     }
-    return launch(forward_kernel<T, kCkpt, W>);
+    return launch(forward_kernel<T, kCkpt, W>, place_scan(p.seqlen, grid, kCtas<W>, smem));
 }
 
 template <typename T, bool kCkpt>

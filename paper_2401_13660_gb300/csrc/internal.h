@@ -75,11 +75,29 @@ struct DeviceLimits {
 const DeviceLimits *device_limits();
 int device_sms();   // 0 if there is no device
 // Dynamic shared memory to ask for, at least `smem`, so that a grid of less
-// than `per` CTAs per SM (the resident limit at `smem`) is spread evenly: left
-// to itself the block scheduler puts up to `per` of them on the SMs that are
-// free first and leaves others idle, above all when the launch overlaps the
-// tail of the kernel before.
+// than `per` CTAs per SM (the resident limit at `smem`) is spread evenly: a
+// launch that overlaps a kernel which lets it launch early puts up to `per` of
+// them on the SMs that have room first and leaves others idle. It also keeps
+// CTAs of other streams off those SMs.
 size_t spread_smem(size_t smem, int64_t grid, int per);
+// How to launch a scan of L steps in `grid` CTAs of one channel tile each, so
+// that it is fast both after a kernel that lets it launch early (a decode step, a
+// cuBLAS GEMM) and beside others on other streams. Grids of at least `per` CTAs
+// per SM need nothing. Microseconds after a decode step (both), and a round of
+// three streams, of 2 x 2048 x 2048 (128 CTAs, one per SM; bf16, 256 bytes of
+// workspace): overlapped 135, 126; overlapped and spread 96, 179; plain 97, 127.
+// 4 x 2048 x 2048 (256 CTAs, two per SM): 157, 218; 121, 245; 122, 218.
+//  * one per SM: plain, which outside a graph costs up to 2.7 us of a long scan;
+//  * two and more: overlapped and spread; others still have room beside it, and
+//    2.7 us would be much of the shorter ones among them;
+//  * under 256 steps: overlapped. Unevenly placed (1 x 128 x 4608 after a step
+//    27.3, spread 25.8) they lose less than a plain launch costs; three streams
+//    12 us a round, spread 17.
+struct Placement {
+    bool overlap;
+    size_t smem;
+};
+Placement place_scan(int64_t L, int64_t grid, int per, size_t smem);
 
 constexpr long long kMaxWaitCycles = 4000000000LL;   // the kernels' wait limit (~2 s at 2 GHz)
 

@@ -586,9 +586,10 @@ cudaError_t launch_typed(const ScanParams &p, cudaStream_t s) {
     if (!lim) return cudaErrorInvalidDevice;
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)lim->smem_optin);
     if (e != cudaSuccess) return e;
-    // verify: overlaps the tail of the kernel before it
-    const size_t ask = kStoreAll ? spread_smem(smem, ctas, kFuse ? MB_VERIFY_FUSED_MINB : MB_VERIFY_MINB) : smem;
-    return launch_pdl(kStoreAll, k, dim3((unsigned)ctas), dim3(kThreads), ask, s, a);
+    const Placement at = kStoreAll
+                             ? place_scan(p.seqlen, ctas, kFuse ? MB_VERIFY_FUSED_MINB : MB_VERIFY_MINB, smem)
+                             : Placement{false, smem};
+    return launch_pdl(at.overlap, k, dim3((unsigned)ctas), dim3(kThreads), at.smem, s, a);
 }
 
 }  // namespace

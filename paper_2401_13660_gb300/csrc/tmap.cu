@@ -92,4 +92,11 @@ size_t spread_smem(size_t smem, int64_t grid, int per) {
     return want > smem && want <= l->smem_optin ? want : smem;
 }
 
+Placement place_scan(int64_t L, int64_t grid, int per, size_t smem) {
+    const int64_t sms = device_sms();
+    if (L < 256 || grid > (per - 1) * sms) return {true, smem};
+    if (grid <= sms) return {false, smem};
+    return {true, spread_smem(smem, grid, per)};
+}
+
 }  // namespace mbscan
