@@ -116,10 +116,10 @@ typedef struct {
  * associative operator); when they fill it unevenly, they run in equal
  * shares that hand the state on where a share ends inside a channel's span.
  * Any workspace of at least 256 bytes is accepted: with a smaller one than
- * this such spans run as they are. The scratch needs no clearing. The caller
- * allocates it (256-byte aligned) and may reuse it across calls on one stream;
- * calls that overlap on the GPU need distinct workspaces. Returns 0 for
- * invalid arguments. */
+ * this, or one whose scratch overlaps an argument, such spans run as they are.
+ * The scratch needs no clearing. The caller allocates the workspace (256-byte
+ * aligned) and may reuse it across calls on one stream; calls that overlap on
+ * the GPU need distinct workspaces. Returns 0 for invalid arguments. */
 size_t mb_workspace_size(const mb_scan_args *args);
 
 /*

@@ -137,38 +137,41 @@ mb_status check_ws(const mb_scan_args *a, void *ws, size_t ws_bytes) {
     return MB_OK;
 }
 
-// Long spans with few channels are split over L, others run in even shares where
-// that is faster, when the workspace holds the scratch (after the status block);
-// else they run as one CTA per channel tile.
-mb_status setup_split(const mb_scan_args *args, ScanParams &p, const float *h_last, void *ws, size_t ws_bytes,
-                      Range ckpt = Range{}) {
-    const bool bf16 = args->dtype == MB_BF16;
-    const int64_t nseg = mbscan::prefill_segments(p, bf16), shares = nseg > 1 ? 0 : mbscan::prefill_shares(p, bf16);
+// Give the scan the workspace's scratch (after the status block) for a time
+// split into nseg segments or for even shares, if it holds as much and overlaps
+// none of the n ranges that the call reads or writes. Otherwise the span runs as
+// one CTA per channel tile, which needs none.
+void use_scratch(ScanParams &p, int64_t nseg, int64_t shares, void *ws, size_t ws_bytes, const Range *used, int n) {
     const size_t scratch = nseg > 1 ? mbscan::prefill_split_bytes(p, nseg) : mbscan::prefill_share_bytes(shares);
-    if (scratch == 0 || ws_bytes < mbscan::kStatusBytes + scratch) return MB_OK;
-    const int64_t es = bf16 ? 2 : 4;
-    const int64_t tok = args->batch * args->seqlen * args->d_inner * es;
-    const int64_t sbytes = args->batch * args->d_inner * args->d_state * 4;
+    if (scratch == 0 || ws_bytes < mbscan::kStatusBytes + scratch) return;
     char *base = static_cast<char *>(ws) + mbscan::kStatusBytes;
-    const Range rs = range_of(base, (int64_t)scratch);
-    const Range others[] = {range_of(args->x, tok), range_of(args->z, tok), range_of(args->dt, tok),
-                            range_of(args->y, tok), range_of(args->B, bc_bytes(args)),
-                            range_of(args->C, bc_bytes(args)), range_of(args->h0, sbytes), range_of(h_last, sbytes),
-                            range_of(args->A, args->d_inner * args->d_state * 4),
-                            range_of(args->D, args->d_inner * 4), range_of(args->dt_bias, args->d_inner * 4), ckpt};
-    bool clear = true;
-    for (const Range &r : others) clear = clear && !overlap(rs, r);
+    for (int i = 0; i < n; ++i)
+        if (overlap(range_of(base, (int64_t)scratch), used[i])) return;
     if (nseg > 1) {
-        if (!clear) return MB_ERR_INVALID_ARG;
         p.nseg = (int32_t)nseg;
         p.seg_h = reinterpret_cast<float *>(base);
         p.seg_p = p.seg_h + scratch / (2 * sizeof(float));
-    } else if (clear) {   // otherwise one CTA per tile, which needs no scratch
+    } else {
         p.shares = (int32_t)shares;
         p.seg_p = reinterpret_cast<float *>(base);
         p.seg_h = reinterpret_cast<float *>(base + mbscan::prefill_share_sync_bytes(shares));
     }
-    return MB_OK;
+}
+
+// Long spans with few channels are split over L, others run in even shares where
+// that is faster (h_ckpt never overlaps ws: mb_scan_prefill_ckpt refuses that).
+void plan_prefill(const mb_scan_args *args, ScanParams &p, const float *h_last, void *ws, size_t ws_bytes) {
+    const bool bf16 = args->dtype == MB_BF16;
+    const int64_t nseg = mbscan::prefill_segments(p, bf16), shares = nseg > 1 ? 0 : mbscan::prefill_shares(p, bf16);
+    const int64_t es = bf16 ? 2 : 4;
+    const int64_t tok = args->batch * args->seqlen * args->d_inner * es;
+    const int64_t sbytes = args->batch * args->d_inner * args->d_state * 4;
+    const Range used[] = {range_of(args->x, tok), range_of(args->z, tok), range_of(args->dt, tok),
+                          range_of(args->y, tok), range_of(args->B, bc_bytes(args)),
+                          range_of(args->C, bc_bytes(args)), range_of(args->h0, sbytes), range_of(h_last, sbytes),
+                          range_of(args->A, args->d_inner * args->d_state * 4),
+                          range_of(args->D, args->d_inner * 4), range_of(args->dt_bias, args->d_inner * 4)};
+    use_scratch(p, nseg, shares, ws, ws_bytes, used, sizeof(used) / sizeof(used[0]));
 }
 
 mb_status from_cuda(cudaError_t e) { return e == cudaSuccess ? MB_OK : MB_ERR_CUDA; }
@@ -221,7 +224,7 @@ mb_status mb_scan_prefill(const mb_scan_args *args, float *h_last, void *ws, siz
     if (args->batch * args->d_inner == 0) return MB_OK;
     ScanParams p = to_params(args, h_last, static_cast<StatusBlock *>(ws));
     const bool bf16 = args->dtype == MB_BF16;
-    if ((st = setup_split(args, p, h_last, ws, ws_bytes)) != MB_OK) return st;
+    plan_prefill(args, p, h_last, ws, ws_bytes);
     return from_cuda(mbscan::launch_prefill(p, bf16, (cudaStream_t)stream));
 }
 
@@ -408,7 +411,7 @@ mb_status mb_scan_prefill_ckpt(const mb_scan_args *args, float *h_last, float *h
         return MB_ERR_INVALID_ARG;
     ScanParams p = to_params(args, h_last, static_cast<StatusBlock *>(ws));
     p.h_ckpt = h_ckpt;
-    if ((st = setup_split(args, p, h_last, ws, ws_bytes, rc)) != MB_OK) return st;
+    plan_prefill(args, p, h_last, ws, ws_bytes);
     return from_cuda(mbscan::launch_prefill_ckpt(p, args->dtype == MB_BF16, (cudaStream_t)stream));
 }
 
@@ -454,24 +457,9 @@ mb_status mb_scan_backward(const mb_scan_args *args, const float *h_ckpt, const 
             if (overlap(outs[i], outs[j])) return MB_ERR_INVALID_ARG;
     }
     ScanParams p = to_params(args, nullptr, static_cast<StatusBlock *>(ws));
-    // Split over L, or even shares, when the workspace holds the scratch and nothing that is read lies there.
     const bool bf16 = args->dtype == MB_BF16;
     const int64_t nseg = mbscan::backward_segments(p, bf16), shares = nseg > 1 ? 0 : mbscan::backward_shares(p, bf16);
-    const size_t scratch = nseg > 1 ? mbscan::prefill_split_bytes(p, nseg) : mbscan::prefill_share_bytes(shares);
-    if (scratch > 0 && ws_bytes >= mbscan::kStatusBytes + scratch) {
-        char *base = static_cast<char *>(ws) + mbscan::kStatusBytes;
-        bool clear = true;
-        for (int i = 0; i < kIns - 1; ++i) clear = clear && !overlap(range_of(base, (int64_t)scratch), ins[i]);
-        if (clear && nseg > 1) {
-            p.nseg = (int32_t)nseg;
-            p.seg_h = reinterpret_cast<float *>(base);
-            p.seg_p = p.seg_h + scratch / (2 * sizeof(float));
-        } else if (clear) {
-            p.shares = (int32_t)shares;
-            p.seg_p = reinterpret_cast<float *>(base);
-            p.seg_h = reinterpret_cast<float *>(base + mbscan::prefill_share_sync_bytes(shares));
-        }
-    }
+    use_scratch(p, nseg, shares, ws, ws_bytes, ins, kIns - 1);   // the outputs do not overlap ws (checked above)
     mbscan::GradParams gp;
     gp.h_ckpt = h_ckpt;
     gp.dout = dout;
