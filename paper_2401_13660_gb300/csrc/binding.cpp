@@ -14,6 +14,8 @@
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/autograd/python_variable.h>
 
+#include <cstring>
+
 #include "mbscan.h"
 
 namespace {
@@ -372,7 +374,7 @@ PyObject *init(ARGS) {
         if (PyErr_Occurred()) return nullptr;
     }
     static_assert(sizeof(p) == sizeof(api), "one address per entry point");
-    memcpy(&api, p, sizeof(api));
+    std::memcpy(&api, p, sizeof(api));
     Py_RETURN_NONE;
 }
 

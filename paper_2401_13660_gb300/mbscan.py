@@ -2,7 +2,8 @@
 
 Calls on plain, well-formed tensors are marshalled natively (csrc/binding.cpp:
 the same checks on the tensors' C++ objects; one mb_step call of one stream 22 -> 3.6 us);
-everything else, errors first of all, takes the Python path below it.
+everything else, errors first of all, takes the Python path below it, as does
+every call where that module is missing or does not load.
 
 Each function has the name of the C entry point it calls (include/mbscan.h)
 and takes torch CUDA tensors in place of device pointers. Every step of the
@@ -18,6 +19,7 @@ import importlib.machinery
 import importlib.util
 import os
 import threading
+import warnings
 
 import torch
 
@@ -64,6 +66,26 @@ class mb_scan_grads(ctypes.Structure):
 MB_CKPT_STEPS = 16
 
 
+class _Declined:
+    """Stands in for the native marshalling where it cannot be had: every call takes the Python path."""
+
+    def __getattr__(self, name):
+        return lambda *a: -1
+
+
+def _load_binding(lib):
+    try:
+        loader = importlib.machinery.ExtensionFileLoader("_mbcall", _build.BINDING)
+        fast = importlib.util.module_from_spec(importlib.util.spec_from_file_location(
+            "_mbcall", _build.BINDING, loader=loader))
+        loader.exec_module(fast)
+        fast.init(*(ctypes.cast(getattr(lib, f), ctypes.c_void_p).value for f in _FAST))
+        return fast
+    except ImportError as e:
+        warnings.warn(f"native argument marshalling not loaded, calls are marshalled in Python: {e}")
+        return _Declined()
+
+
 def library_path() -> str:
     return _build.LIB
 
@@ -107,14 +129,7 @@ def load_library(build_if_needed: bool = True) -> ctypes.CDLL:
             lib.mb_status_string.restype = ctypes.c_char_p
             lib.mb_version.argtypes = []
             lib.mb_version.restype = ctypes.c_char_p
-            if not os.path.exists(_build.BINDING):
-                raise RuntimeError(f"{_build.BINDING} not found; run build() first")
-            loader = importlib.machinery.ExtensionFileLoader("_mbcall", _build.BINDING)
-            fast = importlib.util.module_from_spec(importlib.util.spec_from_file_location(
-                "_mbcall", _build.BINDING, loader=loader))
-            loader.exec_module(fast)
-            fast.init(*(ctypes.cast(getattr(lib, f), ctypes.c_void_p).value for f in _FAST))
-            _fast = fast
+            _fast = _load_binding(lib)
             _lib = lib
     return _lib
 
