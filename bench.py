@@ -230,6 +230,13 @@ def traffic_from_profiles(kernel_key):
     return None
 
 
+def kernel_name(group, prefill_ws_bytes):
+    """The kernel (csrc/) that a group of the step launches. The prefill runs in even shares where the library asked
+    for scratch beyond the 256-byte status block on this GPU, else as one CTA per channel tile."""
+    prefill = "forward_shares_kernel" if prefill_ws_bytes > 256 else "forward_kernel"
+    return {"prefill": prefill, "verify": "prefill_kernel", "rollback": "rollback_kernel", "step": "step_kernel"}[group]
+
+
 def reduce_max(value, dist, device="cpu"):
     """Max of a float over all ranks (the slowest rank sets the job time)."""
     if not dist:
@@ -451,8 +458,7 @@ def gpu_arm(args, rank, world, dist):
     dom_launch_ms = tot[dom] / (K * launches[dom])
     dom_bytes = parts[dom] / launches[dom]
     achieved = dom_bytes / (dom_launch_ms * 1e-3) / 1e9
-    kernel_key = {"prefill": "forward_kernel", "verify": "verify_kernel",
-                  "rollback": "rollback_kernel", "step": "step_kernel"}[dom]
+    kernel_key = kernel_name(dom, P["ws"].numel())
     roofline = {"kernel": kernel_key, "bound": "hbm", "achieved": round(achieved, 1),
                 "peak": peak, "peak_kind": f"{peak_kind} (hbm_gbs)", "unit": "GB/s",
                 "frac": round(achieved / peak, 4), "traffic": traffic_from_profiles(kernel_key),
