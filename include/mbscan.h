@@ -129,7 +129,7 @@ size_t mb_workspace_size(const mb_scan_args *args);
  * h_last[batch, d_inner, d_state] fp32 (the state MambaByte caches to resume
  * generation). h_last may alias h0.
  *   ws, ws_bytes : workspace of at least 256 bytes (mb_workspace_size(args)
- *                  for the split of long few-channel spans); its status block
+ *                  for the spans that run faster with scratch); its status block
  *                  (first 256 bytes) must start zeroed once after allocation
  *                  and is left zeroed by every successful call.
  */

@@ -730,7 +730,7 @@ cudaError_t launch_backward_typed(const ScanParams &p, const GradParams &g, cuda
 // states come from the checkpoints), so the first pass is short: decays and
 // dy C, no sums over channels or states. Every lane folds the segments after
 // its own; beyond sqrt(2 L) segments that costs more than shorter segments
-// give. Measured: 2 x 777 x 1544 (98 CTAs) 156 us unsplit, 66 in 5 segments;
+// give. Measured: 2 x 777 x 1544 (98 CTAs) 156 us unsplit, 62 in 6 segments;
 // 1 x 8192 x 64 1537 us unsplit, 53 in 128, 84 in 256; with the slots nearly
 // filled (8 x 8192 x 2048: 512 CTAs) 2.63 ms unsplit, 2.90 ms in 6. fp32, spans
 // of 2048 steps, tiles per SM 0.5, 1, 1.2, 1.6, 2: 141, 254, 353, 446, 448 us (cut

@@ -79,12 +79,13 @@ __device__ __forceinline__ float2 gld2(const float *p) { return *reinterpret_cas
 // next kernel launch before this one completes (it still waits for it). It is
 // issued early by kernels that leave room for the next one's CTAs (the
 // persistent decode step, the single-wave convolution + x-projection and its
-// reduction, the RMS norm, accept, the clearing of gradients), late by verify
+// reduction, the RMS norm, accept, the clearing of gradients before a grid that
+// fills the SMs), late by verify
 // and the first pass of split spans, and by no other grid of many short-lived
 // CTAs: such a grid that triggers early lets the next one's CTAs take SM slots
 // as they free up, which leaves SMs unevenly loaded when that grid fills less
 // than every slot (measured: back-to-back prefills of 448 CTAs, 822 -> 990 us;
-// spread_smem keeps the scans even when another library's kernel does so).
+// place_scan, internal.h: what the scans do where another kernel does so).
 #ifndef MB_PDL
 #define MB_PDL 1
 #endif

@@ -6,9 +6,9 @@
 // Work decomposition. Every (batch row, channel) is an independent recurrence
 // over L with a 16-float state (A is diagonal). A CTA of four warps owns 32
 // channels of one batch row for its span of L; a warp 8 channels, four lanes
-// per channel, each with 4 states in registers. Chunks of 16 steps come through
-// a ring of TMA tiles (bounded waits); iteration i scans chunk i and converts
-// chunk i + 1.
+// per channel, each with 4 states in registers. Stages of one to four chunks of
+// 16 steps (kSub) come through a ring of TMA tiles (bounded waits); while a chunk
+// is scanned the next one, of the same stage or the next, is converted.
 //
 // What bounds it: per (step, channel) 16 decays on the SFU and 64 multiply-adds,
 // which leave the SM at about 0.6 instructions per scheduler and clock, because
@@ -22,7 +22,7 @@
 //    16-byte slot, B and C are widened to fp32 in pairs (t, t + 1), so decay
 //    exponents, B Delta x and the sum C.h need no copies that duplicate a
 //    scalar and no add across a pair; only the recurrence itself is scalar.
-//    (Pairs of states: 35.3 instructions per lane and step; this: 29.6, 27.3 with 32-step stages.)
+//    (Pairs of states: 35.3 instructions per lane and step; this: 29.6, 27.3 with 32-step stages, 27.0 with 64.)
 //  * A 128-bit shared load takes 2 wavefronts instead of 4 if lanes that differ
 //    in lane bit 0 (or in bit 1) read the same address. Lane bit 0 is a channel
 //    bit and bit 1 a state bit (channel bits 0, 2, 3; state bits 1, 4), so that
@@ -501,7 +501,8 @@ bool make_map(CUtensorMap *m, const void *base, int es, int64_t batch, int64_t L
 }
 
 // Split of a span into at most nseg segments, in whole chunks. The first
-// is scanned for good while the others are summarised, which takes kFirst of its time per step, and is that much shorter.
+// is scanned for good while the others are summarised, which takes kFirst of its time per step, and is that much shorter
+// (0.55 to 0.85 make no difference, bf16 1 x 8192 x 2048 and fp32 3 x 1003 x 1544).
 constexpr double kFirst = 0.7;
 struct Segments {
     int64_t n, len0, len;   // n <= nseg

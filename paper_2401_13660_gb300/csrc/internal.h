@@ -116,7 +116,7 @@ int64_t backward_segments(const ScanParams &p, bool bf16);
 size_t prefill_split_bytes(const ScanParams &p, int64_t nseg);
 // Shares a prefill that is not split is cut into when the workspace has room
 // (0: one CTA per channel tile), and the scratch they need: share_sync (first,
-// prefill_share_sync_bytes) and share_h.
+// prefill_share_sync_bytes) and seg_h.
 int64_t prefill_shares(const ScanParams &p, bool bf16);
 int64_t backward_shares(const ScanParams &p, bool bf16);   // the same for the backward, with the same scratch
 size_t prefill_share_sync_bytes(int64_t shares);

@@ -1,6 +1,8 @@
-// C ABI of the selective-scan layer core: host-side validation, then one
-// kernel launch per call on the caller's stream. Declarations and the
-// contract of every entry point are in include/mbscan.h.
+// C ABI of the selective-scan layer core: host-side validation, the plan of a
+// scan (time split, even shares), then its launches on the caller's stream: one
+// kernel, or two (split spans, mb_conv_xproj), with the clearing of flags or sums
+// before shares and the backward. Declarations and the contract of every entry
+// point are in include/mbscan.h.
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <string.h>

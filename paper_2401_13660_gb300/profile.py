@@ -57,6 +57,7 @@ def main():
                          "decoder.CONFIGS name")
     ap.add_argument("--batch", type=int, default=256, help="streams of --entry decode_model / conv_xproj")
     ap.add_argument("--iters", type=int, default=5)
+    ap.add_argument("--plain", action="store_true", help="a 256-byte workspace: no time split, no even shares")
     ap.add_argument("--layers", type=int, default=4, help="state sets cycled by --entry step / conv_xproj")
     a = ap.parse_args()
     dev = torch.device("cuda:0")
@@ -72,7 +73,9 @@ def main():
         inp = workload_inputs(w, dev, layer=layer)
         x = inp["x"]
         inp["y"] = torch.empty_like(x)
-        inp["ws"] = torch.zeros(256, dtype=torch.uint8, device=dev)
+        args = mb.make_args(x, inp.get("dt"), inp["B"], inp["C"], inp["A"], inp["y"], z=inp.get("z"), h0=inp["h0"],
+                            dt_low=inp.get("dt_low"), W_dt=inp.get("W_dt"))
+        inp["ws"] = torch.zeros(256, dtype=torch.uint8, device=dev) if a.plain else mb.new_workspace(args, dev)
         if inp["h0"] is None and a.entry in ("verify", "rollback", "step"):
             inp["h0"] = torch.zeros(w.batch, w.d_inner, N_STATE, device=dev)
         if a.entry in ("prefill", "backward"):
